@@ -202,28 +202,48 @@ __device__ __forceinline__ void tile_nt_run(const T* __restrict__ A, long long l
     for (int j = 0; j < 4; ++j) acc64[i][j] += (double)acc[i][j];
 }
 
-// G = Cs Cs^T (full K), written (not accumulated) into g[m][n]: tiles on
-// and above the diagonal are computed and also stored transposed, so G is
-// exactly symmetric (inside a diagonal tile both halves use the same k order
-// and commutative products).
-__global__ void k_syrk64(const double* __restrict__ cs, int nao, int K, double* __restrict__ g) {
-  __shared__ double As[16][65];
-  __shared__ double Bs[16][65];
+// G = Cs Cs^T for the occupied (blockIdx.z = 0) and virtual (1) orbitals:
+// tiles on and above the diagonal are computed and also stored transposed, so
+// G is exactly symmetric (inside a diagonal tile both halves use the same k
+// order and commutative products).  16 x 16 tiles of 64 threads: two FMAs per
+// cycle and SM is all there is, so a small G must spread over every SM (124
+// functions: 72 CTAs of 6 us, where 64 x 64 tiles took 80 us on three SMs).
+__global__ void __launch_bounds__(64) k_syrk64(const double* __restrict__ cso, const double* __restrict__ csv,
+                                               int nao, int n_occ, double* __restrict__ go,
+                                               double* __restrict__ gv) {
   if (blockIdx.x < blockIdx.y) return;
-  int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  double acc[4][4] = {};
-  if (K > 0)
-    tile_nt_run<double, double>(cs + (long long)m0 * K, K, min(64, nao - m0), cs + (long long)n0 * K,
-                                K, min(64, nao - n0), 0, K, As, Bs, acc);
-  int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const double* cs = blockIdx.z ? csv : cso;
+  double* g = blockIdx.z ? gv : go;
+  const int K = blockIdx.z ? nao - n_occ : n_occ;
+  __shared__ double As[16][33], Bs[16][33];
+  const int m0 = blockIdx.y * 16, n0 = blockIdx.x * 16;
+  const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+  double acc[2][2] = {};
+  for (int k0 = 0; k0 < K; k0 += 32) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+    for (int e = 0; e < 8; ++e) {
+      const int row = (threadIdx.x >> 5) + 2 * e, kk = threadIdx.x & 31;
+      const bool kin = k0 + kk < K;
+      As[row][kk] = (kin && m0 + row < nao) ? cs[static_cast<long long>(m0 + row) * K + k0 + kk] : 0.0;
+      Bs[row][kk] = (kin && n0 + row < nao) ? cs[static_cast<long long>(n0 + row) * K + k0 + kk] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int kk = 0; kk < 32; ++kk)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int m = m0 + ty + 16 * i, n = n0 + tx + 16 * j;
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) acc[i][j] = fma(As[ty + 8 * i][kk], Bs[tx + 8 * j][kk], acc[i][j]);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int m = m0 + ty + 8 * i, n = n0 + tx + 8 * j;
       if (m < nao && n < nao) {
-        g[(long long)m * nao + n] = acc[i][j];
-        if (m0 != n0) g[(long long)n * nao + m] = acc[i][j];
+        g[static_cast<long long>(m) * nao + n] = acc[i][j];
+        if (m0 != n0) g[static_cast<long long>(n) * nao + m] = acc[i][j];
       }
     }
 }
@@ -507,13 +527,17 @@ void launch_cast_f64_f32(const double* x, float* y, long long n, cudaStream_t st
   k_cast_f64_f32<<<(unsigned)blocks, 256, 0, st>>>(x, y, n);
 }
 
+void launch_scale_orbitals(const double* C, const double* eps, int nao, int n_occ, double mu, double tau,
+                           double* cso, double* csv, cudaStream_t st) {
+  const long long n = (long long)nao * nao;
+  k_scale_orbitals<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(C, eps, nao, n_occ, mu, tau, cso, csv);
+}
+
 void launch_greens(const double* C, const double* eps, int nao, int n_occ, double mu, double tau,
                    double* cso, double* csv, double* g_occ, double* g_virt, cudaStream_t st) {
-  long long n = (long long)nao * nao;
-  k_scale_orbitals<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(C, eps, nao, n_occ, mu, tau, cso, csv);
-  dim3 grid((nao + 63) / 64, (nao + 63) / 64);
-  k_syrk64<<<grid, 256, 0, st>>>(cso, nao, n_occ, g_occ);
-  k_syrk64<<<grid, 256, 0, st>>>(csv, nao, nao - n_occ, g_virt);
+  launch_scale_orbitals(C, eps, nao, n_occ, mu, tau, cso, csv, st);
+  const unsigned t = (nao + 15) / 16;
+  k_syrk64<<<dim3(t, t, 2), 64, 0, st>>>(cso, csv, nao, n_occ, g_occ, g_virt);
 }
 
 void launch_sym_block_filter(double* g, int nao, const int* ao_off, int n_at, double thr,

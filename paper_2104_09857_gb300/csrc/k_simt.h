@@ -17,6 +17,8 @@ void launch_panel_scatter(const double* t3, const int* blk, const long long* off
                           const long long* dstB, const long long* dstA, const int* ldB,
                           const int* ldA, double* pool, cudaStream_t st);
 void launch_cast_f64_f32(const double* x, float* y, long long n, cudaStream_t st);
+void launch_scale_orbitals(const double* C, const double* eps, int nao, int n_occ, double mu, double tau,
+                           double* cso, double* csv, cudaStream_t st);
 void launch_greens(const double* C, const double* eps, int nao, int n_occ, double mu, double tau,
                    double* cso, double* csv, double* g_occ, double* g_virt, cudaStream_t st);
 void launch_sym_block_filter(double* g, int nao, const int* ao_off, int n_at, double thr,
