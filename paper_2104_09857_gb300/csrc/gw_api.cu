@@ -22,6 +22,7 @@
 #include "gw_internal.h"
 #include "k_simt.h"
 #include "k_tc.h"
+#include "k_emu.h"
 #include "k_mlp.h"
 
 using gw::Batch;
@@ -1708,6 +1709,23 @@ int tc_finish_tau(gw_ctx* ctx, std::vector<double>& fc_host) {
 
 namespace gw {
 int build_panels_for(gw_ctx* ctx, double thr) { return build_panels(ctx, thr); }
+int work_buffer(gw_ctx* ctx, const char* name, size_t bytes, void** out) { return ws(ctx, name, bytes, out); }
+void work_trim(gw_ctx* ctx, const char* prefix, size_t keep) {
+  const size_t n = std::strlen(prefix);
+  size_t held = 0;
+  for (const auto& kv : ctx->work)
+    if (kv.first.compare(0, n, prefix) == 0) held += kv.second.second;
+  if (held <= keep) return;
+  cudaStreamSynchronize(ctx->stream);
+  for (auto it = ctx->work.begin(); it != ctx->work.end();) {
+    if (it->first.compare(0, n, prefix) == 0) {
+      cudaFree(it->second.first);
+      it = ctx->work.erase(it);
+    } else {
+      ++it;
+    }
+  }
+}
 }  // namespace gw
 
 // ===========================================================================
@@ -2139,6 +2157,7 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
     if ((rc = wsT(ctx, "g_virt32", (size_t)nao * nao, &gv32))) return rc;
   }
 
+  if ((rc = gw::emu_begin(ctx, ctx->stream))) return rc;
   gw::ScopedEvents<3> ev;
   GW_TRY(ev.create());
   double ms_g = 0, ms_c = 0;
@@ -2146,8 +2165,7 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
     gw::TraceRange trace_tau("chi: one tau point");
     GW_TRY(cudaEventRecord(ev[0], ctx->stream));
     ctx->cur_tau = ctx->tau[j];
-    gw::launch_greens(ctx->d_C, ctx->d_eps, nao, ctx->n_occ, ctx->mu, ctx->tau[j], cso, csv, go, gv,
-                      ctx->stream);
+    if ((rc = gw::greens_fp64(ctx, ctx->tau[j], cso, csv, go, gv, ctx->stream))) return rc;
     GW_CHECK_LAUNCH();
     ctx->stats.kernel_launches += 3;
     if (f16) {
@@ -2241,6 +2259,7 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
     ctx->stats.flops_b += fb;
     ctx->stats.flops_c += fcs;
   }
+  if (tau_count > 0 && (rc = gw::emu_end(ctx, "gw_chi_tau"))) return rc;
   ctx->stats.flops_useful = ctx->stats.flops_a + ctx->stats.flops_b + ctx->stats.flops_c;
   ctx->stats.tasks_seen = ctx->mlp_seen;
   ctx->stats.tasks_skipped = ctx->mlp_skipped;

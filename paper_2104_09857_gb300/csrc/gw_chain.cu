@@ -8,6 +8,7 @@
 
 #include "gw_internal.h"
 #include "k_chain.h"
+#include "k_emu.h"
 
 namespace {
 
@@ -26,6 +27,23 @@ struct DevBuf {
       return e_ == cudaErrorMemoryAllocation ? GW_ERR_OOM : GW_ERR_CUDA;          \
     }                                                                             \
   } while (0)
+
+// count doubles (or as many bytes of another type) of a named work buffer
+template <typename T>
+int chain_buffer(gw_ctx* ctx, const char* name, size_t count, T** out) {
+  void* p = nullptr;
+  const int rc = gw::work_buffer(ctx, name, count * 8, &p);
+  *out = static_cast<T*>(p);
+  return rc;
+}
+
+// g.C = Q Q^T from one set of digits where they are whole
+int square(gw_ctx* ctx, const gw::EmuSrc& q, const gw::EmuGemm& g, cudaStream_t st) {
+  if (gw::emu_dig_bytes(q.rows, q.K) > (size_t(4) << 30)) return gw::emu_product(ctx, q, q, g, nullptr, st);
+  gw::EmuOp op;
+  const int rc = gw::emu_prep(ctx, "a", q, &op, st);
+  return rc ? rc : gw::emu_mm(ctx, op, op, g, st);
+}
 
 }  // namespace
 
@@ -57,26 +75,20 @@ extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const doub
     }
   CH_TRY(cudaSetDevice(ctx->device));
   cudaStream_t st = ctx->stream;
+  gw::WorkTrim trim{ctx};
   const size_t nn = (size_t)n * n;
-  DevBuf b_low, b_chi, b_w, b_cw, b_t1, b_eps, b_z, b_ww, b_g, b_d, b_err;
-  CH_TRY(cudaMalloc(&b_low.p, nn * 8));
-  CH_TRY(cudaMalloc(&b_cw.p, nn * 8));
-  CH_TRY(cudaMalloc(&b_t1.p, nn * 8));
-  CH_TRY(cudaMalloc(&b_eps.p, nn * 8));
-  CH_TRY(cudaMalloc(&b_z.p, nn * 8));
-  CH_TRY(cudaMalloc(&b_ww.p, nn * 8));
-  CH_TRY(cudaMalloc(&b_g.p, (size_t)n_omega * n_tau * 8));
-  CH_TRY(cudaMalloc(&b_d.p, (size_t)n_omega * n_tau * 8));
-  CH_TRY(cudaMalloc(&b_err.p, sizeof(int)));
-  double* low = (double*)b_low.p;
-  double* cw = (double*)b_cw.p;
-  double* t1 = (double*)b_t1.p;
-  double* eps = (double*)b_eps.p;
-  double* z = (double*)b_z.p;
-  double* ww = (double*)b_ww.p;
-  double* g = (double*)b_g.p;
-  double* d = (double*)b_d.p;
-  int* err = (int*)b_err.p;
+  DevBuf b_chi, b_w;
+  // V, its factor L, [eps; L] and one product share the context's work buffers
+  double *v, *low, *m, *t, *ww, *g, *d;
+  int* err;
+  int rc;
+  if ((rc = chain_buffer(ctx, "w.v", nn, &v)) || (rc = chain_buffer(ctx, "w.low", nn, &low)) ||
+      (rc = chain_buffer(ctx, "w.eps_l", 2 * nn, &m)) || (rc = chain_buffer(ctx, "w.t", nn, &t)) ||
+      (rc = chain_buffer(ctx, "w.ww", nn, &ww)) ||
+      (rc = chain_buffer(ctx, "w.gamma", (size_t)n_omega * n_tau, &g)) ||
+      (rc = chain_buffer(ctx, "w.delta", (size_t)n_omega * n_tau, &d)) ||
+      (rc = chain_buffer(ctx, "w.not_spd", 1, &err)) || (rc = gw::emu_begin(ctx, st)))
+    return rc;
   const double* chi;
   if (chi_on_device) {
     chi = chi_tau;
@@ -94,12 +106,12 @@ extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const doub
   }
   CH_TRY(cudaMemsetAsync(wout, 0, (size_t)n_tau * nn * 8, st));
   CH_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
-  CH_TRY(cudaMemcpyAsync(low, V, nn * 8, cudaMemcpyHostToDevice, st));
+  CH_TRY(cudaMemcpyAsync(v, V, nn * 8, cudaMemcpyHostToDevice, st));
   CH_TRY(cudaMemcpyAsync(g, gamma, (size_t)n_omega * n_tau * 8, cudaMemcpyHostToDevice, st));
   CH_TRY(cudaMemcpyAsync(d, delta, (size_t)n_omega * n_tau * 8, cudaMemcpyHostToDevice, st));
   // V = L L^T (Eq. 8)
-  gw::chain_potrf(low, n, err, st);
-  CH_TRY(cudaGetLastError());
+  CH_TRY(cudaMemcpyAsync(low, v, nn * 8, cudaMemcpyDeviceToDevice, st));
+  if ((rc = gw::chain_cholesky(ctx, low, n, n, err, st))) return rc;
   int h_err = 0;
   CH_TRY(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CH_TRY(cudaStreamSynchronize(st));
@@ -107,27 +119,49 @@ extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const doub
     ctx->err = "gw_chi_to_w: the Coulomb matrix is not positive definite";
     return GW_ERR_NOT_SPD;
   }
+  gw::EmuSrc s_lt, s_row;  // L^T, and a matrix by its rows
+  s_lt.src = low;
+  s_lt.ld = s_row.ld = n;
+  s_lt.rows = s_row.rows = n;
+  s_lt.K = s_row.K = n;
+  s_lt.trans = true;
+  gw::EmuOp lt;  // digits of L^T, made once
   for (int k = 0; k < n_omega; ++k) {
     // chi(i omega_k) = sum_j gamma_kj chi(i tau_j)
-    gw::chain_lincomb(chi, n_tau, g + (size_t)k * n_tau, 1, (long long)nn, cw, st);
-    // eps = 1 - L^T (chi L)     (Eq. 7)
-    gw::chain_dgemm(false, false, n, n, n, 1.0, cw, n, low, n, 0.0, t1, n, st);
-    gw::chain_set_identity(eps, n, st);
-    gw::chain_dgemm(true, false, n, n, n, -1.0, low, n, t1, n, 1.0, eps, n, st);
-    // eps = R R^T; Z = R^-1 L^T; W^c = Z^T Z - V   (Eq. 9)
-    gw::chain_potrf(eps, n, err, st);
-    gw::chain_transpose(low, z, n, st);
-    gw::chain_trsm_left_lower(eps, n, z, n, st);
-    gw::chain_dgemm(false, true, n, n, n, 1.0, low, n, low, n, 0.0, ww, n, st);  // V = L L^T
-    gw::chain_dgemm(true, false, n, n, n, 1.0, z, n, z, n, -1.0, ww, n, st);
+    gw::chain_lincomb(chi, n_tau, g + (size_t)k * n_tau, (long long)nn, t, st);
+    // (chi L)^T = L^T chi^T by rows, then eps = 1 - L^T (chi L)  (Eq. 7), its
+    // lower triangle; row r of L^T starts at column r
+    gw::EmuGemm p;
+    p.C = ww;
+    p.ldc = n;
+    p.ktri = 1;
+    s_row.src = t;
+    if ((rc = gw::emu_product(ctx, s_lt, s_row, p, &lt, st))) return rc;
+    p.alpha = -1.0;
+    p.C = m;
+    p.tri = 1;
+    s_row.src = ww;
+    if ((rc = gw::emu_product(ctx, s_lt, s_row, p, &lt, st))) return rc;
+    gw::chain_add_diagonal(m, n, 1.0, st);
+    // eps = R R^T with L below it: its rows become L R^-T = Z, and
+    // W^c = Z Z^T - V  (Eq. 9), lower triangle
+    CH_TRY(cudaMemcpyAsync(m + nn, low, nn * 8, cudaMemcpyDeviceToDevice, st));
+    if ((rc = gw::chain_cholesky(ctx, m, 2LL * n, n, err, st))) return rc;
+    gw::EmuGemm q;
+    q.C = ww;
+    q.ldc = n;
+    q.tri = 1;
+    s_row.src = m + nn;
+    if ((rc = square(ctx, s_row, q, st))) return rc;
     // W^c(i tau_j) += delta_jk W^c(i omega_k)
-    gw::chain_axpy_multi(ww, d, n_omega, k, n_tau, (long long)nn, wout, st);
+    gw::chain_add_symmetric(ww, v, d + k, n_omega, n_tau, n, wout, st);
     CH_TRY(cudaGetLastError());
   }
   CH_TRY(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));
   if (!out_on_device)
     CH_TRY(cudaMemcpyAsync(w_tau_out, wout, (size_t)n_tau * nn * 8, cudaMemcpyDeviceToHost, st));
   CH_TRY(cudaStreamSynchronize(st));
+  if ((rc = gw::emu_end(ctx, "gw_chi_to_w"))) return rc;
   if (h_err) {
     ctx->err = "gw_chi_to_w: eps(i omega) is not positive definite (chi must be negative semidefinite)";
     return GW_ERR_NOT_SPD;
@@ -160,14 +194,15 @@ extern "C" int gw_ri_metric(gw_ctx* ctx, const double* S, int n_mat, const doubl
     }
   CH_TRY(cudaSetDevice(ctx->device));
   cudaStream_t st = ctx->stream;
-  DevBuf b_r, b_ri, b_si, b_t, b_m, b_o, b_err;
-  CH_TRY(cudaMalloc(&b_r.p, nn * 8));
-  CH_TRY(cudaMalloc(&b_ri.p, nn * 8));
-  CH_TRY(cudaMalloc(&b_si.p, nn * 8));
-  CH_TRY(cudaMalloc(&b_t.p, nn * 8));
-  CH_TRY(cudaMalloc(&b_err.p, sizeof(int)));
-  double *r = (double*)b_r.p, *ri = (double*)b_ri.p, *si = (double*)b_si.p, *t = (double*)b_t.p;
-  int* err = (int*)b_err.p;
+  gw::WorkTrim trim{ctx};
+  DevBuf b_m, b_o;
+  double *r, *si, *t;
+  int* err;
+  int rc;
+  if ((rc = chain_buffer(ctx, "w.eps_l", 2 * nn, &r)) || (rc = chain_buffer(ctx, "w.low", nn, &si)) ||
+      (rc = chain_buffer(ctx, "w.t", nn, &t)) || (rc = chain_buffer(ctx, "w.not_spd", 1, &err)) ||
+      (rc = gw::emu_begin(ctx, st)))
+    return rc;
   const double* m = M;
   if (!m_on_device) {
     CH_TRY(cudaMalloc(&b_m.p, (size_t)n_mat * nn * 8));
@@ -181,8 +216,9 @@ extern "C" int gw_ri_metric(gw_ctx* ctx, const double* S, int n_mat, const doubl
   }
   CH_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
   CH_TRY(cudaMemcpyAsync(r, S, nn * 8, cudaMemcpyHostToDevice, st));
-  gw::chain_potrf(r, n, err, st);
-  CH_TRY(cudaGetLastError());
+  // [S; 1] -> [R; R^-T]
+  gw::chain_set_identity(r + nn, n, st);
+  if ((rc = gw::chain_cholesky(ctx, r, 2LL * n, n, err, st))) return rc;
   int h_err = 0;
   CH_TRY(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CH_TRY(cudaStreamSynchronize(st));
@@ -190,16 +226,35 @@ extern "C" int gw_ri_metric(gw_ctx* ctx, const double* S, int n_mat, const doubl
     ctx->err = "gw_ri_metric: the metric is not positive definite";
     return GW_ERR_NOT_SPD;
   }
-  gw::chain_set_identity(ri, n, st);
-  gw::chain_trsm_left_lower(r, n, ri, n, st);                                 // R^-1
-  gw::chain_dgemm(true, false, n, n, n, 1.0, ri, n, ri, n, 0.0, si, n, st);  // S^-1 = R^-T R^-1
+  gw::EmuSrc s_q, s_si, s_m;
+  s_q.src = r + nn;
+  s_q.ld = s_si.ld = s_m.ld = n;
+  s_q.rows = s_si.rows = s_m.rows = n;
+  s_q.K = s_si.K = s_m.K = n;
+  s_si.src = si;
+  // S^-1 = R^-T R^-1; row r of R^-T starts at column r
+  gw::EmuGemm p;
+  p.C = si;
+  p.ldc = n;
+  p.ktri = 1;
+  if ((rc = square(ctx, s_q, p, st))) return rc;
+  gw::EmuOp keep;
   for (int k = 0; k < n_mat; ++k) {
-    gw::chain_dgemm(false, false, n, n, n, 1.0, si, n, m + (size_t)k * nn, n, 0.0, t, n, st);
-    gw::chain_dgemm(false, false, n, n, n, 1.0, t, n, si, n, 0.0, o + (size_t)k * nn, n, st);
+    // t = S^-1 M, then t S^-1 (S^-1 symmetric: its rows are its columns)
+    gw::EmuGemm q;
+    q.C = t;
+    q.ldc = n;
+    s_m.src = m + (size_t)k * nn;
+    s_m.trans = true;  // columns of M
+    if ((rc = gw::emu_product(ctx, s_si, s_m, q, &keep, st))) return rc;
+    q.C = o + (size_t)k * nn;
+    gw::EmuSrc s_t = s_si;
+    s_t.src = t;
+    if ((rc = gw::emu_product(ctx, s_t, s_si, q, nullptr, st))) return rc;
   }
   CH_TRY(cudaGetLastError());
   if (!out_on_device)
     CH_TRY(cudaMemcpyAsync(out, o, (size_t)n_mat * nn * 8, cudaMemcpyDeviceToHost, st));
   CH_TRY(cudaStreamSynchronize(st));
-  return GW_OK;
+  return gw::emu_end(ctx, "gw_ri_metric");
 }

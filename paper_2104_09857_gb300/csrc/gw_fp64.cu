@@ -1,0 +1,155 @@
+// FP64 products of a context: operands and workspaces of the digit engine
+// (k_emu.cu) on the context's named work buffers.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <string>
+
+#include "gw_internal.h"
+#include "k_emu.h"
+#include "k_simt.h"
+
+namespace gw {
+
+namespace {
+// digits of one operand held at a time by emu_product
+constexpr size_t kMaxDigits = size_t(4) << 30;
+
+int flag(gw_ctx* ctx, int** out) {
+  void* p;
+  const int rc = work_buffer(ctx, "w.err", sizeof(int), &p);
+  *out = static_cast<int*>(p);
+  return rc;
+}
+}  // namespace
+
+int emu_begin(gw_ctx* ctx, cudaStream_t st) {
+  int* err;
+  int rc;
+  if ((rc = flag(ctx, &err))) return rc;
+  if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess) {
+    ctx->err = "FP64 products: clearing the error flag failed";
+    return GW_ERR_CUDA;
+  }
+  return GW_OK;
+}
+
+int emu_prep(gw_ctx* ctx, const char* name, const EmuSrc& s, EmuOp* op, cudaStream_t st) {
+  void* p;
+  int rc;
+  const std::string n = std::string("w.dig.") + name;
+  if ((rc = work_buffer(ctx, n.c_str(), std::max<size_t>(emu_dig_bytes(s.rows, s.K), 16), &p))) return rc;
+  op->dig = p;
+  if ((rc = work_buffer(ctx, (n + ".e").c_str(), std::max<size_t>(s.rows, 1) * 2 * sizeof(int), &p))) return rc;
+  op->exps = static_cast<int*>(p);
+  launch_emu_prep(*op, s, st);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    ctx->err = std::string("FP64 operand preparation: ") + cudaGetErrorString(e);
+    return GW_ERR_CUDA;
+  }
+  return GW_OK;
+}
+
+int emu_mm(gw_ctx* ctx, const EmuOp& A, const EmuOp& B, const EmuGemm& g, cudaStream_t st) {
+  void* ws = nullptr;
+  int* err;
+  int rc;
+  const size_t bytes = emu_gemm_ws_bytes(A.s.rows, B.s.rows, A.s.K);
+  if (bytes && (rc = work_buffer(ctx, "w.part", bytes, &ws))) return rc;
+  if ((rc = flag(ctx, &err))) return rc;
+  if (launch_emu_gemm(A, B, g, ws, err, st)) {
+    ctx->err = "FP64 product: launch set-up failed";
+    return GW_ERR_CUDA;
+  }
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    ctx->err = std::string("FP64 product: ") + cudaGetErrorString(e);
+    return GW_ERR_CUDA;
+  }
+  return GW_OK;
+}
+
+int emu_product(gw_ctx* ctx, const EmuSrc& A, const EmuSrc& B, const EmuGemm& g, EmuOp* keep, cudaStream_t st) {
+  auto chunk = [](const EmuSrc& s) {
+    const size_t row = emu_dig_bytes(1, s.K);
+    // whole tiles of rows
+    return static_cast<long long>(std::max<size_t>(kMaxDigits / row / kEmuTileM, 1)) * kEmuTileM;
+  };
+  const long long ca = chunk(A), cb = chunk(B);
+  auto part = [](const EmuSrc& s, long long r0, long long n) {
+    EmuSrc p = s;
+    p.src = s.src + (s.trans ? r0 : r0 * s.ld);
+    p.rows = std::min(n, s.rows - r0);
+    return p;
+  };
+  int rc;
+  for (long long r0 = 0; r0 < A.rows; r0 += ca) {
+    EmuOp a;
+    if (keep && keep->dig && A.rows <= ca) {
+      a = *keep;
+    } else {
+      if ((rc = emu_prep(ctx, keep ? "kept" : "a", part(A, r0, ca), &a, st))) return rc;
+      if (keep && A.rows <= ca) *keep = a;
+    }
+    for (long long c0 = 0; c0 < B.rows; c0 += cb) {
+      EmuOp b;
+      if ((rc = emu_prep(ctx, "b", part(B, c0, cb), &b, st))) return rc;
+      EmuGemm h = g;
+      h.C = g.C + r0 * g.ldc + (g.cblk ? 0 : c0);
+      h.col0 = g.col0 + c0;
+      // for tri, off the diagonal by both chunks' origins; for ktri by the rows'
+      h.tri_off = g.tri_off + r0 - c0;
+      if (g.ktri && c0 > 0) h.ktri = 0;
+      if ((rc = emu_mm(ctx, a, b, h, st))) return rc;
+    }
+  }
+  return GW_OK;
+}
+
+// From kGreensDigits primary functions on, the digit products: about 10 us of
+// preparation and 30 us per product however small, against (n^3 / 2) / 304
+// cycles on the FP64 pipes of all SMs (n = 250: 12 us, 400: 50 us, 602: 175).
+constexpr int kGreensDigits = 448;
+
+int greens_fp64(gw_ctx* ctx, double tau, double* cso, double* csv, double* g_occ, double* g_virt,
+                cudaStream_t st) {
+  const int n = ctx->nao, occ = ctx->n_occ;
+  if (n < kGreensDigits || occ == 0 || occ == n) {
+    launch_greens(ctx->d_C, ctx->d_eps, n, occ, ctx->mu, tau, cso, csv, g_occ, g_virt, st);
+    return GW_OK;
+  }
+  launch_scale_orbitals(ctx->d_C, ctx->d_eps, n, occ, ctx->mu, tau, cso, csv, st);
+  for (int v = 0; v < 2; ++v) {
+    EmuSrc s;
+    s.src = v ? csv : cso;
+    s.K = v ? n - occ : occ;
+    s.ld = s.K;
+    s.rows = n;
+    EmuOp op;
+    int rc = emu_prep(ctx, "orbitals", s, &op, st);
+    if (rc) return rc;
+    EmuGemm g;
+    g.C = v ? g_virt : g_occ;
+    g.ldc = n;
+    if ((rc = emu_mm(ctx, op, op, g, st))) return rc;
+  }
+  return GW_OK;
+}
+
+int emu_end(gw_ctx* ctx, const char* call) {
+  int* err;
+  int rc, h = 0;
+  if ((rc = flag(ctx, &err))) return rc;
+  if (cudaMemcpy(&h, err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) {
+    ctx->err = std::string(call) + ": reading the error flag failed";
+    return GW_ERR_CUDA;
+  }
+  if (h) {
+    ctx->err = std::string(call) + ": a bounded wait of the FP64 product kernel gave up";
+    return GW_ERR_TIMEOUT;
+  }
+  return GW_OK;
+}
+
+}  // namespace gw

@@ -100,6 +100,21 @@ struct Batch {
 // thr; defined with the chi orchestration.
 int build_panels_for(gw_ctx* ctx, double thr);
 
+// Named device work buffer of the context, grown on demand and kept between
+// calls.  work_trim gives back every buffer whose name starts with prefix when
+// together they hold more than `keep` bytes (0: always): the buffers of the
+// FP64 calls ("w." names) stay only while they are small beside the operand
+// batches of chi.
+int work_buffer(gw_ctx* ctx, const char* name, size_t bytes, void** out);
+void work_trim(gw_ctx* ctx, const char* prefix, size_t keep);
+constexpr size_t kWorkKeep = size_t(1) << 30;
+
+// the same when a call ends, on every path
+struct WorkTrim {
+  gw_ctx* ctx;
+  ~WorkTrim() { work_trim(ctx, "w.", kWorkKeep); }
+};
+
 // Learned-screening hook of a tensor-core batch, called after the task lists
 // are built and before step C (defined in gw_mlp.cu).  Mode 1 logs
 // (features, log10 contribution norm) of every task; mode 2 drops the tasks

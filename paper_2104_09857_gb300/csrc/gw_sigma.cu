@@ -12,14 +12,17 @@
 #include <vector>
 
 #include "gw_internal.h"
-#include "k_chain.h"
+#include "k_emu.h"
 #include "k_simt.h"
 #include "k_tc.h"
 
 namespace gw {
 namespace sigma {
 
-// Bn[j][ao(s) + s'][p0 + pw] = sum_k Csel[lam[k]][j] panel_s[k][pw * nsig + s']
+// Bn[j][ao(s) + s'][p0 + pw] = sum_k Csel[lam[k]][j] panel_s[k][pw * nsig + s'],
+// kBnOrb orbitals j per thread: the panels, the bulk of the bytes, are read
+// once for that many orbitals.
+constexpr int kBnOrb = 4;
 __global__ void k_bn_panels(const double* __restrict__ pool, const PanelDesc* __restrict__ panels,
                             const int* __restrict__ owners, const int* __restrict__ lam,
                             const int* __restrict__ ao_off, const double* __restrict__ csel,
@@ -27,14 +30,24 @@ __global__ void k_bn_panels(const double* __restrict__ pool, const PanelDesc* __
   const PanelDesc d = panels[owners[blockIdx.y]];
   const int N = d.npw * d.nsig;
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.z;
+  const int j0 = blockIdx.z * kBnOrb;
   if (n >= N) return;
   const double* p = pool + d.off;
   const int* lk = lam + d.lam_off;
-  double acc = 0.0;
-  for (int k = 0; k < d.K; ++k) acc = fma(csel[static_cast<long long>(lk[k]) * n_orb + j], p[static_cast<long long>(k) * N + n], acc);
+  double acc[kBnOrb] = {};
+#pragma unroll 4
+  for (int k = 0; k < d.K; ++k) {
+    const double v = p[static_cast<long long>(k) * N + n];
+    const double* c = csel + static_cast<long long>(lk[k]) * n_orb + j0;
+#pragma unroll
+    for (int j = 0; j < kBnOrb; ++j)
+      if (j0 + j < n_orb) acc[j] = fma(c[j], v, acc[j]);
+  }
   const int pw = n / d.nsig, sp = n - pw * d.nsig;
-  bn[(static_cast<long long>(j) * nao + ao_off[d.owner] + sp) * nri + d.p0 + pw] = acc;
+#pragma unroll
+  for (int j = 0; j < kBnOrb; ++j)
+    if (j0 + j < n_orb)
+      bn[(static_cast<long long>(j0 + j) * nao + ao_off[d.owner] + sp) * nri + d.p0 + pw] = acc[j];
 }
 
 // zero the (mu-atom, P-atom) blocks of Bn_j with norm < thr (warp per block)
@@ -138,6 +151,7 @@ int sigma_impl(gw_ctx* ctx, const double* W_tau, int w_on_device, const int* orb
   int rc = gw::build_panels_for(ctx, thr);
   if (rc) return rc;
   cudaStream_t st = ctx->stream;
+  gw::WorkTrim trim{ctx};
   const size_t nn_ri = (size_t)nri * nri, nn_ao = (size_t)nao * nao;
   DevBuf b_w, b_csel, b_bn, b_y, b_z, b_cso, b_csv, b_go, b_gv, b_fl, b_part, b_own, b_aooff;
   const double* w;
@@ -173,7 +187,7 @@ int sigma_impl(gw_ctx* ctx, const double* W_tau, int w_on_device, const int* orb
     SG_TRY(cudaMemcpyAsync(b_own.p, owners.data(), owners.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   double* bn = (double*)b_bn.p;
   if (!owners.empty()) {
-    dim3 g((maxN + 127) / 128, (unsigned)owners.size(), n_orb);
+    dim3 g((maxN + 127) / 128, (unsigned)owners.size(), (n_orb + gw::sigma::kBnOrb - 1) / gw::sigma::kBnOrb);
     gw::sigma::k_bn_panels<<<g, 128, 0, st>>>(ctx->d_panel64, (const gw::PanelDesc*)b_pd.p,
                                               (const int*)b_own.p, ctx->d_lam, ctx->d_ao_off,
                                               (const double*)b_csel.p, n_orb, nao, nri, bn);
@@ -185,16 +199,23 @@ int sigma_impl(gw_ctx* ctx, const double* W_tau, int w_on_device, const int* orb
                                                                        ctx->d_ao_off, ctx->d_ri_off, thr);
     SG_TRY(cudaGetLastError());
   }
-  SG_TRY(cudaMalloc(&b_y.p, (size_t)nao * nri * 8));
+  // FP64: the product with W for as many orbitals at a time as keep its digits
+  // within 1 GB
+  const int orb_step =
+      mixed ? 1
+            : std::max(1, std::min<int>(n_orb, (int)((size_t(1) << 30) / gw::emu_dig_bytes(nao, nri))));
+  SG_TRY(cudaMalloc(&b_y.p, (size_t)orb_step * nao * nri * 8));
   SG_TRY(cudaMalloc(&b_z.p, nn_ao * 8));
+  if ((rc = gw::emu_begin(ctx, st))) return rc;
   SG_TRY(cudaMalloc(&b_cso.p, (size_t)nao * std::max(ctx->n_occ, 1) * 8));
   SG_TRY(cudaMalloc(&b_csv.p, (size_t)nao * std::max(nao - ctx->n_occ, 1) * 8));
   SG_TRY(cudaMalloc(&b_go.p, nn_ao * 8));
   SG_TRY(cudaMalloc(&b_gv.p, nn_ao * 8));
   SG_TRY(cudaMalloc(&b_fl.p, (size_t)n_at * n_at));
-  SG_TRY(cudaMalloc(&b_part.p, (size_t)kDotBlocks * 2 * 8));
+  // the traces' partial sums of every (orbital, tau), read once at the end
+  SG_TRY(cudaMalloc(&b_part.p, (size_t)n_orb * n_tau * kDotBlocks * 2 * 8));
   double *y = (double*)b_y.p, *z = (double*)b_z.p, *go = (double*)b_go.p, *gv = (double*)b_gv.p;
-  std::vector<double> part((size_t)kDotBlocks * 2);
+  std::vector<double> part((size_t)n_orb * n_tau * kDotBlocks * 2);
   // tensor-core route: both products as step-C style tile jobs on bf16 slices
   //   y = -(B W)     (rows mu, columns Q, K = P)
   //   z = -(y B^T)   (rows mu, columns nu, K = Q)  = B W B^T
@@ -251,19 +272,50 @@ int sigma_impl(gw_ctx* ctx, const double* W_tau, int w_on_device, const int* orb
     }
     m_bq = m_b;
   }
+  gw::EmuOp op_b, op_y;  // FP64: digits of B and Y
   for (int jt = 0; jt < n_tau; ++jt) {
-    gw::launch_greens(ctx->d_C, ctx->d_eps, nao, ctx->n_occ, ctx->mu, taus[jt], (double*)b_cso.p,
-                      (double*)b_csv.p, go, gv, st);
+    if ((rc = gw::greens_fp64(ctx, taus[jt], (double*)b_cso.p, (double*)b_csv.p, go, gv, st))) return rc;
     if (thr > 0.0) {
       gw::launch_sym_block_filter(go, nao, ctx->d_ao_off, n_at, thr, (unsigned char*)b_fl.p, st);
       gw::launch_sym_block_filter(gv, nao, ctx->d_ao_off, n_at, thr, (unsigned char*)b_fl.p, st);
     }
     const double* wt = w + (size_t)jt * nn_ri;
+    gw::EmuOp op_w;  // FP64: the columns of W as rows
+    if (!mixed) {
+      gw::EmuSrc sw;
+      sw.src = wt;
+      sw.ld = sw.rows = nri;
+      sw.K = nri;
+      sw.trans = true;
+      if ((rc = gw::emu_prep(ctx, "w", sw, &op_w, st))) return rc;
+    }
     for (int a = 0; a < n_orb; ++a) {
       const double* b = bn + (size_t)a * nao * nri;
       if (!mixed) {
-        gw::chain_dgemm(false, false, nao, nri, nri, 1.0, b, nri, wt, nri, 0.0, y, nri, st);  // Y = B W
-        gw::chain_dgemm(false, true, nao, nao, nri, 1.0, y, nri, b, nri, 0.0, z, nao, st);    // Z = Y B^T
+        const int i = a % orb_step;
+        if (i == 0) {
+          // Y = B W for orb_step orbitals (the digits of B made once if that is all of them)
+          const int cnt = std::min(orb_step, n_orb - a);
+          gw::EmuSrc sb, sy;
+          sb.src = b;
+          sb.ld = sy.ld = nri;
+          sb.rows = sy.rows = (long long)cnt * nao;
+          sb.K = sy.K = nri;
+          if ((jt == 0 || orb_step < n_orb) && (rc = gw::emu_prep(ctx, "b", sb, &op_b, st))) return rc;
+          gw::EmuGemm g;
+          g.C = y;
+          g.ldc = nri;
+          if ((rc = gw::emu_mm(ctx, op_b, op_w, g, st))) return rc;
+          sy.src = y;
+          if ((rc = gw::emu_prep(ctx, "y", sy, &op_y, st))) return rc;
+        }
+        // Z = Y B^T
+        gw::EmuGemm g;
+        g.C = z;
+        g.ldc = nao;
+        if ((rc = gw::emu_mm(ctx, op_y.slice_rows((long long)i * nao, nao), op_b.slice_rows((long long)i * nao, nao), g,
+                             st)))
+          return rc;
       } else {
         // binary16 scales: max |B|, max |W| and the bound |B W| <= max_mu
         // sum_P |B[mu][P]| * max |W| (all 1 for bf16 slices)
@@ -303,19 +355,23 @@ int sigma_impl(gw_ctx* ctx, const double* W_tau, int w_on_device, const int* orb
         }
         SG_TRY(cudaGetLastError());
       }
-      gw::sigma::k_dot2<<<kDotBlocks, 256, 0, st>>>(go, gv, z, (long long)nn_ao, (double*)b_part.p);
+      gw::sigma::k_dot2<<<kDotBlocks, 256, 0, st>>>(go, gv, z, (long long)nn_ao,
+                                                    (double*)b_part.p + ((size_t)a * n_tau + jt) * kDotBlocks * 2);
       SG_TRY(cudaGetLastError());
-      SG_TRY(cudaMemcpyAsync(part.data(), b_part.p, part.size() * 8, cudaMemcpyDeviceToHost, st));
-      SG_TRY(cudaStreamSynchronize(st));
-      double so = 0.0, sv = 0.0;
-      for (int bl = 0; bl < kDotBlocks; ++bl) {
-        so += part[2 * bl];
-        sv += part[2 * bl + 1];
-      }
-      sigma_out[((size_t)a * n_tau + jt) * 2 + 0] = -so;
-      sigma_out[((size_t)a * n_tau + jt) * 2 + 1] = sv;
     }
   }
+  SG_TRY(cudaMemcpyAsync(part.data(), b_part.p, part.size() * 8, cudaMemcpyDeviceToHost, st));
+  SG_TRY(cudaStreamSynchronize(st));
+  for (size_t i = 0; i < (size_t)n_orb * n_tau; ++i) {
+    double so = 0.0, sv = 0.0;
+    for (int bl = 0; bl < kDotBlocks; ++bl) {
+      so += part[(i * kDotBlocks + bl) * 2];
+      sv += part[(i * kDotBlocks + bl) * 2 + 1];
+    }
+    sigma_out[i * 2 + 0] = -so;
+    sigma_out[i * 2 + 1] = sv;
+  }
+  if ((rc = gw::emu_end(ctx, "gw_sigma_tau"))) return rc;
   if (mixed) {
     int h_err = 0;
     SG_TRY(cudaMemcpy(&h_err, b_err.p, sizeof(int), cudaMemcpyDeviceToHost));
@@ -495,7 +551,7 @@ int sigma_batch_mixed(gw_ctx* const* ctxs, int n_mol, const double* const* W_tau
     SB_TRY(cudaMalloc(&own.p, std::max<size_t>(owners.size(), 1) * sizeof(int)));
     if (!owners.empty()) {
       SB_TRY(cudaMemcpyAsync(own.p, owners.data(), owners.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-      dim3 g((maxN + 127) / 128, (unsigned)owners.size(), n_orb[i]);
+      dim3 g((maxN + 127) / 128, (unsigned)owners.size(), (n_orb[i] + gw::sigma::kBnOrb - 1) / gw::sigma::kBnOrb);
       gw::sigma::k_bn_panels<<<g, 128, 0, st>>>(c->d_panel64, (const gw::PanelDesc*)pd.p,
                                                 (const int*)own.p, c->d_lam, c->d_ao_off,
                                                 (const double*)csel.p, n_orb[i], c->nao, c->nri,

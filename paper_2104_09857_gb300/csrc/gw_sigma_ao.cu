@@ -5,12 +5,14 @@
 // (the real representation of gw_sigma_tau: C_n^T Sigma C_n is Sigma^c_n).
 //
 // FP64 dense route for molecules: T[mu][lam][P] is scattered once from the
-// stored atom blocks, then per tau point three products on the CUDA cores,
-//   Z = T W            (n_AO^2 x n_RI by n_RI x n_RI),
-//   U = G Z            (n_AO x n_AO by n_AO x n_AO n_RI),
-//   Sigma = -+ sum_lam T[:, lam, :] U[lam]^T   (n_AO products of n_AO x n_RI).
-// Memory is 3 n_AO^2 n_RI doubles; the filter drops 3c blocks and G blocks
-// with Frobenius norm < thr, like the other contractions.
+// stored atom blocks, then per tau point three products (k_emu.cu),
+//   Z[sig][nu][P] = T W               (n_AO^2 x n_RI by n_RI x n_RI),
+//   M[mu][sig][P] = sum_lam G T       (n_AO x n_AO by n_AO x n_AO n_RI),
+//   Sigma[mu][nu] = -+ sum_(sig, P) M[mu][sig][P] Z[nu][sig][P],
+// the last one product of length n_AO n_RI (T symmetric in its primary
+// indices, so Z is too).  Memory is 3 n_AO^2 n_RI doubles and the operands'
+// digits; the filter drops 3c blocks and G blocks with Frobenius norm < thr,
+// like the other contractions.
 
 #include <cuda_runtime.h>
 
@@ -20,7 +22,7 @@
 #include <vector>
 
 #include "gw_internal.h"
-#include "k_chain.h"
+#include "k_emu.h"
 #include "k_simt.h"
 
 namespace gw {
@@ -100,7 +102,7 @@ extern "C" int gw_sigma_ao_tau(gw_ctx* ctx, const double* W_tau, int w_on_device
   const int nao = ctx->nao, nri = ctx->nri, n_at = ctx->n_at;
   const int n_tau = static_cast<int>(ctx->tau.size());
   const long long dense = static_cast<long long>(nao) * nao * nri;
-  // the products' grids: n_AO^2 rows of 64 (at most 65535 row tiles), n_AO n_RI columns in an int
+  // n_AO n_RI is a reduction length (an int)
   if (dense > kMaxDense || ctx->n_blocks > 0x7fffffffLL ||
       static_cast<long long>(nao) * nao > 65535LL * 64 || static_cast<long long>(nao) * nri > 0x7fffffffLL) {
     ctx->err = "gw_sigma_ao_tau: the dense route holds n_AO^2 n_RI <= 3*2^30 elements and n_AO <= 2047";
@@ -115,6 +117,9 @@ extern "C" int gw_sigma_ao_tau(gw_ctx* ctx, const double* W_tau, int w_on_device
       }
   SA_TRY(cudaSetDevice(ctx->device));
   cudaStream_t st = ctx->stream;
+  gw::WorkTrim trim{ctx};
+  int rc = gw::emu_begin(ctx, st);
+  if (rc) return rc;
   DevBuf b_t, b_z, b_u, b_go, b_gv, b_cso, b_csv, b_fl, b_w, b_out;
   SA_TRY(cudaMalloc(&b_t.p, std::max<long long>(dense, 1) * 8));
   SA_TRY(cudaMalloc(&b_z.p, std::max<long long>(dense, 1) * 8));
@@ -139,10 +144,23 @@ extern "C" int gw_sigma_ao_tau(gw_ctx* ctx, const double* W_tau, int w_on_device
         nri, dense, T);
     SA_TRY(cudaGetLastError());
   }
-  const long long row = static_cast<long long>(nao) * nri;  // one lambda (or sigma) slab of T, Z, U
+  const long long row = static_cast<long long>(nao) * nri;  // one slab of T, Z, M
+  auto rows_of = [](const double* p, long long ld, long long rows, int K, bool trans) {
+    gw::EmuSrc s;
+    s.src = p;
+    s.ld = ld;
+    s.rows = rows;
+    s.K = K;
+    s.trans = trans;
+    return s;
+  };
+  const gw::EmuSrc t_p = rows_of(T, nri, static_cast<long long>(nao) * nao, nri, false);  // rows (sig, nu)
+  const gw::EmuSrc t_lam = rows_of(T, row, row, nao, true);                               // rows (mu, P)
+  gw::EmuOp keep_t;
   for (int j = 0; j < n_tau; ++j) {
-    gw::launch_greens(ctx->d_C, ctx->d_eps, nao, ctx->n_occ, ctx->mu, ctx->tau[j],
-                      static_cast<double*>(b_cso.p), static_cast<double*>(b_csv.p), go, gv, st);
+    if ((rc = gw::greens_fp64(ctx, ctx->tau[j], static_cast<double*>(b_cso.p), static_cast<double*>(b_csv.p), go, gv,
+                              st)))
+      return rc;
     if (thr > 0.0) {
       gw::launch_sym_block_filter(go, nao, ctx->d_ao_off, n_at, thr, static_cast<unsigned char*>(b_fl.p), st);
       gw::launch_sym_block_filter(gv, nao, ctx->d_ao_off, n_at, thr, static_cast<unsigned char*>(b_fl.p), st);
@@ -152,22 +170,27 @@ extern "C" int gw_sigma_ao_tau(gw_ctx* ctx, const double* W_tau, int w_on_device
       SA_TRY(cudaMemcpyAsync(b_w.p, wj, nn_ri * 8, cudaMemcpyHostToDevice, st));
       wj = static_cast<const double*>(b_w.p);
     }
-    // Z[sig][nu][P] = sum_Q T[sig][nu][Q] W[Q][P]
-    gw::chain_dgemm(false, false, nao * nao, nri, nri, 1.0, T, nri, wj, nri, 0.0, Z, nri, st);
+    gw::EmuGemm z;
+    z.C = Z;
+    z.ldc = nri;
+    if ((rc = gw::emu_product(ctx, t_p, rows_of(wj, nri, nri, nri, true), z, &keep_t, st))) return rc;
     double* dst = out_on_device ? sigma_out + static_cast<size_t>(j) * 2 * nn_ao
                                 : static_cast<double*>(b_out.p);
     for (int k = 0; k < 2; ++k) {
-      const double* g = k == 0 ? go : gv;
-      const double sign = k == 0 ? -1.0 : 1.0;
-      // U[lam][nu][P] = sum_sig G[lam][sig] Z[sig][nu][P]
-      gw::chain_dgemm(false, false, nao, static_cast<int>(row), nao, 1.0, g, nao, Z, static_cast<int>(row),
-                      0.0, U, static_cast<int>(row), st);
-      // Sigma[mu][nu] = sign sum_lam sum_P T[mu][lam][P] U[lam][nu][P]
-      double* out = dst + static_cast<size_t>(k) * nn_ao;
-      for (int lam = 0; lam < nao; ++lam)
-        gw::chain_dgemm(false, true, nao, nao, nri, sign, T + static_cast<size_t>(lam) * nri,
-                        static_cast<int>(row), U + static_cast<size_t>(lam) * row, nri, lam == 0 ? 0.0 : 1.0,
-                        out, nao, st);
+      gw::EmuGemm m;
+      m.C = U;
+      m.ldc = nri;
+      m.cblk = nri;
+      m.cblk_stride = row;
+      if ((rc = gw::emu_product(ctx, rows_of(k == 0 ? go : gv, nao, nao, nao, false), t_lam, m, nullptr, st)))
+        return rc;
+      gw::EmuGemm g;
+      g.alpha = k == 0 ? -1.0 : 1.0;
+      g.C = dst + static_cast<size_t>(k) * nn_ao;
+      g.ldc = nao;
+      if ((rc = gw::emu_product(ctx, rows_of(U, row, nao, static_cast<int>(row), false),
+                                rows_of(Z, row, nao, static_cast<int>(row), false), g, nullptr, st)))
+        return rc;
     }
     SA_TRY(cudaGetLastError());
     if (!out_on_device)
@@ -175,5 +198,5 @@ extern "C" int gw_sigma_ao_tau(gw_ctx* ctx, const double* W_tau, int w_on_device
                              cudaMemcpyDeviceToHost, st));
   }
   SA_TRY(cudaStreamSynchronize(st));
-  return GW_OK;
+  return gw::emu_end(ctx, "gw_sigma_ao_tau");
 }

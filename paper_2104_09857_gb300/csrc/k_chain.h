@@ -3,22 +3,24 @@
 
 #include <cuda_runtime.h>
 
+#include "gw_internal.h"
+
 namespace gw {
 
-// out[k][e] = sum_j w[k * nin + j] in[j][e], n elements per matrix
-void chain_lincomb(const double* in, int nin, const double* w, int nout, long long n, double* out,
-                   cudaStream_t st);
-// out[j][e] += w[j * ldw + k] x[e] for j < nout
-void chain_axpy_multi(const double* x, const double* w, int ldw, int k, int nout, long long n,
-                      double* out, cudaStream_t st);
+// out[e] = sum_j w[j] in[j][e], n elements per matrix
+void chain_lincomb(const double* in, int nin, const double* w, long long n, double* out, cudaStream_t st);
+// x = w - v on the lower triangles of two n x n matrices, taken as symmetric:
+// out[j] += d[j * ldd] x for j < nout, both triangles of out written
+void chain_add_symmetric(const double* w, const double* v, const double* d, int ldd, int nout, int n, double* out,
+                         cudaStream_t st);
+// a[i][i] += x
+void chain_add_diagonal(double* a, int n, double x, cudaStream_t st);
+// a = identity
 void chain_set_identity(double* a, int n, cudaStream_t st);
-void chain_transpose(const double* a, double* b, int n, cudaStream_t st);
-// C = alpha op(A) op(B) + beta C (row-major; op transposes when ta / tb)
-void chain_dgemm(bool ta, bool tb, int m, int n, int k, double alpha, const double* A, int lda,
-                 const double* B, int ldb, double beta, double* C, int ldc, cudaStream_t st);
-// in-place lower Cholesky; err[0] |= 1 on a non-positive pivot
-void chain_potrf(double* a, int n, int* err, cudaStream_t st);
-// B <- R^-1 B with R lower triangular (n x n), B n x m
-void chain_trsm_left_lower(const double* r, int n, double* bm, int m, cudaStream_t st);
+// a[rows][n], rows >= n: the leading n x n block (its lower triangle is read)
+// becomes its Cholesky factor R, the rows below become B R^-T; the strict
+// upper triangle of the leading block is zeroed.  err[0] |= 1 on a pivot that
+// is not positive.  Uses the context's work buffers (emu_begin before).
+int chain_cholesky(gw_ctx* ctx, double* a, long long rows, int n, int* err, cudaStream_t st);
 
 }  // namespace gw

@@ -50,6 +50,7 @@
 
 #include "gw_internal.h"
 #include "k_tc.h"
+#include "tc_ptx.h"
 
 namespace gw {
 namespace tc {
@@ -57,96 +58,11 @@ namespace tc {
 constexpr int kTileM = 128;
 constexpr int kTileN = 128;
 constexpr int kStageK = 64;   // bf16 elements per K step: one 128-byte swizzled row
-constexpr int kMmaK = 16;
 constexpr int kEpiWarps = 16;                 // 4 TMEM lane quadrants x 4 column groups
 constexpr int kEpiCols = kTileN / 4;          // accumulator columns per epilogue warp
 constexpr int kWriteK = 2048;  // reduction elements between ChiJob write-outs (one per split-K unit)
 constexpr int kTmemCols = 512;
 constexpr int kAccBufs = 4;   // accumulators: TMEM columns [128 b, 128 b + 128)
-constexpr uint32_t kSuspendNs = 20000;            // longest suspension of one try_wait
-constexpr uint64_t kWaitLimitNs = 2000000000ull;  // a wait gives up after 2 s
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// try_wait with a suspend-time hint: a thread whose phase is not complete
-// sleeps in hardware (up to kSuspendNs) instead of spinning on issue slots.
-__device__ __forceinline__ bool mbar_try_wait_sleep(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendNs)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// Bounded wait for the phase of the given parity; false on time-out
-// (kWaitLimitNs) or abort.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try_wait_sleep(bar, parity)) return true;
-  const uint64_t t0 = global_ns();
-  for (;;) {
-    if (mbar_try_wait_sleep(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (global_ns() - t0 > kWaitLimitNs) return false;
-  }
-}
-// Bounded wait without abort check (clean-up after an abort).
-__device__ __forceinline__ void mbar_wait_cleanup(uint64_t* bar, uint32_t parity) {
-  const uint64_t t0 = global_ns();
-  while (!mbar_try_wait_sleep(bar, parity) && global_ns() - t0 < kWaitLimitNs) {
-  }
-}
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z,
-                                            uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
-      : "memory");
-}
-// Bulk copy of `bytes` (a multiple of 16) from shared to global memory, both
-// addresses 16-byte aligned, as a bulk async-group of the issuing thread.
-__device__ __forceinline__ void bulk_store(void* gdst, const void* ssrc, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst),
-               "r"(smem_u32(ssrc)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// the shared-memory sources of this thread's bulk groups have been read
-__device__ __forceinline__ void bulk_wait_read() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-// this thread's bulk groups have completed
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-// order this thread's shared-memory writes before later async-proxy reads
-__device__ __forceinline__ void fence_proxy_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 128-byte rows
 // (64 bf16), 8-row groups 1024 bytes apart, 1024-aligned tile base.
 __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
@@ -157,12 +73,6 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
   d |= static_cast<uint64_t>(1) << 46;
   d |= static_cast<uint64_t>(2) << 61;
   return d;
-}
-// Instruction descriptor of kind::f16: BF16 x BF16 (or F16 x F16) -> FP32,
-// both operands K-major.
-__host__ __device__ constexpr uint32_t idesc_f32(int m, int n, bool f16) {
-  return (1u << 4) | (f16 ? 0u : ((1u << 7) | (1u << 10))) | (static_cast<uint32_t>(n >> 3) << 17) |
-         (static_cast<uint32_t>(m >> 4) << 24);
 }
 // One slice of v (bf16, or binary16 when f16): returns its bits and leaves
 // the remainder v - slice in v (exact).
@@ -185,20 +95,6 @@ __device__ __forceinline__ uint16_t take_slice(double& v, bool f16) {
   const __nv_bfloat16 h = __double2bfloat16(v);
   v -= static_cast<double>(__bfloat162float(h));
   return __bfloat16_as_ushort(h);
-}
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
-}
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_u32(bar))
-      : "memory");
 }
 // acc[j] += TMEM[lane row][taddr column + j], j < 32: one 32-column load and
 // its wait, or (kHalves = 2) two 16-column loads and waits, which keeps 16
@@ -1847,6 +1743,26 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
+// 3-D map over [slices][rows][k_len] 16-bit elements
+int encode_map(CUtensorMap* map, const void* base, long long k_len, long long rows, long long stride_rows,
+               int slices, int box_k, int box_rows, int box_slices, int f16, CUtensorMapSwizzle swizzle) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return -1;
+  if ((reinterpret_cast<uintptr_t>(base) & 15) != 0 || (k_len * 2) % 16 != 0) return -2;
+  cuuint64_t dims[3] = {static_cast<cuuint64_t>(k_len), static_cast<cuuint64_t>(rows),
+                        static_cast<cuuint64_t>(slices)};
+  cuuint64_t strides[2] = {static_cast<cuuint64_t>(k_len * 2),
+                           static_cast<cuuint64_t>(k_len * 2 * stride_rows)};
+  cuuint32_t box[3] = {static_cast<cuuint32_t>(box_k), static_cast<cuuint32_t>(box_rows),
+                       static_cast<cuuint32_t>(box_slices)};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = fn(map, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
+                  const_cast<void*>(base), dims, strides,
+                  box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? 0 : -3;
+}
+
 thread_local int g_stall_test = 0;  // test hook, per host thread
 
 // SM count of the current device (queried per call: contexts of one process
@@ -1901,20 +1817,12 @@ int launch_persistent(int slices, int f16, const CUtensorMap& ma, const CUtensor
 
 int make_slice_map(CUtensorMap* map, const void* base, long long k_len, long long rows, int slices,
                    int box_rows, int f16) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return -1;
-  if ((reinterpret_cast<uintptr_t>(base) & 15) != 0 || (k_len * 2) % 16 != 0) return -2;
-  cuuint64_t dims[3] = {static_cast<cuuint64_t>(k_len), static_cast<cuuint64_t>(rows),
-                        static_cast<cuuint64_t>(slices)};
-  cuuint64_t strides[2] = {static_cast<cuuint64_t>(k_len * 2),
-                           static_cast<cuuint64_t>(k_len * 2 * rows)};
-  cuuint32_t box[3] = {static_cast<cuuint32_t>(tc::kStageK), static_cast<cuuint32_t>(box_rows), 1};
-  cuuint32_t estr[3] = {1, 1, 1};
-  CUresult r = fn(map, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
-                  const_cast<void*>(base), dims, strides,
-                  box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? 0 : -3;
+  return encode_map(map, base, k_len, rows, rows, slices, tc::kStageK, box_rows, 1, f16, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
+int make_digit_map(CUtensorMap* map, const void* base, long long k_len, long long rows, long long stride_rows,
+                   int slices, int box_k, int box_rows) {
+  return encode_map(map, base, k_len, rows, stride_rows, slices, box_k, box_rows, slices, 1, CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
 int tc_tile_rows() { return tc::kTileM; }
