@@ -20,7 +20,7 @@
 //             Frobenius norms of its atom blocks accumulated on the way.
 // Warp roles (576 threads):
 //   warp 0      TMA producer (one thread): A and B slices of each K step
-//   warp 1      TMEM allocator and MMA issuer (one thread)
+//   warp 1      TMEM allocator and MMA issuer (one elected lane)
 //   warps 2..17 epilogue (4 lane quadrants x 4 groups of 32 columns): the
 //               TMEM accumulators are read into an FP32
 //               register sum per element; the job writes it out at the end
@@ -955,19 +955,7 @@ struct Sched {
     advance();
     return v;
   }
-  // the MMA issuer (one thread)
-  __device__ int consume_one(bool& ok) {
-    if (!counter) return next_static();
-    if (!mbar_wait(&full[s], ph, abort)) {
-      ok = false;
-      return -1;
-    }
-    const int v = slot[s];
-    mbar_arrive(&empty[s]);
-    advance();
-    return v;
-  }
-  // an epilogue warp (all 32 lanes)
+  // the MMA issuer warp and the epilogue warps (all 32 lanes)
   __device__ int consume_warp(int lane, bool& ok) {
     if (!counter) return next_static();
     if (!mbar_wait(&full[s], ph, abort)) {
@@ -1019,7 +1007,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   int* sched_slot = reinterpret_cast<int*>(sched_empty + kSchedSlots);  // [kSchedSlots]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sched_slot + kSchedSlots);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
+  const int warp = __reduce_max_sync(0xffffffffu, threadIdx.x / 32), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -1104,86 +1092,102 @@ __global__ void __launch_bounds__(kThreads, 1)
     // the next accumulator buffer; within the part of an interval that lies
     // in one K step, the small slice products come first, then the main
     // product (0, 0).
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_f32(kTileM, kTileN, F16);
-      // slice tiles are kTileBytes apart: descriptor start addresses
-      // advance by kTileBytes >> 4
-      constexpr uint64_t kStep = static_cast<uint64_t>(L::kTileBytes >> 4);
-      int stage = 0;
-      uint32_t phase = 0;
-      int chunk = 0;
-      bool ok = true, issued_any = false;
-      for (int t = sch.consume_one(ok); t >= 0 && ok; t = sch.consume_one(ok)) {
-        const typename Job::Tile T = job.tile(t);
-        const long long n = job.nsteps(T);
-        const long long nsub = n * kSub;
-        long long js = 0;
-        int sub = 0;  // MMA steps into the drain interval
-        for (long long i = 0; i < n && ok; ++i) {
-          if (!mbar_wait(&full[stage], phase, abort_flag)) {
-            ok = false;
-            break;
+    // The whole warp runs the loop and one elected lane issues: in converged
+    // control flow the descriptors live in uniform registers and an MMA
+    // issues as fast as the tensor core takes it (64 cycles for 128 x 128 x
+    // 16).  Issued from a branch on lane 0, every MMA first moved its
+    // descriptors to uniform registers: 85 cycles and more.
+    constexpr uint32_t idesc = idesc_f32(kTileM, kTileN, F16);
+    // slice tiles are kTileBytes apart: descriptor start addresses advance
+    // by kTileBytes >> 4
+    constexpr uint32_t kStep = static_cast<uint32_t>(L::kTileBytes >> 4);
+    constexpr uint32_t kAll = 0xffffffffu;
+    const uint32_t lead = elect_one();
+    const uint32_t tmu = __reduce_max_sync(kAll, tmem);
+    int stage = 0;
+    uint32_t phase = 0;
+    int chunk = 0;
+    bool ok = true, issued_any = false;
+    for (int t = sch.consume_warp(lane, ok); __all_sync(kAll, t >= 0 && ok); t = sch.consume_warp(lane, ok)) {
+      const typename Job::Tile T = job.tile(t);
+      const int n = __reduce_max_sync(kAll, static_cast<int>(job.nsteps(T)));
+      const int nsub = n * kSub;
+      int js = 0;
+      int sub = 0;  // MMA steps into the drain interval
+      for (int i = 0; i < n; ++i) {
+        ok = __all_sync(kAll, mbar_wait(&full[stage], phase, abort_flag));
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t da = desc_sw128(smem_u32(operands + stage * L::kStageBytes));
+        const uint32_t a_lo = static_cast<uint32_t>(da), hi = static_cast<uint32_t>(da >> 32);
+        const uint32_t b_lo = a_lo + S * kStep;
+        int k = 0;
+        while (k < kSub) {
+          const int mb = chunk % kAccBufs;
+          if (sub == 0) {
+            ok = __all_sync(kAll, mbar_wait(&acc_empty[mb], ((static_cast<uint32_t>(chunk / kAccBufs)) & 1u) ^ 1u,
+                                            abort_flag));
+            if (!ok) break;
+            tc_fence_after();
           }
-          tc_fence_after();
-          const uint32_t st = smem_u32(operands + stage * L::kStageBytes);
-          const uint64_t da = desc_sw128(st), db = desc_sw128(st + S * L::kTileBytes);
-          int k = 0;
-          while (k < kSub) {
-            const int mb = chunk % kAccBufs;
-            if (sub == 0) {
-              ok = mbar_wait(&acc_empty[mb], ((static_cast<uint32_t>(chunk / kAccBufs)) & 1u) ^ 1u,
-                             abort_flag);
-              tc_fence_after();
-              if (!ok) break;
-            }
-            // MMA steps [k, ke) of this K step belong to the current interval
-            const int ke = min(kSub, k + (cad.main - sub));
-            const uint32_t d = tmem + static_cast<uint32_t>(mb * 128);
+          // MMA steps [k, ke) of this K step belong to the current interval
+          const int ke = min(kSub, k + (cad.main - sub));
+          js += ke - k;
+          const bool close = sub + ke - k == cad.main || js == nsub;
+          if (lead) {
+            const uint32_t d = tmu + static_cast<uint32_t>(mb * 128);
             uint32_t accf = sub == 0 ? 0u : 1u;
-            for (int kk = k; kk < ke; ++kk) {
-              const uint64_t koff = static_cast<uint64_t>((kk * kMmaK * 2) >> 4);
+#pragma unroll
+            for (int kk = 0; kk < kSub; ++kk) {
+              if (kk < k || kk >= ke) continue;
+              const uint32_t koff = static_cast<uint32_t>((kk * kMmaK * 2) >> 4);
 #pragma unroll
               for (int a = 0; a < S; ++a) {
 #pragma unroll
                 for (int b = 0; b < S - a; ++b) {
                   if (a == 0 && b == 0) continue;
-                  mma_bf16(d, da + a * kStep + koff, db + b * kStep + koff, idesc, accf);
+                  mma_f16_lo(d, a_lo + a * kStep + koff, b_lo + b * kStep + koff, hi, idesc, accf);
                   accf = 1u;
                 }
               }
             }
-            for (int kk = k; kk < ke; ++kk) {
-              const uint64_t koff = static_cast<uint64_t>((kk * kMmaK * 2) >> 4);
-              mma_bf16(d, da + koff, db + koff, idesc, accf);
-              accf = 1u;
+#pragma unroll
+            for (int kk = 0; kk < kSub; ++kk) {
+              if (kk < k || kk >= ke) continue;
+              const uint32_t koff = static_cast<uint32_t>((kk * kMmaK * 2) >> 4);
+              mma_f16_lo(d, a_lo + koff, b_lo + koff, hi, idesc, 1u);
             }
-            issued_any = true;
-            js += ke - k;
-            sub += ke - k;
-            k = ke;
-            if (sub == cad.main || js == nsub) {
-              mma_commit(&acc_full[mb]);
-              ++chunk;
-              sub = 0;
-            }
+            if (close) mma_commit(&acc_full[mb]);
           }
-          if (!ok) break;
-          mma_commit(&empty[stage]);
-          if (++stage == kStages) {
-            stage = 0;
-            phase ^= 1u;
+          __syncwarp();
+          issued_any = true;
+          sub += ke - k;
+          k = ke;
+          if (close) {
+            ++chunk;
+            sub = 0;
           }
+        }
+        if (!ok) break;
+        if (lead) mma_commit(&empty[stage]);
+        __syncwarp();
+        if (++stage == kStages) {
+          stage = 0;
+          phase ^= 1u;
         }
       }
-      if (!ok) {
-        *abort_flag = 1;
-        atomicOr(err_flag, 2);
-        if (issued_any) {
-          mma_commit(drain);
-          mbar_wait_cleanup(drain, 0);
-        }
+      if (!ok) break;
+    }
+    ok = __all_sync(kAll, ok);
+    if (!ok && lead) {
+      *abort_flag = 1;
+      atomicOr(err_flag, 2);
+      if (issued_any) {
+        mma_commit(drain);
+        mbar_wait_cleanup(drain, 0);
       }
     }
+    __syncwarp();
   } else {
     // ---------------- epilogue (warps 2..17) ----------------
     const int quad = warp & 3;

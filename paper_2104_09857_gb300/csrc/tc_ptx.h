@@ -100,17 +100,9 @@ __host__ __device__ constexpr uint32_t idesc_f32(int m, int n, bool f16) {
   return (1u << 4) | (f16 ? 0u : ((1u << 7) | (1u << 10))) | (static_cast<uint32_t>(n >> 3) << 17) |
          (static_cast<uint32_t>(m >> 4) << 24);
 }
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
-}
-// The same with the low words of the two descriptors and their common high
-// word: 32-bit adds step a descriptor, and in uniform control flow it stays in
-// uniform registers.
+// kind::f16 MMA from the low words of the two descriptors and their common
+// high word: 32-bit adds step a descriptor, and in uniform control flow it
+// stays in uniform registers.
 __device__ __forceinline__ void mma_f16_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
                                            uint32_t idesc, uint32_t accumulate) {
   asm volatile(
