@@ -122,6 +122,14 @@ void free_dev(void* p) {
   if (p) cudaFree(p);
 }
 
+void free_panel_digits(gw_ctx* ctx) {
+  free_dev(ctx->d_pd);
+  free_dev(ctx->d_pd_exps);
+  ctx->d_pd = nullptr;
+  ctx->d_pd_exps = nullptr;
+  ctx->pd_ok = false;
+}
+
 void reset_tensor(gw_ctx* ctx) {
   free_dev(ctx->d_t3);
   free_dev(ctx->d_t3f);
@@ -149,6 +157,7 @@ void reset_tensor(gw_ctx* ctx) {
   free_dev(ctx->d_pt);
   ctx->d_pt = nullptr;
   ctx->pt_ok = false;
+  free_panel_digits(ctx);
   ctx->ycov_valid = false;
 }
 
@@ -180,6 +189,7 @@ int plan_panels(gw_ctx* ctx, double thr) {
   ctx->panels_ok = false;
   ctx->panels_thr = -1.0;
   ctx->pt_ok = false;
+  ctx->pd_ok = false;
   ctx->panel32_ok = false;
   ctx->ycov_valid = false;
   const int n = ctx->n_at;
@@ -744,7 +754,7 @@ int chi_one_batch(gw_ctx* ctx, const Batch& b, const T* g_occ, const T* g_virt, 
   if ((rc = wsT(ctx, "counts", (size_t)npt * nqt, &counts))) return rc;
   if ((rc = wsT(ctx, "kacc", (size_t)npt * nqt, &kacc))) return rc;
   gw::launch_build_tasks(fx, fy, nslab, npt, nqt, b.P0, prow, 0, ctx->nri, ctx->d_atom_of_ri, d_len,
-                         tasks, counts, kacc, tile, per, 0, ctx->n_at, 0, ctx->nao, ctx->d_atom_of_ao,
+                         tasks, counts, kacc, tile, tile, per, 0, ctx->n_at, 0, ctx->nao, ctx->d_atom_of_ao,
                          ctx->stream);
   GW_CHECK_LAUNCH();
   double* d_fc;
@@ -804,6 +814,285 @@ int chi_one_batch(gw_ctx* ctx, const Batch& b, const T* g_occ, const T* g_virt, 
   (void)tcpath;
   (void)slices;
   ctx->stats.flops_issued += 2.0 * tile * tile * ksum;
+  return GW_OK;
+}
+
+// ---------------------------------------------------------------------------
+// FP64 route on the tensor cores: panels as digits (k_emu.h), once per thr
+// ---------------------------------------------------------------------------
+// Bytes of an operand element there: FP64 and eight 16-bit digits.
+constexpr size_t kDigitElem = 8 + 2 * gw::kEmuSlices;
+
+// ctx->pd_ok afterwards: the digits are there.  They take 16 bytes per panel
+// element beside the FP64 pool's 8; where that and one batch of operands do
+// not fit in free memory the call stays on the CUDA-core kernels.
+int ensure_panel_digits(gw_ctx* ctx) {
+  if (ctx->pd_ok) return GW_OK;
+  free_panel_digits(ctx);
+  const int n = ctx->n_at;
+  ctx->pd_row0.assign(n, 0);
+  long long rows = 0;
+  int kmax = 1, max_n = 0;
+  for (int s = 0; s < n; ++s) {
+    const PanelDesc& d = ctx->panels[s];
+    ctx->pd_row0[s] = rows;
+    if (d.K == 0) continue;
+    rows += (long long)d.npw * d.nsig;
+    kmax = std::max(kmax, d.K);
+    max_n = std::max(max_n, d.npw * d.nsig);
+  }
+  if (rows == 0 || rows > INT32_MAX) return GW_OK;
+  const int kp = gw::emu_kp(kmax);
+  const size_t bytes = gw::emu_dig_bytes(rows, kmax);
+  size_t free_b = 0, total_b = 0;
+  cudaMemGetInfo(&free_b, &total_b);
+  const double operands = std::min(ctx->batch_bytes, (double)kDigitElem * 2.0 * ctx->nri * ctx->naop * (double)ctx->nao);
+  const double need = (double)bytes + 8.0 * rows + operands + 32.0 * ctx->nri * (double)ctx->nri +
+                      64.0 * ctx->nao * (double)ctx->nao + 1e9;
+  if (need > (double)free_b) return GW_OK;
+  void *dig = nullptr, *exps = nullptr;
+  if (cudaMalloc(&dig, bytes) != cudaSuccess || cudaMalloc(&exps, (size_t)rows * sizeof(int)) != cudaSuccess) {
+    cudaGetLastError();
+    free_dev(dig);
+    return GW_OK;
+  }
+  ctx->d_pd = dig;
+  ctx->d_pd_exps = static_cast<int*>(exps);
+  ctx->pd_rows = rows;
+  ctx->pd_kp = kp;
+  // panels without rows are left out of the launch
+  std::vector<PanelDesc> pd;
+  std::vector<long long> row0;
+  for (int s = 0; s < n; ++s)
+    if (ctx->panels[s].K > 0) {
+      pd.push_back(ctx->panels[s]);
+      row0.push_back(ctx->pd_row0[s]);
+    }
+  PanelDesc* d_desc;
+  long long* d_row0;
+  int *d_be, rc;
+  if ((rc = upload(ctx, "pd_desc", pd, &d_desc)) || (rc = upload(ctx, "pd_row0", row0, &d_row0)) ||
+      (rc = wsT(ctx, "pd_be", (size_t)rows, &d_be)))
+    return rc;
+  gw::launch_panel_digits(ctx->d_panel64, d_desc, d_row0, (int)pd.size(), max_n, kmax, rows, kp, d_be, ctx->d_pd,
+                          ctx->d_pd_exps, ctx->stream);
+  GW_CHECK_LAUNCH();
+  GW_TRY(cudaStreamSynchronize(ctx->stream));  // the host tables go out of scope
+  ctx->pd_ok = true;
+  return GW_OK;
+}
+
+// One batch in FP64 by digit products.  op_o, op_v: digits of G^occ, G^virt.
+int chi_one_batch_digits(gw_ctx* ctx, const Batch& b, const double* g_occ, const double* g_virt,
+                         const gw::EmuOp& op_o, const gw::EmuOp& op_v, double thr, double* acc,
+                         std::vector<double>& fc_host, size_t batch_idx) {
+  gw::TraceRange trace("chi: batch, FP64 digits");
+  const int ns = b.s1 - b.s0, prow = b.P1 - b.P0, n_at = ctx->n_at, nri = ctx->nri, nao = ctx->nao;
+  const long long Kb = b.Kb;
+  int rc, *d_err;
+  if (prow == 0 || Kb == 0) return GW_OK;
+  if ((rc = gw::emu_flag(ctx, &d_err))) return rc;
+  const int tm = gw::kEmuTileM, tn = gw::kEmuTileN;
+  double *X, *Y;
+  if ((rc = wsT(ctx, "X", (size_t)prow * Kb, &X)) || (rc = wsT(ctx, "Y", (size_t)nri * Kb, &Y))) return rc;
+  GW_TRY(cudaMemsetAsync(X, 0, (size_t)prow * Kb * sizeof(double), ctx->stream));
+  GW_TRY(cudaMemsetAsync(Y, 0, (size_t)nri * Kb * sizeof(double), ctx->stream));
+  // where every panel's lambda functions are all of them, G's own digits serve
+  bool whole = true;
+  for (const PanelDesc& d : ctx->panels) whole = whole && (d.K == 0 || d.K == nao);
+  const int r0 = ctx->ao_off[b.s0], R = ctx->ao_off[b.s1] - r0;
+  std::vector<gw::PanelTask64> tasks[2];
+  std::vector<int4> tiles[2];
+  for (int mode = 0; mode < 2; ++mode) {
+    const int first = mode == 0 ? b.s0 : 0, last = mode == 0 ? b.s1 : n_at;
+    const int grows = mode == 0 ? nao : R;  // G rows of a task
+    for (int s = first; s < last; ++s) {
+      const PanelDesc& d = ctx->panels[s];
+      if (d.K == 0) continue;
+      const int id = (int)tasks[mode].size();
+      gw::PanelTask64 t{};
+      t.panel_off = d.off;
+      t.seg = mode == 0 ? b.seg[s - b.s0] : 0;
+      t.p_row0 = (int)ctx->pd_row0[s];
+      t.g_row0 = whole ? (mode == 0 ? 0 : r0) : id * grows;
+      t.K = d.K;
+      t.N = d.npw * d.nsig;
+      t.npw = d.npw;
+      t.nsig = d.nsig;
+      t.p0 = d.p0;
+      t.aom = ctx->ao_off[s];
+      t.lam_off = d.lam_off;
+      tasks[mode].push_back(t);
+      const int na = mode == 0 ? t.N : grows, nb = mode == 0 ? grows : t.N;
+      for (int i = 0; i * tm < na; ++i)
+        for (int j = 0; j * tn < nb; ++j) tiles[mode].push_back(make_int4(id, i, j, 0));
+    }
+  }
+  std::vector<long long> rowbase(R);
+  std::vector<int> rowmul(R);
+  for (int s = b.s0; s < b.s1; ++s)
+    for (int i = 0; i < ctx->n_ao[s]; ++i) {
+      rowbase[ctx->ao_off[s] - r0 + i] = b.seg[s - b.s0] + i;
+      rowmul[ctx->ao_off[s] - r0 + i] = ctx->n_ao[s];
+    }
+  long long* d_rowbase;
+  int* d_rowmul;
+  if ((rc = upload(ctx, "rowbase", rowbase, &d_rowbase)) || (rc = upload(ctx, "rowmul", rowmul, &d_rowmul)))
+    return rc;
+  for (int mode = 0; mode < 2; ++mode) {
+    if (tasks[mode].empty()) continue;
+    const gw::EmuOp& op = mode == 0 ? op_o : op_v;
+    gw::PanelTask64* d_tasks;
+    int4* d_tiles;
+    if ((rc = upload(ctx, mode == 0 ? "d64_tasksA" : "d64_tasksB", tasks[mode], &d_tasks)) ||
+        (rc = upload(ctx, mode == 0 ? "d64_tilesA" : "d64_tilesB", tiles[mode], &d_tiles)))
+      return rc;
+    gw::Panel64Args p{};
+    p.tiles = d_tiles;
+    p.n_tiles = (int)tiles[mode].size();
+    p.mode = mode;
+    p.R = mode == 0 ? nao : R;
+    p.r0 = mode == 0 ? 0 : r0;
+    p.P0b = mode == 0 ? b.P0 : 0;
+    p.tasks = d_tasks;
+    p.ldk = Kb;
+    p.rowbase = d_rowbase;
+    p.rowmul = d_rowmul;
+    p.panel_dig = ctx->d_pd;
+    p.panel_exps = ctx->d_pd_exps;
+    p.panel_rows = ctx->pd_rows;
+    p.kp = ctx->pd_kp;
+    p.g_dig = op.dig;
+    p.g_exps = op.exps;
+    p.g_rows = nao;
+    p.g_kp = op.kp;
+    if (!whole) {
+      p.g_rows = (long long)tasks[mode].size() * p.R;
+      p.g_kp = ctx->pd_kp;
+      void* gg;
+      if ((rc = ws(ctx, "d64_gg", gw::emu_dig_bytes(p.g_rows, p.g_kp), &gg))) return rc;
+      gw::launch_gather_digits(op, p.r0, p.R, d_tasks, (int)tasks[mode].size(), ctx->d_lam, p.g_rows, p.g_kp, gg,
+                               ctx->stream);
+      p.g_dig = gg;
+      ctx->stats.kernel_launches += 1;
+    }
+    p.out = mode == 0 ? X : Y;
+    p.pool = ctx->d_panel64;
+    p.G = mode == 0 ? g_occ : g_virt;
+    p.lam = ctx->d_lam;
+    p.nao = nao;
+    if (gw::launch_panel64(p, d_err, ctx->stream))
+      return fail(ctx, GW_ERR_CUDA, "FP64 steps A/B: launch setup failed");
+    GW_CHECK_LAUNCH();
+    ctx->stats.kernel_launches += 1;
+  }
+  ctx->stats.bytes_operands += (double)(prow + nri) * Kb * sizeof(double);
+
+  // block filter of X and Y, occupancy flags, digits of what is kept
+  const int nslab = b.nslab;
+  const int npt = (prow + tm - 1) / tm, nqt = (nri + tn - 1) / tn, ntiles = npt * nqt;
+  int pa0 = 0;
+  while (ctx->ri_off[pa0 + 1] <= b.P0) ++pa0;
+  int pa1 = pa0;
+  while (pa1 < n_at && ctx->ri_off[pa1] < b.P1) ++pa1;
+  const int npa = pa1 - pa0;
+  unsigned char *bx, *by, *fx, *fy;
+  if ((rc = wsT(ctx, "bx", (size_t)ns * n_at * npa, &bx)) || (rc = wsT(ctx, "by", (size_t)ns * n_at * n_at, &by)) ||
+      (rc = wsT(ctx, "fx", (size_t)ns * n_at * npt, &fx)) || (rc = wsT(ctx, "fy", (size_t)ns * n_at * nqt, &fy)))
+    return rc;
+  GW_TRY(cudaMemsetAsync(fx, 0, (size_t)ns * n_at * npt, ctx->stream));
+  GW_TRY(cudaMemsetAsync(fy, 0, (size_t)ns * n_at * nqt, ctx->stream));
+  long long* d_seg;
+  int *d_nao, *d_nri;
+  if ((rc = upload(ctx, "seg", b.seg, &d_seg)) || (rc = upload(ctx, "n_ao_b", ctx->n_ao, &d_nao)) ||
+      (rc = upload(ctx, "n_ri_b", ctx->n_ri, &d_nri)))
+    return rc;
+  gw::launch_operand_block_filter<double>(X, Kb, b.P0, ctx->d_ri_off, ctx->d_ao_off, d_nao, b.s0, ns, d_seg, pa0,
+                                          npa, n_at, thr, ctx->naop, bx, fx, npt, tm, ctx->stream);
+  gw::launch_operand_block_filter<double>(Y, Kb, 0, ctx->d_ri_off, ctx->d_ao_off, d_nao, b.s0, ns, d_seg, 0, n_at,
+                                          n_at, thr, ctx->naop, by, fy, nqt, tn, ctx->stream);
+  GW_CHECK_LAUNCH();
+  gw::EmuOp ox, oy;
+  gw::EmuSrc sx;
+  sx.src = X;
+  sx.ld = Kb;
+  sx.rows = prow;
+  sx.K = (int)Kb;
+  gw::EmuSrc sy = sx;
+  sy.src = Y;
+  sy.rows = nri;
+  if ((rc = gw::emu_prep(ctx, "X", sx, &ox, ctx->stream)) || (rc = gw::emu_prep(ctx, "Y", sy, &oy, ctx->stream)))
+    return rc;
+  // task lists, work units, step C
+  std::vector<long long> slab_k0(nslab);
+  std::vector<int> slab_len(nslab);
+  const int per = ctx->naop / kSlabAO;
+  for (int sl = 0; sl < ns; ++sl)
+    for (int c = 0; c < per; ++c) {
+      const int nsig = ctx->n_ao[b.s0 + sl];
+      slab_k0[sl * per + c] = b.seg[sl] + (long long)c * kSlabAO * nsig;
+      slab_len[sl * per + c] = kSlabAO * nsig;
+    }
+  long long *d_k0, *kacc;
+  int *d_len, *tlist, *counts;
+  double* d_fc;
+  unsigned long long* tstat;
+  gw::UnitScratch w{};
+  const size_t cap = std::max<size_t>((size_t)ntiles * nslab, 1);
+  if ((rc = upload(ctx, "slab_k0", slab_k0, &d_k0)) || (rc = upload(ctx, "slab_len", slab_len, &d_len)) ||
+      (rc = wsT(ctx, "tasks", cap, &tlist)) || (rc = wsT(ctx, "counts", ntiles, &counts)) ||
+      (rc = wsT(ctx, "kacc", ntiles, &kacc)) || (rc = wsT(ctx, "fc", (size_t)ns * n_at, &d_fc)) ||
+      (rc = wsT(ctx, "task_stats", 3, &tstat)) || (rc = wsT(ctx, "u_ucnt", ntiles, &w.ucnt)) ||
+      (rc = wsT(ctx, "u_uoff", ntiles, &w.uoff)) || (rc = wsT(ctx, "u_ttile", cap, &w.t_tile)) ||
+      (rc = wsT(ctx, "u_tfirst", cap, &w.t_first)) || (rc = wsT(ctx, "u_tcount", cap, &w.t_count)) ||
+      (rc = wsT(ctx, "u_tkey", cap, &w.t_key)) || (rc = wsT(ctx, "u_tile", cap, &w.u_tile)) ||
+      (rc = wsT(ctx, "u_first", cap, &w.u_first)) || (rc = wsT(ctx, "u_count", cap, &w.u_count)) ||
+      (rc = wsT(ctx, "u_hist", std::max(nslab, 1), &w.hist)) ||
+      (rc = wsT(ctx, "u_start", std::max(nslab, 1), &w.start)) || (rc = wsT(ctx, "u_nunits", 1, &w.n_units)) ||
+      (rc = wsT(ctx, "u_nkeys", 1, &w.total_keys)))
+    return rc;
+  gw::launch_build_tasks(fx, fy, nslab, npt, nqt, b.P0, prow, 0, nri, ctx->d_atom_of_ri, d_len, tlist, counts, kacc,
+                         tm, tn, per, 0, n_at, 0, nao, ctx->d_atom_of_ao, ctx->stream);
+  gw::launch_count_c(bx, by, ns, 0, n_at, pa0, npa, 0, n_at, d_nri, d_nao, b.s0, d_fc, ctx->stream);
+  // Units of about 1/8 of an SM's share, at least 1024 elements (a unit's
+  // atomics cost about as much as 64); with many tiles a unit is a tile, and
+  // adds into chi itself.  Partial sums are integers, so either way chi is
+  // the same to the last bit, run after run.
+  int split = INT32_MAX;
+  if (ntiles < 152 * 16)
+    split = (int)std::min<double>(std::max(1024.0, 0.6 * ntiles * (double)Kb / (152 * 8)), 1 << 30);
+  void* part = nullptr;
+  if (split != INT32_MAX && (rc = ws(ctx, "d64_part", (size_t)prow * nri * 16, &part))) return rc;
+  GW_TRY(cudaMemsetAsync(tstat, 0, 3 * sizeof(unsigned long long), ctx->stream));
+  gw::launch_plan_units(tlist, counts, kacc, d_len, ntiles, nslab, split, w, tstat, ctx->stream);
+  GW_CHECK_LAUNCH();
+  cudaEvent_t ec0, ec1;
+  if ((rc = c_event_pair(ctx, 2 * batch_idx, &ec0, &ec1))) return rc;
+  GW_TRY(cudaEventRecord(ec0, ctx->stream));
+  gw::Chi64Args c{w, tlist, counts, nslab, nqt, b.P0, prow, nri, d_k0, d_len, acc, part};
+  if (gw::launch_chi64(ox, oy, c, d_err, ctx->stream))
+    return fail(ctx, GW_ERR_CUDA, "FP64 step C: launch setup failed");
+  GW_CHECK_LAUNCH();
+  GW_TRY(cudaEventRecord(ec1, ctx->stream));
+  ctx->stats.c_launches += 1;
+  ctx->stats.kernel_launches += 13;
+  std::vector<double> h_fc((size_t)ns * n_at);
+  unsigned long long h_stat[3];
+  GW_TRY(cudaMemcpyAsync(h_fc.data(), d_fc, h_fc.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+  GW_TRY(cudaMemcpyAsync(h_stat, tstat, sizeof(h_stat), cudaMemcpyDeviceToHost, ctx->stream));
+  GW_TRY(cudaStreamSynchronize(ctx->stream));
+  float ms_ck = 0.f;
+  GW_TRY(cudaEventElapsedTime(&ms_ck, ec0, ec1));
+  ctx->stats.ms_step_c_kernel += ms_ck;
+  ctx->stats.tiles_total += ntiles;
+  ctx->stats.tiles_active += (long long)h_stat[0];
+  ctx->stats.slabs_total += (long long)ntiles * nslab;
+  ctx->stats.slabs_active += (long long)h_stat[1];
+  for (double v : h_fc) fc_host.push_back(v);
+  ctx->stats.flops_issued += 2.0 * tm * tn * gw::kEmuProducts * (double)h_stat[2];
+  for (int mode = 0; mode < 2; ++mode)
+    for (const int4& t : tiles[mode])
+      ctx->stats.flops_issued += 2.0 * tm * tn * gw::kEmuProducts * ((tasks[mode][t.x].K + 31) / 32 * 32);
   return GW_OK;
 }
 
@@ -1416,7 +1705,7 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const double* g_occ, const dou
   if ((rc = wsT(ctx, "counts", (size_t)npt * nqt, &counts))) return rc;
   if ((rc = wsT(ctx, "kacc", (size_t)npt * nqt, &kacc))) return rc;
   gw::launch_build_tasks(fx, fy, nslab, npt, nqt, b.P0, prow, b.Q0, qrow, ctx->d_atom_of_ri, d_len,
-                         tasks, counts, kacc, tile, per, b.m0, nmc, b.mu0, b.nmu, ctx->d_atom_of_ao,
+                         tasks, counts, kacc, tile, tile, per, b.m0, nmc, b.mu0, b.nmu, ctx->d_atom_of_ao,
                          ctx->stream);
   double* d_fc;
   int* d_nri;
@@ -2128,13 +2417,16 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
   const int f16 = precision == GW_FP16X3;
   if (ctx->last_precision != precision) {
     ws_release_all(ctx);
+    if (!f64) free_panel_digits(ctx);
     ctx->last_precision = precision;
   }
+  if (f64 && (rc = ensure_panel_digits(ctx))) return rc;
+  const bool digits = f64 && ctx->pd_ok;
   if (!f64 && !tcpath && (rc = ensure_panel32(ctx))) return rc;
   if (tcpath && (rc = ensure_pt(ctx, precision == GW_BF16X6 ? 3 : 2, f16))) return rc;
   const int nao = ctx->nao, nri = ctx->nri, n_at = ctx->n_at;
-  // device bytes per operand element: FP64, FP32, or FP32 plus bf16 slices
-  const size_t esz = f64 ? sizeof(double)
+  // device bytes per operand element: FP64 (and its digits), FP32, or slices
+  const size_t esz = f64 ? (digits ? kDigitElem : sizeof(double))
                          : precision == GW_BF16X6 ? 6 : tcpath ? 4 : sizeof(float);
   std::vector<Batch> batches =
       tcpath ? plan_batches_tc(ctx, esz, ctx->batch_bytes, gw::tc_tile_rows())
@@ -2205,6 +2497,17 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
     GW_TRY(cudaEventRecord(ev[1], ctx->stream));
     std::vector<double> fc;
     if (tcpath && (rc = tc_begin_tau(ctx))) return rc;
+    gw::EmuOp op_o, op_v;  // digits of the filtered G
+    if (digits) {
+      gw::EmuSrc s;
+      s.src = go;
+      s.ld = s.rows = nao;
+      s.K = nao;
+      if ((rc = gw::emu_prep(ctx, "go", s, &op_o, ctx->stream))) return rc;
+      s.src = gv;
+      if ((rc = gw::emu_prep(ctx, "gv", s, &op_v, ctx->stream))) return rc;
+      ctx->stats.kernel_launches += 2;
+    }
     double fa = 0.0, fb = 0.0;
     std::vector<double> kao;
     int kao_m0 = -1;
@@ -2226,7 +2529,9 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
       }
       fa += ba;
       fb += bb;
-      if (f64)
+      if (digits)
+        rc = chi_one_batch_digits(ctx, b, go, gv, op_o, op_v, thr, acc, fc, bi);
+      else if (f64)
         rc = chi_one_batch<double>(ctx, b, go, gv, ctx->d_panel64, thr, acc, fc, precision, bi);
       else if (tcpath)
         rc = chi_one_batch_tc(ctx, b, go, gv, thr, acc, fc, precision, bi);

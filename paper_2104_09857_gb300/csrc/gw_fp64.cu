@@ -14,19 +14,19 @@ namespace gw {
 namespace {
 // digits of one operand held at a time by emu_product
 constexpr size_t kMaxDigits = size_t(4) << 30;
+}  // namespace
 
-int flag(gw_ctx* ctx, int** out) {
+int emu_flag(gw_ctx* ctx, int** err) {
   void* p;
   const int rc = work_buffer(ctx, "w.err", sizeof(int), &p);
-  *out = static_cast<int*>(p);
+  *err = static_cast<int*>(p);
   return rc;
 }
-}  // namespace
 
 int emu_begin(gw_ctx* ctx, cudaStream_t st) {
   int* err;
   int rc;
-  if ((rc = flag(ctx, &err))) return rc;
+  if ((rc = emu_flag(ctx, &err))) return rc;
   if (cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess) {
     ctx->err = "FP64 products: clearing the error flag failed";
     return GW_ERR_CUDA;
@@ -57,7 +57,7 @@ int emu_mm(gw_ctx* ctx, const EmuOp& A, const EmuOp& B, const EmuGemm& g, cudaSt
   int rc;
   const size_t bytes = emu_gemm_ws_bytes(A.s.rows, B.s.rows, A.s.K);
   if (bytes && (rc = work_buffer(ctx, "w.part", bytes, &ws))) return rc;
-  if ((rc = flag(ctx, &err))) return rc;
+  if ((rc = emu_flag(ctx, &err))) return rc;
   if (launch_emu_gemm(A, B, g, ws, err, st)) {
     ctx->err = "FP64 product: launch set-up failed";
     return GW_ERR_CUDA;
@@ -140,7 +140,7 @@ int greens_fp64(gw_ctx* ctx, double tau, double* cso, double* csv, double* g_occ
 int emu_end(gw_ctx* ctx, const char* call) {
   int* err;
   int rc, h = 0;
-  if ((rc = flag(ctx, &err))) return rc;
+  if ((rc = emu_flag(ctx, &err))) return rc;
   if (cudaMemcpy(&h, err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) {
     ctx->err = std::string(call) + ": reading the error flag failed";
     return GW_ERR_CUDA;

@@ -205,6 +205,14 @@ struct gw_ctx {
   int* d_lam = nullptr;
   long long lam_total = 0;
 
+  // the panels as digits for the FP64 products (row pd_row0[owner] + n)
+  bool pd_ok = false;
+  void* d_pd = nullptr;
+  int* d_pd_exps = nullptr;
+  long long pd_rows = 0;
+  int pd_kp = 0;
+  std::vector<long long> pd_row0;
+
   // transposed, split panels for the tensor-core steps A/B
   bool pt_ok = false;
   int pt_slices = 0, pt_f16 = 0;

@@ -358,7 +358,7 @@ extern "C" int gw_chi_tau_noalloc(gw_ctx* ctx, int tau_index, double thr, double
                                             d_seg, 0, n_at, n_at, thr, naop, by, fy, nqt, 64, st);
     NA_LAUNCHED();
     gw::launch_build_tasks(fx, fy, nslab, npt, nqt, b.P0, prow, 0, nri, ctx->d_atom_of_ri, d_len, tasks,
-                           counts, kacc, 64, per, 0, n_at, 0, nao, ctx->d_atom_of_ao, st);
+                           counts, kacc, 64, 64, per, 0, n_at, 0, nao, ctx->d_atom_of_ao, st);
     gw::launch_chi_tiles<double, double>(X, Y, Kb, b.P0, prow, nri, tasks, counts, nslab, npt, nqt,
                                          d_k0, d_len, acc, st);
     NA_LAUNCHED();

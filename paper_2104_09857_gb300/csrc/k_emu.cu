@@ -218,6 +218,75 @@ __global__ void __launch_bounds__(256) k_prep_cols(const double* __restrict__ sr
     *reinterpret_cast<uint4*>(dig + (i * rows + r) * kp + k0 + 8 * g) = q[i];
 }
 
+// The same for the owner panels of the 3c tensor ([K][N] each, blockIdx.z =
+// panel): operand row row0[panel] + n, pitch kp.
+__global__ void __launch_bounds__(256) k_panel_exps(const double* __restrict__ pool, const PanelDesc* __restrict__ pd,
+                                                    const long long* __restrict__ row0, int* __restrict__ be) {
+  const PanelDesc d = pd[blockIdx.z];
+  const int N = d.npw * d.nsig;
+  if (static_cast<int>(blockIdx.x) * 32 >= N) return;
+  const int c = threadIdx.x & 31, kk = threadIdx.x >> 5;
+  const int col = blockIdx.x * 32 + c;
+  int m = 0;
+  if (col < N)
+    for (int k = blockIdx.y * 8 + kk; k < d.K; k += 8 * gridDim.y)
+      m = max(m, biased_exp(pool[d.off + static_cast<long long>(k) * N + col]));
+  __shared__ int red[8][32];
+  red[kk][c] = m;
+  __syncthreads();
+  if (kk == 0 && col < N) {
+#pragma unroll
+    for (int i = 1; i < 8; ++i) m = max(m, red[i][c]);
+    if (m) atomicMax(be + row0[blockIdx.z] + col, m);
+  }
+}
+__global__ void __launch_bounds__(256) k_panel_prep(const double* __restrict__ pool, const PanelDesc* __restrict__ pd,
+                                                    const long long* __restrict__ row0, long long rows, int kp,
+                                                    const int* __restrict__ be, __half* __restrict__ dig,
+                                                    int* __restrict__ exps) {
+  const PanelDesc d = pd[blockIdx.z];
+  const int N = d.npw * d.nsig, c0 = blockIdx.x * 32, k0 = blockIdx.y * 64;
+  if (c0 >= N || k0 >= d.K) return;
+  __shared__ double t[64][33];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int k = (threadIdx.x >> 5) + 8 * i, c = threadIdx.x & 31;
+    t[k][c] = (k0 + k < d.K && c0 + c < N) ? pool[d.off + static_cast<long long>(k0 + k) * N + c0 + c] : 0.0;
+  }
+  __syncthreads();
+  const int c = threadIdx.x >> 3, g = threadIdx.x & 7;
+  if (c0 + c >= N) return;
+  const long long r = row0[blockIdx.z] + c0 + c;
+  const int e = row_exp(be[r]);
+  if (blockIdx.y == 0 && g == 0) exps[r] = e;
+  double v[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = t[8 * g + i][c];
+  uint4 q[kS];
+  digits8(v, e, q);
+#pragma unroll
+  for (int i = 0; i < kS; ++i) *reinterpret_cast<uint4*>(dig + (i * rows + r) * kp + k0 + 8 * g) = q[i];
+}
+
+// Digits of G gathered on each task's lambda functions: out row
+// g_row0 + r, column k = digits of G[rbase + r][lam[lam_off + k]], zero for
+// k >= K up to the task's last 64 columns.  blockIdx.y = task, z = digit.
+__global__ void __launch_bounds__(256) k_gather_digits(const __half* __restrict__ g, int nao, int gkp, int rbase,
+                                                       int R, const PanelTask64* __restrict__ tasks,
+                                                       const int* __restrict__ lam, long long out_rows, int kp,
+                                                       __half* __restrict__ out) {
+  const PanelTask64 tk = tasks[blockIdx.y];
+  const int kt = (tk.K + 63) / 64 * 64;
+  const __half* src = g + (static_cast<long long>(blockIdx.z) * nao + rbase) * gkp;
+  __half* dst = out + (blockIdx.z * out_rows + tk.g_row0) * kp;
+  const int n = R * kt;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int r = i / kt, k = i - r * kt;
+    dst[static_cast<long long>(r) * kp + k] =
+        k < tk.K ? src[static_cast<long long>(r) * gkp + lam[tk.lam_off + k]] : __half(0.f);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // integers back to FP64
 // ---------------------------------------------------------------------------
@@ -369,6 +438,212 @@ __global__ void k_gemm_finish(const GemmJob j) {
     j.store(r, c, a == kBad || b == kBad ? j.direct(r, c)
                                          : fixed_to_double(static_cast<long long>(v.x), static_cast<long long>(v.y),
                                                            a + b + kUnit));
+  }
+}
+
+// ---------------------------------------------------------------------------
+// steps A / B of Eq. 3 in FP64: one tile = 128 rows of the A operand x 64 of
+// the B operand of one panel task
+//   mode 0 (X): A = panel rows n = (pw, s'), B = G^occ rows mu
+//   mode 1 (Y): A = G^virt rows sigma (batch), B = panel rows n = (pw, mu')
+// A thread owns one A row, so consecutive lanes write along the contiguous
+// index of the operand's K layout (s, mu, s').
+// ---------------------------------------------------------------------------
+struct Panel64Job {
+  const int4* tiles;  // (task, A tile, B tile, 0)
+  int n_tiles, mode, R, r0, P0b;
+  const PanelTask64* tasks;
+  long long ldk;
+  const long long* rowbase;
+  const int* rowmul;
+  const int *pe, *ge;  // exponents of the panel rows and of G's rows
+  double* out;
+  const double *pool, *G;
+  const int* lam;
+  int nao;
+  struct Tile {
+    int ya, yb, n, task, a0, b0;
+  };
+  __device__ int items() const { return n_tiles; }
+  __device__ Tile tile(int t) const {
+    const int4 e = tiles[t];
+    const PanelTask64& tk = tasks[e.x];
+    Tile T;
+    T.task = e.x;
+    T.a0 = e.y * kM;
+    T.b0 = e.z * kN;
+    T.ya = (mode == 0 ? tk.p_row0 : tk.g_row0) + T.a0;
+    T.yb = (mode == 0 ? tk.g_row0 : tk.p_row0) + T.b0;
+    T.n = (tk.K + kChunk - 1) / kChunk;
+    return T;
+  }
+  __device__ int nchunks(const Tile& T) const { return T.n; }
+  struct Iter {
+    int x;
+    __device__ void init(const Panel64Job*, const Tile&) { x = 0; }
+    __device__ int next() {
+      const int v = x;
+      x += kChunk;
+      return v;
+    }
+  };
+  // panel row n against G row r (global AO) from the FP64 values
+  __device__ double direct(const PanelTask64& tk, int n, int r) const {
+    double s = 0.0;
+    for (int k = 0; k < tk.K; ++k)
+      s = fma(G[static_cast<long long>(lam[tk.lam_off + k]) * nao + r],
+              pool[tk.panel_off + static_cast<long long>(k) * tk.N + n], s);
+    return s;
+  }
+  __device__ void write(long long (&hi)[kCols], long long (&lo)[kCols], const Tile& T, int row, int c0) const {
+    const PanelTask64& tk = tasks[T.task];
+    const int a = T.a0 + row, b = T.b0 + c0;
+    const int nsig = tk.nsig;
+    unsigned bad = 0;
+    if (mode == 0) {
+      if (a >= tk.N) return;
+      const int pw = a / nsig, sp = a - pw * nsig;
+      const int ea = pe[tk.p_row0 + a];
+      double* o = out + static_cast<long long>(tk.p0 + pw - P0b) * ldk + tk.seg + sp;
+#pragma unroll
+      for (int j = 0; j < kCols; ++j) {
+        const int mu = b + j;
+        if (mu >= R) break;
+        const int eb = ge[r0 + mu];
+        if (ea == kBad || eb == kBad)
+          bad |= 1u << j;
+        else
+          o[static_cast<long long>(r0 + mu) * nsig] = fixed_to_double(hi[j], lo[j], ea + eb + kUnit);
+      }
+      for (; bad; bad &= bad - 1) {
+        const int mu = b + __ffs(bad) - 1;
+        o[static_cast<long long>(r0 + mu) * nsig] = direct(tk, a, r0 + mu);
+      }
+    } else {
+      if (a >= R) return;
+      const int ea = ge[r0 + a];
+      const long long rb = rowbase[a], rm = rowmul[a];
+      int pw = b / nsig, sp = b - pw * nsig;
+      double* o = out + static_cast<long long>(tk.p0 + pw - P0b) * ldk + rb + tk.aom * rm;
+#pragma unroll
+      for (int j = 0; j < kCols; ++j) {
+        const int n = b + j;
+        if (n >= tk.N) break;
+        const int eb = pe[tk.p_row0 + n];
+        o[sp * rm] = (ea == kBad || eb == kBad) ? direct(tk, n, r0 + a)
+                                                : fixed_to_double(hi[j], lo[j], ea + eb + kUnit);
+        if (++sp == nsig) {
+          sp = 0;
+          o += ldk;
+        }
+      }
+    }
+  }
+};
+
+// ---------------------------------------------------------------------------
+// step C in FP64: chi[P][Q] -= sum over the unit's slabs of X[P][k] Y[Q][k]
+// ---------------------------------------------------------------------------
+struct Chi64Job {
+  const int *unit_tile, *unit_first, *unit_count, *n_units;
+  const int* tasks;
+  const int* counts;
+  int nslab, nqt, P0, prow, nri;
+  const long long* slab_k0;
+  const int* slab_len;
+  const int *ex, *ey;
+  double* chi;
+  unsigned long long* part;  // units of one tile add here; null: a unit is a whole tile
+  const double *X, *Y;
+  long long ldk;
+  struct Tile {
+    int ya, yb, n, cnt, id;
+    const int* list;
+  };
+  __device__ int items() const { return *n_units; }
+  __device__ Tile tile(int u) const {
+    Tile T;
+    T.id = unit_tile[u];
+    T.ya = T.id / nqt * kM;
+    T.yb = T.id % nqt * kN;
+    T.cnt = unit_count[u];
+    T.list = tasks + static_cast<long long>(T.id) * nslab + unit_first[u];
+    T.n = 0;
+    for (int i = 0; i < T.cnt; ++i) T.n += slab_len[T.list[i]] / kChunk;
+    return T;
+  }
+  __device__ int nchunks(const Tile& T) const { return T.n; }
+  struct Iter {
+    const Chi64Job* j;
+    const int* list;
+    int cnt, i, kk, len;
+    long long k0;
+    __device__ void init(const Chi64Job* jj, const Tile& T) {
+      j = jj;
+      list = T.list;
+      cnt = T.cnt;
+      i = kk = 0;
+      len = cnt > 0 ? j->slab_len[list[0]] : 0;
+      k0 = cnt > 0 ? j->slab_k0[list[0]] : 0;
+    }
+    __device__ int next() {
+      const int x = static_cast<int>(k0 + kk);
+      kk += kChunk;
+      if (kk >= len) {
+        ++i;
+        kk = 0;
+        if (i < cnt) {
+          len = j->slab_len[list[i]];
+          k0 = j->slab_k0[list[i]];
+        }
+      }
+      return x;
+    }
+  };
+  // the element from the FP64 operands, over the tile's whole list
+  __device__ double direct(int id, int p, int q) const {
+    double s = 0.0;
+    const int* l = tasks + static_cast<long long>(id) * nslab;
+    for (int i = 0; i < counts[id]; ++i)
+      for (int k = 0; k < slab_len[l[i]]; ++k)
+        s = fma(X[p * ldk + slab_k0[l[i]] + k], Y[q * ldk + slab_k0[l[i]] + k], s);
+    return s;
+  }
+  __device__ void add(int id, int p, int q, long long hi, long long lo) const {
+    const int a = ex[p], b = ey[q];
+    double* c = chi + static_cast<long long>(P0 + p) * nri + q;
+    *c -= (a == kBad || b == kBad) ? direct(id, p, q) : fixed_to_double(hi, lo, a + b + kUnit);
+  }
+  __device__ void write(long long (&hi)[kCols], long long (&lo)[kCols], const Tile& T, int row, int c0) const {
+    const int p = T.ya + row;
+    if (p >= prow) return;
+    if (part) {
+      unsigned long long* o = part + (static_cast<long long>(p) * nri + T.yb + c0) * 2;
+#pragma unroll
+      for (int j = 0; j < kCols; ++j) {
+        if (T.yb + c0 + j >= nri) break;
+        carry(hi[j], lo[j]);
+        atomicAdd(o + 2 * j, static_cast<unsigned long long>(hi[j]));
+        atomicAdd(o + 2 * j + 1, static_cast<unsigned long long>(lo[j]));
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < kCols; ++j) {
+        if (T.yb + c0 + j >= nri) break;
+        add(T.id, p, T.yb + c0 + j, hi[j], lo[j]);
+      }
+    }
+  }
+};
+__global__ void k_chi64_finish(const Chi64Job j) {
+  const long long n = static_cast<long long>(j.prow) * j.nri;
+  for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
+       i += static_cast<long long>(gridDim.x) * blockDim.x) {
+    const int p = static_cast<int>(i / j.nri), q = static_cast<int>(i % j.nri);
+    const int id = p / kM * j.nqt + q / kN;
+    if (j.counts[id] == 0) continue;
+    const ulonglong2 v = reinterpret_cast<const ulonglong2*>(j.part)[i];
+    j.add(id, p, q, static_cast<long long>(v.x), static_cast<long long>(v.y));
   }
 }
 
@@ -695,6 +970,60 @@ int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, 
   if (j.ks > 1) {
     const long long blocks = (static_cast<long long>(m) * n + 255) / 256;
     emu::k_gemm_finish<<<static_cast<unsigned>(std::min<long long>(blocks, 152 * 16)), 256, 0, st>>>(j);
+  }
+  return 0;
+}
+
+void launch_panel_digits(const double* pool, const PanelDesc* panels, const long long* row0, int n_panels, int max_n,
+                         int max_k, long long rows, int kp, int* be, void* dig, int* exps, cudaStream_t st) {
+  if (n_panels == 0 || max_n == 0) return;
+  cudaMemsetAsync(be, 0, static_cast<size_t>(rows) * sizeof(int), st);
+  const unsigned gx = (max_n + 31) / 32, gy = (max_k + 63) / 64;
+  for (int z = 0; z < n_panels; z += 65535) {
+    const unsigned nz = std::min(n_panels - z, 65535);
+    emu::k_panel_exps<<<dim3(gx, std::min(gy, 4u), nz), 256, 0, st>>>(pool, panels + z, row0 + z, be);
+    emu::k_panel_prep<<<dim3(gx, gy, nz), 256, 0, st>>>(pool, panels + z, row0 + z, rows, kp, be,
+                                                        static_cast<__half*>(dig), exps);
+  }
+}
+
+void launch_gather_digits(const EmuOp& g, int rbase, int R, const PanelTask64* tasks, int n_tasks, const int* lam,
+                          long long out_rows, int kp, void* out, cudaStream_t st) {
+  if (n_tasks == 0 || R == 0) return;
+  const unsigned bx = static_cast<unsigned>(std::min<long long>((static_cast<long long>(R) * kp + 255) / 256, 256));
+  for (int t = 0; t < n_tasks; t += 65535)
+    emu::k_gather_digits<<<dim3(bx, std::min(n_tasks - t, 65535), kEmuSlices), 256, 0, st>>>(
+        static_cast<const __half*>(g.dig), static_cast<int>(g.stride_rows), g.kp, rbase, R, tasks + t, lam, out_rows,
+        kp, static_cast<__half*>(out));
+}
+
+int launch_panel64(const Panel64Args& p, int* err_flag, cudaStream_t st) {
+  if (p.n_tiles == 0) return 0;
+  CUtensorMap mp, mg;
+  const bool x = p.mode == 0;
+  if (make_digit_map(&mp, p.panel_dig, p.kp, p.panel_rows, p.panel_rows, kEmuSlices, emu::kChunk,
+                     x ? emu::kM : emu::kN) ||
+      make_digit_map(&mg, p.g_dig, p.g_kp, p.g_rows, p.g_rows, kEmuSlices, emu::kChunk, x ? emu::kN : emu::kM))
+    return -2;
+  emu::Panel64Job j{p.tiles, p.n_tiles, p.mode, p.R,  p.r0,   p.P0b, p.tasks, p.ldk, p.rowbase,
+                    p.rowmul, p.panel_exps, p.g_exps, p.out, p.pool, p.G, p.lam, p.nao};
+  return x ? emu::launch(mp, mg, j, p.n_tiles, err_flag, st) : emu::launch(mg, mp, j, p.n_tiles, err_flag, st);
+}
+
+int launch_chi64(const EmuOp& x, const EmuOp& y, const Chi64Args& c, int* err_flag, cudaStream_t st) {
+  CUtensorMap mx, my;
+  if (make_digit_map(&mx, x.dig, x.kp, x.s.rows, x.stride_rows, kEmuSlices, emu::kChunk, emu::kM) ||
+      make_digit_map(&my, y.dig, y.kp, y.s.rows, y.stride_rows, kEmuSlices, emu::kChunk, emu::kN))
+    return -2;
+  emu::Chi64Job j{c.units.u_tile, c.units.u_first, c.units.u_count, c.units.n_units, c.tasks, c.counts, c.nslab,
+                  c.nqt, c.P0, c.prow, c.nri, c.slab_k0, c.slab_len, x.exps, y.exps, c.chi,
+                  static_cast<unsigned long long*>(c.part), x.s.src, y.s.src, x.s.ld};
+  if (c.part) cudaMemsetAsync(c.part, 0, static_cast<size_t>(c.prow) * c.nri * 16, st);
+  const int rc = emu::launch(mx, my, j, INT32_MAX, err_flag, st);
+  if (rc) return rc;
+  if (c.part) {
+    const long long blocks = (static_cast<long long>(c.prow) * c.nri + 255) / 256;
+    emu::k_chi64_finish<<<static_cast<unsigned>(std::min<long long>(blocks, 152 * 16)), 256, 0, st>>>(j);
   }
   return 0;
 }

@@ -6,10 +6,12 @@
 #include <cuda_runtime.h>
 
 #include "gw_internal.h"
+#include "k_tc.h"
 
 namespace gw {
 
 constexpr int kEmuSlices = 8;   // digits per operand element
+constexpr int kEmuProducts = 36;  // digit pairs of a product
 constexpr int kEmuTileM = 128;  // rows (A operand) and columns (B operand) of a tile
 constexpr int kEmuTileN = 64;
 
@@ -69,9 +71,60 @@ size_t emu_gemm_ws_bytes(long long m, long long n, int K);
 int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, int* err_flag,
                     cudaStream_t st);
 
+// One panel problem of the FP64 steps A / B: digits of the panel's rows from
+// p_row0, of G's rows (gathered on its lambda functions) from g_row0.
+struct PanelTask64 {
+  long long panel_off, seg;  // seg: K offset of the owner's segment in X (mode 0)
+  int p_row0, g_row0, K, N, npw, nsig, p0, aom, lam_off, pad;
+};
+// Digits of all owner panels ([K][N] each in pool): rows row0[i].., pitch kp;
+// be, exps: one int per row.
+void launch_panel_digits(const double* pool, const PanelDesc* panels, const long long* row0, int n_panels, int max_n,
+                         int max_k, long long rows, int kp, int* be, void* dig, int* exps, cudaStream_t st);
+// Digits of G gathered per task: rows rbase .. rbase + R of g to rows g_row0..
+void launch_gather_digits(const EmuOp& g, int rbase, int R, const PanelTask64* tasks, int n_tasks, const int* lam,
+                          long long out_rows, int kp, void* out, cudaStream_t st);
+// Steps A (mode 0, X) and B (mode 1, Y): rows r0 .. r0 + R of G, output as
+// k_panel_gemm's (k_simt.cu).
+struct Panel64Args {
+  const int4* tiles;  // (task, A tile of 128 rows, B tile of 64, 0)
+  int n_tiles, mode, R, r0, P0b;
+  const PanelTask64* tasks;
+  long long ldk;
+  const long long* rowbase;
+  const int* rowmul;
+  const void* panel_dig;
+  const int* panel_exps;
+  long long panel_rows;
+  int kp;
+  const void* g_dig;
+  const int* g_exps;
+  long long g_rows;
+  int g_kp;
+  double* out;
+  const double *pool, *G;
+  const int* lam;
+  int nao;
+};
+int launch_panel64(const Panel64Args& p, int* err_flag, cudaStream_t st);
+// Step C over work units (k_tc.h, launch_plan_units) of 128 x 64 tiles.  part:
+// 16 bytes per (X row, RI function) of partial sums, or null when a unit is a
+// whole tile.
+struct Chi64Args {
+  UnitScratch units;
+  const int *tasks, *counts;
+  int nslab, nqt, P0, prow, nri;
+  const long long* slab_k0;
+  const int* slab_len;
+  double* chi;
+  void* part;
+};
+int launch_chi64(const EmuOp& x, const EmuOp& y, const Chi64Args& c, int* err_flag, cudaStream_t st);
+
 // The same on the work buffers of a context (gw_fp64.cu).  Between emu_begin
 // and emu_end of one call; names tell apart operands in use together.
 int emu_begin(gw_ctx* ctx, cudaStream_t st);
+int emu_flag(gw_ctx* ctx, int** err);  // the error flag of the launchers
 int emu_prep(gw_ctx* ctx, const char* name, const EmuSrc& s, EmuOp* op, cudaStream_t st);
 int emu_mm(gw_ctx* ctx, const EmuOp& A, const EmuOp& B, const EmuGemm& g, cudaStream_t st);
 // Product of two matrices.  Operands beyond 4 GB of digits go in row chunks;

@@ -417,12 +417,12 @@ __global__ void k_build_tasks(const unsigned char* __restrict__ fx, const unsign
                               int nslab, int npt, int nqt, int P0, int prow, int Q0, int qrow,
                               const int* __restrict__ atom_of_ri, const int* __restrict__ slab_len,
                               int* __restrict__ tasks, int* __restrict__ counts,
-                              long long* __restrict__ kacc, int tile_rows, int per, int m0, int nmc,
-                              int mu0, int nmu, const int* __restrict__ atom_of_ao) {
+                              long long* __restrict__ kacc, int tile_rows, int tile_cols, int per,
+                              int m0, int nmc, int mu0, int nmu, const int* __restrict__ atom_of_ao) {
   int tile = blockIdx.x;
   int pt = tile / nqt, qt = tile % nqt;
   int pfirst = P0 + pt * tile_rows;
-  int qlast = Q0 + min(qrow, (qt + 1) * tile_rows) - 1;
+  int qlast = Q0 + min(qrow, (qt + 1) * tile_cols) - 1;
   bool upper = atom_of_ri[pfirst] <= atom_of_ri[qlast];
   // warp-serial compaction in slab order (deterministic)
   if (threadIdx.x >= 32) return;
@@ -588,11 +588,11 @@ template void launch_operand_block_filter<float>(float*, long long, int, const i
 void launch_build_tasks(const unsigned char* fx, const unsigned char* fy, int nslab, int npt,
                         int nqt, int P0, int prow, int Q0, int qrow, const int* atom_of_ri,
                         const int* slab_len, int* tasks, int* counts, long long* kacc,
-                        int tile_rows, int per, int m0, int nmc, int mu0, int nmu,
+                        int tile_rows, int tile_cols, int per, int m0, int nmc, int mu0, int nmu,
                         const int* atom_of_ao, cudaStream_t st) {
   if (npt * nqt == 0) return;
   k_build_tasks<<<npt * nqt, 32, 0, st>>>(fx, fy, nslab, npt, nqt, P0, prow, Q0, qrow, atom_of_ri,
-                                          slab_len, tasks, counts, kacc, tile_rows, per, m0, nmc, mu0,
+                                          slab_len, tasks, counts, kacc, tile_rows, tile_cols, per, m0, nmc, mu0,
                                           nmu, atom_of_ao);
 }
 

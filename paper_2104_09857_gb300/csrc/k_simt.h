@@ -40,7 +40,7 @@ void launch_operand_block_filter(T* Z, long long ldk, int rowoff, const int* ri_
 void launch_build_tasks(const unsigned char* fx, const unsigned char* fy, int nslab, int npt,
                         int nqt, int P0, int prow, int Q0, int qrow, const int* atom_of_ri,
                         const int* slab_len, int* tasks, int* counts, long long* kacc,
-                        int tile_rows, int per, int m0, int nmc, int mu0, int nmu,
+                        int tile_rows, int tile_cols, int per, int m0, int nmc, int mu0, int nmu,
                         const int* atom_of_ao, cudaStream_t st);
 void launch_count_c(const unsigned char* bx, const unsigned char* by, int ns, int m0, int nmc, int pa0,
                     int npa, int qa0, int nqa, const int* n_ri, const int* n_ao, int s0, double* out,
