@@ -2,6 +2,7 @@
 // (Eq. 7, with V = L L^T, Eq. 8) -> W^c(i omega) (Eq. 9) -> W^c(i tau).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <string>
 #include <vector>
@@ -78,12 +79,16 @@ extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const doub
   gw::WorkTrim trim{ctx};
   const size_t nn = (size_t)n * n;
   DevBuf b_chi, b_w;
-  // V, its factor L, [eps; L] and one product share the context's work buffers
+  // V, its factor L, [eps; L] of nb frequencies and one product share the
+  // context's work buffers.  nb frequencies are factored together: all of
+  // them within 1 GB (the sweep's chain of small kernels is then paid once),
+  // one at a time for large matrices, whose sweeps fill the chip by themselves.
+  const int nb = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_omega, (size_t(1) << 30) / (2 * nn * 8)));
   double *v, *low, *m, *t, *ww, *g, *d;
   int* err;
   int rc;
   if ((rc = chain_buffer(ctx, "w.v", nn, &v)) || (rc = chain_buffer(ctx, "w.low", nn, &low)) ||
-      (rc = chain_buffer(ctx, "w.eps_l", 2 * nn, &m)) || (rc = chain_buffer(ctx, "w.t", nn, &t)) ||
+      (rc = chain_buffer(ctx, "w.eps_l", 2 * nn * nb, &m)) || (rc = chain_buffer(ctx, "w.t", nn, &t)) ||
       (rc = chain_buffer(ctx, "w.ww", nn, &ww)) ||
       (rc = chain_buffer(ctx, "w.gamma", (size_t)n_omega * n_tau, &g)) ||
       (rc = chain_buffer(ctx, "w.delta", (size_t)n_omega * n_tau, &d)) ||
@@ -111,7 +116,7 @@ extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const doub
   CH_TRY(cudaMemcpyAsync(d, delta, (size_t)n_omega * n_tau * 8, cudaMemcpyHostToDevice, st));
   // V = L L^T (Eq. 8)
   CH_TRY(cudaMemcpyAsync(low, v, nn * 8, cudaMemcpyDeviceToDevice, st));
-  if ((rc = gw::chain_cholesky(ctx, low, n, n, err, st))) return rc;
+  if ((rc = gw::chain_cholesky(ctx, low, n, n, 1, 0, err, st))) return rc;
   int h_err = 0;
   CH_TRY(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CH_TRY(cudaStreamSynchronize(st));
@@ -126,36 +131,42 @@ extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const doub
   s_lt.K = s_row.K = n;
   s_lt.trans = true;
   gw::EmuOp lt;  // digits of L^T, made once
-  for (int k = 0; k < n_omega; ++k) {
-    // chi(i omega_k) = sum_j gamma_kj chi(i tau_j)
-    gw::chain_lincomb(chi, n_tau, g + (size_t)k * n_tau, (long long)nn, t, st);
-    // (chi L)^T = L^T chi^T by rows, then eps = 1 - L^T (chi L)  (Eq. 7), its
-    // lower triangle; row r of L^T starts at column r
-    gw::EmuGemm p;
-    p.C = ww;
-    p.ldc = n;
-    p.ktri = 1;
-    s_row.src = t;
-    if ((rc = gw::emu_product(ctx, s_lt, s_row, p, &lt, st))) return rc;
-    p.alpha = -1.0;
-    p.C = m;
-    p.tri = 1;
-    s_row.src = ww;
-    if ((rc = gw::emu_product(ctx, s_lt, s_row, p, &lt, st))) return rc;
-    gw::chain_add_diagonal(m, n, 1.0, st);
+  for (int k0 = 0; k0 < n_omega; k0 += nb) {
+    const int nk = std::min(nb, n_omega - k0);
+    for (int k = k0; k < k0 + nk; ++k) {
+      double* mk = m + (size_t)(k - k0) * 2 * nn;
+      // chi(i omega_k) = sum_j gamma_kj chi(i tau_j)
+      gw::chain_lincomb(chi, n_tau, g + (size_t)k * n_tau, (long long)nn, t, st);
+      // (chi L)^T = L^T chi^T by rows, then eps = 1 - L^T (chi L)  (Eq. 7), its
+      // lower triangle; row r of L^T starts at column r
+      gw::EmuGemm p;
+      p.C = ww;
+      p.ldc = n;
+      p.ktri = 1;
+      s_row.src = t;
+      if ((rc = gw::emu_product(ctx, s_lt, s_row, p, &lt, st))) return rc;
+      p.alpha = -1.0;
+      p.C = mk;
+      p.tri = 1;
+      s_row.src = ww;
+      if ((rc = gw::emu_product(ctx, s_lt, s_row, p, &lt, st))) return rc;
+      gw::chain_add_diagonal(mk, n, 1.0, st);
+      CH_TRY(cudaMemcpyAsync(mk + nn, low, nn * 8, cudaMemcpyDeviceToDevice, st));
+    }
     // eps = R R^T with L below it: its rows become L R^-T = Z, and
     // W^c = Z Z^T - V  (Eq. 9), lower triangle
-    CH_TRY(cudaMemcpyAsync(m + nn, low, nn * 8, cudaMemcpyDeviceToDevice, st));
-    if ((rc = gw::chain_cholesky(ctx, m, 2LL * n, n, err, st))) return rc;
-    gw::EmuGemm q;
-    q.C = ww;
-    q.ldc = n;
-    q.tri = 1;
-    s_row.src = m + nn;
-    if ((rc = square(ctx, s_row, q, st))) return rc;
-    // W^c(i tau_j) += delta_jk W^c(i omega_k)
-    gw::chain_add_symmetric(ww, v, d + k, n_omega, n_tau, n, wout, st);
-    CH_TRY(cudaGetLastError());
+    if ((rc = gw::chain_cholesky(ctx, m, 2LL * n, n, nk, 2LL * nn, err, st))) return rc;
+    for (int k = k0; k < k0 + nk; ++k) {
+      gw::EmuGemm q;
+      q.C = ww;
+      q.ldc = n;
+      q.tri = 1;
+      s_row.src = m + (size_t)(k - k0) * 2 * nn + nn;
+      if ((rc = square(ctx, s_row, q, st))) return rc;
+      // W^c(i tau_j) += delta_jk W^c(i omega_k)
+      gw::chain_add_symmetric(ww, v, d + k, n_omega, n_tau, n, wout, st);
+      CH_TRY(cudaGetLastError());
+    }
   }
   CH_TRY(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));
   if (!out_on_device)
@@ -218,7 +229,7 @@ extern "C" int gw_ri_metric(gw_ctx* ctx, const double* S, int n_mat, const doubl
   CH_TRY(cudaMemcpyAsync(r, S, nn * 8, cudaMemcpyHostToDevice, st));
   // [S; 1] -> [R; R^-T]
   gw::chain_set_identity(r + nn, n, st);
-  if ((rc = gw::chain_cholesky(ctx, r, 2LL * n, n, err, st))) return rc;
+  if ((rc = gw::chain_cholesky(ctx, r, 2LL * n, n, 1, 0, err, st))) return rc;
   int h_err = 0;
   CH_TRY(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CH_TRY(cudaStreamSynchronize(st));

@@ -38,9 +38,9 @@ int emu_prep(gw_ctx* ctx, const char* name, const EmuSrc& s, EmuOp* op, cudaStre
   void* p;
   int rc;
   const std::string n = std::string("w.dig.") + name;
-  if ((rc = work_buffer(ctx, n.c_str(), std::max<size_t>(emu_dig_bytes(s.rows, s.K), 16), &p))) return rc;
+  if ((rc = work_buffer(ctx, n.c_str(), std::max<size_t>(emu_dig_bytes(s.rows * s.nz, s.K), 16), &p))) return rc;
   op->dig = p;
-  if ((rc = work_buffer(ctx, (n + ".e").c_str(), std::max<size_t>(s.rows, 1) * 2 * sizeof(int), &p))) return rc;
+  if ((rc = work_buffer(ctx, (n + ".e").c_str(), std::max<size_t>(s.rows * s.nz, 1) * 2 * sizeof(int), &p))) return rc;
   op->exps = static_cast<int*>(p);
   launch_emu_prep(*op, s, st);
   const cudaError_t e = cudaGetLastError();
@@ -55,7 +55,7 @@ int emu_mm(gw_ctx* ctx, const EmuOp& A, const EmuOp& B, const EmuGemm& g, cudaSt
   void* ws = nullptr;
   int* err;
   int rc;
-  const size_t bytes = emu_gemm_ws_bytes(A.s.rows, B.s.rows, A.s.K);
+  const size_t bytes = emu_gemm_ws_bytes(A.s.rows, B.s.rows, A.s.K, A.s.nz);
   if (bytes && (rc = work_buffer(ctx, "w.part", bytes, &ws))) return rc;
   if ((rc = emu_flag(ctx, &err))) return rc;
   if (launch_emu_gemm(A, B, g, ws, err, st)) {

@@ -78,89 +78,111 @@ __global__ void k_set_identity(double* __restrict__ a, int n) {
 // ---------------------------------------------------------------------------
 // Cholesky
 // ---------------------------------------------------------------------------
-// Blocks of 128 columns, each in four steps of 32.  A step is one kernel that
-// factors the 32 x 32 diagonal block and solves for the rows below, and one
-// that applies the 32 columns to the block's remaining columns on the FP64
-// pipe; the 128 columns are then applied to everything to their right as one
-// product of the digit engine.  128: the FP64 pipe does rows x 128 x 96
-// multiply-adds per block (9 us at 1400 rows, spread over the chip), the
-// product costs about 40 us however narrow it is, so wider blocks shift work
-// to the slow pipe and narrower ones add launches.
+// Blocks of 64 columns in two steps of 32.  A step factors the 32 x 32
+// diagonal block and solves for the rows below; the first 32 columns are
+// applied to the other 32 on the FP64 pipe, the 64 then to everything to their
+// right as one product of the digit engine.  Several matrices go through the
+// sweep together (blockIdx.z): at the sizes where it matters the chain of
+// small dependent kernels is what takes the time, not their work.  The FP64
+// pipe of an SM quarter takes 64 cycles for one warp-wide operation, so every
+// phase spreads its work over the four warps of a CTA and over many CTAs:
+// with one warp per diagonal block and a row per thread a step took 88 us.
+// 64 columns and not 128: the FP64 work inside a block grows with its width
+// (rows x 32 x 32 multiply-adds here, six times that at 128).
 constexpr int kNb = 32;
-constexpr int kOuter = 128;
+constexpr int kOuter = 2 * kNb;
+
+// 1 / sqrt(p) for a normal p > 0: the FP32 reciprocal square root of the
+// mantissa (exponent made even and taken apart), then one third-order step
+// y (1 + e/2 + 3 e^2/8), e = 1 - p y^2, which leaves e^3 ~ 2^-66.
+__device__ __forceinline__ double inv_sqrt(double p) {
+  const int hi = __double2hiint(p);
+  const int ex = ((hi >> 20) - 1023) & ~1;  // even exponent
+  const double m = __hiloint2double(hi - (ex << 20), __double2loint(p));  // in [1, 4)
+  const double y0 = static_cast<double>(rsqrtf(static_cast<float>(m)));
+  const double e = fma(-m * y0, y0, 1.0);
+  const double y = fma(y0 * e, fma(e, 0.375, 0.5), y0);
+  return __hiloint2double(__double2hiint(y) - ((ex / 2) << 20), __double2loint(y));
+}
 
 // Rows i >= k0 + b: a[i][k0:k0+b] <- a[i][k0:k0+b] D^-T, D the Cholesky factor
 // of the diagonal block at (k0, k0), which every CTA forms for itself (one
-// warp, a row per lane: one launch fewer on the serial chain); CTA 0 writes
-// it to fac[k0 * 32..] (row-major, pitch 32), not in place: other CTAs still
-// read the block.  One thread per row below, its 32 values in registers.
-__global__ void __launch_bounds__(128) k_chol_step(double* __restrict__ a, long long rows, int n, int k0, int b,
-                                                   double* __restrict__ fac, int* __restrict__ err) {
+// launch fewer on the serial chain); CTA 0 writes it to fac[k0 * 32..]
+// (row-major, pitch 32), not in place: other CTAs still read the block.  32
+// rows per CTA, 8 per warp, a row on four lanes that hold every fourth column.
+__global__ void __launch_bounds__(128) k_chol_step(double* __restrict__ a0, long long rows, int n, long long z_stride,
+                                                   int k0, int b, double* __restrict__ fac0, long long fac_z,
+                                                   int* __restrict__ err) {
   __shared__ double d[kNb][kNb + 1];
   __shared__ double rd[kNb];  // reciprocals of the diagonal
-  const int lane = threadIdx.x & 31;
+  double* a = a0 + blockIdx.z * z_stride;
+  double* fac = fac0 + blockIdx.z * fac_z;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int i = threadIdx.x; i < kNb * kNb; i += blockDim.x) {
     const int r = i >> 5, c = i & 31;
     d[r][c] = (r < b && c <= r) ? a[static_cast<long long>(k0 + r) * n + k0 + c] : (r == c ? 1.0 : 0.0);
   }
+  // this thread's part of a row below: columns g, g + 4, ...
+  const long long row = k0 + b + static_cast<long long>(blockIdx.x) * kNb + warp * 8 + (lane >> 2);
+  const int g = lane & 3;
+  double x[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) x[i] = (row < rows && g + 4 * i < b) ? a[row * n + k0 + g + 4 * i] : 0.0;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double x[kNb];
-#pragma unroll
-    for (int c = 0; c < kNb; ++c) x[c] = d[lane][c];
-    bool bad = false;
-#pragma unroll
-    for (int j = 0; j < kNb; ++j) {
-      double p = __shfl_sync(0xffffffffu, x[j], j);
-      if (!(p > 0.0) || !isfinite(p)) {
-        bad = bad || j < b;
-        p = 1.0;
-      }
-      const double l = sqrt(p), inv = 1.0 / l;
-      x[j] = lane == j ? l : (lane > j ? x[j] * inv : x[j]);
-      if (lane == j) rd[j] = inv;
-      d[lane][j] = x[j];  // column j, read below by every lane
-      __syncwarp();
-#pragma unroll
-      for (int c = j + 1; c < kNb; ++c)
-        if (lane >= c) x[c] = fma(-x[j], d[c][j], x[c]);
+  bool bad = false;
+  for (int j = 0; j < b; ++j) {
+    double p = d[j][j];
+    if (!(p > 0.0) || !isfinite(p)) {
+      bad = true;
+      p = 1.0;
     }
-    if (lane == 0 && bad && blockIdx.x == 0) atomicOr(err, 1);
+    // a subnormal pivot (outside inv_sqrt's range) by the library's root
+    const double y = p < 2.2250738585072014e-308 ? 1.0 / sqrt(p) : inv_sqrt(p);
+    __syncthreads();  // every thread has read the pivot
+    if (warp == 0) {
+      if (lane > j) d[lane][j] *= y;
+      if (lane == j) {
+        d[j][j] = p * y;
+        rd[j] = y;
+      }
+    }
+    __syncthreads();
+    const double l = d[lane][j];
+    for (int c = j + 1 + warp; c < b; c += 4)
+      if (lane >= c) d[lane][c] = fma(-l, d[c][j], d[lane][c]);
+    __syncthreads();
   }
-  __syncthreads();
+  if (bad && threadIdx.x == 0 && blockIdx.x == 0) atomicOr(err, 1);
   if (blockIdx.x == 0)
     for (int i = threadIdx.x; i < kNb * kNb; i += blockDim.x)
       fac[static_cast<long long>(k0) * kNb + i] = d[i >> 5][i & 31];
-  const long long row = k0 + b + static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (row >= rows) return;
-  double* r = a + row * n + k0;
-  double x[kNb];
-#pragma unroll
-  for (int c = 0; c < kNb; ++c) x[c] = c < b ? r[c] : 0.0;
 #pragma unroll
   for (int j = 0; j < kNb; ++j) {
-    x[j] *= rd[j];
+    if (j >= b) break;
+    if (g == (j & 3)) x[j >> 2] *= rd[j];
+    const double xj = __shfl_sync(0xffffffffu, x[j >> 2], (lane & ~3) | (j & 3));
 #pragma unroll
-    for (int c = j + 1; c < kNb; ++c) x[c] = fma(-x[j], d[c][j], x[c]);
+    for (int i = j >> 2; i < 8; ++i)
+      if (g + 4 * i > j) x[i] = fma(-xj, d[g + 4 * i][j], x[i]);
   }
+  if (row < rows)
 #pragma unroll
-  for (int c = 0; c < kNb; ++c)
-    if (c < b) r[c] = x[c];
+    for (int i = 0; i < 8; ++i)
+      if (g + 4 * i < b) a[row * n + k0 + g + 4 * i] = x[i];
 }
 
-// a[r][c] -= sum_{t < 32} a[r][k0 + t] a[c][k0 + t] for rows r >= c0 and
-// columns c of [c0, c1), 32 x 32 tiles (small, so that the FP64 pipes of all
-// SMs take part), tiles above the diagonal left out.
-__global__ void __launch_bounds__(256) k_chol_update(double* __restrict__ a, long long rows, int n, int k0, int c0,
-                                                     int c1) {
-  const int cb = c0 + blockIdx.x * 32;
-  const long long rb = c0 + static_cast<long long>(blockIdx.y) * 32;
-  if (rb + 31 < cb) return;
-  __shared__ double x[32][33], y[32][33];
+// a[r][c] -= sum_{t < 32} a[r][k0 + t] a[c][k0 + t] for rows r >= c0 and the
+// columns c of [c0, c1), c1 - c0 <= 32: 16 x 32 tiles (small, so that the FP64
+// pipes of all SMs take part), nothing above the diagonal.
+__global__ void __launch_bounds__(128) k_chol_update(double* __restrict__ a0, long long rows, int n,
+                                                     long long z_stride, int k0, int c0, int c1) {
+  double* a = a0 + blockIdx.z * z_stride;
+  const long long rb = c0 + static_cast<long long>(blockIdx.x) * 16;
+  __shared__ double x[16][33], y[32][33];
   for (int i = threadIdx.x; i < 32 * 32; i += blockDim.x) {
     const int r = i >> 5, t = i & 31;
-    x[r][t] = rb + r < rows ? a[(rb + r) * n + k0 + t] : 0.0;
-    y[r][t] = cb + r < c1 ? a[static_cast<long long>(cb + r) * n + k0 + t] : 0.0;
+    if (r < 16) x[r][t] = rb + r < rows ? a[(rb + r) * n + k0 + t] : 0.0;
+    y[r][t] = c0 + r < c1 ? a[static_cast<long long>(c0 + r) * n + k0 + t] : 0.0;
   }
   __syncthreads();
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -169,18 +191,21 @@ __global__ void __launch_bounds__(256) k_chol_update(double* __restrict__ a, lon
   for (int t = 0; t < 32; ++t) {
     const double v = y[tx][t];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) acc[i] = fma(x[ty + 8 * i][t], v, acc[i]);
+    for (int i = 0; i < 4; ++i) acc[i] = fma(x[ty + 4 * i][t], v, acc[i]);
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const long long r = rb + ty + 8 * i;
-    const int c = cb + tx;
+    const long long r = rb + ty + 4 * i;
+    const int c = c0 + tx;
     if (r < rows && c < c1 && r >= c) a[r * n + c] -= acc[i];
   }
 }
 
 // the factored diagonal blocks into place, zeros above the diagonal
-__global__ void k_chol_finish(double* __restrict__ a, int n, const double* __restrict__ fac) {
+__global__ void k_chol_finish(double* __restrict__ a0, int n, long long z_stride, const double* __restrict__ fac0,
+                              long long fac_z) {
+  double* a = a0 + blockIdx.z * z_stride;
+  const double* fac = fac0 + blockIdx.z * fac_z;
   long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   const long long nn = static_cast<long long>(n) * n;
   if (i >= nn) return;
@@ -220,22 +245,23 @@ void chain_set_identity(double* a, int n, cudaStream_t st) {
   chain::k_set_identity<<<static_cast<unsigned>((nn + 255) / 256), 256, 0, st>>>(a, n);
 }
 
-int chain_cholesky(gw_ctx* ctx, double* a, long long rows, int n, int* err, cudaStream_t st) {
+int chain_cholesky(gw_ctx* ctx, double* a, long long rows, int n, int nz, long long z_stride, int* err,
+                   cudaStream_t st) {
   void* p;
   int rc;
-  if ((rc = work_buffer(ctx, "w.chol.fac", (static_cast<size_t>(n) + chain::kNb) * chain::kNb * sizeof(double), &p)))
-    return rc;
+  const long long fac_z = (static_cast<long long>(n) + chain::kNb) * chain::kNb;
+  if ((rc = work_buffer(ctx, "w.chol.fac", static_cast<size_t>(fac_z) * nz * sizeof(double), &p))) return rc;
   double* fac = static_cast<double*>(p);
   for (int k0 = 0; k0 < n; k0 += chain::kOuter) {
     const int k1 = std::min(n, k0 + chain::kOuter);
     for (int j0 = k0; j0 < k1; j0 += chain::kNb) {
       const int b = std::min(chain::kNb, k1 - j0);
       const long long below = rows - j0 - b;
-      chain::k_chol_step<<<static_cast<unsigned>(std::max(1ll, (below + 127) / 128)), 128, 0, st>>>(a, rows, n, j0, b,
-                                                                                                   fac, err);
+      chain::k_chol_step<<<dim3(static_cast<unsigned>(std::max(1ll, (below + 31) / 32)), 1, nz), 128, 0, st>>>(
+          a, rows, n, z_stride, j0, b, fac, fac_z, err);
       if (j0 + b < k1)
-        chain::k_chol_update<<<dim3((k1 - j0 - b + 31) / 32, static_cast<unsigned>((below + 31) / 32)), 256, 0, st>>>(
-            a, rows, n, j0, j0 + b, k1);
+        chain::k_chol_update<<<dim3(static_cast<unsigned>((below + 15) / 16), 1, nz), 128, 0, st>>>(
+            a, rows, n, z_stride, j0, j0 + b, k1);
     }
     if (k1 < n) {
       // a[k1:, k1:n] -= X X^T, X = a[k1:, k0:k1]
@@ -245,6 +271,8 @@ int chain_cholesky(gw_ctx* ctx, double* a, long long rows, int n, int* err, cuda
       s.ld = n;
       s.rows = rows - k1;
       s.K = k1 - k0;
+      s.nz = nz;
+      s.z_stride = z_stride;
       if ((rc = emu_prep(ctx, "panel", s, &x, st))) return rc;
       y = x;
       y.s.rows = n - k1;
@@ -253,12 +281,14 @@ int chain_cholesky(gw_ctx* ctx, double* a, long long rows, int n, int* err, cuda
       g.beta = 1.0;
       g.C = a + static_cast<long long>(k1) * n + k1;
       g.ldc = n;
+      g.c_zstride = z_stride;
       g.tri = 1;
       if ((rc = emu_mm(ctx, x, y, g, st))) return rc;
     }
   }
   const long long nn = static_cast<long long>(n) * n;
-  chain::k_chol_finish<<<static_cast<unsigned>((nn + 255) / 256), 256, 0, st>>>(a, n, fac);
+  chain::k_chol_finish<<<dim3(static_cast<unsigned>((nn + 255) / 256), 1, nz), 256, 0, st>>>(a, n, z_stride, fac,
+                                                                                          fac_z);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     ctx->err = std::string("Cholesky factorisation: ") + cudaGetErrorString(e);

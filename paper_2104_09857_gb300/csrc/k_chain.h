@@ -19,8 +19,10 @@ void chain_add_diagonal(double* a, int n, double x, cudaStream_t st);
 void chain_set_identity(double* a, int n, cudaStream_t st);
 // a[rows][n], rows >= n: the leading n x n block (its lower triangle is read)
 // becomes its Cholesky factor R, the rows below become B R^-T; the strict
-// upper triangle of the leading block is zeroed.  err[0] |= 1 on a pivot that
-// is not positive.  Uses the context's work buffers (emu_begin before).
-int chain_cholesky(gw_ctx* ctx, double* a, long long rows, int n, int* err, cudaStream_t st);
+// upper triangle of the leading block is zeroed.  nz such matrices z_stride
+// elements apart in one sweep.  err[0] |= 1 on a pivot that is not positive.
+// Uses the context's work buffers (emu_begin before).
+int chain_cholesky(gw_ctx* ctx, double* a, long long rows, int n, int nz, long long z_stride, int* err,
+                   cudaStream_t st);
 
 }  // namespace gw

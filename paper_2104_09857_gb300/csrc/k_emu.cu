@@ -134,8 +134,8 @@ __device__ __forceinline__ int biased_exp(double x) {
 // consecutive elements per lane.
 template <int kWarps>
 __global__ void __launch_bounds__(256) k_prep_rows(const double* __restrict__ src, long long ld, long long rows,
-                                                   int K, int kp, __half* __restrict__ dig,
-                                                   int* __restrict__ exps) {
+                                                   int K, int kp, long long zrows, long long z_stride,
+                                                   __half* __restrict__ dig, int* __restrict__ exps) {
   constexpr int kPer = 8 / kWarps;  // rows of a CTA
   __shared__ int red[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(256) k_prep_rows(const double* __restrict__ sr
        r0 += static_cast<long long>(gridDim.x) * kPer) {
     const long long r = r0 + warp / kWarps;
     const bool on = r < rows;
-    const double* x = src + r * ld;
+    const double* x = zrows == rows ? src + r * ld : src + r / zrows * z_stride + r % zrows * ld;
     int be = 0;
     if (on)
       for (int k = t; k < K; k += nt) be = max(be, biased_exp(x[k]));
@@ -338,21 +338,27 @@ struct GemmJob {
   long long ldc, cblk_stride, col0;
   int cblk;
   const int *ea, *eb;
-  unsigned long long* part;  // ks > 1: [m][n][2] integer sums
+  int per_z, za, zb;         // items and operand rows of one product of a batch
+  long long c_z, a_z, b_z;   // C, A, B from one product to the next
+  unsigned long long* part;  // ks > 1: [nz][m][n][2] integer sums
   const double *A, *B;
   long long lda, ldb;
   int ta, tb;
 
   struct Tile {
-    int ya, yb, c0, n;
+    int ya, yb, c0, n;  // rows of the stacked digits
+    int ra, rb, z;      // ... and of the product's own operands
   };
   __device__ int items() const { return n_items; }
   __device__ Tile tile(int t) const {
-    const int s = t % ks, x = t / ks;
     Tile T;
-    T.ya = x / nt * kM;
-    T.yb = x % nt * kN;
-    const int from = ktri ? min(max(T.ya + tri_off, 0) / kChunk, stages) : 0;
+    T.z = t / per_z;
+    const int u = t - T.z * per_z, s = u % ks, x = u / ks;
+    T.ra = x / nt * kM;
+    T.rb = x % nt * kN;
+    T.ya = T.ra + T.z * za;
+    T.yb = T.rb + T.z * zb;
+    const int from = ktri ? min(max(T.ra + tri_off, 0) / kChunk, stages) : 0;
     const int per = (stages - from + ks - 1) / ks;
     T.c0 = from + s * per;
     T.n = max(min(per, stages - T.c0), 0);
@@ -361,7 +367,7 @@ struct GemmJob {
       T.c0 = stages - 1;
       T.n = 1;
     }
-    if (skip(T.ya, T.yb)) T.n = 0;
+    if (skip(T.ra, T.rb)) T.n = 0;
     return T;
   }
   __device__ bool skip(int ya, int yb) const { return tri && yb >= ya + kM + tri_off; }
@@ -379,65 +385,67 @@ struct GemmJob {
     return t ? p[k * ld + r] : p[r * ld + k];
   }
   // the element from the FP64 operands (a row with an Inf or NaN)
-  __device__ double direct(int r, int c) const {
+  __device__ double direct(int z, int r, int c) const {
     double s = 0.0;
-    for (int k = 0; k < K; ++k) s = fma(at(A, lda, ta, r, k), at(B, ldb, tb, c, k), s);
+    for (int k = 0; k < K; ++k) s = fma(at(A + z * a_z, lda, ta, r, k), at(B + z * b_z, ldb, tb, c, k), s);
     return s;
   }
-  __device__ void store(int r, int c, double v) const {
+  __device__ void store(int z, int r, int c, double v) const {
     long long at = c;
     if (cblk) {
       const uint32_t q = static_cast<uint32_t>(c + col0), b = static_cast<uint32_t>(cblk);
       at = q / b * cblk_stride + q % b;
     }
-    double* p = C + r * ldc + at;
+    double* p = C + z * c_z + r * ldc + at;
     const double w = alpha == 1.0 ? v : (alpha == -1.0 ? -v : alpha * v);  // most calls spare the FP64 pipe
     *p = beta == 0.0 ? w : fma(beta, *p, w);
   }
   __device__ void write(long long (&hi)[kCols], long long (&lo)[kCols], const Tile& T, int row, int c0) const {
-    const int r = T.ya + row;
+    const int r = T.ra + row;
     if (r >= m) return;
     if (part) {
-      unsigned long long* p = part + (static_cast<long long>(r) * n + T.yb + c0) * 2;
+      unsigned long long* p = part + ((static_cast<long long>(T.z) * m + r) * n + T.rb + c0) * 2;
 #pragma unroll
       for (int j = 0; j < kCols; ++j) {
-        if (T.yb + c0 + j >= n) break;
+        if (T.rb + c0 + j >= n) break;
         carry(hi[j], lo[j]);
         atomicAdd(p + 2 * j, static_cast<unsigned long long>(hi[j]));
         atomicAdd(p + 2 * j + 1, static_cast<unsigned long long>(lo[j]));
       }
       return;
     }
-    const int a = ea[r];
+    const int a = ea[T.z * za + r];
     unsigned bad = 0;  // columns that need the FP64 operands
 #pragma unroll
     for (int j = 0; j < kCols; ++j) {
-      const int c = T.yb + c0 + j;
+      const int c = T.rb + c0 + j;
       if (c >= n) break;
-      const int b = eb[c];
+      const int b = eb[T.z * zb + c];
       if (a == kBad || b == kBad)
         bad |= 1u << j;
       else
-        store(r, c, fixed_to_double(hi[j], lo[j], a + b + kUnit));
+        store(T.z, r, c, fixed_to_double(hi[j], lo[j], a + b + kUnit));
     }
     while (bad) {
-      const int c = T.yb + c0 + __ffs(bad) - 1;
-      store(r, c, direct(r, c));
+      const int c = T.rb + c0 + __ffs(bad) - 1;
+      store(T.z, r, c, direct(T.z, r, c));
       bad &= bad - 1;
     }
   }
 };
-__global__ void k_gemm_finish(const GemmJob j) {
-  const long long n = static_cast<long long>(j.m) * j.n;
-  for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
+__global__ void k_gemm_finish(const GemmJob j, int nz) {
+  const long long mn = static_cast<long long>(j.m) * j.n;
+  for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < mn * nz;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int r = static_cast<int>(i / j.n), c = static_cast<int>(i % j.n);
+    const int z = static_cast<int>(i / mn);
+    const long long e = i - z * mn;
+    const int r = static_cast<int>(e / j.n), c = static_cast<int>(e % j.n);
     if (j.skip(r / kM * kM, c / kN * kN)) continue;
     const ulonglong2 v = reinterpret_cast<const ulonglong2*>(j.part)[i];
-    const int a = j.ea[r], b = j.eb[c];
-    j.store(r, c, a == kBad || b == kBad ? j.direct(r, c)
-                                         : fixed_to_double(static_cast<long long>(v.x), static_cast<long long>(v.y),
-                                                           a + b + kUnit));
+    const int a = j.ea[z * j.za + r], b = j.eb[z * j.zb + c];
+    j.store(z, r, c, a == kBad || b == kBad ? j.direct(z, r, c)
+                                            : fixed_to_double(static_cast<long long>(v.x),
+                                                              static_cast<long long>(v.y), a + b + kUnit));
   }
 }
 
@@ -881,8 +889,8 @@ int launch(const CUtensorMap& ma, const CUtensorMap& mb, const Job& job, int n_i
 // over the SMs short.  Costs in stages (about 2 us each): a unit's start and
 // end about 3 (the write, or 128 KB of atomics), clearing and converting the
 // partial sums about 5 in all.
-int k_splits(long long m, long long n, int K) {
-  const long long tiles = ((m + kM - 1) / kM) * ((n + kN - 1) / kN);
+int k_splits(long long m, long long n, int K, int nz) {
+  const long long tiles = ((m + kM - 1) / kM) * ((n + kN - 1) / kN) * nz;
   const long long stages = (K + kChunk - 1) / kChunk;
   long long best = 1, cost = 0;
   for (long long ks = 1; ks <= 64 && ks * 4 <= std::max(stages, 4ll); ++ks) {
@@ -899,18 +907,19 @@ int k_splits(long long m, long long n, int K) {
 
 void launch_emu_prep(EmuOp& op, const EmuSrc& s, cudaStream_t st) {
   op.s = s;
-  op.stride_rows = s.rows;
+  const long long rows = s.rows * s.nz;
+  op.stride_rows = rows;
   op.kp = emu_kp(s.K);
-  if (s.rows <= 0) return;
+  if (rows <= 0) return;
   __half* dig = static_cast<__half*>(op.dig);
   if (!s.trans) {
     const bool wide = s.K >= 2048;  // a CTA per row, else a warp
-    const long long blocks = wide ? s.rows : (s.rows + 7) / 8;
+    const long long blocks = wide ? rows : (rows + 7) / 8;
     const unsigned grid = static_cast<unsigned>(std::min<long long>(blocks, 152 * 64));
     if (wide)
-      emu::k_prep_rows<8><<<grid, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, op.kp, dig, op.exps);
+      emu::k_prep_rows<8><<<grid, 256, 0, st>>>(s.src, s.ld, rows, s.K, op.kp, s.rows, s.z_stride, dig, op.exps);
     else
-      emu::k_prep_rows<1><<<grid, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, op.kp, dig, op.exps);
+      emu::k_prep_rows<1><<<grid, 256, 0, st>>>(s.src, s.ld, rows, s.K, op.kp, s.rows, s.z_stride, dig, op.exps);
   } else {
     int* be = op.exps + s.rows;
     cudaMemsetAsync(be, 0, static_cast<size_t>(s.rows) * sizeof(int), st);
@@ -921,8 +930,8 @@ void launch_emu_prep(EmuOp& op, const EmuSrc& s, cudaStream_t st) {
   }
 }
 
-size_t emu_gemm_ws_bytes(long long m, long long n, int K) {
-  return emu::k_splits(m, n, K) > 1 ? static_cast<size_t>(m) * n * 16 : 0;
+size_t emu_gemm_ws_bytes(long long m, long long n, int K, int nz) {
+  return emu::k_splits(m, n, K, nz) > 1 ? static_cast<size_t>(m) * n * 16 * nz : 0;
 }
 
 int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, int* err_flag,
@@ -930,8 +939,9 @@ int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, 
   const int m = static_cast<int>(A.s.rows), n = static_cast<int>(B.s.rows);
   if (m <= 0 || n <= 0) return 0;
   CUtensorMap ma, mb;
-  if (make_digit_map(&ma, A.dig, A.kp, A.s.rows, A.stride_rows, kEmuSlices, emu::kChunk, emu::kM) ||
-      make_digit_map(&mb, B.dig, B.kp, B.s.rows, B.stride_rows, kEmuSlices, emu::kChunk, emu::kN))
+  if (make_digit_map(&ma, A.dig, A.kp, A.s.nz > 1 ? A.stride_rows : A.s.rows, A.stride_rows, kEmuSlices, emu::kChunk, emu::kM) ||
+      make_digit_map(&mb, B.dig, B.kp, B.s.nz > 1 ? B.stride_rows : B.s.rows, B.stride_rows, kEmuSlices, emu::kChunk,
+                     emu::kN))
     return -2;
   emu::GemmJob j{};
   j.m = m;
@@ -939,8 +949,16 @@ int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, 
   j.K = A.s.K;
   j.nt = (n + emu::kN - 1) / emu::kN;
   j.stages = std::max(1, (A.s.K + emu::kChunk - 1) / emu::kChunk);
-  j.ks = ws ? emu::k_splits(m, n, A.s.K) : 1;
-  const long long items = static_cast<long long>((m + emu::kM - 1) / emu::kM) * j.nt * j.ks;
+  const int nz = A.s.nz;
+  j.ks = ws ? emu::k_splits(m, n, A.s.K, nz) : 1;
+  j.per_z = (m + emu::kM - 1) / emu::kM * j.nt * j.ks;
+  // rows of one matrix in the stacked digits (a slice of rows of each keeps the whole stack's)
+  j.za = nz > 1 ? static_cast<int>(A.stride_rows / nz) : 0;
+  j.zb = B.s.nz > 1 ? static_cast<int>(B.stride_rows / B.s.nz) : 0;
+  j.c_z = g.c_zstride;
+  j.a_z = A.s.z_stride;
+  j.b_z = B.s.z_stride;
+  const long long items = static_cast<long long>(j.per_z) * nz;
   if (items > INT32_MAX) return -3;
   j.n_items = static_cast<int>(items);
   j.tri = g.tri;
@@ -963,13 +981,13 @@ int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, 
   j.tb = B.s.trans;
   if (j.ks > 1) {
     j.part = static_cast<unsigned long long*>(ws);
-    cudaMemsetAsync(ws, 0, static_cast<size_t>(m) * n * 16, st);
+    cudaMemsetAsync(ws, 0, static_cast<size_t>(m) * n * 16 * nz, st);
   }
   const int rc = emu::launch(ma, mb, j, j.n_items, err_flag, st);
   if (rc) return rc;
   if (j.ks > 1) {
-    const long long blocks = (static_cast<long long>(m) * n + 255) / 256;
-    emu::k_gemm_finish<<<static_cast<unsigned>(std::min<long long>(blocks, 152 * 16)), 256, 0, st>>>(j);
+    const long long blocks = (static_cast<long long>(m) * n * nz + 255) / 256;
+    emu::k_gemm_finish<<<static_cast<unsigned>(std::min<long long>(blocks, 152 * 16)), 256, 0, st>>>(j, nz);
   }
   return 0;
 }

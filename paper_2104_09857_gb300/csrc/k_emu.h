@@ -22,6 +22,10 @@ struct EmuSrc {
   long long ld = 0, rows = 0;
   int K = 0;
   bool trans = false;
+  // several matrices of `rows` rows each, z_stride elements apart, one below
+  // the other in the digits (not with trans)
+  int nz = 1;
+  long long z_stride = 0;
 };
 // The same as digits: [kEmuSlices][stride_rows][kp] binary16, kp a multiple of
 // 64, zero for k >= K, and per row the power of two above its largest
@@ -47,14 +51,16 @@ inline int emu_kp(int k) { return (k + 63) / 64 * 64; }
 inline size_t emu_dig_bytes(long long rows, int k) {
   return static_cast<size_t>(kEmuSlices) * rows * emu_kp(k) * 2;
 }
-// Digits and exponents of s into op.dig (emu_dig_bytes) and op.exps (s.rows
-// ints; twice that when trans).
+// Digits and exponents of s into op.dig (emu_dig_bytes) and op.exps (s.nz *
+// s.rows ints; twice that when trans).
 void launch_emu_prep(EmuOp& op, const EmuSrc& s, cudaStream_t st);
 
 // C[r * ldc + c] = alpha * sum_k A[r][k] B[c][k] + beta * C, with C's columns
 // in blocks of cblk (0: one block) cblk_stride elements apart.
 //   tri 1: only the tiles that touch r + tri_off >= c are computed
 //   ktri 1: A[r][k] is zero for k < r + tri_off: those stages are left out
+// With A.s.nz > 1 the same for every pair of matrices (B may be one matrix),
+// C's c_zstride elements apart.
 struct EmuGemm {
   double alpha = 1.0, beta = 0.0;
   double* C = nullptr;
@@ -63,9 +69,10 @@ struct EmuGemm {
   long long tri_off = 0;
   int cblk = 0;
   long long cblk_stride = 0, col0 = 0;  // col0: index of B's first row in the blocks
+  long long c_zstride = 0;
 };
 // Bytes of the partial-sum workspace of a product (0: not split along K).
-size_t emu_gemm_ws_bytes(long long m, long long n, int K);
+size_t emu_gemm_ws_bytes(long long m, long long n, int K, int nz = 1);
 // Returns 0, or a negative set-up error.  err_flag as for the other
 // tensor-core launchers (k_tc.h).
 int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, int* err_flag,
