@@ -79,7 +79,7 @@ __global__ void k_set_identity(double* __restrict__ a, int n) {
 // Cholesky
 // ---------------------------------------------------------------------------
 // Blocks of 64 columns in two steps of 32.  A step factors the 32 x 32
-// diagonal block and solves for the rows below; the first 32 columns are
+// diagonal block, then solves for the rows below; the first 32 columns are
 // applied to the other 32 on the FP64 pipe, the 64 then to everything to their
 // right as one product of the digit engine.  Several matrices go through the
 // sweep together (blockIdx.z): at the sizes where it matters the chain of
@@ -105,29 +105,22 @@ __device__ __forceinline__ double inv_sqrt(double p) {
   return __hiloint2double(__double2hiint(y) - ((ex / 2) << 20), __double2loint(y));
 }
 
-// Rows i >= k0 + b: a[i][k0:k0+b] <- a[i][k0:k0+b] D^-T, D the Cholesky factor
-// of the diagonal block at (k0, k0), which every CTA forms for itself (one
-// launch fewer on the serial chain); CTA 0 writes it to fac[k0 * 32..]
-// (row-major, pitch 32), not in place: other CTAs still read the block.  32
-// rows per CTA, 8 per warp, a row on four lanes that hold every fourth column.
-__global__ void __launch_bounds__(128) k_chol_step(double* __restrict__ a0, long long rows, int n, long long z_stride,
-                                                   int k0, int b, double* __restrict__ fac0, long long fac_z,
-                                                   int* __restrict__ err) {
+// Cholesky factor of the b x b diagonal block at (k0, k0) of every matrix, to
+// fac[k0 * 32..] (row-major, pitch 32) and the reciprocals of its diagonal to
+// fac[(n + 32) * 32 + k0..].  One CTA per matrix; formed by every CTA of the
+// solve below instead, the CTAs of an SM would queue for its FP64 pipe.
+__global__ void __launch_bounds__(128) k_chol_factor(const double* __restrict__ a0, int n, long long z_stride, int k0,
+                                                     int b, double* __restrict__ fac0, long long fac_z,
+                                                     int* __restrict__ err) {
   __shared__ double d[kNb][kNb + 1];
-  __shared__ double rd[kNb];  // reciprocals of the diagonal
-  double* a = a0 + blockIdx.z * z_stride;
-  double* fac = fac0 + blockIdx.z * fac_z;
+  const double* a = a0 + blockIdx.x * z_stride;
+  double* fac = fac0 + blockIdx.x * fac_z;
+  double* rd = fac + (static_cast<long long>(n) + kNb) * kNb + k0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int i = threadIdx.x; i < kNb * kNb; i += blockDim.x) {
     const int r = i >> 5, c = i & 31;
     d[r][c] = (r < b && c <= r) ? a[static_cast<long long>(k0 + r) * n + k0 + c] : (r == c ? 1.0 : 0.0);
   }
-  // this thread's part of a row below: columns g, g + 4, ...
-  const long long row = k0 + b + static_cast<long long>(blockIdx.x) * kNb + warp * 8 + (lane >> 2);
-  const int g = lane & 3;
-  double x[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) x[i] = (row < rows && g + 4 * i < b) ? a[row * n + k0 + g + 4 * i] : 0.0;
   __syncthreads();
   bool bad = false;
   for (int j = 0; j < b; ++j) {
@@ -152,10 +145,30 @@ __global__ void __launch_bounds__(128) k_chol_step(double* __restrict__ a0, long
       if (lane >= c) d[lane][c] = fma(-l, d[c][j], d[lane][c]);
     __syncthreads();
   }
-  if (bad && threadIdx.x == 0 && blockIdx.x == 0) atomicOr(err, 1);
-  if (blockIdx.x == 0)
-    for (int i = threadIdx.x; i < kNb * kNb; i += blockDim.x)
-      fac[static_cast<long long>(k0) * kNb + i] = d[i >> 5][i & 31];
+  if (bad && threadIdx.x == 0) atomicOr(err, 1);
+  for (int i = threadIdx.x; i < kNb * kNb; i += blockDim.x)
+    fac[static_cast<long long>(k0) * kNb + i] = d[i >> 5][i & 31];
+}
+
+// Rows i >= k0 + b: a[i][k0:k0+b] <- a[i][k0:k0+b] D^-T, D the factor.  32
+// rows per CTA, 8 per warp, a row on four lanes that hold every fourth column.
+__global__ void __launch_bounds__(128) k_chol_solve(double* __restrict__ a0, long long rows, int n, long long z_stride,
+                                                    int k0, int b, const double* __restrict__ fac0, long long fac_z) {
+  __shared__ double d[kNb][kNb + 1];
+  __shared__ double rd[kNb];
+  double* a = a0 + blockIdx.z * z_stride;
+  const double* fac = fac0 + blockIdx.z * fac_z;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < kNb * kNb; i += blockDim.x)
+    d[i >> 5][i & 31] = fac[static_cast<long long>(k0) * kNb + i];
+  if (threadIdx.x < b) rd[threadIdx.x] = fac[(static_cast<long long>(n) + kNb) * kNb + k0 + threadIdx.x];
+  // this thread's part of a row: columns g, g + 4, ...
+  const long long row = k0 + b + static_cast<long long>(blockIdx.x) * kNb + warp * 8 + (lane >> 2);
+  const int g = lane & 3;
+  double x[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) x[i] = (row < rows && g + 4 * i < b) ? a[row * n + k0 + g + 4 * i] : 0.0;
+  __syncthreads();
 #pragma unroll
   for (int j = 0; j < kNb; ++j) {
     if (j >= b) break;
@@ -249,7 +262,7 @@ int chain_cholesky(gw_ctx* ctx, double* a, long long rows, int n, int nz, long l
                    cudaStream_t st) {
   void* p;
   int rc;
-  const long long fac_z = (static_cast<long long>(n) + chain::kNb) * chain::kNb;
+  const long long fac_z = (static_cast<long long>(n) + chain::kNb) * (chain::kNb + 1);
   if ((rc = work_buffer(ctx, "w.chol.fac", static_cast<size_t>(fac_z) * nz * sizeof(double), &p))) return rc;
   double* fac = static_cast<double*>(p);
   for (int k0 = 0; k0 < n; k0 += chain::kOuter) {
@@ -257,8 +270,10 @@ int chain_cholesky(gw_ctx* ctx, double* a, long long rows, int n, int nz, long l
     for (int j0 = k0; j0 < k1; j0 += chain::kNb) {
       const int b = std::min(chain::kNb, k1 - j0);
       const long long below = rows - j0 - b;
-      chain::k_chol_step<<<dim3(static_cast<unsigned>(std::max(1ll, (below + 31) / 32)), 1, nz), 128, 0, st>>>(
-          a, rows, n, z_stride, j0, b, fac, fac_z, err);
+      chain::k_chol_factor<<<nz, 128, 0, st>>>(a, n, z_stride, j0, b, fac, fac_z, err);
+      if (below > 0)
+        chain::k_chol_solve<<<dim3(static_cast<unsigned>((below + 31) / 32), 1, nz), 128, 0, st>>>(
+            a, rows, n, z_stride, j0, b, fac, fac_z);
       if (j0 + b < k1)
         chain::k_chol_update<<<dim3(static_cast<unsigned>((below + 15) / 16), 1, nz), 128, 0, st>>>(
             a, rows, n, z_stride, j0, j0 + b, k1);

@@ -19,17 +19,26 @@
 // closer to the exact value, and it does not depend on how K is split:
 // partial sums are integers, so split units may add in any order.
 //
-// Layout of a tile: 128 x 64 outputs; stages of 32 reduction elements with
-// all eight digits of both operands (96 KB, two stages), one TMA box per
-// operand and stage.  64 columns and not 128: the two integers of 128 x 128
-// outputs would take the whole register file.  Each diagonal has its own 64
-// accumulator columns; a diagonal of the next 128 elements starts as soon as
-// the epilogue has drained it.  Eight-bit digits and not nine: seven nine-bit
-// digits need 28 products but a drain every 32 elements, and the drains'
-// float-to-integer conversions (16 per cycle and SM) were then the limit.
-// The MMA warp runs converged with one elected thread issuing, so that the
-// descriptors stay in uniform registers: issued from a divergent branch an
-// MMA took 85 cycles, now the 48 that its 6 KB of operands need.
+// Layout: a cluster of two CTAs takes 128 x 128 outputs, 64 columns each;
+// stages of 32 reduction elements with all eight digits of both operands
+// (96 KB, two stages).  64 columns per CTA and not 128: the two integers of
+// 128 x 128 outputs would take the whole register file.  The A operand is the
+// same for both: each CTA loads four of its digits and multicasts them to the
+// pair, which cuts the L2 traffic of a stage from 96 to 64 KB per CTA.
+// MMAs: a digit of A meets two neighbouring digits of B at once, whose rows
+// follow one another in shared memory, and adds into two neighbouring
+// diagonals, 64 accumulator columns each: N = 128 takes 64 cycles where two
+// N = 64 take 48 each (each reads the 4 KB of A again).  32 N = 128 and 8 N =
+// 64 MMAs per stage: 2430 cycles.  The diagonals go pair by pair, so that the
+// epilogue drains one pair while the next is computed.  The MMA warp runs
+// converged with one elected lane issuing: the descriptors stay in uniform
+// registers (from a divergent branch an MMA took 85 cycles).
+// Eight-bit digits and not nine: seven nine-bit digits need 28 products but a
+// drain every 32 elements, and the drains' float-to-integer conversions (16
+// per cycle and SM) were then the limit.
+// Measured at 4096^3: 3.2 ms, 43 TFLOP/s (one digit pair per MMA: 4.2 ms;
+// without the elected lane and with nine-bit digits: 6.2 ms; the FP64 pipe:
+// 137 ms).
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -49,21 +58,25 @@ namespace emu {
 using namespace gw::tc;
 
 constexpr int kS = kEmuSlices;
-constexpr int kM = kEmuTileM, kN = kEmuTileN;
+constexpr int kM = kEmuTileM, kN = kEmuTileN / 2;  // a CTA takes half of a cluster's columns
+constexpr int kN2 = kEmuTileN;
 constexpr int kChunk = 32;  // reduction elements of a stage (64-byte rows)
 constexpr int kSub = kChunk / kMmaK;
 constexpr int kStages = 2;
 constexpr int kGroup = 4;  // stages of one exact accumulation
+constexpr int kPairs = kS / 2;  // pairs of diagonals (2p, 2p + 1)
 constexpr int kTmemCols = 512;
 constexpr int kEpiWarps = 16;              // 4 lane quadrants x 4 column groups
 constexpr int kCols = kN / (kEpiWarps / 4);  // 16 columns per epilogue warp
 constexpr int kThreads = (2 + kEpiWarps) * 32;
 constexpr int kABytes = kM * kChunk * 2, kBBytes = kN * kChunk * 2;  // one digit of one operand
 constexpr int kStageBytes = kS * (kABytes + kBBytes);
-constexpr int kSmem = kStages * kStageBytes + 256 + 1024;
+constexpr int kStgBytes = 32 * 8 * 8;  // per epilogue warp: 32 rows x 8 values on the way out
+constexpr int kSmem = kStages * kStageBytes + kEpiWarps * kStgBytes + 256 + 1024;
 constexpr int kLoBits = 32;   // value = (hi * 2^32 + lo) * 2^(ea + eb - 68)
 constexpr int kUnit = -68;
 constexpr int kBad = INT32_MAX;  // exponent of a row that holds an Inf or NaN
+constexpr int kOut = INT32_MIN;  // ... of a row outside the operand
 
 // K-major tile of 64-byte rows (32 binary16), 64-byte swizzle: 8-row groups
 // 512 bytes apart.
@@ -290,42 +303,123 @@ __global__ void __launch_bounds__(256) k_gather_digits(const __half* __restrict_
 // ---------------------------------------------------------------------------
 // integers back to FP64
 // ---------------------------------------------------------------------------
-// lo into [0, 2^32), the carry into hi.
-__device__ __forceinline__ void carry(long long& hi, long long& lo) {
-  hi += lo >> kLoBits;
-  lo &= (1ll << kLoBits) - 1;
-}
-// (hi 2^32 + lo) 2^e rounded to nearest even, in 32-bit integer arithmetic:
-// the FP64 pipe takes 16 cycles per warp and operation.
-__device__ __forceinline__ double fixed_to_double(long long hi, long long lo, int e) {
-  carry(hi, lo);
-  uint32_t w2 = static_cast<uint32_t>(static_cast<unsigned long long>(hi) >> 32);
-  uint32_t w1 = static_cast<uint32_t>(hi), w0 = static_cast<uint32_t>(lo);
-  const uint32_t sign = w2 & 0x80000000u;
-  if (sign) {  // 96-bit negation
-    w0 = 0u - w0;
-    w1 = ~w1 + (w0 == 0u);
-    w2 = ~w2 + (w0 == 0u && w1 == 0u);
+// Exponents of a warp's 32 rows (one per lane) and 16 columns (lanes 0-15, and
+// again 16-31), with kOut and kBad taken out.
+struct Exps {
+  int row, col;
+  bool row_in, row_bad;
+  unsigned col_in, col_bad;  // per column
+  __device__ Exps(int er, int ec) {
+    row_in = er != kOut;
+    row_bad = er == kBad;
+    row = row_in && !row_bad ? er + kUnit : 0;
+    col = ec != kOut && ec != kBad ? ec : 0;
+    col_in = __ballot_sync(0xffffffffu, ec != kOut);
+    col_bad = __ballot_sync(0xffffffffu, ec == kBad);
   }
+  __device__ int sum(int j) const { return row + __shfl_sync(0xffffffffu, col, j); }
+  __device__ bool in(int j) const { return row_in && ((col_in >> j) & 1u); }
+  __device__ bool bad(int j) const { return row_bad || ((col_bad >> j) & 1u); }
+};
+// (hi 2^32 + lo) 2^e from a sum of partial sums, whose low parts are not
+// carried yet.
+__device__ __forceinline__ double sums_to_double(long long hi, long long lo, int e);
+// (hi 2^32 + lo) 2^e rounded to nearest (ties away from zero), in about 35
+// 32-bit integer operations: three on the FP64 pipe, 64 cycles each per warp
+// and SM quarter, would take longer.
+__device__ __forceinline__ double fixed_to_double(long long hi, uint32_t lo, int e) {
+  const uint32_t sg = static_cast<uint32_t>(static_cast<int32_t>(static_cast<unsigned long long>(hi) >> 32) >> 31);
+  uint32_t w2 = static_cast<uint32_t>(static_cast<unsigned long long>(hi) >> 32) ^ sg;
+  uint32_t w1 = static_cast<uint32_t>(hi) ^ sg, w0 = lo ^ sg;
+  asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, 0;\n\taddc.u32 %2, %2, 0;"
+      : "+r"(w0), "+r"(w1), "+r"(w2)
+      : "r"(sg & 1u));
+  // leading word first; its first 64 significant bits (what follows is below
+  // the rounding by 2^-11 of a unit)
   const bool z2 = w2 == 0u, z1 = z2 && w1 == 0u;
-  if (z1 && w0 == 0u) return 0.0;
-  // leading word first
   const uint32_t a = z1 ? w0 : (z2 ? w1 : w2), b = z1 ? 0u : (z2 ? w0 : w1), c = z2 ? 0u : w0;
   const int s = __clz(static_cast<int>(a));
-  const uint32_t m1 = __funnelshift_l(b, a, s), m0 = __funnelshift_l(c, b, s), rest = c << s;
-  uint32_t f1 = m1 >> 11, f0 = __funnelshift_l(m0, m1, 21);
-  const uint32_t cut = m0 & 0x7ffu;
-  const uint32_t up = cut > 0x400u || (cut == 0x400u && (rest != 0u || (f0 & 1u)));
-  f0 += up;
-  f1 += up && f0 == 0u;
+  uint32_t m1 = __funnelshift_l(b, a, s), m0 = __funnelshift_l(c, b, s), over;
+  asm("add.cc.u32 %0, %0, 0x400;\n\taddc.cc.u32 %1, %1, 0;\n\taddc.u32 %2, 0, 0;"
+      : "+r"(m0), "+r"(m1), "=r"(over));
+  const uint32_t f1 = (m1 >> 11) | (over << 21), f0 = __funnelshift_r(m0, m1, 11);
   // (f1 : f0) in [2^52, 2^53], value (f1 : f0) 2^ex
   const int ex = 43 - s - (z1 ? 64 : (z2 ? 32 : 0)) + e;
   const int be = ex + 1075;
-  if (be > 0 && be < 2046)
+  const uint32_t sign = sg & 0x80000000u;
+  if (a != 0u && static_cast<unsigned>(be - 1) < 2045u)
     return __hiloint2double(static_cast<int>(((static_cast<uint32_t>(be - 1) << 20) + f1) | sign),
                             static_cast<int>(f0));
+  if (a == 0u) return 0.0;
   const double d = ldexp(__hiloint2double(static_cast<int>((1074u << 20) + f1), static_cast<int>(f0)), ex);
   return sign ? -d : d;
+}
+
+__device__ __forceinline__ double sums_to_double(long long hi, long long lo, int e) {
+  return fixed_to_double(hi + (lo >> kLoBits), static_cast<uint32_t>(lo), e);
+}
+
+// FP64 operations that are not to be speculated: an FP64 instruction takes the
+// SM quarter's pipe for 64 cycles per warp, also where its result is not used.
+__device__ __forceinline__ double mul_here(double a, double b) {
+  double d;
+  asm volatile("mul.rn.f64 %0, %1, %2;" : "=d"(d) : "d"(a), "d"(b));
+  return d;
+}
+__device__ __forceinline__ double fma_here(double a, double b, double c) {
+  double d;
+  asm volatile("fma.rn.f64 %0, %1, %2, %3;" : "=d"(d) : "d"(a), "d"(b), "d"(c));
+  return d;
+}
+
+// A lane holds eight consecutive values of its row; they leave row by row: lane
+// l takes value l % 8 of rows l / 8, + 4, ... (item i of f(i, x)), so that a
+// warp's access covers four rows of 64 contiguous bytes and not 32 rows of 8.
+// All lanes call it.
+// load(i) first, for all items together: what the values are to be added to.
+template <class L, class F>
+__device__ __forceinline__ void by_rows(unsigned long long* stg, int lane, const unsigned long long (&v)[8],
+                                        const L& load, const F& f) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) stg[lane * 8 + (j ^ (lane & 7))] = v[j];
+  __syncwarp();
+  double old[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) old[i] = load(i);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = 4 * i + (lane >> 3);
+    f(i, stg[r * 8 + ((lane & 7) ^ (r & 7))], old[i]);
+  }
+  __syncwarp();
+}
+// The (hi, lo) of 32 rows into 64-bit partial sums: element (r, c) at part +
+// 2 (r * n + c) for r < rows, c < n; r, c: the warp's first row and column.
+// only: the one unit of its tile, which stores and does not add.
+__device__ __forceinline__ void add_partial(unsigned long long* part, bool only, long long n, int rows, int r, int c,
+                                            int lane, long long (&hi)[kCols], uint32_t (&lo)[kCols],
+                                            unsigned long long* stg) {
+  const int k = lane & 7;
+  unsigned long long* p = part + ((r + (lane >> 3)) * n + c + (k >> 1)) * 2 + (k & 1);
+  const int left = rows - r - (lane >> 3);
+#pragma unroll
+  for (int h = 0; h < kCols; h += 4) {
+    unsigned long long v[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      v[2 * j] = static_cast<unsigned long long>(hi[h + j]);
+      v[2 * j + 1] = lo[h + j];
+    }
+    const bool in = c + h + (k >> 1) < n;
+    by_rows(stg, lane, v, [](int) { return 0.0; }, [&](int i, unsigned long long x, double) {
+      unsigned long long* q = p + 8 * i * n + 2 * h;
+      if (!in || 4 * i >= left) return;
+      if (only)
+        *q = x;
+      else
+        atomicAdd(q, x);
+    });
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -334,13 +428,14 @@ __device__ __forceinline__ double fixed_to_double(long long hi, long long lo, in
 struct GemmJob {
   int m, n, K, nt, n_items, ks, stages, tri, ktri, tri_off;
   double alpha, beta;
+  int a_kind, accumulate;  // alpha 1 (0), -1 (1) or another (2); beta not 0
   double* C;
   long long ldc, cblk_stride, col0;
   int cblk;
   const int *ea, *eb;
   int per_z, za, zb;         // items and operand rows of one product of a batch
   long long c_z, a_z, b_z;   // C, A, B from one product to the next
-  unsigned long long* part;  // ks > 1: [nz][m][n][2] integer sums
+  unsigned long long* part;  // [nz][m][n][2] integer sums, or null: C is written directly
   const double *A, *B;
   long long lda, ldb;
   int ta, tb;
@@ -355,7 +450,7 @@ struct GemmJob {
     T.z = t / per_z;
     const int u = t - T.z * per_z, s = u % ks, x = u / ks;
     T.ra = x / nt * kM;
-    T.rb = x % nt * kN;
+    T.rb = x % nt * kN2;
     T.ya = T.ra + T.z * za;
     T.yb = T.rb + T.z * zb;
     const int from = ktri ? min(max(T.ra + tri_off, 0) / kChunk, stages) : 0;
@@ -371,6 +466,10 @@ struct GemmJob {
     return T;
   }
   __device__ bool skip(int ya, int yb) const { return tri && yb >= ya + kM + tri_off; }
+  __device__ void half(Tile& T, int rank) const {
+    T.yb += rank * kN;
+    T.rb += rank * kN;
+  }
   __device__ int nchunks(const Tile& T) const { return T.n; }
   struct Iter {
     int x;
@@ -390,46 +489,59 @@ struct GemmJob {
     for (int k = 0; k < K; ++k) s = fma(at(A + z * a_z, lda, ta, r, k), at(B + z * b_z, ldb, tb, c, k), s);
     return s;
   }
-  __device__ void store(int z, int r, int c, double v) const {
+  __device__ double* place(int z, int r, int c) const {
     long long at = c;
     if (cblk) {
       const uint32_t q = static_cast<uint32_t>(c + col0), b = static_cast<uint32_t>(cblk);
       at = q / b * cblk_stride + q % b;
     }
-    double* p = C + z * c_z + r * ldc + at;
-    const double w = alpha == 1.0 ? v : (alpha == -1.0 ? -v : alpha * v);  // most calls spare the FP64 pipe
-    *p = beta == 0.0 ? w : fma(beta, *p, w);
+    return C + z * c_z + r * ldc + at;
   }
-  __device__ void write(long long (&hi)[kCols], long long (&lo)[kCols], const Tile& T, int row, int c0) const {
-    const int r = T.ra + row;
-    if (r >= m) return;
+  __device__ double combine(double v, double old) const {
+    double w = a_kind == 0 ? v : -v;
+    if (a_kind == 2) w = mul_here(alpha, v);
+    if (accumulate) w = fma_here(beta, old, w);
+    return w;
+  }
+  __device__ void store(int z, int r, int c, double v) const {
+    double* p = place(z, r, c);
+    *p = combine(v, accumulate ? *p : 0.0);
+  }
+  __device__ int row_exp(const Tile& T, int row) const { return T.ra + row < m ? ea[T.z * za + T.ra + row] : kOut; }
+  __device__ int col_exp(const Tile& T, int c) const { return T.rb + c < n ? eb[T.z * zb + T.rb + c] : kOut; }
+  __device__ void write(long long (&hi)[kCols], uint32_t (&lo)[kCols], const Tile& T, int row0, int lane, int c0,
+                        int er, int ec, unsigned long long* stg) const {
+    const int r = T.ra + row0, c = T.rb + c0;
     if (part) {
-      unsigned long long* p = part + ((static_cast<long long>(T.z) * m + r) * n + T.rb + c0) * 2;
-#pragma unroll
-      for (int j = 0; j < kCols; ++j) {
-        if (T.rb + c0 + j >= n) break;
-        carry(hi[j], lo[j]);
-        atomicAdd(p + 2 * j, static_cast<unsigned long long>(hi[j]));
-        atomicAdd(p + 2 * j + 1, static_cast<unsigned long long>(lo[j]));
-      }
+      add_partial(part + static_cast<long long>(T.z) * m * n * 2, ks == 1, n, m, r, c, lane, hi, lo, stg);
       return;
     }
-    const int a = ea[T.z * za + r];
-    unsigned bad = 0;  // columns that need the FP64 operands
+    const int left = m - r - (lane >> 3);
+    const Exps ex(er, ec);
 #pragma unroll
-    for (int j = 0; j < kCols; ++j) {
-      const int c = T.rb + c0 + j;
-      if (c >= n) break;
-      const int b = eb[T.z * zb + c];
-      if (a == kBad || b == kBad)
-        bad |= 1u << j;
-      else
-        store(T.z, r, c, fixed_to_double(hi[j], lo[j], a + b + kUnit));
-    }
-    while (bad) {
-      const int c = T.rb + c0 + __ffs(bad) - 1;
-      store(T.z, r, c, direct(T.z, r, c));
-      bad &= bad - 1;
+    for (int h = 0; h < kCols; h += 8) {
+      unsigned long long v[8];
+      unsigned bad = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        v[j] = static_cast<unsigned long long>(
+            __double_as_longlong(fixed_to_double(hi[h + j], lo[h + j], ex.sum(h + j))));
+        if (ex.in(h + j) && ex.bad(h + j)) bad |= 1u << j;
+      }
+      if (__any_sync(0xffffffffu, bad != 0)) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if ((bad >> j) & 1u) v[j] = static_cast<unsigned long long>(
+              __double_as_longlong(direct(T.z, r + lane, c + h + j)));
+      }
+      const int cc = c + h + (lane & 7);
+      const bool in = cc < n;
+      double* p = place(T.z, r + (lane >> 3), cc);
+      by_rows(
+          stg, lane, v, [&](int i) { return accumulate && in && 4 * i < left ? p[4 * i * ldc] : 0.0; },
+          [&](int i, unsigned long long x, double old) {
+            if (in && 4 * i < left) p[4 * i * ldc] = combine(__longlong_as_double(static_cast<long long>(x)), old);
+          });
     }
   }
 };
@@ -437,20 +549,21 @@ __global__ void k_gemm_finish(const GemmJob j, int nz) {
   const long long mn = static_cast<long long>(j.m) * j.n;
   for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < mn * nz;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int z = static_cast<int>(i / mn);
-    const long long e = i - z * mn;
-    const int r = static_cast<int>(e / j.n), c = static_cast<int>(e % j.n);
-    if (j.skip(r / kM * kM, c / kN * kN)) continue;
+    // m n nz <= 2^28 here (k_splits)
+    const int z = static_cast<int>(static_cast<unsigned>(i) / static_cast<unsigned>(mn));
+    const unsigned e = static_cast<unsigned>(i - z * mn);
+    const int r = static_cast<int>(e / static_cast<unsigned>(j.n)), c = static_cast<int>(e % static_cast<unsigned>(j.n));
+    if (j.skip(r / kM * kM, c / kN2 * kN2)) continue;
     const ulonglong2 v = reinterpret_cast<const ulonglong2*>(j.part)[i];
     const int a = j.ea[z * j.za + r], b = j.eb[z * j.zb + c];
     j.store(z, r, c, a == kBad || b == kBad ? j.direct(z, r, c)
-                                            : fixed_to_double(static_cast<long long>(v.x),
-                                                              static_cast<long long>(v.y), a + b + kUnit));
+                                            : sums_to_double(static_cast<long long>(v.x),
+                                                             static_cast<long long>(v.y), a + b + kUnit));
   }
 }
 
 // ---------------------------------------------------------------------------
-// steps A / B of Eq. 3 in FP64: one tile = 128 rows of the A operand x 64 of
+// steps A / B of Eq. 3 in FP64: one tile = 128 rows of the A operand x 128 of
 // the B operand of one panel task
 //   mode 0 (X): A = panel rows n = (pw, s'), B = G^occ rows mu
 //   mode 1 (Y): A = G^virt rows sigma (batch), B = panel rows n = (pw, mu')
@@ -465,7 +578,7 @@ struct Panel64Job {
   const long long* rowbase;
   const int* rowmul;
   const int *pe, *ge;  // exponents of the panel rows and of G's rows
-  double* out;
+  double* out_;
   const double *pool, *G;
   const int* lam;
   int nao;
@@ -479,11 +592,15 @@ struct Panel64Job {
     Tile T;
     T.task = e.x;
     T.a0 = e.y * kM;
-    T.b0 = e.z * kN;
+    T.b0 = e.z * kN2;
     T.ya = (mode == 0 ? tk.p_row0 : tk.g_row0) + T.a0;
     T.yb = (mode == 0 ? tk.g_row0 : tk.p_row0) + T.b0;
     T.n = (tk.K + kChunk - 1) / kChunk;
     return T;
+  }
+  __device__ void half(Tile& T, int rank) const {
+    T.yb += rank * kN;
+    T.b0 += rank * kN;
   }
   __device__ int nchunks(const Tile& T) const { return T.n; }
   struct Iter {
@@ -503,47 +620,44 @@ struct Panel64Job {
               pool[tk.panel_off + static_cast<long long>(k) * tk.N + n], s);
     return s;
   }
-  __device__ void write(long long (&hi)[kCols], long long (&lo)[kCols], const Tile& T, int row, int c0) const {
+  __device__ int row_exp(const Tile& T, int row) const {
     const PanelTask64& tk = tasks[T.task];
-    const int a = T.a0 + row, b = T.b0 + c0;
-    const int nsig = tk.nsig;
-    unsigned bad = 0;
+    const int a = T.a0 + row;
+    return mode == 0 ? (a < tk.N ? pe[tk.p_row0 + a] : kOut) : (a < R ? ge[r0 + a] : kOut);
+  }
+  __device__ int col_exp(const Tile& T, int c) const {
+    const PanelTask64& tk = tasks[T.task];
+    const int b = T.b0 + c;
+    return mode == 0 ? (b < R ? ge[r0 + b] : kOut) : (b < tk.N ? pe[tk.p_row0 + b] : kOut);
+  }
+  __device__ void write(long long (&hi)[kCols], uint32_t (&lo)[kCols], const Tile& T, int row0, int lane, int c0,
+                        int er, int ec, unsigned long long*) const {
+    const PanelTask64& tk = tasks[T.task];
+    const int a = T.a0 + row0 + lane, b = T.b0 + c0, nsig = tk.nsig;
+    const int pw = (mode == 0 ? a : b) / nsig;
+    int sp = (mode == 0 ? a : b) - pw * nsig;
+    double* o = out_ + static_cast<long long>(tk.p0 + pw - P0b) * ldk;  // where the first column goes,
+    long long next, wrap = 0;  // from one column to the next, and (mode 1) on to the next RI row
     if (mode == 0) {
-      if (a >= tk.N) return;
-      const int pw = a / nsig, sp = a - pw * nsig;
-      const int ea = pe[tk.p_row0 + a];
-      double* o = out + static_cast<long long>(tk.p0 + pw - P0b) * ldk + tk.seg + sp;
-#pragma unroll
-      for (int j = 0; j < kCols; ++j) {
-        const int mu = b + j;
-        if (mu >= R) break;
-        const int eb = ge[r0 + mu];
-        if (ea == kBad || eb == kBad)
-          bad |= 1u << j;
-        else
-          o[static_cast<long long>(r0 + mu) * nsig] = fixed_to_double(hi[j], lo[j], ea + eb + kUnit);
-      }
-      for (; bad; bad &= bad - 1) {
-        const int mu = b + __ffs(bad) - 1;
-        o[static_cast<long long>(r0 + mu) * nsig] = direct(tk, a, r0 + mu);
-      }
+      next = nsig;
+      o += tk.seg + sp + (r0 + b) * next;
     } else {
-      if (a >= R) return;
-      const int ea = ge[r0 + a];
-      const long long rb = rowbase[a], rm = rowmul[a];
-      int pw = b / nsig, sp = b - pw * nsig;
-      double* o = out + static_cast<long long>(tk.p0 + pw - P0b) * ldk + rb + tk.aom * rm;
+      next = er == kOut ? 0 : rowmul[a];
+      o += (er == kOut ? 0 : rowbase[a]) + (tk.aom + sp) * next;
+      wrap = ldk - nsig * next;
+    }
+    const Exps ex(er, ec);
 #pragma unroll
-      for (int j = 0; j < kCols; ++j) {
-        const int n = b + j;
-        if (n >= tk.N) break;
-        const int eb = pe[tk.p_row0 + n];
-        o[sp * rm] = (ea == kBad || eb == kBad) ? direct(tk, n, r0 + a)
-                                                : fixed_to_double(hi[j], lo[j], ea + eb + kUnit);
-        if (++sp == nsig) {
-          sp = 0;
-          o += ldk;
-        }
+    for (int j = 0; j < kCols; ++j) {
+      double x = fixed_to_double(hi[j], lo[j], ex.sum(j));
+      if (ex.in(j)) {
+        if (ex.bad(j)) x = mode == 0 ? direct(tk, a, r0 + b + j) : direct(tk, b + j, r0 + a);
+        *o = x;
+      }
+      o += next;
+      if (mode == 1 && ++sp == nsig) {
+        sp = 0;
+        o += wrap;
       }
     }
   }
@@ -573,13 +687,14 @@ struct Chi64Job {
     Tile T;
     T.id = unit_tile[u];
     T.ya = T.id / nqt * kM;
-    T.yb = T.id % nqt * kN;
+    T.yb = T.id % nqt * kN2;
     T.cnt = unit_count[u];
     T.list = tasks + static_cast<long long>(T.id) * nslab + unit_first[u];
     T.n = 0;
     for (int i = 0; i < T.cnt; ++i) T.n += slab_len[T.list[i]] / kChunk;
     return T;
   }
+  __device__ void half(Tile& T, int rank) const { T.yb += rank * kN; }
   __device__ int nchunks(const Tile& T) const { return T.n; }
   struct Iter {
     const Chi64Job* j;
@@ -617,29 +732,38 @@ struct Chi64Job {
         s = fma(X[p * ldk + slab_k0[l[i]] + k], Y[q * ldk + slab_k0[l[i]] + k], s);
     return s;
   }
-  __device__ void add(int id, int p, int q, long long hi, long long lo) const {
-    const int a = ex[p], b = ey[q];
-    double* c = chi + static_cast<long long>(P0 + p) * nri + q;
-    *c -= (a == kBad || b == kBad) ? direct(id, p, q) : fixed_to_double(hi, lo, a + b + kUnit);
+  __device__ double value(int id, int p, int q, long long hi, long long lo, int a, int b) const {
+    return (a == kBad || b == kBad) ? direct(id, p, q) : sums_to_double(hi, lo, a + b + kUnit);
   }
-  __device__ void write(long long (&hi)[kCols], long long (&lo)[kCols], const Tile& T, int row, int c0) const {
-    const int p = T.ya + row;
-    if (p >= prow) return;
+  __device__ int row_exp(const Tile& T, int row) const { return T.ya + row < prow ? ex[T.ya + row] : kOut; }
+  __device__ int col_exp(const Tile& T, int c) const { return T.yb + c < nri ? ey[T.yb + c] : kOut; }
+  __device__ void write(long long (&hi)[kCols], uint32_t (&lo)[kCols], const Tile& T, int row0, int lane, int c0,
+                        int er, int ec, unsigned long long* stg) const {
+    const int p0 = T.ya + row0, q0 = T.yb + c0;
     if (part) {
-      unsigned long long* o = part + (static_cast<long long>(p) * nri + T.yb + c0) * 2;
+      add_partial(part, false, nri, prow, p0, q0, lane, hi, lo, stg);
+      return;
+    }
+    const int left = prow - p0 - (lane >> 3);
+    const Exps es(er, ec);
 #pragma unroll
-      for (int j = 0; j < kCols; ++j) {
-        if (T.yb + c0 + j >= nri) break;
-        carry(hi[j], lo[j]);
-        atomicAdd(o + 2 * j, static_cast<unsigned long long>(hi[j]));
-        atomicAdd(o + 2 * j + 1, static_cast<unsigned long long>(lo[j]));
-      }
-    } else {
+    for (int h = 0; h < kCols; h += 8) {
+      unsigned long long v[8];
 #pragma unroll
-      for (int j = 0; j < kCols; ++j) {
-        if (T.yb + c0 + j >= nri) break;
-        add(T.id, p, T.yb + c0 + j, hi[j], lo[j]);
+      for (int j = 0; j < 8; ++j) {
+        double x = fixed_to_double(hi[h + j], lo[h + j], es.sum(h + j));
+        if (es.in(h + j) && es.bad(h + j)) x = direct(T.id, p0 + lane, q0 + h + j);
+        v[j] = static_cast<unsigned long long>(__double_as_longlong(x));
       }
+      const int q = q0 + h + (lane & 7);
+      const bool in = q < nri;
+      const long long ld = nri;
+      double* c = chi + (P0 + p0 + (lane >> 3)) * ld + q;
+      by_rows(
+          stg, lane, v, [&](int i) { return in && 4 * i < left ? c[4 * i * ld] : 0.0; },
+          [&](int i, unsigned long long x, double old) {
+            if (in && 4 * i < left) c[4 * i * ld] = old - __longlong_as_double(static_cast<long long>(x));
+          });
     }
   }
 };
@@ -648,10 +772,11 @@ __global__ void k_chi64_finish(const Chi64Job j) {
   for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
     const int p = static_cast<int>(i / j.nri), q = static_cast<int>(i % j.nri);
-    const int id = p / kM * j.nqt + q / kN;
+    const int id = p / kM * j.nqt + q / kN2;
     if (j.counts[id] == 0) continue;
     const ulonglong2 v = reinterpret_cast<const ulonglong2*>(j.part)[i];
-    j.add(id, p, q, static_cast<long long>(v.x), static_cast<long long>(v.y));
+    j.chi[static_cast<long long>(j.P0 + p) * j.nri + q] -=
+        j.value(id, p, q, static_cast<long long>(v.x), static_cast<long long>(v.y), j.ex[p], j.ey[q]);
   }
 }
 
@@ -659,37 +784,97 @@ __global__ void k_chi64_finish(const Chi64Job j) {
 // the persistent kernel: warp 0 TMA producer, warp 1 MMA issuer, warps 2-17
 // epilogue; every wait is bounded (tc_ptx.h)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+// eight columns from each of two addresses, both loads in flight together
+__device__ __forceinline__ void tmem_ld8x2(uint32_t a0, uint32_t a1, uint32_t (&r)[8], uint32_t (&s)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
+               : "r"(a0));
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(s[0]), "=r"(s[1]), "=r"(s[2]), "=r"(s[3]), "=r"(s[4]), "=r"(s[5]), "=r"(s[6]), "=r"(s[7])
+               : "r"(a1));
   asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(s[0]), "+r"(s[1]), "+r"(s[2]), "+r"(s[3]), "+r"(s[4]), "+r"(s[5]), "+r"(s[6]), "+r"(s[7])
                :
                : "memory");
 }
+// An accumulator (an integer in FP32) as int.  small: |v| <= 2^22, as for
+// diagonals 0-2 (the leading digits are at most 64): adding 1.5 2^23 puts the
+// integer in the low bits, on the FP32 pipe at eight times the rate of the
+// conversion.
+__device__ __forceinline__ int to_int(uint32_t v, bool small) {
+  if (small) return __float_as_int(__uint_as_float(v) + 12582912.f) - 0x4B400000;
+  return __float2int_rn(__uint_as_float(v));
+}
+
+// Adds the accumulators of diagonals 2p and 2p + 1 into this thread's columns:
+// pairs 0 and 1, times 2^24, 2^16, 2^8 and 1, into hi; pairs 2 and 3 the same
+// into lo, with the carry into hi at once (lo as 64 bits would cost the
+// registers that the way out needs).
+template <bool kHi>
+__device__ __forceinline__ bool add_pair(int p, int q, uint64_t* acc_full, uint64_t* acc_empty, uint32_t parity,
+                                         volatile int* abort_flag, uint32_t row_addr, int lane,
+                                         long long (&hi)[kCols], uint32_t (&lo)[kCols]) {
+  if (!mbar_wait(&acc_full[p], parity, abort_flag)) return false;
+  tc_fence_after();
+  const int w0 = q ? 1 << 8 : 1 << 24, w1 = q ? 1 : 1 << 16;
+#pragma unroll
+  for (int h = 0; h < kCols; h += 8) {  // 16 columns at once would spill
+    uint32_t r0[8], r1[8];
+    tmem_ld8x2(row_addr + static_cast<uint32_t>(2 * p * kN + h),
+               row_addr + static_cast<uint32_t>((2 * p + 1) * kN + h), r0, r1);
+    if (h + 8 == kCols) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acc_empty[p]);
+    }
+    // diagonals 0 to 2 are at most 2^22
+    if (kHi && q == 0) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        hi[h + j] += static_cast<long long>(to_int(r0[j], true)) * w0;
+        hi[h + j] += static_cast<long long>(to_int(r1[j], true)) * w1;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        long long t = kHi ? hi[h + j] : static_cast<long long>(lo[h + j]);
+        t += static_cast<long long>(to_int(r0[j], false)) * w0;
+        t += static_cast<long long>(to_int(r1[j], false)) * w1;
+        if (kHi) {
+          hi[h + j] = t;
+        } else {
+          hi[h + j] += t >> kLoBits;
+          lo[h + j] = static_cast<uint32_t>(t);
+        }
+      }
+    }
+  }
+  return true;
+}
 
 template <class Job>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     k_emu(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const Job job,
           int* __restrict__ err_flag) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
+  uint8_t* staging = smem + kStages * kStageBytes;
+  uint64_t* full = reinterpret_cast<uint64_t*>(staging + kEpiWarps * kStgBytes);
   uint64_t* empty = full + kStages;
   uint64_t* acc_full = empty + kStages;
-  uint64_t* acc_empty = acc_full + kS;
-  uint64_t* drain = acc_empty + kS;
+  uint64_t* acc_empty = acc_full + kPairs;
+  uint64_t* drain = acc_empty + kPairs;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = __reduce_max_sync(0xffffffffu, threadIdx.x / 32), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+      mbar_init(&empty[s], 2);  // both CTAs have read their copy of the stage
     }
-    for (int b = 0; b < kS; ++b) {
+    for (int b = 0; b < kPairs; ++b) {
       mbar_init(&acc_full[b], 1);
       mbar_init(&acc_empty[b], kEpiWarps);
     }
@@ -704,9 +889,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // the peer's barriers are initialised
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const int n_items = job.items();
+  const int rank = blockIdx.x & 1, first = blockIdx.x >> 1, step = gridDim.x >> 1;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -715,8 +902,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool armed[kStages] = {};
       uint32_t armed_parity[kStages] = {};
       bool ok = true;
-      for (int t = blockIdx.x; t < n_items && ok; t += gridDim.x) {
-        const typename Job::Tile T = job.tile(t);
+      for (int t = first; t < n_items && ok; t += step) {
+        typename Job::Tile T = job.tile(t);
+        job.half(T, rank);
         const int n = job.nchunks(T);
         typename Job::Iter it;
         it.init(&job, T);
@@ -730,7 +918,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           armed[stage] = true;
           armed_parity[stage] = phase;
           const int x = it.next();
-          tma_load_3d(st, &map_a, x, T.ya, 0, &full[stage]);
+          // this CTA's half of A's digits to both CTAs, its own columns of B
+          const int s0 = rank * (kS / 2);
+          tma_load_3d_pair(st + s0 * kABytes, &map_a, x, T.ya, s0, &full[stage]);
           tma_load_3d(st + kS * kABytes, &map_b, x, T.yb, 0, &full[stage]);
           if (++stage == kStages) {
             stage = 0;
@@ -738,6 +928,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
+      // both CTAs' releases of the last stages have arrived here: none is on
+      // its way to a CTA that has left
+      for (int s = 0; s < kStages && ok; ++s)
+        if (armed[s]) ok = mbar_wait(&empty[s], armed_parity[s], abort_flag);
       if (!ok) {
         *abort_flag = 1;
         atomicOr(err_flag, 1);
@@ -748,13 +942,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == 1) {
     // the whole warp runs the loop: uniform control flow keeps the
     // descriptors in uniform registers; one elected lane issues
-    constexpr uint32_t idesc = idesc_f32(kM, kN, true);
+    constexpr uint32_t one = idesc_f32(kM, kN, true), two = idesc_f32(kM, 2 * kN, true);
     const uint32_t lead = elect_one();
     const uint32_t tmu = __reduce_max_sync(0xffffffffu, tmem);
     int stage = 0;
     uint32_t phase = 0, aphase = 1;
     bool ok = true, issued = false;
-    for (int t = blockIdx.x; t < n_items && ok; t += gridDim.x) {
+    for (int t = first; t < n_items && ok; t += step) {
       const typename Job::Tile T = job.tile(t);
       const int n = __reduce_max_sync(0xffffffffu, job.nchunks(T));
       for (int i = 0; i < n && ok; ++i) {
@@ -766,28 +960,35 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t a_lo = static_cast<uint32_t>(da), hi = static_cast<uint32_t>(da >> 32);
         const uint32_t b_lo = a_lo + static_cast<uint32_t>((kS * kABytes) >> 4);
 #pragma unroll
-        for (int d = 0; d < kS; ++d) {
+        for (int p = 0; p < kPairs; ++p) {
           if (first) {
-            ok = __all_sync(0xffffffffu, mbar_wait(&acc_empty[d], aphase, abort_flag));
+            ok = __all_sync(0xffffffffu, mbar_wait(&acc_empty[p], aphase, abort_flag));
             if (!ok) break;
             tc_fence_after();
           }
           if (lead) {
-            const uint32_t acc = tmu + static_cast<uint32_t>(d * kN);
+            // digit a of A with digits 2p - a and 2p - a + 1 of B, whose rows
+            // follow one another, into the two accumulators side by side; the
+            // last digit of A only meets digit 0
+            const uint32_t acc = tmu + static_cast<uint32_t>(2 * p * kN);
 #pragma unroll
-            for (int a = 0; a <= d; ++a)
+            for (int a = 0; a <= 2 * p + 1; ++a)
 #pragma unroll
-              for (int k = 0; k < kSub; ++k)
-                mma_f16_lo(acc, a_lo + static_cast<uint32_t>((a * kABytes + k * kMmaK * 2) >> 4),
-                           b_lo + static_cast<uint32_t>(((d - a) * kBBytes + k * kMmaK * 2) >> 4), hi, idesc,
-                           (a | k) ? 1u : (first ? 0u : 1u));
-            if (last) mma_commit(&acc_full[d]);
+              for (int k = 0; k < kSub; ++k) {
+                const uint32_t da_lo = a_lo + static_cast<uint32_t>((a * kABytes + k * kMmaK * 2) >> 4);
+                if (a <= 2 * p)
+                  mma_f16_lo(acc, da_lo, b_lo + static_cast<uint32_t>(((2 * p - a) * kBBytes + k * kMmaK * 2) >> 4),
+                             hi, two, (a | k) ? 1u : (first ? 0u : 1u));
+                else
+                  mma_f16_lo(acc + kN, da_lo, b_lo + static_cast<uint32_t>((k * kMmaK * 2) >> 4), hi, one, 1u);
+              }
+            if (last) mma_commit(&acc_full[p]);
           }
           __syncwarp();
           issued = true;
         }
         if (!ok) break;
-        if (lead) mma_commit(&empty[stage]);
+        if (lead) mma_commit_pair(&empty[stage]);
         __syncwarp();
         if (last) aphase ^= 1u;
         if (++stage == kStages) {
@@ -808,51 +1009,38 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else {
     const int quad = warp & 3;
     const int c0 = ((warp - 2) >> 2) * kCols;
+    unsigned long long* stg = reinterpret_cast<unsigned long long*>(staging + (warp - 2) * kStgBytes);
     const uint32_t row_addr = tmem + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(c0);
     uint32_t aphase = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < n_items && ok; t += gridDim.x) {
-      const typename Job::Tile T = job.tile(t);
+    for (int t = first; t < n_items && ok; t += step) {
+      typename Job::Tile T = job.tile(t);
       const int n = job.nchunks(T);
       if (n == 0) continue;
-      long long hi[kCols], lo[kCols];
+      job.half(T, rank);
+      // exponents of this lane's row and of column c0 + lane % 16, loaded here:
+      // beside the stores they would be fetched one by one
+      const int er = job.row_exp(T, quad * 32 + lane), ec = job.col_exp(T, c0 + lane % kCols);
+      // value = hi 2^32 + lo: 48 registers for 16 columns
+      long long hi[kCols];
+      uint32_t lo[kCols];
 #pragma unroll
-      for (int j = 0; j < kCols; ++j) hi[j] = lo[j] = 0;
+      for (int j = 0; j < kCols; ++j) {
+        hi[j] = 0;
+        lo[j] = 0;
+      }
       for (int i = 0; i < n && ok; i += kGroup, aphase ^= 1u) {
-#pragma unroll
-        for (int d = 0; d < kS; ++d) {
-          if (!mbar_wait(&acc_full[d], aphase, abort_flag)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {  // two halves: 16 columns at once would spill
-            uint32_t r[8];
-            tmem_ld8(row_addr + static_cast<uint32_t>(d * kN + 8 * h), r);
-            if (h == 1) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(&acc_empty[d]);
-            }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const int v = __float2int_rn(__uint_as_float(r[j]));
-              if (d < 4)
-                hi[8 * h + j] += static_cast<long long>(v) * (1 << (24 - 8 * d));
-              else
-                lo[8 * h + j] += static_cast<long long>(v) * (1 << (56 - 8 * d));
-            }
-          }
-        }
-        // a group adds less than 2^48 to lo
-        if ((i & 16383) == 16384 - kGroup) {
-#pragma unroll
-          for (int j = 0; j < kCols; ++j) carry(hi[j], lo[j]);
-        }
+        // pairs 0 and 1 (diagonals 0-3) into hi, 2 and 3 into lo; rolled, for
+        // the instruction cache
+#pragma unroll 1
+        for (int p = 0; p < kPairs / 2 && ok; ++p)
+          ok = add_pair<true>(p, p, acc_full, acc_empty, aphase, abort_flag, row_addr, lane, hi, lo);
+#pragma unroll 1
+        for (int p = 0; p < kPairs / 2 && ok; ++p)
+          ok = add_pair<false>(kPairs / 2 + p, p, acc_full, acc_empty, aphase, abort_flag, row_addr, lane, hi, lo);
       }
       if (!ok) break;
-      job.write(hi, lo, T, quad * 32 + lane, c0);
+      job.write(hi, lo, T, quad * 32, lane, c0, er, ec, stg);
     }
     if (!ok) {
       *abort_flag = 1;
@@ -861,6 +1049,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // neither CTA leaves while the other may write to it
   tc_fence_after();
   if (warp == 1) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
@@ -881,20 +1070,20 @@ int launch(const CUtensorMap& ma, const CUtensorMap& mb, const Job& job, int n_i
       return -1;
     attr_set.fetch_or(bit, std::memory_order_release);
   }
-  k_emu<Job><<<std::min(n_items, sms), kThreads, kSmem, st>>>(ma, mb, job, err_flag);
+  k_emu<Job><<<2 * std::min(n_items, std::max(sms / 2, 1)), kThreads, kSmem, st>>>(ma, mb, job, err_flag);
   return 0;
 }
 
 // K splits of an m x n product: the number of units that makes the last wave
-// over the SMs short.  Costs in stages (about 2 us each): a unit's start and
-// end about 3 (the write, or 128 KB of atomics), clearing and converting the
-// partial sums about 5 in all.
+// over the 76 clusters short.  Costs in stages (about 1.7 us each): a unit's
+// start and end about 3, clearing the partial sums about 3 in all.
 int k_splits(long long m, long long n, int K, int nz) {
-  const long long tiles = ((m + kM - 1) / kM) * ((n + kN - 1) / kN) * nz;
+  const long long tiles = ((m + kM - 1) / kM) * ((n + kN2 - 1) / kN2) * nz;
   const long long stages = (K + kChunk - 1) / kChunk;
+  if (m * n * nz > (1ll << 28)) return 1;  // 4 GB of partial sums
   long long best = 1, cost = 0;
   for (long long ks = 1; ks <= 64 && ks * 4 <= std::max(stages, 4ll); ++ks) {
-    const long long c = (tiles * ks + 151) / 152 * ((stages + ks - 1) / ks + 3) + (ks > 1 ? 5 : 0);
+    const long long c = (tiles * ks + 75) / 76 * ((stages + ks - 1) / ks + 3) + (ks > 1 ? 3 : 0);
     if (ks == 1 || c < cost) {
       cost = c;
       best = ks;
@@ -930,8 +1119,13 @@ void launch_emu_prep(EmuOp& op, const EmuSrc& s, cudaStream_t st) {
   }
 }
 
+// Sums go out as integers and a second kernel rounds them, also where K is not
+// split, as long as they stay in the L2 cache: beside the accumulators there
+// are few registers left for the conversion, which takes 20000 cycles per tile
+// there (a stage takes 3400), the integers alone 3500.
 size_t emu_gemm_ws_bytes(long long m, long long n, int K, int nz) {
-  return emu::k_splits(m, n, K, nz) > 1 ? static_cast<size_t>(m) * n * 16 * nz : 0;
+  const size_t bytes = static_cast<size_t>(m) * n * 16 * nz;
+  return bytes <= (size_t(96) << 20) || emu::k_splits(m, n, K, nz) > 1 ? bytes : 0;
 }
 
 int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, int* err_flag,
@@ -939,15 +1133,15 @@ int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, 
   const int m = static_cast<int>(A.s.rows), n = static_cast<int>(B.s.rows);
   if (m <= 0 || n <= 0) return 0;
   CUtensorMap ma, mb;
-  if (make_digit_map(&ma, A.dig, A.kp, A.s.nz > 1 ? A.stride_rows : A.s.rows, A.stride_rows, kEmuSlices, emu::kChunk, emu::kM) ||
+  if (make_digit_map(&ma, A.dig, A.kp, A.s.nz > 1 ? A.stride_rows : A.s.rows, A.stride_rows, kEmuSlices, emu::kChunk, emu::kM, kEmuSlices / 2) ||
       make_digit_map(&mb, B.dig, B.kp, B.s.nz > 1 ? B.stride_rows : B.s.rows, B.stride_rows, kEmuSlices, emu::kChunk,
-                     emu::kN))
+                     emu::kN, kEmuSlices))
     return -2;
   emu::GemmJob j{};
   j.m = m;
   j.n = n;
   j.K = A.s.K;
-  j.nt = (n + emu::kN - 1) / emu::kN;
+  j.nt = (n + emu::kN2 - 1) / emu::kN2;
   j.stages = std::max(1, (A.s.K + emu::kChunk - 1) / emu::kChunk);
   const int nz = A.s.nz;
   j.ks = ws ? emu::k_splits(m, n, A.s.K, nz) : 1;
@@ -966,6 +1160,8 @@ int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, 
   j.tri_off = static_cast<int>(g.tri_off);
   j.alpha = g.alpha;
   j.beta = g.beta;
+  j.a_kind = g.alpha == 1.0 ? 0 : (g.alpha == -1.0 ? 1 : 2);
+  j.accumulate = g.beta != 0.0;
   j.C = g.C;
   j.ldc = g.ldc;
   j.cblk = g.cblk;
@@ -979,13 +1175,13 @@ int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, 
   j.B = B.s.src;
   j.ldb = B.s.ld;
   j.tb = B.s.trans;
+  j.part = static_cast<unsigned long long*>(ws);
   if (j.ks > 1) {
-    j.part = static_cast<unsigned long long*>(ws);
     cudaMemsetAsync(ws, 0, static_cast<size_t>(m) * n * 16 * nz, st);
   }
   const int rc = emu::launch(ma, mb, j, j.n_items, err_flag, st);
   if (rc) return rc;
-  if (j.ks > 1) {
+  if (j.part) {
     const long long blocks = (static_cast<long long>(m) * n * nz + 255) / 256;
     emu::k_gemm_finish<<<static_cast<unsigned>(std::min<long long>(blocks, 152 * 16)), 256, 0, st>>>(j, nz);
   }
@@ -1019,9 +1215,11 @@ int launch_panel64(const Panel64Args& p, int* err_flag, cudaStream_t st) {
   if (p.n_tiles == 0) return 0;
   CUtensorMap mp, mg;
   const bool x = p.mode == 0;
+  const int whole = kEmuSlices, part = kEmuSlices / 2;  // digits per load of the B and A operand
   if (make_digit_map(&mp, p.panel_dig, p.kp, p.panel_rows, p.panel_rows, kEmuSlices, emu::kChunk,
-                     x ? emu::kM : emu::kN) ||
-      make_digit_map(&mg, p.g_dig, p.g_kp, p.g_rows, p.g_rows, kEmuSlices, emu::kChunk, x ? emu::kN : emu::kM))
+                     x ? emu::kM : emu::kN, x ? part : whole) ||
+      make_digit_map(&mg, p.g_dig, p.g_kp, p.g_rows, p.g_rows, kEmuSlices, emu::kChunk, x ? emu::kN : emu::kM,
+                     x ? whole : part))
     return -2;
   emu::Panel64Job j{p.tiles, p.n_tiles, p.mode, p.R,  p.r0,   p.P0b, p.tasks, p.ldk, p.rowbase,
                     p.rowmul, p.panel_exps, p.g_exps, p.out, p.pool, p.G, p.lam, p.nao};
@@ -1030,8 +1228,9 @@ int launch_panel64(const Panel64Args& p, int* err_flag, cudaStream_t st) {
 
 int launch_chi64(const EmuOp& x, const EmuOp& y, const Chi64Args& c, int* err_flag, cudaStream_t st) {
   CUtensorMap mx, my;
-  if (make_digit_map(&mx, x.dig, x.kp, x.s.rows, x.stride_rows, kEmuSlices, emu::kChunk, emu::kM) ||
-      make_digit_map(&my, y.dig, y.kp, y.s.rows, y.stride_rows, kEmuSlices, emu::kChunk, emu::kN))
+  if (make_digit_map(&mx, x.dig, x.kp, x.s.rows, x.stride_rows, kEmuSlices, emu::kChunk, emu::kM,
+                     kEmuSlices / 2) ||
+      make_digit_map(&my, y.dig, y.kp, y.s.rows, y.stride_rows, kEmuSlices, emu::kChunk, emu::kN, kEmuSlices))
     return -2;
   emu::Chi64Job j{c.units.u_tile, c.units.u_first, c.units.u_count, c.units.n_units, c.tasks, c.counts, c.nslab,
                   c.nqt, c.P0, c.prow, c.nri, c.slab_k0, c.slab_len, x.exps, y.exps, c.chi,

@@ -13,7 +13,7 @@ namespace gw {
 constexpr int kEmuSlices = 8;   // digits per operand element
 constexpr int kEmuProducts = 36;  // digit pairs of a product
 constexpr int kEmuTileM = 128;  // rows (A operand) and columns (B operand) of a tile
-constexpr int kEmuTileN = 64;
+constexpr int kEmuTileN = 128;
 
 // A matrix to be used as an operand: rows x K, element (r, k) at
 // src[r * ld + k], or src[k * ld + r] when trans.
@@ -94,7 +94,7 @@ void launch_gather_digits(const EmuOp& g, int rbase, int R, const PanelTask64* t
 // Steps A (mode 0, X) and B (mode 1, Y): rows r0 .. r0 + R of G, output as
 // k_panel_gemm's (k_simt.cu).
 struct Panel64Args {
-  const int4* tiles;  // (task, A tile of 128 rows, B tile of 64, 0)
+  const int4* tiles;  // (task, A tile of 128 rows, B tile of 128, 0)
   int n_tiles, mode, R, r0, P0b;
   const PanelTask64* tasks;
   long long ldk;
@@ -114,7 +114,7 @@ struct Panel64Args {
   int nao;
 };
 int launch_panel64(const Panel64Args& p, int* err_flag, cudaStream_t st);
-// Step C over work units (k_tc.h, launch_plan_units) of 128 x 64 tiles.  part:
+// Step C over work units (k_tc.h, launch_plan_units) of 128 x 128 tiles.  part:
 // 16 bytes per (X row, RI function) of partial sums, or null when a unit is a
 // whole tile.
 struct Chi64Args {

@@ -1825,8 +1825,8 @@ int make_slice_map(CUtensorMap* map, const void* base, long long k_len, long lon
 }
 
 int make_digit_map(CUtensorMap* map, const void* base, long long k_len, long long rows, long long stride_rows,
-                   int slices, int box_k, int box_rows) {
-  return encode_map(map, base, k_len, rows, stride_rows, slices, box_k, box_rows, slices, 1, CU_TENSOR_MAP_SWIZZLE_64B);
+                   int slices, int box_k, int box_rows, int box_slices) {
+  return encode_map(map, base, k_len, rows, stride_rows, slices, box_k, box_rows, box_slices, 1, CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
 int tc_tile_rows() { return tc::kTileM; }

@@ -19,10 +19,10 @@ namespace gw {
 int make_slice_map(CUtensorMap* map, const void* base, long long k_len, long long rows, int slices,
                    int box_rows, int f16);
 // The same for the digit operands of the FP64 products (k_emu.cu): binary16,
-// box = box_k (32: 64-byte rows, 64-byte swizzle) x box_rows x every slice;
+// box = box_k (32: 64-byte rows, 64-byte swizzle) x box_rows x box_slices;
 // slices stride_rows rows apart.
 int make_digit_map(CUtensorMap* map, const void* base, long long k_len, long long rows, long long stride_rows,
-                   int slices, int box_k, int box_rows);
+                   int slices, int box_k, int box_rows, int box_slices);
 // Rows (and columns) of one step-C tile of the tensor-core kernel.
 int tc_tile_rows();
 // Test hook (process-wide): while on, every tensor-core kernel launched has
