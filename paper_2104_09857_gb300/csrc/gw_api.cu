@@ -158,6 +158,10 @@ void reset_tensor(gw_ctx* ctx) {
   ctx->d_pt = nullptr;
   ctx->pt_ok = false;
   free_panel_digits(ctx);
+  free_dev(ctx->d_bn_bucket);
+  free_dev(ctx->d_bn_list);
+  ctx->d_bn_bucket = ctx->d_bn_list = nullptr;
+  ctx->bn_ok = false;
   ctx->ycov_valid = false;
 }
 
@@ -190,6 +194,7 @@ int plan_panels(gw_ctx* ctx, double thr) {
   ctx->panels_thr = -1.0;
   ctx->pt_ok = false;
   ctx->pd_ok = false;
+  ctx->bn_ok = false;
   ctx->panel32_ok = false;
   ctx->ycov_valid = false;
   const int n = ctx->n_at;
@@ -1997,7 +2002,40 @@ int tc_finish_tau(gw_ctx* ctx, std::vector<double>& fc_host) {
 }  // namespace
 
 namespace gw {
-int build_panels_for(gw_ctx* ctx, double thr) { return build_panels(ctx, thr); }
+int plan_bn_lists(gw_ctx* ctx, double thr) {
+  if (ctx->d_t3f)
+    return fail(ctx, GW_ERR_UNSUPPORTED,
+                "the self-energy needs the tensor in FP64 (it is kept in FP32: option tensor_fp32)");
+  int rc;
+  if ((rc = plan_panels(ctx, thr))) return rc;
+  if (ctx->bn_ok) return GW_OK;
+  const int n = ctx->n_at;
+  // kept blocks are in the order (A, B, P): a bucket's entries come sorted by
+  // their partner atom
+  std::vector<int> bucket((size_t)n * n + 1, 0);
+  for (int b : ctx->plan_kept) {
+    const int A = ctx->blk[3 * b], B = ctx->blk[3 * b + 1], p = ctx->blk[3 * b + 2];
+    ++bucket[(size_t)B * n + p + 1];
+    if (A != B) ++bucket[(size_t)A * n + p + 1];
+  }
+  for (size_t i = 0; i < (size_t)n * n; ++i) bucket[i + 1] += bucket[i];
+  std::vector<int> list(bucket.back()), at(bucket.begin(), bucket.end() - 1);
+  for (int b : ctx->plan_kept) {
+    const int A = ctx->blk[3 * b], B = ctx->blk[3 * b + 1], p = ctx->blk[3 * b + 2];
+    list[at[(size_t)B * n + p]++] = b << 1;
+    if (A != B) list[at[(size_t)A * n + p]++] = b << 1 | 1;
+  }
+  free_dev(ctx->d_bn_bucket);
+  free_dev(ctx->d_bn_list);
+  ctx->d_bn_bucket = ctx->d_bn_list = nullptr;
+  GW_TRY(cudaMalloc(&ctx->d_bn_bucket, bucket.size() * sizeof(int)));
+  GW_TRY(cudaMalloc(&ctx->d_bn_list, std::max<size_t>(list.size(), 1) * sizeof(int)));
+  GW_TRY(cudaMemcpy(ctx->d_bn_bucket, bucket.data(), bucket.size() * sizeof(int), cudaMemcpyHostToDevice));
+  if (!list.empty())
+    GW_TRY(cudaMemcpy(ctx->d_bn_list, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice));
+  ctx->bn_ok = true;
+  return GW_OK;
+}
 int work_buffer(gw_ctx* ctx, const char* name, size_t bytes, void** out) { return ws(ctx, name, bytes, out); }
 void work_trim(gw_ctx* ctx, const char* prefix, size_t keep) {
   const size_t n = std::strlen(prefix);
@@ -2457,7 +2495,7 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
     gw::TraceRange trace_tau("chi: one tau point");
     GW_TRY(cudaEventRecord(ev[0], ctx->stream));
     ctx->cur_tau = ctx->tau[j];
-    if ((rc = gw::greens_fp64(ctx, ctx->tau[j], cso, csv, go, gv, ctx->stream))) return rc;
+    if ((rc = gw::greens_fp64(ctx, *ctx, ctx->tau[j], cso, csv, go, gv, ctx->stream))) return rc;
     GW_CHECK_LAUNCH();
     ctx->stats.kernel_launches += 3;
     if (f16) {
@@ -2479,10 +2517,9 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
     }
     std::vector<unsigned char> hfo((size_t)n_at * n_at, 1), hfv((size_t)n_at * n_at, 1);
     if (thr > 0.0) {
-      gw::launch_sym_block_filter(go, nao, ctx->d_ao_off, n_at, thr, flo, ctx->stream);
-      gw::launch_sym_block_filter(gv, nao, ctx->d_ao_off, n_at, thr, flv, ctx->stream);
+      gw::launch_sym_block_filter(go, gv, nao, ctx->d_ao_off, n_at, thr, flo, flv, ctx->stream);
       GW_CHECK_LAUNCH();
-      ctx->stats.kernel_launches += 2;
+      ctx->stats.kernel_launches += 1;
       GW_TRY(cudaMemcpyAsync(hfo.data(), flo, hfo.size(), cudaMemcpyDeviceToHost, ctx->stream));
       GW_TRY(cudaMemcpyAsync(hfv.data(), flv, hfv.size(), cudaMemcpyDeviceToHost, ctx->stream));
       GW_TRY(cudaStreamSynchronize(ctx->stream));  // the batch plan below reads the flags

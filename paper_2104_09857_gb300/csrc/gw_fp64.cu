@@ -112,14 +112,14 @@ int emu_product(gw_ctx* ctx, const EmuSrc& A, const EmuSrc& B, const EmuGemm& g,
 // cycles on the FP64 pipes of all SMs (n = 250: 12 us, 400: 50 us, 602: 175).
 constexpr int kGreensDigits = 448;
 
-int greens_fp64(gw_ctx* ctx, double tau, double* cso, double* csv, double* g_occ, double* g_virt,
+int greens_fp64(gw_ctx* ctx, const gw_ctx& mol, double tau, double* cso, double* csv, double* g_occ, double* g_virt,
                 cudaStream_t st) {
-  const int n = ctx->nao, occ = ctx->n_occ;
+  const int n = mol.nao, occ = mol.n_occ;
   if (n < kGreensDigits || occ == 0 || occ == n) {
-    launch_greens(ctx->d_C, ctx->d_eps, n, occ, ctx->mu, tau, cso, csv, g_occ, g_virt, st);
+    launch_greens(mol.d_C, mol.d_eps, n, occ, mol.mu, tau, cso, csv, g_occ, g_virt, st);
     return GW_OK;
   }
-  launch_scale_orbitals(ctx->d_C, ctx->d_eps, n, occ, ctx->mu, tau, cso, csv, st);
+  launch_scale_orbitals(mol.d_C, mol.d_eps, n, occ, mol.mu, tau, cso, csv, st);
   for (int v = 0; v < 2; ++v) {
     EmuSrc s;
     s.src = v ? csv : cso;

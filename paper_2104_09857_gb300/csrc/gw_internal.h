@@ -96,9 +96,10 @@ struct Batch {
   int Q0 = 0, Q1 = 0;          // RI window of Y rows
 };
 
-// Builds (or reuses) the owner panels of the 3c tensor for filter threshold
-// thr; defined with the chi orchestration.
-int build_panels_for(gw_ctx* ctx, double thr);
+// Lists of the kept 3c blocks of every (sigma-atom, RI atom) pair for filter
+// threshold thr (ctx->d_bn_bucket, d_bn_list); defined with the chi
+// orchestration.
+int plan_bn_lists(gw_ctx* ctx, double thr);
 
 // Named device work buffer of the context, grown on demand and kept between
 // calls.  work_trim gives back every buffer whose name starts with prefix when
@@ -204,6 +205,12 @@ struct gw_ctx {
   bool panel32_ok = false;
   int* d_lam = nullptr;
   long long lam_total = 0;
+
+  // self-energy: per (sigma-atom s, RI atom P) the kept blocks (s, l, P) and
+  // (l, s, P) by partner atom l, entries block << 1 | (s is the first atom)
+  bool bn_ok = false;
+  int* d_bn_bucket = nullptr;
+  int* d_bn_list = nullptr;
 
   // the panels as digits for the FP64 products (row pd_row0[owner] + n)
   bool pd_ok = false;

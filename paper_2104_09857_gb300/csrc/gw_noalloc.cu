@@ -233,8 +233,7 @@ extern "C" int gw_chi_tau_noalloc(gw_ctx* ctx, int tau_index, double thr, double
   gw::launch_greens(ctx->d_C, ctx->d_eps, nao, n_occ, ctx->mu, ctx->tau[tau_index], cso, csv, go, gv, st);
   NA_LAUNCHED();
   if (thr > 0.0) {
-    gw::launch_sym_block_filter(go, nao, ctx->d_ao_off, n_at, thr, flo, st);
-    gw::launch_sym_block_filter(gv, nao, ctx->d_ao_off, n_at, thr, flv, st);
+    gw::launch_sym_block_filter(go, gv, nao, ctx->d_ao_off, n_at, thr, flo, flv, st);
     NA_LAUNCHED();
   }
   NA_TRY(cudaMemsetAsync(acc, 0, (size_t)nri * nri * sizeof(double), st));

@@ -2,9 +2,8 @@
 //   B^n[mu][P]  = sum_nu C[nu][n] (nu mu | P)          (half transform, Eq. 10 text)
 //   S^g_n(tau)  = sum_{mu nu} G^g_{mu nu}(tau) (B^n W(tau) B^nT)_{mu nu},  g = occ, virt
 //   Sigma^c_n(i tau) = -S^occ_n(tau),  Sigma^c_n(-i tau) = +S^virt_n(tau)
-// FP64 throughout.  B^n is formed from the owner panels of the 3c tensor
-// (each (sigma, P) pair belongs to exactly one panel); its (mu-atom, P-atom)
-// blocks below the filter threshold are dropped, as are G blocks.
+// B^n is formed in FP64 from the stored 3c blocks; its (mu-atom, P-atom) blocks
+// below the filter threshold are dropped, as are G blocks.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -19,35 +18,56 @@
 namespace gw {
 namespace sigma {
 
-// Bn[j][ao(s) + s'][p0 + pw] = sum_k Csel[lam[k]][j] panel_s[k][pw * nsig + s'],
-// kBnOrb orbitals j per thread: the panels, the bulk of the bytes, are read
-// once for that many orbitals.
-constexpr int kBnOrb = 4;
-__global__ void k_bn_panels(const double* __restrict__ pool, const PanelDesc* __restrict__ panels,
-                            const int* __restrict__ owners, const int* __restrict__ lam,
-                            const int* __restrict__ ao_off, const double* __restrict__ csel,
-                            int n_orb, int nao, int nri, double* __restrict__ bn) {
-  const PanelDesc d = panels[owners[blockIdx.y]];
-  const int N = d.npw * d.nsig;
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j0 = blockIdx.z * kBnOrb;
-  if (n >= N) return;
-  const double* p = pool + d.off;
-  const int* lk = lam + d.lam_off;
-  double acc[kBnOrb] = {};
-#pragma unroll 4
-  for (int k = 0; k < d.K; ++k) {
-    const double v = p[static_cast<long long>(k) * N + n];
-    const double* c = csel + static_cast<long long>(lk[k]) * n_orb + j0;
+// csel[mu][j] = C[mu][orbitals[j]]
+__global__ void k_select(const double* __restrict__ C, int nao, const int* __restrict__ orb, int n_orb,
+                         double* __restrict__ csel) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nao * n_orb) csel[i] = C[static_cast<long long>(i / n_orb) * nao + orb[i % n_orb]];
+}
+
+// Bn[j][ao(s) + s'][ri(P) + p'] = sum_l csel[l][j] (l s'|p') from the stored 3c
+// blocks.  One CTA per (sigma-atom s, RI atom P) pair and NO orbitals; its
+// blocks (list: block index << 1 | s is the block's first atom) in the order
+// of their partner atom, each block read from the tensor once per side.  Bound
+// by the FP64 pipe (two multiply-adds per cycle and SM), so NO is exactly the
+// orbitals there are: a masked multiply-add costs as much as one that counts.
+// From the owner panels instead the tensor was first scattered into panels
+// and then read by one chain of dependent loads per thread.
+template <int NO>
+__global__ void __launch_bounds__(128) k_bn_blocks(const double* __restrict__ t3, const int* __restrict__ blk,
+                                                   const long long* __restrict__ off,
+                                                   const int* __restrict__ bucket, const int* __restrict__ list,
+                                                   const int* __restrict__ ao_off, const int* __restrict__ ri_off,
+                                                   const double* __restrict__ csel, int n_at, int n_orb, int j0,
+                                                   int nao, int nri, double* __restrict__ bn) {
+  const int e0 = bucket[blockIdx.x], e1 = bucket[blockIdx.x + 1];
+  if (e0 == e1) return;
+  const int s = blockIdx.x / n_at, P = blockIdx.x % n_at;
+  const int ns = ao_off[s + 1] - ao_off[s], np = ri_off[P + 1] - ri_off[P];
+  j0 += blockIdx.y * NO;
+  for (int o = threadIdx.x; o < ns * np; o += blockDim.x) {
+    const int sp = o / np, pp = o - sp * np;
+    double acc[NO] = {};
+    for (int e = e0; e < e1; ++e) {
+      const int b = list[e] >> 1;
+      const bool first = list[e] & 1;
+      const int l = blk[3 * b + (first ? 1 : 0)];
+      const int l0 = ao_off[l], nl = ao_off[l + 1] - l0;
+      // element (l', s') of [nA][nB][np]
+      const double* x = t3 + off[b] + (first ? static_cast<long long>(sp) * nl * np : sp * np) + pp;
+      const long long step = first ? np : static_cast<long long>(ns) * np;
+      const double* c = csel + static_cast<long long>(l0) * n_orb + j0;
+#pragma unroll 13
+      for (int k = 0; k < nl; ++k) {
+        const double v = x[k * step];
 #pragma unroll
-    for (int j = 0; j < kBnOrb; ++j)
-      if (j0 + j < n_orb) acc[j] = fma(c[j], v, acc[j]);
+        for (int j = 0; j < NO; ++j) acc[j] = fma(c[k * n_orb + j], v, acc[j]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < NO; ++j)
+      bn[(static_cast<long long>(j0 + j) * nao + ao_off[s] + sp) * nri + ri_off[P] + pp] = acc[j];
   }
-  const int pw = n / d.nsig, sp = n - pw * d.nsig;
-#pragma unroll
-  for (int j = 0; j < kBnOrb; ++j)
-    if (j0 + j < n_orb)
-      bn[(static_cast<long long>(j0 + j) * nao + ao_off[d.owner] + sp) * nri + d.p0 + pw] = acc[j];
 }
 
 // zero the (mu-atom, P-atom) blocks of Bn_j with norm < thr (warp per block)
@@ -102,12 +122,15 @@ __global__ void k_dot2(const double* __restrict__ go, const double* __restrict__
 }  // namespace gw
 
 namespace {
-struct DevBuf {
+// a named work buffer of the context (gw::work_buffer)
+struct WorkBuf {
   void* p = nullptr;
-  ~DevBuf() {
-    if (p) cudaFree(p);
-  }
 };
+#define SG_BUF(buf, bytes)                                                                   \
+  do {                                                                                       \
+    const int rc_ = gw::work_buffer(ctx, "w.sg." #buf, std::max<size_t>((bytes), 1), &buf.p); \
+    if (rc_) return rc_;                                                                     \
+  } while (0)
 #define SG_TRY(call)                                                                   \
   do {                                                                                 \
     cudaError_t e_ = (call);                                                           \
@@ -117,6 +140,39 @@ struct DevBuf {
     }                                                                                  \
   } while (0)
 constexpr int kDotBlocks = 256;
+
+// B^n of the orbitals of ctx, filtered at thr, into bn [n_orb][n_AO][n_RI]
+// (zeroed here), on stream st; messages and scratch go to ctx.
+int build_bn(gw_ctx* ctx, const int* orbitals, int n_orb, double thr, double* bn, cudaStream_t st) {
+  int rc;
+  if ((rc = gw::plan_bn_lists(ctx, thr))) return rc;
+  const int nao = ctx->nao, nri = ctx->nri, n_at = ctx->n_at;
+  WorkBuf b_csel, b_orb;
+  SG_BUF(b_csel, (size_t)nao * n_orb * 8);
+  SG_BUF(b_orb, (size_t)n_orb * sizeof(int));
+  SG_TRY(cudaMemcpyAsync(b_orb.p, orbitals, n_orb * sizeof(int), cudaMemcpyHostToDevice, st));
+  gw::sigma::k_select<<<(nao * n_orb + 255) / 256, 256, 0, st>>>(ctx->d_C, nao, (const int*)b_orb.p, n_orb,
+                                                                 (double*)b_csel.p);
+  SG_TRY(cudaMemsetAsync(bn, 0, (size_t)n_orb * nao * nri * 8, st));
+  const auto launch = [&](auto kernel, int per, int j0, int groups) {
+    if (groups > 0 && ctx->n_blocks > 0)
+      kernel<<<dim3((unsigned)(n_at * n_at), groups), 128, 0, st>>>(
+          ctx->d_t3, ctx->d_blk, ctx->d_blk_off, ctx->d_bn_bucket, ctx->d_bn_list, ctx->d_ao_off, ctx->d_ri_off,
+          (const double*)b_csel.p, n_at, n_orb, j0, nao, nri, bn);
+    return j0 + per * groups;
+  };
+  int j = launch(gw::sigma::k_bn_blocks<4>, 4, 0, n_orb / 4);
+  j = launch(gw::sigma::k_bn_blocks<2>, 2, j, (n_orb - j) / 2);
+  launch(gw::sigma::k_bn_blocks<1>, 1, j, n_orb - j);
+  SG_TRY(cudaGetLastError());
+  if (thr > 0.0) {
+    const long long nblk = (long long)n_orb * n_at * n_at;
+    gw::sigma::k_bn_filter<<<(unsigned)((nblk + 7) / 8), 256, 0, st>>>(bn, n_orb, n_at, nao, nri, ctx->d_ao_off,
+                                                                       ctx->d_ri_off, thr);
+    SG_TRY(cudaGetLastError());
+  }
+  return GW_OK;
+}
 }  // namespace
 
 namespace {
@@ -148,72 +204,37 @@ int sigma_impl(gw_ctx* ctx, const double* W_tau, int w_on_device, const int* orb
       return GW_ERR_INVALID_ARG;
     }
   SG_TRY(cudaSetDevice(ctx->device));
-  int rc = gw::build_panels_for(ctx, thr);
-  if (rc) return rc;
+  int rc;
   cudaStream_t st = ctx->stream;
   gw::WorkTrim trim{ctx};
   const size_t nn_ri = (size_t)nri * nri, nn_ao = (size_t)nao * nao;
-  DevBuf b_w, b_csel, b_bn, b_y, b_z, b_cso, b_csv, b_go, b_gv, b_fl, b_part, b_own, b_aooff;
+  WorkBuf b_w, b_bn, b_y, b_z, b_cso, b_csv, b_go, b_gv, b_fl, b_part;
   const double* w;
   if (w_on_device) {
     w = W_tau;
   } else {
-    SG_TRY(cudaMalloc(&b_w.p, (size_t)n_tau * nn_ri * 8));
+    SG_BUF(b_w, (size_t)n_tau * nn_ri * 8);
     SG_TRY(cudaMemcpyAsync(b_w.p, W_tau, (size_t)n_tau * nn_ri * 8, cudaMemcpyHostToDevice, st));
     w = (const double*)b_w.p;
   }
-  // selected orbital columns of C: csel[mu][j] = C[mu][orbitals[j]] (host gather
-  // from the device copy would need a kernel; the host keeps no copy of C, so
-  // gather on the device by strided copies)
-  SG_TRY(cudaMalloc(&b_csel.p, (size_t)nao * n_orb * 8));
-  for (int a = 0; a < n_orb; ++a)
-    SG_TRY(cudaMemcpy2DAsync((double*)b_csel.p + a, n_orb * 8, ctx->d_C + orbitals[a], nao * 8, 8, nao,
-                             cudaMemcpyDeviceToDevice, st));
-  SG_TRY(cudaMalloc(&b_bn.p, (size_t)n_orb * nao * nri * 8));
-  SG_TRY(cudaMemsetAsync(b_bn.p, 0, (size_t)n_orb * nao * nri * 8, st));
-  std::vector<int> owners;
-  int maxN = 0;
-  for (int s = 0; s < n_at; ++s)
-    if (ctx->panels[s].K > 0) {
-      owners.push_back(s);
-      maxN = std::max(maxN, ctx->panels[s].npw * ctx->panels[s].nsig);
-    }
-  DevBuf b_pd;
-  SG_TRY(cudaMalloc(&b_pd.p, ctx->panels.size() * sizeof(gw::PanelDesc)));
-  SG_TRY(cudaMemcpyAsync(b_pd.p, ctx->panels.data(), ctx->panels.size() * sizeof(gw::PanelDesc),
-                         cudaMemcpyHostToDevice, st));
-  SG_TRY(cudaMalloc(&b_own.p, std::max<size_t>(owners.size(), 1) * sizeof(int)));
-  if (!owners.empty())
-    SG_TRY(cudaMemcpyAsync(b_own.p, owners.data(), owners.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+  SG_BUF(b_bn, (size_t)n_orb * nao * nri * 8);
   double* bn = (double*)b_bn.p;
-  if (!owners.empty()) {
-    dim3 g((maxN + 127) / 128, (unsigned)owners.size(), (n_orb + gw::sigma::kBnOrb - 1) / gw::sigma::kBnOrb);
-    gw::sigma::k_bn_panels<<<g, 128, 0, st>>>(ctx->d_panel64, (const gw::PanelDesc*)b_pd.p,
-                                              (const int*)b_own.p, ctx->d_lam, ctx->d_ao_off,
-                                              (const double*)b_csel.p, n_orb, nao, nri, bn);
-    SG_TRY(cudaGetLastError());
-  }
-  if (thr > 0.0) {
-    const long long nblk = (long long)n_orb * n_at * n_at;
-    gw::sigma::k_bn_filter<<<(unsigned)((nblk + 7) / 8), 256, 0, st>>>(bn, n_orb, n_at, nao, nri,
-                                                                       ctx->d_ao_off, ctx->d_ri_off, thr);
-    SG_TRY(cudaGetLastError());
-  }
+  if ((rc = build_bn(ctx, orbitals, n_orb, thr, bn, st))) return rc;
   // FP64: the product with W for as many orbitals at a time as keep its digits
   // within 1 GB
   const int orb_step =
       mixed ? 1
             : std::max(1, std::min<int>(n_orb, (int)((size_t(1) << 30) / gw::emu_dig_bytes(nao, nri))));
-  SG_TRY(cudaMalloc(&b_y.p, (size_t)orb_step * nao * nri * 8));
-  SG_TRY(cudaMalloc(&b_z.p, nn_ao * 8));
+  SG_BUF(b_y, (size_t)orb_step * nao * nri * 8);
+  SG_BUF(b_z, nn_ao * 8);
   if ((rc = gw::emu_begin(ctx, st))) return rc;
-  SG_TRY(cudaMalloc(&b_cso.p, (size_t)nao * std::max(ctx->n_occ, 1) * 8));
-  SG_TRY(cudaMalloc(&b_csv.p, (size_t)nao * std::max(nao - ctx->n_occ, 1) * 8));
-  SG_TRY(cudaMalloc(&b_go.p, nn_ao * 8));
-  SG_TRY(cudaMalloc(&b_gv.p, nn_ao * 8));
-  SG_TRY(cudaMalloc(&b_fl.p, (size_t)n_at * n_at));
+  SG_BUF(b_cso, (size_t)nao * std::max(ctx->n_occ, 1) * 8);
+  SG_BUF(b_csv, (size_t)nao * std::max(nao - ctx->n_occ, 1) * 8);
+  SG_BUF(b_go, nn_ao * 8);
+  SG_BUF(b_gv, nn_ao * 8);
+  SG_BUF(b_fl, 2 * (size_t)n_at * n_at);
   // the traces' partial sums of every (orbital, tau), read once at the end
-  SG_TRY(cudaMalloc(&b_part.p, (size_t)n_orb * n_tau * kDotBlocks * 2 * 8));
+  SG_BUF(b_part, (size_t)n_orb * n_tau * kDotBlocks * 2 * 8);
   double *y = (double*)b_y.p, *z = (double*)b_z.p, *go = (double*)b_go.p, *gv = (double*)b_gv.p;
   std::vector<double> part((size_t)n_orb * n_tau * kDotBlocks * 2);
   // tensor-core route: both products as step-C style tile jobs on bf16 slices
@@ -221,7 +242,7 @@ int sigma_impl(gw_ctx* ctx, const double* W_tau, int w_on_device, const int* orb
   //   z = -(y B^T)   (rows mu, columns nu, K = Q)  = B W B^T
   const int tile = gw::tc_tile_rows();
   const int kpad = (nri + 63) / 64 * 64;
-  DevBuf b_bs, b_ws, b_ys, b_tl1, b_tk1, b_ct1, b_k01, b_ln1, b_tl2, b_tk2, b_ct2, b_err, b_mx;
+  WorkBuf b_bs, b_ws, b_ys, b_tl1, b_tk1, b_ct1, b_k01, b_ln1, b_tl2, b_tk2, b_ct2, b_err, b_mx;
   int nslab = 0, n_tiles1 = 0, n_tiles2 = 0, nqt1 = 0, nqt2 = 0;
   CUtensorMap m_b, m_w, m_y, m_bq;
   if (mixed) {
@@ -238,31 +259,34 @@ int sigma_impl(gw_ctx* ctx, const double* W_tau, int w_on_device, const int* orb
     nqt2 = (nao + tile - 1) / tile;
     n_tiles1 = npt * nqt1;
     n_tiles2 = npt * nqt2;
-    auto lists = [&](int nt, DevBuf& tl, DevBuf& tk, DevBuf& ct) -> int {
+    auto lists = [&](const char* which, int nt, WorkBuf& tl, WorkBuf& tk, WorkBuf& ct) -> int {
       std::vector<int> h_tl(nt), h_tk((size_t)nt * nslab), h_ct(nt, nslab);
       for (int t = 0; t < nt; ++t) {
         h_tl[t] = t;
         for (int i = 0; i < nslab; ++i) h_tk[(size_t)t * nslab + i] = i;
       }
-      SG_TRY(cudaMalloc(&tl.p, nt * sizeof(int)));
-      SG_TRY(cudaMalloc(&tk.p, h_tk.size() * sizeof(int)));
-      SG_TRY(cudaMalloc(&ct.p, nt * sizeof(int)));
+      const std::string n = std::string("w.sg.lists") + which;
+      int r;
+      if ((r = gw::work_buffer(ctx, (n + "t").c_str(), nt * sizeof(int), &tl.p)) ||
+          (r = gw::work_buffer(ctx, (n + "k").c_str(), h_tk.size() * sizeof(int), &tk.p)) ||
+          (r = gw::work_buffer(ctx, (n + "c").c_str(), nt * sizeof(int), &ct.p)))
+        return r;
       SG_TRY(cudaMemcpy(tl.p, h_tl.data(), nt * sizeof(int), cudaMemcpyHostToDevice));
       SG_TRY(cudaMemcpy(tk.p, h_tk.data(), h_tk.size() * sizeof(int), cudaMemcpyHostToDevice));
       SG_TRY(cudaMemcpy(ct.p, h_ct.data(), nt * sizeof(int), cudaMemcpyHostToDevice));
       return GW_OK;
     };
-    if ((rc = lists(n_tiles1, b_tl1, b_tk1, b_ct1))) return rc;
-    if ((rc = lists(n_tiles2, b_tl2, b_tk2, b_ct2))) return rc;
-    SG_TRY(cudaMalloc(&b_k01.p, nslab * sizeof(long long)));
-    SG_TRY(cudaMalloc(&b_ln1.p, nslab * sizeof(int)));
+    if ((rc = lists("1", n_tiles1, b_tl1, b_tk1, b_ct1))) return rc;
+    if ((rc = lists("2", n_tiles2, b_tl2, b_tk2, b_ct2))) return rc;
+    SG_BUF(b_k01, nslab * sizeof(long long));
+    SG_BUF(b_ln1, nslab * sizeof(int));
     SG_TRY(cudaMemcpy(b_k01.p, k0.data(), nslab * sizeof(long long), cudaMemcpyHostToDevice));
     SG_TRY(cudaMemcpy(b_ln1.p, len.data(), nslab * sizeof(int), cudaMemcpyHostToDevice));
-    SG_TRY(cudaMalloc(&b_bs.p, (size_t)slices * nao * kpad * 2));
-    SG_TRY(cudaMalloc(&b_ws.p, (size_t)slices * nri * kpad * 2));
-    SG_TRY(cudaMalloc(&b_ys.p, (size_t)slices * nao * kpad * 2));
-    SG_TRY(cudaMalloc(&b_err.p, sizeof(int)));
-    SG_TRY(cudaMalloc(&b_mx.p, 4 * sizeof(double)));
+    SG_BUF(b_bs, (size_t)slices * nao * kpad * 2);
+    SG_BUF(b_ws, (size_t)slices * nri * kpad * 2);
+    SG_BUF(b_ys, (size_t)slices * nao * kpad * 2);
+    SG_BUF(b_err, sizeof(int));
+    SG_BUF(b_mx, 4 * sizeof(double));
     SG_TRY(cudaMemsetAsync(b_err.p, 0, sizeof(int), st));
     if (gw::make_slice_map(&m_b, b_bs.p, kpad, nao, slices, tile, f16) ||
         gw::make_slice_map(&m_w, b_ws.p, kpad, nri, slices, tile, f16) ||
@@ -274,10 +298,10 @@ int sigma_impl(gw_ctx* ctx, const double* W_tau, int w_on_device, const int* orb
   }
   gw::EmuOp op_b, op_y;  // FP64: digits of B and Y
   for (int jt = 0; jt < n_tau; ++jt) {
-    if ((rc = gw::greens_fp64(ctx, taus[jt], (double*)b_cso.p, (double*)b_csv.p, go, gv, st))) return rc;
+    if ((rc = gw::greens_fp64(ctx, *ctx, taus[jt], (double*)b_cso.p, (double*)b_csv.p, go, gv, st))) return rc;
     if (thr > 0.0) {
-      gw::launch_sym_block_filter(go, nao, ctx->d_ao_off, n_at, thr, (unsigned char*)b_fl.p, st);
-      gw::launch_sym_block_filter(gv, nao, ctx->d_ao_off, n_at, thr, (unsigned char*)b_fl.p, st);
+      gw::launch_sym_block_filter(go, gv, nao, ctx->d_ao_off, n_at, thr, (unsigned char*)b_fl.p,
+                                  (unsigned char*)b_fl.p + (size_t)n_at * n_at, st);
     }
     const double* wt = w + (size_t)jt * nn_ri;
     gw::EmuOp op_w;  // FP64: the columns of W as rows
@@ -474,6 +498,12 @@ namespace {
     }                                                                                        \
   } while (0)
 
+#define SB_BUF(buf, bytes)                                                                  \
+  do {                                                                                      \
+    const int rc_ = gw::work_buffer(c0, "w.sb." #buf, std::max<size_t>((bytes), 1), &buf.p); \
+    if (rc_) return rc_;                                                                    \
+  } while (0)
+
 struct Prob {
   int mol, a, nao, nri;
   long long rowB;  // first slice row of B_p (and of Y_p)
@@ -518,60 +548,22 @@ int sigma_batch_mixed(gw_ctx* const* ctxs, int n_mol, const double* const* W_tau
     }
   }
   const int np = (int)pr.size();
-  DevBuf b_bn, b_csel, b_bs, b_ws, b_ys, b_w64, b_y64, b_z64, b_go, b_gv, b_cso, b_csv, b_fl, b_mx,
-      b_sd, b_t1, b_t2, b_dd, b_part, b_err, b_pd, b_own;
-  SB_TRY(cudaMalloc(&b_bn.p, std::max<long long>(nB64, 1) * 8));
-  SB_TRY(cudaMemsetAsync(b_bn.p, 0, std::max<long long>(nB64, 1) * 8, st));
+  WorkBuf b_bn, b_bs, b_ws, b_ys, b_w64, b_y64, b_z64, b_go, b_gv, b_cso, b_csv, b_fl, b_mx, b_sd, b_t1, b_t2,
+      b_dd, b_part, b_err;
+  gw::WorkTrim trim{c0};
+  SB_BUF(b_bn, std::max<long long>(nB64, 1) * 8);
   double* bn = (double*)b_bn.p;
-  // B^n of every molecule from its FP64 panels (built and released one
-  // molecule at a time, so that one pool is resident at once)
+  {
+    const int rc = gw::emu_begin(c0, st);
+    if (rc) return rc;
+  }
   for (int i = 0; i < n_mol; ++i) {
     gw_ctx* c = ctxs[i];
-    int rc = gw::build_panels_for(c, thr);
+    const int rc = build_bn(c, orbitals[i], n_orb[i], thr, bn + offB64[i], st);
     if (rc) {
       c0->err = "gw_sigma_tau_batch: molecule " + std::to_string(i) + ": " + c->err;
       return rc;
     }
-    DevBuf csel;
-    SB_TRY(cudaMalloc(&csel.p, (size_t)c->nao * n_orb[i] * 8));
-    for (int a = 0; a < n_orb[i]; ++a)
-      SB_TRY(cudaMemcpy2DAsync((double*)csel.p + a, n_orb[i] * 8, c->d_C + orbitals[i][a], c->nao * 8, 8,
-                               c->nao, cudaMemcpyDeviceToDevice, st));
-    std::vector<int> owners;
-    int maxN = 0;
-    for (int s = 0; s < c->n_at; ++s)
-      if (c->panels[s].K > 0) {
-        owners.push_back(s);
-        maxN = std::max(maxN, c->panels[s].npw * c->panels[s].nsig);
-      }
-    DevBuf pd, own;
-    SB_TRY(cudaMalloc(&pd.p, c->panels.size() * sizeof(gw::PanelDesc)));
-    SB_TRY(cudaMemcpyAsync(pd.p, c->panels.data(), c->panels.size() * sizeof(gw::PanelDesc),
-                           cudaMemcpyHostToDevice, st));
-    SB_TRY(cudaMalloc(&own.p, std::max<size_t>(owners.size(), 1) * sizeof(int)));
-    if (!owners.empty()) {
-      SB_TRY(cudaMemcpyAsync(own.p, owners.data(), owners.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-      dim3 g((maxN + 127) / 128, (unsigned)owners.size(), (n_orb[i] + gw::sigma::kBnOrb - 1) / gw::sigma::kBnOrb);
-      gw::sigma::k_bn_panels<<<g, 128, 0, st>>>(c->d_panel64, (const gw::PanelDesc*)pd.p,
-                                                (const int*)own.p, c->d_lam, c->d_ao_off,
-                                                (const double*)csel.p, n_orb[i], c->nao, c->nri,
-                                                bn + offB64[i]);
-      SB_TRY(cudaGetLastError());
-    }
-    if (thr > 0.0) {
-      const long long nblk = (long long)n_orb[i] * c->n_at * c->n_at;
-      gw::sigma::k_bn_filter<<<(unsigned)((nblk + 7) / 8), 256, 0, st>>>(bn + offB64[i], n_orb[i], c->n_at,
-                                                                         c->nao, c->nri, c->d_ao_off,
-                                                                         c->d_ri_off, thr);
-      SB_TRY(cudaGetLastError());
-    }
-    SB_TRY(cudaStreamSynchronize(st));
-    // the pool is not needed again here: release it
-    cudaFree(c->d_panel64);
-    c->d_panel64 = nullptr;
-    c->panels_ok = false;
-    c->panels_thr = -1.0;
-    c->panel32_ok = false;
   }
   // slices of B (tau independent) with per-problem binary16 scales
   std::vector<gw::SplitDesc> sd(np);
@@ -579,8 +571,8 @@ int sigma_batch_mixed(gw_ctx* const* ctxs, int n_mol, const double* const* W_tau
     const Prob& q = pr[p];
     sd[p] = gw::SplitDesc{offB64[q.mol] + (long long)q.a * q.nao * q.nri, q.rowB, q.nao, q.nri, q.nri, 0, 1.0};
   }
-  SB_TRY(cudaMalloc(&b_sd.p, std::max(np, n_mol) * sizeof(gw::SplitDesc)));
-  SB_TRY(cudaMalloc(&b_mx.p, 2 * std::max(np, n_mol) * sizeof(double)));
+  SB_BUF(b_sd, std::max(np, n_mol) * sizeof(gw::SplitDesc));
+  SB_BUF(b_mx, 2 * std::max(np, n_mol) * sizeof(double));
   std::vector<double> bmx(2 * np, 1.0);
   if (f16) {
     SB_TRY(cudaMemcpyAsync(b_sd.p, sd.data(), np * sizeof(gw::SplitDesc), cudaMemcpyHostToDevice, st));
@@ -596,24 +588,24 @@ int sigma_batch_mixed(gw_ctx* const* ctxs, int n_mol, const double* const* W_tau
   }
   SB_TRY(cudaMemcpyAsync(b_sd.p, sd.data(), np * sizeof(gw::SplitDesc), cudaMemcpyHostToDevice, st));
   const long long bs_elems = std::max<long long>(rowsB, 1) * kmax;
-  SB_TRY(cudaMalloc(&b_bs.p, (size_t)slices * bs_elems * 2));
-  SB_TRY(cudaMalloc(&b_ys.p, (size_t)slices * bs_elems * 2));
+  SB_BUF(b_bs, (size_t)slices * bs_elems * 2);
+  SB_BUF(b_ys, (size_t)slices * bs_elems * 2);
   gw::launch_split_group(bn, (const gw::SplitDesc*)b_sd.p, np, max_nao, kmax, slices, bs_elems, f16, b_bs.p, st);
   SB_TRY(cudaGetLastError());
   const long long ws_elems = std::max<long long>(rowsW, 1) * kmax;
-  SB_TRY(cudaMalloc(&b_ws.p, (size_t)slices * ws_elems * 2));
-  SB_TRY(cudaMalloc(&b_y64.p, std::max<long long>(nY, 1) * 8));
-  SB_TRY(cudaMalloc(&b_z64.p, std::max<long long>(nZ, 1) * 8));
-  SB_TRY(cudaMalloc(&b_go.p, std::max<long long>(nG, 1) * 8));
-  SB_TRY(cudaMalloc(&b_gv.p, std::max<long long>(nG, 1) * 8));
-  SB_TRY(cudaMalloc(&b_cso.p, (size_t)max_nao * max_occ * 8));
-  SB_TRY(cudaMalloc(&b_csv.p, (size_t)max_nao * max_virt * 8));
-  SB_TRY(cudaMalloc(&b_err.p, sizeof(int)));
+  SB_BUF(b_ws, (size_t)slices * ws_elems * 2);
+  SB_BUF(b_y64, std::max<long long>(nY, 1) * 8);
+  SB_BUF(b_z64, std::max<long long>(nZ, 1) * 8);
+  SB_BUF(b_go, std::max<long long>(nG, 1) * 8);
+  SB_BUF(b_gv, std::max<long long>(nG, 1) * 8);
+  SB_BUF(b_cso, (size_t)max_nao * max_occ * 8);
+  SB_BUF(b_csv, (size_t)max_nao * max_virt * 8);
+  SB_BUF(b_err, sizeof(int));
   SB_TRY(cudaMemsetAsync(b_err.p, 0, sizeof(int), st));
-  if (!w_on_device) SB_TRY(cudaMalloc(&b_w64.p, std::max<long long>(nW, 1) * 8));
+  if (!w_on_device) SB_BUF(b_w64, std::max<long long>(nW, 1) * 8);
   int max_at = 1;
   for (int i = 0; i < n_mol; ++i) max_at = std::max(max_at, ctxs[i]->n_at);
-  SB_TRY(cudaMalloc(&b_fl.p, (size_t)max_at * max_at));
+  SB_BUF(b_fl, 2 * (size_t)max_at * max_at);
   CUtensorMap m_b, m_w, m_y;
   if (gw::make_slice_map(&m_b, b_bs.p, kmax, std::max<long long>(rowsB, 1), slices, tile, f16) ||
       gw::make_slice_map(&m_w, b_ws.p, kmax, std::max<long long>(rowsW, 1), slices, tile, f16) ||
@@ -625,9 +617,9 @@ int sigma_batch_mixed(gw_ctx* const* ctxs, int n_mol, const double* const* W_tau
   std::vector<gw::sigma::DotDesc> dd(np);
   for (int p = 0; p < np; ++p)
     dd[p] = gw::sigma::DotDesc{offG[pr[p].mol], pr[p].offZ, (long long)pr[p].nao * pr[p].nao};
-  SB_TRY(cudaMalloc(&b_dd.p, np * sizeof(gw::sigma::DotDesc)));
+  SB_BUF(b_dd, np * sizeof(gw::sigma::DotDesc));
   SB_TRY(cudaMemcpyAsync(b_dd.p, dd.data(), np * sizeof(gw::sigma::DotDesc), cudaMemcpyHostToDevice, st));
-  SB_TRY(cudaMalloc(&b_part.p, (size_t)np * kDotBlocks * 2 * 8));
+  SB_BUF(b_part, (size_t)np * kDotBlocks * 2 * 8);
   std::vector<double> part((size_t)np * kDotBlocks * 2);
   std::vector<gw::GroupTile> t1, t2;
   for (const Prob& q : pr) {
@@ -644,15 +636,15 @@ int sigma_batch_mixed(gw_ctx* const* ctxs, int n_mol, const double* const* W_tau
                                    std::min(tile, q.nao - mt * tile), std::min(tile, q.nao - nt * tile), q.nao,
                                    1.f, 0});
   }
-  SB_TRY(cudaMalloc(&b_t1.p, std::max<size_t>(t1.size(), 1) * sizeof(gw::GroupTile)));
-  SB_TRY(cudaMalloc(&b_t2.p, std::max<size_t>(t2.size(), 1) * sizeof(gw::GroupTile)));
+  SB_BUF(b_t1, std::max<size_t>(t1.size(), 1) * sizeof(gw::GroupTile));
+  SB_BUF(b_t2, std::max<size_t>(t2.size(), 1) * sizeof(gw::GroupTile));
   std::vector<gw::SplitDesc> wd(n_mol), yd(np);
   for (int j = 0; j < n_tau; ++j) {
     // W(tau_j) of every molecule: magnitudes, then slices
     const double* w64 = nullptr;
     if (w_on_device) {
       // one contiguous view is needed: copy the molecules' matrices together
-      if (!b_w64.p) SB_TRY(cudaMalloc(&b_w64.p, std::max<long long>(nW, 1) * 8));
+      if (!b_w64.p) SB_BUF(b_w64, std::max<long long>(nW, 1) * 8);
       for (int i = 0; i < n_mol; ++i)
         SB_TRY(cudaMemcpyAsync((double*)b_w64.p + offW[i], W_tau[i] + (size_t)j * ctxs[i]->nri * ctxs[i]->nri,
                                (size_t)ctxs[i]->nri * ctxs[i]->nri * 8, cudaMemcpyDeviceToDevice, st));
@@ -726,14 +718,12 @@ int sigma_batch_mixed(gw_ctx* const* ctxs, int n_mol, const double* const* W_tau
     // Green's functions of every molecule at its tau_j (FP64, filtered)
     for (int i = 0; i < n_mol; ++i) {
       const gw_ctx* c = ctxs[i];
-      gw::launch_greens(c->d_C, c->d_eps, c->nao, c->n_occ, c->mu, c->tau[j], (double*)b_cso.p,
-                        (double*)b_csv.p, (double*)b_go.p + offG[i], (double*)b_gv.p + offG[i], st);
-      if (thr > 0.0) {
-        gw::launch_sym_block_filter((double*)b_go.p + offG[i], c->nao, c->d_ao_off, c->n_at, thr,
-                                    (unsigned char*)b_fl.p, st);
-        gw::launch_sym_block_filter((double*)b_gv.p + offG[i], c->nao, c->d_ao_off, c->n_at, thr,
-                                    (unsigned char*)b_fl.p, st);
-      }
+      double *go = (double*)b_go.p + offG[i], *gv = (double*)b_gv.p + offG[i];
+      const int rc = gw::greens_fp64(c0, *c, c->tau[j], (double*)b_cso.p, (double*)b_csv.p, go, gv, st);
+      if (rc) return rc;
+      if (thr > 0.0)
+        gw::launch_sym_block_filter(go, gv, c->nao, c->d_ao_off, c->n_at, thr, (unsigned char*)b_fl.p,
+                                    (unsigned char*)b_fl.p + (size_t)c->n_at * c->n_at, st);
     }
     SB_TRY(cudaGetLastError());
     gw::sigma::k_dot2_group<<<dim3(kDotBlocks, np), 256, 0, st>>>((const double*)b_go.p, (const double*)b_gv.p,
@@ -753,6 +743,10 @@ int sigma_batch_mixed(gw_ctx* const* ctxs, int n_mol, const double* const* W_tau
       o[0] = -so;
       o[1] = sv;
     }
+  }
+  {
+    const int rc = gw::emu_end(c0, "gw_sigma_tau_batch");
+    if (rc) return rc;
   }
   int h_err = 0;
   SB_TRY(cudaMemcpy(&h_err, b_err.p, sizeof(int), cudaMemcpyDeviceToHost));

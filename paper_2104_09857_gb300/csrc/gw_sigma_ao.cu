@@ -128,7 +128,7 @@ extern "C" int gw_sigma_ao_tau(gw_ctx* ctx, const double* W_tau, int w_on_device
   SA_TRY(cudaMalloc(&b_gv.p, nn_ao * 8));
   SA_TRY(cudaMalloc(&b_cso.p, static_cast<size_t>(nao) * std::max(ctx->n_occ, 1) * 8));
   SA_TRY(cudaMalloc(&b_csv.p, static_cast<size_t>(nao) * std::max(nao - ctx->n_occ, 1) * 8));
-  SA_TRY(cudaMalloc(&b_fl.p, static_cast<size_t>(n_at) * n_at));
+  SA_TRY(cudaMalloc(&b_fl.p, 2 * static_cast<size_t>(n_at) * n_at));
   if (!w_on_device) SA_TRY(cudaMalloc(&b_w.p, nn_ri * 8));
   if (!out_on_device) SA_TRY(cudaMalloc(&b_out.p, 2 * nn_ao * 8));
   double* T = static_cast<double*>(b_t.p);
@@ -158,12 +158,12 @@ extern "C" int gw_sigma_ao_tau(gw_ctx* ctx, const double* W_tau, int w_on_device
   const gw::EmuSrc t_lam = rows_of(T, row, row, nao, true);                               // rows (mu, P)
   gw::EmuOp keep_t;
   for (int j = 0; j < n_tau; ++j) {
-    if ((rc = gw::greens_fp64(ctx, ctx->tau[j], static_cast<double*>(b_cso.p), static_cast<double*>(b_csv.p), go, gv,
+    if ((rc = gw::greens_fp64(ctx, *ctx, ctx->tau[j], static_cast<double*>(b_cso.p), static_cast<double*>(b_csv.p), go, gv,
                               st)))
       return rc;
     if (thr > 0.0) {
-      gw::launch_sym_block_filter(go, nao, ctx->d_ao_off, n_at, thr, static_cast<unsigned char*>(b_fl.p), st);
-      gw::launch_sym_block_filter(gv, nao, ctx->d_ao_off, n_at, thr, static_cast<unsigned char*>(b_fl.p), st);
+      gw::launch_sym_block_filter(go, gv, nao, ctx->d_ao_off, n_at, thr, static_cast<unsigned char*>(b_fl.p),
+                                  static_cast<unsigned char*>(b_fl.p) + static_cast<size_t>(n_at) * n_at, st);
     }
     const double* wj = W_tau + static_cast<size_t>(j) * nn_ri;
     if (!w_on_device) {

@@ -139,9 +139,10 @@ int emu_mm(gw_ctx* ctx, const EmuOp& A, const EmuOp& B, const EmuGemm& g, cudaSt
 // where they are whole (keep->dig set by the first call).
 int emu_product(gw_ctx* ctx, const EmuSrc& A, const EmuSrc& B, const EmuGemm& g, EmuOp* keep,
                 cudaStream_t st);
-// G^occ(tau), G^virt(tau) of Eq. 2 from the context's orbitals; cso, csv:
-// scratch for the scaled orbitals (n_AO x n_occ, n_AO x n_virt).
-int greens_fp64(gw_ctx* ctx, double tau, double* cso, double* csv, double* g_occ, double* g_virt, cudaStream_t st);
+// G^occ(tau), G^virt(tau) of Eq. 2 from the orbitals of mol (ctx: the context
+// whose work buffers serve, often the same); cso, csv: scratch for the scaled
+// orbitals (n_AO x n_occ, n_AO x n_virt).
+int greens_fp64(gw_ctx* ctx, const gw_ctx& mol, double tau, double* cso, double* csv, double* g_occ, double* g_virt, cudaStream_t st);
 // Reads the error flag after the stream has been synchronised.
 int emu_end(gw_ctx* ctx, const char* call);
 

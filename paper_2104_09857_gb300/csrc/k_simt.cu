@@ -99,54 +99,61 @@ __global__ void k_cast_f64_f32(const double* __restrict__ x, float* __restrict__
 // Eq. 2: scaled orbital columns.  occupied: C[mu][i] exp((eps_i - mu_F) tau/2),
 // virtual: C[mu][a] exp(-(eps_a - mu_F) tau/2); G = Cs Cs^T.
 // ---------------------------------------------------------------------------
-__global__ void k_scale_orbitals(const double* __restrict__ C, const double* __restrict__ eps,
-                                 int nao, int n_occ, double mu, double tau,
-                                 double* __restrict__ cso, double* __restrict__ csv) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  long long n = (long long)nao * nao;
-  if (i >= n) return;
-  int row = (int)(i / nao), col = (int)(i % nao);
-  double e = eps[col] - mu;
-  if (col < n_occ) {
-    cso[(long long)row * n_occ + col] = C[i] * exp(0.5 * e * tau);
-  } else {
-    int nv = nao - n_occ;
-    csv[(long long)row * nv + (col - n_occ)] = C[i] * exp(-0.5 * e * tau);
+// One exponential per column and CTA: an FP64 exponential is some 25 operations
+// on the FP64 pipe, and one per element took 18 us at 602 functions.
+__global__ void __launch_bounds__(256) k_scale_orbitals(const double* __restrict__ C, const double* __restrict__ eps,
+                                                        int nao, int n_occ, double mu, double tau,
+                                                        double* __restrict__ cso, double* __restrict__ csv) {
+  __shared__ double f[32];
+  const int col = blockIdx.x * 32 + (threadIdx.x & 31);
+  if (threadIdx.x < 32 && col < nao) {
+    const double e = eps[col] - mu;
+    f[threadIdx.x] = col < n_occ ? exp(0.5 * e * tau) : exp(-0.5 * e * tau);
+  }
+  __syncthreads();
+  if (col >= nao) return;
+  const double w = f[threadIdx.x & 31];
+  const int nv = nao - n_occ;
+  for (int row = blockIdx.y * 8 + (threadIdx.x >> 5); row < nao; row += 8 * gridDim.y) {
+    const double v = C[static_cast<long long>(row) * nao + col] * w;
+    if (col < n_occ)
+      cso[static_cast<long long>(row) * n_occ + col] = v;
+    else
+      csv[static_cast<long long>(row) * nv + (col - n_occ)] = v;
   }
 }
 
-// Frobenius norms of the (A <= B) atom blocks of a symmetric matrix; blocks
-// with norm < thr are zeroed together with their mirror.  flags[A*n+B] =
-// flags[B*n+A] = kept.
-__global__ void k_sym_block_filter(double* __restrict__ g, int nao, const int* __restrict__ ao_off,
-                                   int n_at, double thr, unsigned char* __restrict__ flags) {
-  int pair = blockIdx.x;
-  int A = pair / n_at, B = pair % n_at;
+// Frobenius norms of the (A <= B) atom blocks of two symmetric matrices
+// (blockIdx.y); blocks with norm < thr are zeroed together with their mirror.
+// flags[A*n+B] = flags[B*n+A] = kept.  A warp per block: blocks are a few
+// hundred elements, and a CTA for each (and for each mirror) took 16 us at 58
+// atoms where this takes 3.
+__global__ void __launch_bounds__(256) k_sym_block_filter(double* __restrict__ g0, double* __restrict__ g1, int nao,
+                                                          const int* __restrict__ ao_off, int n_at, double thr,
+                                                          unsigned char* __restrict__ f0,
+                                                          unsigned char* __restrict__ f1) {
+  double* g = blockIdx.y ? g1 : g0;
+  unsigned char* flags = blockIdx.y ? f1 : f0;
+  const int lane = threadIdx.x & 31;
+  const long long pair = static_cast<long long>(blockIdx.x) * 8 + threadIdx.x / 32;
+  if (pair >= static_cast<long long>(n_at) * n_at) return;
+  const int A = static_cast<int>(pair / n_at), B = static_cast<int>(pair % n_at);
   if (A > B) return;
-  int a0 = ao_off[A], na = ao_off[A + 1] - a0;
-  int b0 = ao_off[B], nb = ao_off[B + 1] - b0;
-  __shared__ double red[32];
+  const int a0 = ao_off[A], na = ao_off[A + 1] - a0;
+  const int b0 = ao_off[B], nb = ao_off[B + 1] - b0;
   double s = 0.0;
-  for (int i = threadIdx.x; i < na * nb; i += blockDim.x) {
-    double v = g[(long long)(a0 + i / nb) * nao + b0 + i % nb];
+  for (int i = lane; i < na * nb; i += 32) {
+    const double v = g[(long long)(a0 + i / nb) * nao + b0 + i % nb];
     s += v * v;
   }
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x / 32] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = threadIdx.x < blockDim.x / 32 ? red[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (threadIdx.x == 0) red[0] = t;
-  }
-  __syncthreads();
-  bool keep = !(sqrt(red[0]) < thr);
-  if (threadIdx.x == 0) {
-    flags[A * n_at + B] = keep;
-    flags[B * n_at + A] = keep;
+  const bool keep = !(sqrt(s) < thr);
+  if (lane == 0) {
+    flags[(long long)A * n_at + B] = keep;
+    flags[(long long)B * n_at + A] = keep;
   }
   if (!keep) {
-    for (int i = threadIdx.x; i < na * nb; i += blockDim.x) {
+    for (int i = lane; i < na * nb; i += 32) {
       g[(long long)(a0 + i / nb) * nao + b0 + i % nb] = 0.0;
       g[(long long)(b0 + i % nb) * nao + a0 + i / nb] = 0.0;
     }
@@ -529,8 +536,8 @@ void launch_cast_f64_f32(const double* x, float* y, long long n, cudaStream_t st
 
 void launch_scale_orbitals(const double* C, const double* eps, int nao, int n_occ, double mu, double tau,
                            double* cso, double* csv, cudaStream_t st) {
-  const long long n = (long long)nao * nao;
-  k_scale_orbitals<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(C, eps, nao, n_occ, mu, tau, cso, csv);
+  const unsigned gx = (nao + 31) / 32;
+  k_scale_orbitals<<<dim3(gx, (304 + gx - 1) / gx), 256, 0, st>>>(C, eps, nao, n_occ, mu, tau, cso, csv);
 }
 
 void launch_greens(const double* C, const double* eps, int nao, int n_occ, double mu, double tau,
@@ -540,9 +547,11 @@ void launch_greens(const double* C, const double* eps, int nao, int n_occ, doubl
   k_syrk64<<<dim3(t, t, 2), 64, 0, st>>>(cso, csv, nao, n_occ, g_occ, g_virt);
 }
 
-void launch_sym_block_filter(double* g, int nao, const int* ao_off, int n_at, double thr,
-                             unsigned char* flags, cudaStream_t st) {
-  k_sym_block_filter<<<n_at * n_at, 256, 0, st>>>(g, nao, ao_off, n_at, thr, flags);
+void launch_sym_block_filter(double* g0, double* g1, int nao, const int* ao_off, int n_at, double thr,
+                             unsigned char* flags0, unsigned char* flags1, cudaStream_t st) {
+  const long long pairs = static_cast<long long>(n_at) * n_at;
+  k_sym_block_filter<<<dim3(static_cast<unsigned>((pairs + 7) / 8), 2), 256, 0, st>>>(g0, g1, nao, ao_off, n_at, thr,
+                                                                                      flags0, flags1);
 }
 
 template <typename T>

@@ -21,8 +21,9 @@ void launch_scale_orbitals(const double* C, const double* eps, int nao, int n_oc
                            double* cso, double* csv, cudaStream_t st);
 void launch_greens(const double* C, const double* eps, int nao, int n_occ, double mu, double tau,
                    double* cso, double* csv, double* g_occ, double* g_virt, cudaStream_t st);
-void launch_sym_block_filter(double* g, int nao, const int* ao_off, int n_at, double thr,
-                             unsigned char* flags, cudaStream_t st);
+// Both Green's functions: blocks of norm < thr zeroed, flags of the kept ones.
+void launch_sym_block_filter(double* g0, double* g1, int nao, const int* ao_off, int n_at, double thr,
+                             unsigned char* flags0, unsigned char* flags1, cudaStream_t st);
 template <typename T>
 void launch_panel_gemm(const T* G, int nao, const T* pool, const int* lam, const PanelTask* tasks,
                        int ntasks, int maxN, int mode, int r0, int R, int P0b, long long ldk,

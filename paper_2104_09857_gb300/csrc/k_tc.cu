@@ -1466,34 +1466,55 @@ __global__ void k_zero_dead_y(uint16_t* __restrict__ Y, int slices, long long sl
   }
 }
 
+// Eight consecutive elements into 16-byte stores of each slice.
+__device__ __forceinline__ void store_slices8(double (&v)[8], int slices, long long slice_elems, bool f16,
+                                              uint16_t* __restrict__ dst) {
+  for (int s = 0; s < slices; ++s) {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t lo = take_slice(v[2 * i], f16);
+      w[i] = lo | (static_cast<uint32_t>(take_slice(v[2 * i + 1], f16)) << 16);
+    }
+    *reinterpret_cast<uint4*>(dst + s * slice_elems) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
 // FP64 [rows][cols] (row stride ld), times scale -> 16-bit slices
-// [S][rows][kpad], zero for k >= cols
-__global__ void k_split_f64(const double* __restrict__ a, long long ld, int rows, int cols, int kpad,
-                            int slices, int f16, double scale, uint16_t* __restrict__ out) {
-  const long long n = static_cast<long long>(rows) * kpad;
-  const long long slice = n;
+// [S][rows][kpad], zero for k >= cols; kpad a multiple of 64.
+__global__ void __launch_bounds__(256) k_split_f64(const double* __restrict__ a, long long ld, int rows, int cols,
+                                                   int kpad, int slices, int f16, double scale,
+                                                   uint16_t* __restrict__ out) {
+  const long long per = kpad / 8, n = rows * per;
   for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int r = static_cast<int>(i / kpad), k = static_cast<int>(i % kpad);
-    double v = k < cols ? scale * a[static_cast<long long>(r) * ld + k] : 0.0;
-    for (int s = 0; s < slices; ++s) out[s * slice + i] = take_slice(v, f16 != 0);
+    const long long r = i / per;
+    const int k = static_cast<int>(i - r * per) * 8;
+    double v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = k + j < cols ? scale * a[r * ld + k + j] : 0.0;
+    store_slices8(v, slices, static_cast<long long>(rows) * kpad, f16 != 0, out + r * kpad + k);
   }
 }
 
 // Grouped split: problem p's FP64 matrix src[off + r * ld + k] (r < rows,
 // k < cols), times its scale, into slice rows dst_row + r of [S][..][kmax],
-// zero for k >= cols.  blockIdx.y = problem.
-__global__ void k_split_group(const double* __restrict__ src, const SplitDesc* __restrict__ desc,
-                              int kmax, int slices, long long slice_elems, int f16,
-                              uint16_t* __restrict__ out) {
+// zero for cols <= k < the next multiple of 64 (no product reads beyond it).
+// blockIdx.y = problem; eight elements of a row per thread (kmax and the
+// problems' padded widths are multiples of 64, the rows 16-byte aligned).
+__global__ void __launch_bounds__(256) k_split_group(const double* __restrict__ src,
+                                                     const SplitDesc* __restrict__ desc, int kmax, int slices,
+                                                     long long slice_elems, int f16, uint16_t* __restrict__ out) {
   const SplitDesc d = desc[blockIdx.y];
-  const long long n = static_cast<long long>(d.rows) * kmax;
-  for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-       i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int r = static_cast<int>(i / kmax), k = static_cast<int>(i % kmax);
-    double v = k < d.cols ? d.scale * src[d.src_off + static_cast<long long>(r) * d.ld + k] : 0.0;
-    const long long dst = (d.dst_row + r) * kmax + k;
-    for (int s = 0; s < slices; ++s) out[s * slice_elems + dst] = take_slice(v, f16 != 0);
+  const int per = (d.cols + 63) / 64 * 8;  // groups of eight per row
+  const int n = d.rows * per;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int r = i / per, k = (i - r * per) * 8;
+    const double* x = src + d.src_off + static_cast<long long>(r) * d.ld + k;
+    double v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = k + j < d.cols ? d.scale * x[j] : 0.0;
+    store_slices8(v, slices, slice_elems, f16 != 0, out + (d.dst_row + r) * kmax + k);
   }
 }
 
@@ -1718,7 +1739,7 @@ void launch_split_f64(const double* a, long long ld, int rows, int cols, int kpa
                       int f16, double scale, void* out, cudaStream_t st) {
   const long long n = static_cast<long long>(rows) * kpad;
   if (n == 0) return;
-  long long blocks = (n + 255) / 256;
+  long long blocks = (n / 8 + 255) / 256;
   if (blocks > 152 * 32) blocks = 152 * 32;
   tc::k_split_f64<<<static_cast<unsigned>(blocks), 256, 0, st>>>(a, ld, rows, cols, kpad, slices, f16,
                                                                 scale, static_cast<uint16_t*>(out));
@@ -1874,7 +1895,7 @@ int launch_panel_tc(int slices, int f16, float unscale, float out_scale, const C
 void launch_split_group(const double* src, const SplitDesc* desc, int n_prob, int max_rows, int kmax,
                         int slices, long long slice_elems, int f16, void* out, cudaStream_t st) {
   if (n_prob == 0 || max_rows == 0) return;
-  long long bx = (static_cast<long long>(max_rows) * kmax + 255) / 256;
+  long long bx = (static_cast<long long>(max_rows) * kmax / 8 + 255) / 256;
   if (bx > 256) bx = 256;
   for (int p0 = 0; p0 < n_prob; p0 += 65535) {
     const int np = n_prob - p0 < 65535 ? n_prob - p0 : 65535;

@@ -108,7 +108,7 @@ struct SplitDesc {
   double scale;
 };
 // scale * matrix -> 16-bit slices [S][..][kmax] for every problem in one launch
-// (zero for k >= cols); max_rows bounds the problems' row counts.
+// (zero from cols to the next multiple of 64); max_rows bounds the problems' row counts.
 void launch_split_group(const double* src, const SplitDesc* desc, int n_prob, int max_rows, int kmax,
                         int slices, long long slice_elems, int f16, void* out, cudaStream_t st);
 // out2[2p] = max |x|, out2[2p + 1] = max row sum |x| of every problem.
