@@ -65,6 +65,7 @@ int ws(gw_ctx* ctx, const char* name, size_t bytes, void** out) {
     return GW_OK;
   }
   if (it != wb.end()) {
+    ctx->uploaded.erase(name);
     cudaFree(it->second.first);
     wb.erase(it);
   }
@@ -98,6 +99,7 @@ void ws_release_all(gw_ctx* ctx) {
   cudaStreamSynchronize(ctx->stream);
   for (auto& kv : wb) cudaFree(kv.second.first);
   wb.clear();
+  ctx->uploaded.clear();
 }
 
 template <typename T>
@@ -108,13 +110,26 @@ int wsT(gw_ctx* ctx, const char* name, size_t count, T** out) {
   return rc;
 }
 
+// Copies a host table into its named buffer, unless the buffer already holds
+// exactly these bytes: a table of the plan is the same at every tau point (and,
+// as a rule, in the next call), and a copy from pageable memory costs some 5 us
+// of host time, twenty of them per batch.  Compared by content; the buffers of
+// tables are written nowhere else.
 template <typename T>
 int upload(gw_ctx* ctx, const char* name, const std::vector<T>& v, T** out) {
   int rc = wsT<T>(ctx, name, std::max<size_t>(v.size(), 1), out);
-  if (rc) return rc;
-  if (!v.empty())
-    GW_TRY(cudaMemcpyAsync(*out, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice,
-                           ctx->stream));
+  if (rc || v.empty()) return rc;
+  constexpr size_t kMaxHeld = size_t(4) << 20;
+  const size_t bytes = v.size() * sizeof(T);
+  auto& held = ctx->uploaded[name];
+  const char* p = reinterpret_cast<const char*>(v.data());
+  if (held.first == *out && held.second.size() == bytes && !std::memcmp(held.second.data(), p, bytes)) return GW_OK;
+  held.first = nullptr;
+  GW_TRY(cudaMemcpyAsync(*out, p, bytes, cudaMemcpyHostToDevice, ctx->stream));
+  if (bytes <= kMaxHeld) {
+    held.second.assign(p, p + bytes);
+    held.first = *out;
+  }
   return GW_OK;
 }
 
@@ -1348,9 +1363,12 @@ int ensure_ycover(gw_ctx* ctx) {
   return GW_OK;
 }
 
+int tc_results(gw_ctx* ctx, int** err, unsigned long long** stat, double** fc);
+
 // One batch on the tensor cores: steps A and B straight into bf16 slices,
-// block filter from the accumulated norms, task lists, step C.
-int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const double* g_occ, const double* g_virt,
+// block filter from the accumulated norms, task lists, step C.  gs_occ,
+// gs_virt: slices of G^occ and G^virt, [slices][n_AO][n_AO rounded to 64].
+int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void* gs_virt,
                      double thr, double* acc, std::vector<double>& fc_host, int precision,
                      size_t batch_idx) {
   const int slices = precision == GW_BF16X6 ? 3 : 2;
@@ -1370,7 +1388,7 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const double* g_occ, const dou
   const int n_at = ctx->n_at, nri = ctx->nri;
   int rc;
   if (prow == 0 || qrow == 0 || Kb == 0) return GW_OK;
-  const int kmax = ctx->pt_kmax;
+  const int kmax = ctx->pt_kmax, gkp = (ctx->nao + 63) / 64 * 64;
   void *xs, *ys;
   if ((rc = ws(ctx, "Xs", (size_t)slices * prow * Kb * 2, &xs))) return rc;
   if ((rc = ws(ctx, "Ys", (size_t)slices * qrow * Kb * 2, &ys))) return rc;
@@ -1412,7 +1430,7 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const double* g_occ, const dou
   GW_TRY(cudaMemsetAsync(bx2, 0, (size_t)ns * nmc * npa * sizeof(float), ctx->stream));
   GW_TRY(cudaMemsetAsync(by2, 0, (size_t)ns * nmc * nqa * sizeof(float), ctx->stream));
   int* d_err;  // zeroed once per tau point by gw_chi_tau
-  if ((rc = wsT(ctx, "tc_err", 1, &d_err))) return rc;
+  if ((rc = tc_results(ctx, &d_err, nullptr, nullptr))) return rc;
   // split panels: the resident set for both steps, or streamed regions (A:
   // the batch's owners, rebuilt per batch; B: the chunk's atoms, rebuilt when
   // the chunk changes)
@@ -1515,8 +1533,8 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const double* g_occ, const dou
       if ((rc = upload(ctx, "tc_tilesA", tiles, &d_tiles))) return rc;
       const long long g_elems = (long long)ta.size() * rows_a * kmax;
       if ((rc = ws(ctx, "GgA", (size_t)slices * g_elems * 2, &gg))) return rc;
-      gw::launch_gather_g(g_occ, ctx->nao, d_ta, (int)ta.size(), ctx->d_lam, b.mu0, b.nmu, rows_a, kmax,
-                          slices, g_elems, f16, s_go, gg, ctx->stream);
+      gw::launch_gather_g(gs_occ, ctx->nao, gkp, d_ta, (int)ta.size(), ctx->d_lam, b.mu0, b.nmu, rows_a, kmax,
+                          slices, g_elems, gg, ctx->stream);
       GW_CHECK_LAUNCH();
       CUtensorMap mg;
       if (gw::make_slice_map(&mg, gg, kmax, (long long)ta.size() * rows_a, slices, tile, f16))
@@ -1631,8 +1649,8 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const double* g_occ, const dou
       if ((rc = upload(ctx, "rowsl", rowsl, &d_rowsl))) return rc;
       const long long g_elems = (long long)tb.size() * rows_b * kmax;
       if ((rc = ws(ctx, "GgB", (size_t)slices * g_elems * 2, &gg))) return rc;
-      gw::launch_gather_g(g_virt, ctx->nao, d_tb, (int)tb.size(), ctx->d_lam, r0, R, rows_b, kmax, slices,
-                          g_elems, f16, s_gv, gg, ctx->stream);
+      gw::launch_gather_g(gs_virt, ctx->nao, gkp, d_tb, (int)tb.size(), ctx->d_lam, r0, R, rows_b, kmax, slices,
+                          g_elems, gg, ctx->stream);
       GW_CHECK_LAUNCH();
       CUtensorMap mg;
       if (gw::make_slice_map(&mg, gg, kmax, (long long)tb.size() * rows_b, slices, tile, f16))
@@ -1791,7 +1809,7 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const double* g_occ, const dou
         (rc = wsT(ctx, "u_hist", std::max(nslab, 1), &w.hist)) ||
         (rc = wsT(ctx, "u_start", std::max(nslab, 1), &w.start)) ||
         (rc = wsT(ctx, "u_nunits", 1, &w.n_units)) || (rc = wsT(ctx, "u_nkeys", 1, &w.total_keys)) ||
-        (rc = wsT(ctx, "task_stats", 3, &tstat)))
+        (rc = tc_results(ctx, nullptr, &tstat, nullptr)))
       return rc;
     gw::launch_plan_units(tasks, counts, kacc, d_len, ntiles, nslab, ctx->c_split_k, w, tstat,
                           ctx->stream);
@@ -1811,7 +1829,7 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const double* g_occ, const dou
     ctx->stats.c_launches += 1;
     ctx->stats.kernel_launches += 1;
     double* d_fc_all;
-    if ((rc = wsT(ctx, "fc_all", (size_t)n_at * n_at, &d_fc_all))) return rc;
+    if ((rc = tc_results(ctx, nullptr, nullptr, &d_fc_all))) return rc;
     GW_TRY(cudaMemcpyAsync(d_fc_all + ctx->tc_fc_used, d_fc, (size_t)ns * nmc * sizeof(double),
                            cudaMemcpyDeviceToDevice, ctx->stream));
     ctx->tc_pending.push_back({batch_idx, ctx->tc_fc_used, ns * nmc, fc_scale_dev});
@@ -1919,8 +1937,8 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const double* g_occ, const dou
   ctx->stats.kernel_launches += 1;
   // this batch's flop counts, error flag and timings are read at the end of
   // the tau point (tc_finish_tau), so the next batch is queued without a wait
-  double* d_fc_all;  // sized n_at * n_at by gw_chi_tau
-  if ((rc = wsT(ctx, "fc_all", (size_t)n_at * n_at, &d_fc_all))) return rc;
+  double* d_fc_all;
+  if ((rc = tc_results(ctx, nullptr, nullptr, &d_fc_all))) return rc;
   GW_TRY(cudaMemcpyAsync(d_fc_all + ctx->tc_fc_used, d_fc, (size_t)ns * nmc * sizeof(double),
                          cudaMemcpyDeviceToDevice, ctx->stream));
   ctx->tc_pending.push_back({batch_idx, ctx->tc_fc_used, ns * nmc, fc_scale});
@@ -1941,45 +1959,55 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const double* g_occ, const dou
   return GW_OK;
 }
 
+// What the tensor-core batches of a tau point leave for the host, in one buffer
+// that is read with one copy: the error flag (8 bytes), three task statistics,
+// and the flop counts of step C.
+int tc_results(gw_ctx* ctx, int** err, unsigned long long** stat, double** fc) {
+  unsigned long long* p;
+  const int rc = wsT(ctx, "tc_results", 4 + (size_t)ctx->n_at * ctx->n_at, &p);
+  if (rc) return rc;
+  if (err) *err = reinterpret_cast<int*>(p);
+  if (stat) *stat = p + 1;
+  if (fc) *fc = reinterpret_cast<double*>(p + 4);
+  return GW_OK;
+}
+
 // Start of a tau point on the tensor-core route: error flag and flop-count
 // staging for its batches.
 int tc_begin_tau(gw_ctx* ctx) {
   int* d_err;
-  double* d_fc_all;
   int rc;
-  if ((rc = wsT(ctx, "tc_err", 1, &d_err))) return rc;
-  if ((rc = wsT(ctx, "fc_all", (size_t)ctx->n_at * ctx->n_at, &d_fc_all))) return rc;
-  GW_TRY(cudaMemsetAsync(d_err, 0, sizeof(int), ctx->stream));
-  unsigned long long* tstat;
-  if ((rc = wsT(ctx, "task_stats", 3, &tstat))) return rc;
-  GW_TRY(cudaMemsetAsync(tstat, 0, 3 * sizeof(unsigned long long), ctx->stream));
+  if ((rc = tc_results(ctx, &d_err, nullptr, nullptr))) return rc;
+  GW_TRY(cudaMemsetAsync(d_err, 0, 4 * sizeof(unsigned long long), ctx->stream));
   ctx->tc_pending.clear();
   ctx->tc_fc_used = 0;
   ctx->tc_issue_per_k = 0.0;
   return GW_OK;
 }
 
+// The results of a tau point's batches, on their way to the host.
+int tc_fetch_tau(gw_ctx* ctx, std::vector<unsigned long long>& h) {
+  int* d_res;
+  int rc;
+  if ((rc = tc_results(ctx, &d_res, nullptr, nullptr))) return rc;
+  h.assign(4 + (size_t)ctx->tc_fc_used, 0);
+  GW_TRY(cudaMemcpyAsync(h.data(), d_res, h.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                         ctx->stream));
+  return GW_OK;
+}
+
 // End of a tau point (after the stream is synchronised): error flag, step
 // timings and step-C flop counts of its tensor-core batches.
-int tc_finish_tau(gw_ctx* ctx, std::vector<double>& fc_host) {
-  int* d_err;
-  double* d_fc_all;
+int tc_finish_tau(gw_ctx* ctx, const std::vector<unsigned long long>& h, std::vector<double>& fc_host) {
   int rc;
-  if ((rc = wsT(ctx, "tc_err", 1, &d_err))) return rc;
-  if ((rc = wsT(ctx, "fc_all", (size_t)ctx->n_at * ctx->n_at, &d_fc_all))) return rc;
-  int h_err = 0;
-  GW_TRY(cudaMemcpy(&h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost));
+  int h_err;
+  std::memcpy(&h_err, h.data(), sizeof(int));
   if (h_err)
     return fail(ctx, GW_ERR_TIMEOUT,
                 "tensor-core kernel: a bounded wait gave up (flags " + std::to_string(h_err) + ")");
-  std::vector<double> h_fc((size_t)ctx->tc_fc_used);
-  if (!h_fc.empty())
-    GW_TRY(cudaMemcpy(h_fc.data(), d_fc_all, h_fc.size() * sizeof(double), cudaMemcpyDeviceToHost));
-  // task statistics of the batches whose units were planned on the device
-  unsigned long long* tstat;
-  unsigned long long h_stat[3] = {0, 0, 0};
-  if ((rc = wsT(ctx, "task_stats", 3, &tstat))) return rc;
-  GW_TRY(cudaMemcpy(h_stat, tstat, sizeof(h_stat), cudaMemcpyDeviceToHost));
+  const unsigned long long* h_stat = h.data() + 1;
+  std::vector<double> h_fc(h.size() - 4);
+  std::memcpy(h_fc.data(), h.data() + 4, h_fc.size() * sizeof(double));
   ctx->stats.tiles_active += (long long)h_stat[0];
   ctx->stats.slabs_active += (long long)h_stat[1];
   ctx->stats.flops_issued += ctx->tc_issue_per_k * (double)h_stat[2];
@@ -2046,6 +2074,7 @@ void work_trim(gw_ctx* ctx, const char* prefix, size_t keep) {
   cudaStreamSynchronize(ctx->stream);
   for (auto it = ctx->work.begin(); it != ctx->work.end();) {
     if (it->first.compare(0, n, prefix) == 0) {
+      ctx->uploaded.erase(it->first);
       cudaFree(it->second.first);
       it = ctx->work.erase(it);
     } else {
@@ -2498,22 +2527,17 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
     if ((rc = gw::greens_fp64(ctx, *ctx, ctx->tau[j], cso, csv, go, gv, ctx->stream))) return rc;
     GW_CHECK_LAUNCH();
     ctx->stats.kernel_launches += 3;
+    double h[4] = {0, 0, 0, 0};
     if (f16) {
       // binary16 scales of this tau: max |G| for the G slices, and the bounds
       // |X| <= max_mu sum_lambda |G^occ| * max |T| (Y alike with G^virt)
       double* gst;
-      double h[4];
       if ((rc = wsT(ctx, "g_absmax", 4, &gst))) return rc;
       gw::launch_absmax_rowsum(go, nao, nao, nao, gst, ctx->stream);
       gw::launch_absmax_rowsum(gv, nao, nao, nao, gst + 2, ctx->stream);
       GW_CHECK_LAUNCH();
       ctx->stats.kernel_launches += 2;
       GW_TRY(cudaMemcpyAsync(h, gst, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
-      GW_TRY(cudaStreamSynchronize(ctx->stream));
-      ctx->tc_scale[0] = gw::pow2_scale(h[0]);
-      ctx->tc_scale[1] = gw::pow2_scale(h[2]);
-      ctx->tc_scale[2] = gw::pow2_scale(h[1] * ctx->t_absmax);
-      ctx->tc_scale[3] = gw::pow2_scale(h[3] * ctx->t_absmax);
     }
     std::vector<unsigned char> hfo((size_t)n_at * n_at, 1), hfv((size_t)n_at * n_at, 1);
     if (thr > 0.0) {
@@ -2522,7 +2546,14 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
       ctx->stats.kernel_launches += 1;
       GW_TRY(cudaMemcpyAsync(hfo.data(), flo, hfo.size(), cudaMemcpyDeviceToHost, ctx->stream));
       GW_TRY(cudaMemcpyAsync(hfv.data(), flv, hfv.size(), cudaMemcpyDeviceToHost, ctx->stream));
-      GW_TRY(cudaStreamSynchronize(ctx->stream));  // the batch plan below reads the flags
+    }
+    // one wait for the scales and for the flags that the batch plan below reads
+    if (f16 || thr > 0.0) GW_TRY(cudaStreamSynchronize(ctx->stream));
+    if (f16) {
+      ctx->tc_scale[0] = gw::pow2_scale(h[0]);
+      ctx->tc_scale[1] = gw::pow2_scale(h[2]);
+      ctx->tc_scale[2] = gw::pow2_scale(h[1] * ctx->t_absmax);
+      ctx->tc_scale[3] = gw::pow2_scale(h[3] * ctx->t_absmax);
     }
     if (!f64 && !tcpath) {
       gw::launch_cast_f64_f32(go, go32, (long long)nao * nao, ctx->stream);
@@ -2534,6 +2565,17 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
     GW_TRY(cudaEventRecord(ev[1], ctx->stream));
     std::vector<double> fc;
     if (tcpath && (rc = tc_begin_tau(ctx))) return rc;
+    void *gs_occ = nullptr, *gs_virt = nullptr;  // slices of the filtered G
+    if (tcpath) {
+      const int sl = precision == GW_BF16X6 ? 3 : 2, gkp = (nao + 63) / 64 * 64;
+      if ((rc = ws(ctx, "gs_occ", (size_t)sl * nao * gkp * 2, &gs_occ)) ||
+          (rc = ws(ctx, "gs_virt", (size_t)sl * nao * gkp * 2, &gs_virt)))
+        return rc;
+      gw::launch_split_f64(go, nao, nao, nao, gkp, sl, f16, f16 ? ctx->tc_scale[0] : 1.0, gs_occ, ctx->stream);
+      gw::launch_split_f64(gv, nao, nao, nao, gkp, sl, f16, f16 ? ctx->tc_scale[1] : 1.0, gs_virt, ctx->stream);
+      GW_CHECK_LAUNCH();
+      ctx->stats.kernel_launches += 2;
+    }
     gw::EmuOp op_o, op_v;  // digits of the filtered G
     if (digits) {
       gw::EmuSrc s;
@@ -2571,7 +2613,7 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
       else if (f64)
         rc = chi_one_batch<double>(ctx, b, go, gv, ctx->d_panel64, thr, acc, fc, precision, bi);
       else if (tcpath)
-        rc = chi_one_batch_tc(ctx, b, go, gv, thr, acc, fc, precision, bi);
+        rc = chi_one_batch_tc(ctx, b, gs_occ, gs_virt, thr, acc, fc, precision, bi);
       else
         rc = chi_one_batch<float>(ctx, b, go32, gv32, ctx->d_panel32, thr, acc, fc, precision, bi);
       if (rc) {
@@ -2588,8 +2630,10 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
     if (!out_on_device)
       GW_TRY(cudaMemcpyAsync(chi_out + (size_t)(j - tau_first) * nri * nri, stage,
                              (size_t)nri * nri * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    std::vector<unsigned long long> h_res;
+    if (tcpath && (rc = tc_fetch_tau(ctx, h_res))) return rc;
     GW_TRY(cudaStreamSynchronize(ctx->stream));
-    if (tcpath && (rc = tc_finish_tau(ctx, fc))) return rc;
+    if (tcpath && (rc = tc_finish_tau(ctx, h_res, fc))) return rc;
     float t01, t12;
     GW_TRY(cudaEventElapsedTime(&t01, ev[0], ev[1]));
     GW_TRY(cudaEventElapsedTime(&t12, ev[1], ev[2]));

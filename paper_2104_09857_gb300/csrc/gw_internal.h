@@ -301,6 +301,8 @@ struct gw_ctx {
   // named device work buffers (grown on demand) and the step timing events
   // of this context; a context is used by one host thread at a time
   std::map<std::string, std::pair<void*, size_t>> work;
+  // host tables last copied into a work buffer: the buffer and the bytes
+  std::map<std::string, std::pair<void*, std::vector<char>>> uploaded;
   std::vector<cudaEvent_t> events;
 
   // test hooks (options "test_fail_alloc", "test_stall_tc")

@@ -166,9 +166,12 @@ void launch_zero_unwritten_y(void* Y, int slices, long long slice_elems, long lo
 // zero-padded in k.
 void launch_split_f64(const double* a, long long ld, int rows, int cols, int kpad, int slices,
                       int f16, double scale, void* out, cudaStream_t st);
-void launch_gather_g(const double* g, int nao, const PanelTaskTC* tasks, int ntasks, const int* lam,
-                     int rbase, int rows_valid, int rows_per_task, int kmax, int slices,
-                     long long slice_elems, int f16, double scale, void* out, cudaStream_t st);
+// The rows of G that step A / B's panel tasks multiply, gathered on each
+// panel's lambda functions from the slices gs [slices][nao][gkp] of G (k_gather_g
+// in k_tc.cu); kmax a multiple of 64.
+void launch_gather_g(const void* gs, int nao, int gkp, const PanelTaskTC* tasks, int ntasks, const int* lam,
+                     int rbase, int rows_valid, int rows_per_task, int kmax, int slices, long long slice_elems,
+                     void* out, cudaStream_t st);
 // The same from the tensor kept in FP32 (option tensor_fp32).
 void launch_pt_scatter_f32(const float* t3, const int* blk, const long long* off, const int* n_ao,
                            const int* n_ri, const int* kept, long long n_kept, const long long* rowB,
