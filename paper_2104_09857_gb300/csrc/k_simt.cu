@@ -9,6 +9,8 @@
 #include "gw_internal.h"
 #include "k_simt.h"
 
+#include <cooperative_groups.h>
+
 namespace gw {
 
 // ---------------------------------------------------------------------------
@@ -255,6 +257,171 @@ __global__ void __launch_bounds__(64) k_syrk64(const double* __restrict__ cso, c
     }
 }
 
+// ---------------------------------------------------------------------------
+// FP32: 64 x 64 tile, 128 threads, thread (tx, ty) owns rows 8 ty .. + 7 and
+// columns 4 tx .. + 3, two products per instruction (fma.rn.f32x2).  Three
+// 16-byte shared loads feed 32 multiply-adds, where the 4 x 4 tile of
+// tile_nt_run needs eight 4-byte ones for 16.  Per element the products enter
+// one by one in the order of k, as there: the sums are the same to the bit.
+// ---------------------------------------------------------------------------
+constexpr int kF32K = 16;      // reduction elements per stage
+constexpr int kF32Pitch = 68;  // floats per k row of a stage (16-byte aligned)
+using F32Stage = float[kF32K][kF32Pitch];
+
+__device__ __forceinline__ void fma2(unsigned long long& c, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long pack2(float x, float y) {
+  unsigned long long v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+  return v;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+// acc[i][j]: rows r = 8 ty + 2 i and r + 1 at columns c = 4 tx + (j & ~1) and
+// c + 1: (r, c), (r + 1, c + 1) for even j and (r, c + 1), (r + 1, c) for odd,
+// which takes one swapped copy of B's pair and no duplicated operand.
+__device__ __forceinline__ void f32_stage(const F32Stage& A, const F32Stage& B, int tx, int ty,
+                                          unsigned long long (&acc)[4][4]) {
+#pragma unroll
+  for (int kk = 0; kk < kF32K; ++kk) {
+    const float4 a0 = *reinterpret_cast<const float4*>(&A[kk][8 * ty]);
+    const float4 a1 = *reinterpret_cast<const float4*>(&A[kk][8 * ty + 4]);
+    const float4 b = *reinterpret_cast<const float4*>(&B[kk][4 * tx]);
+    const unsigned long long av[4] = {pack2(a0.x, a0.y), pack2(a0.z, a0.w), pack2(a1.x, a1.y), pack2(a1.z, a1.w)};
+    const unsigned long long bv[4] = {pack2(b.x, b.y), pack2(b.y, b.x), pack2(b.z, b.w), pack2(b.w, b.z)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) fma2(acc[i][j], av[i], bv[j]);
+  }
+}
+
+// v[i][j]: row 8 ty + i, column 4 tx + j
+__device__ __forceinline__ void f32_unpack(const unsigned long long (&acc)[4][4], float (&v)[8][4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; j += 2) {
+      const float2 d = unpack2(acc[i][j]), s = unpack2(acc[i][j + 1]);
+      v[2 * i][j] = d.x;
+      v[2 * i + 1][j + 1] = d.y;
+      v[2 * i][j + 1] = s.x;
+      v[2 * i + 1][j] = s.y;
+    }
+}
+
+// Step C in FP32: chi[P][Q] -= sum over the tile's slab list of X[P][k] Y[Q][k],
+// each slab summed in FP32 and the slabs in FP64.  ldk and every slab's start
+// and length are multiples of 16 elements.  A cluster shares a tile, each block
+// a contiguous part of its slabs: 58 atoms have 272 tiles of work, less than two
+// blocks per SM.  Bound by the FP32 pipe.
+constexpr int kF32Split = 8;
+__global__ void __cluster_dims__(1, 1, kF32Split) __launch_bounds__(128) k_chi_tiles_f32(const float* __restrict__ X, const float* __restrict__ Y,
+                                                       long long ldk, int P0, int prow, int nri,
+                                                       const int* __restrict__ tasks, const int* __restrict__ counts,
+                                                       int max_slab, int nqt, const long long* __restrict__ slab_k0,
+                                                       const int* __restrict__ slab_len, double* __restrict__ chi) {
+  __shared__ __align__(16) union {
+    struct {
+      F32Stage a[2], b[2];
+    } st;
+    double part[64][64];
+  } sm;
+  auto& As = sm.st.a;
+  auto& Bs = sm.st.b;
+  auto& part = sm.part;  // after the last stage
+  const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int rank = static_cast<int>(cluster.block_rank());
+  const int tile = blockIdx.y * nqt + blockIdx.x;
+  const int total = counts[tile];
+  if (total == 0) return;  // the whole cluster
+  const int p0 = blockIdx.y * 64, q0 = blockIdx.x * 64;
+  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+  // this thread fetches k 4 (t % 4) .. + 3 of rows t / 4 and t / 4 + 32
+  const int fr = t >> 2, fk = (t & 3) * 4;
+  const float* xr[2];
+  const float* yr[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int r = fr + 32 * h;
+    xr[h] = p0 + r < prow ? X + static_cast<long long>(p0 + r) * ldk + fk : nullptr;
+    yr[h] = q0 + r < nri ? Y + static_cast<long long>(q0 + r) * ldk + fk : nullptr;
+  }
+  float4 fx[2], fy[2];
+  auto fetch = [&](long long k) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      fx[h] = xr[h] ? *reinterpret_cast<const float4*>(xr[h] + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+      fy[h] = yr[h] ? *reinterpret_cast<const float4*>(yr[h] + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  auto put = [&](int s) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = fr + 32 * h;
+      As[s][fk][r] = fx[h].x;
+      As[s][fk + 1][r] = fx[h].y;
+      As[s][fk + 2][r] = fx[h].z;
+      As[s][fk + 3][r] = fx[h].w;
+      Bs[s][fk][r] = fy[h].x;
+      Bs[s][fk + 1][r] = fy[h].y;
+      Bs[s][fk + 2][r] = fy[h].z;
+      Bs[s][fk + 3][r] = fy[h].w;
+    }
+  };
+  const int first = static_cast<int>(static_cast<long long>(total) * rank / kF32Split);
+  const int cnt = static_cast<int>(static_cast<long long>(total) * (rank + 1) / kF32Split) - first;
+  const int* list = tasks + static_cast<long long>(tile) * max_slab + first;
+  double sum[8][4] = {};
+  int s = 0;
+  if (cnt > 0) {
+    fetch(slab_k0[list[0]]);
+    put(0);
+  }
+  __syncthreads();
+  for (int i = 0; i < cnt; ++i) {
+    const long long k0 = slab_k0[list[i]];
+    const int len = slab_len[list[i]];
+    const long long next = i + 1 < cnt ? slab_k0[list[i + 1]] : -1;
+    unsigned long long acc[4][4] = {};
+    for (int kk = 0; kk < len; kk += kF32K) {
+      // the next stage on its way while this one is multiplied
+      const long long k = kk + kF32K < len ? k0 + kk + kF32K : next;
+      if (k >= 0) fetch(k);
+      f32_stage(As[s], Bs[s], tx, ty, acc);
+      if (k >= 0) put(s ^ 1);
+      __syncthreads();
+      s ^= 1;
+    }
+    float v[8][4];
+    f32_unpack(acc, v);
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) sum[a][j] += static_cast<double>(v[a][j]);
+  }
+  // the cluster's partial tiles, eight rows of each added up by every rank in
+  // the order of the slabs
+#pragma unroll
+  for (int a = 0; a < 8; ++a)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) part[8 * ty + a][4 * tx + j] = sum[a][j];
+  cluster.sync();
+  for (int e = t; e < 8 * 64; e += 128) {
+    const int r = 8 * rank + e / 64, c = e % 64;
+    double v = 0.0;
+#pragma unroll
+    for (int o = 0; o < kF32Split; ++o) v += cluster.map_shared_rank(&part[r][c], o)[0];
+    const int m = p0 + r, n = q0 + c;
+    if (m < prow && n < nri) chi[static_cast<long long>(P0 + m) * nri + n] -= v;
+  }
+  cluster.sync();  // no rank leaves while its tile is read
+}
+
 // Step C: chi[P][Q] -= sum over the tile's slab list of X[P][k] Y[Q][k].
 // Tile (pt, qt) covers P in [P0 + 64 pt, ...) and Q in [64 qt, ...).
 template <typename T, typename AccT>
@@ -362,6 +529,73 @@ __global__ void k_panel_gemm(const T* __restrict__ G, int nao, const T* __restri
   }
 }
 
+// The same in FP32 on the 8 x 4 tiles of f32_stage: rows n of the panel along
+// the threads' columns, rows r of G along their rows.
+__global__ void __launch_bounds__(128) k_panel_gemm_f32(const float* __restrict__ G, int nao,
+                                                        const float* __restrict__ pool, const int* __restrict__ lam,
+                                                        const PanelTask* __restrict__ tasks, int mode, int r0, int R,
+                                                        int P0b, long long ldk, const long long* __restrict__ rowbase,
+                                                        const int* __restrict__ rowmul, float* __restrict__ out) {
+  __shared__ __align__(16) F32Stage As[2], Bs[2];
+  const PanelTask tk = tasks[blockIdx.z];
+  const int n0 = blockIdx.x * 64, m0 = blockIdx.y * 64;
+  if (n0 >= tk.N || m0 >= R) return;
+  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+  const float* P = pool + tk.panel_off;
+  const int* lk = lam + tk.lam_off;
+  // this thread fetches column c of k rows kr, kr + 2, ..
+  const int c = t & 63, kr = t >> 6;
+  const bool rin = m0 + c < R, nin = n0 + c < tk.N;
+  float fa[8], fb[8];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int k = k0 + kr + 2 * e;
+      const bool kin = k < tk.K;
+      fa[e] = (kin && rin) ? G[static_cast<long long>(lk[k]) * nao + r0 + m0 + c] : 0.f;
+      fb[e] = (kin && nin) ? P[static_cast<long long>(k) * tk.N + n0 + c] : 0.f;
+    }
+  };
+  auto put = [&](int s) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      As[s][kr + 2 * e][c] = fa[e];
+      Bs[s][kr + 2 * e][c] = fb[e];
+    }
+  };
+  unsigned long long acc[4][4] = {};
+  int s = 0;
+  fetch(0);
+  put(0);
+  __syncthreads();
+  for (int k0 = 0; k0 < tk.K; k0 += kF32K) {
+    const bool more = k0 + kF32K < tk.K;
+    if (more) fetch(k0 + kF32K);
+    f32_stage(As[s], Bs[s], tx, ty, acc);
+    if (more) put(s ^ 1);
+    __syncthreads();
+    s ^= 1;
+  }
+  float v[8][4];
+  f32_unpack(acc, v);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int n = n0 + 4 * tx + j;
+    if (n >= tk.N) continue;
+    const int pw = n / tk.nsig, sp = n - pw * tk.nsig;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = m0 + 8 * ty + i;
+      if (r >= R) continue;
+      const long long dst = mode == 0 ? static_cast<long long>(tk.p0 + pw - P0b) * ldk + tk.seg +
+                                            static_cast<long long>(r0 + r) * tk.nsig + sp
+                                      : static_cast<long long>(tk.p0 + pw) * ldk + rowbase[r] +
+                                            static_cast<long long>(tk.aom + sp) * rowmul[r];
+      out[dst] = v[i][j];
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Block filter of the intermediates and slab/tile occupancy.
 // Block (m, s, p) of an operand buffer Z[row][k]: rows = RI functions of atom
@@ -369,6 +603,20 @@ __global__ void k_panel_gemm(const T* __restrict__ G, int nao, const T* __restri
 // Norm < thr -> zeroed.  Kept and nonzero -> flag byte of the block and of
 // every (slab, row tile) it touches.
 // ---------------------------------------------------------------------------
+// |v| as FP32 within 2^-22, by integer operations (an FP64 conversion takes the
+// SM quarter's FP64 pipe for 64 cycles per warp); below FP32's range 0.
+__device__ __forceinline__ float magnitude(float v) { return fabsf(v); }
+__device__ __forceinline__ float magnitude(double v) {
+  const unsigned hi = static_cast<unsigned>(__double2hiint(v)) & 0x7fffffffu;
+  if (hi < 0x38100000u) return 0.f;
+  if (hi >= 0x47f00000u) return INFINITY;
+  return __uint_as_float(((hi - 0x38000000u) << 3) | (static_cast<unsigned>(__double2loint(v)) >> 29));
+}
+
+// One warp per block.  The norm is first taken in FP32 (a relative error below
+// 1e-3 for blocks of up to 10^4 rows); only a block within 1 % of the threshold, one
+// outside FP32's range or one with an Inf or NaN has it taken in FP64, so every decision is the FP64 one.
+// In FP64 throughout, the kernel was bound by that pipe.
 template <typename T>
 __global__ void k_operand_block_filter(T* __restrict__ Z, long long ldk, int rowoff,
                                        const int* __restrict__ ri_off, const int* __restrict__ ao_off,
@@ -390,24 +638,50 @@ __global__ void k_operand_block_filter(T* __restrict__ Z, long long ldk, int row
   int rows0 = ri_off[p] - rowoff, nrows = ri_off[p + 1] - ri_off[p];
   long long c0 = seg[sl] + (long long)ao_off[m] * nsig;
   int ncols = n_ao[m] * nsig;
-  double acc = 0.0;
+  float sum = 0.f;
+  bool any = false;
   for (int r = 0; r < nrows; ++r) {
     const T* row = Z + (long long)(rows0 + r) * ldk + c0;
+    float part = 0.f;
+#pragma unroll 4
     for (int c = lane; c < ncols; c += 32) {
-      double v = (double)row[c];
-      acc += v * v;
+      const T v = row[c];
+      any = any || !(v == T(0));
+      const float m = magnitude(v);
+      part = fmaf(m, m, part);
     }
+    sum += part;
   }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  double nrm = sqrt(acc);
-  bool kept = !(nrm < thr);
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  any = __any_sync(0xffffffffu, any);
+  const float t2 = (float)(thr * thr);
+  bool kept, nz = false;
+  if (!any) {
+    kept = !(0.0 < thr);
+  } else if (sum > fmaxf(1.01f * t2, 1e-30f) && sum < 1e37f) {
+    kept = nz = true;
+  } else if (t2 > 1e-30f && sum < 0.99f * t2) {
+    kept = false;
+  } else {
+    double acc = 0.0;
+    for (int r = 0; r < nrows; ++r) {
+      const T* row = Z + (long long)(rows0 + r) * ldk + c0;
+      for (int c = lane; c < ncols; c += 32) {
+        const double v = (double)row[c];
+        acc += v * v;
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    const double nrm = sqrt(acc);
+    kept = !(nrm < thr);
+    nz = kept && nrm > 0.0;
+  }
   if (!kept) {
     for (int r = 0; r < nrows; ++r) {
       T* row = Z + (long long)(rows0 + r) * ldk + c0;
       for (int c = lane; c < ncols; c += 32) row[c] = T(0);
     }
   }
-  bool nz = kept && nrm > 0.0;
   if (lane == 0) blockflag[w] = nz;
   if (nz) {
     // flag (sigma-atom, mu-atom, tile) for every tile the block's rows touch
@@ -562,8 +836,12 @@ void launch_panel_gemm(const T* G, int nao, const T* pool, const int* lam, const
   for (int z0 = 0; z0 < ntasks; z0 += 65535) {
     int nz = ntasks - z0 < 65535 ? ntasks - z0 : 65535;
     dim3 grid((maxN + 63) / 64, (R + 63) / 64, nz);
-    k_panel_gemm<T><<<grid, 256, 0, st>>>(G, nao, pool, lam, tasks + z0, mode, r0, R, P0b, ldk,
-                                         rowbase, rowmul, out);
+    if constexpr (sizeof(T) == 4)
+      k_panel_gemm_f32<<<grid, 128, 0, st>>>(G, nao, pool, lam, tasks + z0, mode, r0, R, P0b, ldk, rowbase, rowmul,
+                                             out);
+    else
+      k_panel_gemm<T><<<grid, 256, 0, st>>>(G, nao, pool, lam, tasks + z0, mode, r0, R, P0b, ldk,
+                                           rowbase, rowmul, out);
   }
 }
 template void launch_panel_gemm<double>(const double*, int, const double*, const int*,
@@ -619,8 +897,12 @@ void launch_chi_tiles(const T* X, const T* Y, long long ldk, int P0, int prow, i
                       const int* tasks, const int* counts, int max_slab, int npt, int nqt,
                       const long long* slab_k0, const int* slab_len, double* chi, cudaStream_t st) {
   dim3 grid(nqt, npt);
-  k_chi_tiles<T, AccT><<<grid, 256, 0, st>>>(X, Y, ldk, P0, prow, nri, tasks, counts, max_slab, nqt,
-                                             slab_k0, slab_len, chi);
+  if constexpr (sizeof(T) == 4)
+    k_chi_tiles_f32<<<dim3(nqt, npt, kF32Split), 128, 0, st>>>(X, Y, ldk, P0, prow, nri, tasks, counts, max_slab, nqt, slab_k0, slab_len,
+                                          chi);
+  else
+    k_chi_tiles<T, AccT><<<grid, 256, 0, st>>>(X, Y, ldk, P0, prow, nri, tasks, counts, max_slab, nqt,
+                                               slab_k0, slab_len, chi);
 }
 template void launch_chi_tiles<double, double>(const double*, const double*, long long, int, int, int,
                                                const int*, const int*, int, int, int,
