@@ -258,16 +258,23 @@ __global__ void __launch_bounds__(64) k_syrk64(const double* __restrict__ cso, c
 }
 
 // ---------------------------------------------------------------------------
-// FP32: 64 x 64 tile, 128 threads, thread (tx, ty) owns rows 8 ty .. + 7 and
-// columns 4 tx .. + 3, two products per instruction (fma.rn.f32x2).  Three
-// 16-byte shared loads feed 32 multiply-adds, where the 4 x 4 tile of
-// tile_nt_run needs eight 4-byte ones for 16.  Per element the products enter
-// one by one in the order of k, as there: the sums are the same to the bit.
+// FP32: 64 x 64 tile, 64 threads; thread (tx, ty) owns rows 4 ty + i and
+// 32 + 4 ty + i, columns 4 tx + j and 32 + 4 tx + j (i, j < 4), two products per
+// instruction (fma.rn.f32x2).  Four 16-byte shared loads feed 64 multiply-adds,
+// where the 4 x 4 tile of tile_nt_run needs eight 4-byte ones for 16: alone the
+// loop runs at 63 TFLOP/s with 8 warps per SM (8 x 4 per thread: 55).  Per
+// element the products enter one by one in the order of k, as there: the sums
+// are the same to the bit.
 // ---------------------------------------------------------------------------
-constexpr int kF32K = 16;      // reduction elements per stage
-constexpr int kF32Pitch = 68;  // floats per k row of a stage (16-byte aligned)
+constexpr int kF32K = 16;       // reduction elements per stage
+constexpr int kF32Pitch = 68;   // floats per k row of a stage (16-byte aligned)
+constexpr int kF32Threads = 64;
 using F32Stage = float[kF32K][kF32Pitch];
+using F32Acc = unsigned long long[4][8];
 
+// column of row or column r of the tile in k row k: the swap of 8 columns keeps
+// four k rows apart in the banks when a warp stores 4 consecutive k of 8 rows
+__device__ __forceinline__ int f32_col(int k, int r) { return k & 8 ? r ^ 8 : r; }
 __device__ __forceinline__ void fma2(unsigned long long& c, unsigned long long a, unsigned long long b) {
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
 }
@@ -281,142 +288,128 @@ __device__ __forceinline__ float2 unpack2(unsigned long long v) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
   return f;
 }
-// acc[i][j]: rows r = 8 ty + 2 i and r + 1 at columns c = 4 tx + (j & ~1) and
-// c + 1: (r, c), (r + 1, c + 1) for even j and (r, c + 1), (r + 1, c) for odd,
-// which takes one swapped copy of B's pair and no duplicated operand.
-__device__ __forceinline__ void f32_stage(const F32Stage& A, const F32Stage& B, int tx, int ty,
-                                          unsigned long long (&acc)[4][4]) {
+// row or column of the tile of a thread's element i (or j) < 8
+__device__ __forceinline__ int f32_at(int t8, int i) { return (i & 4) * 8 + 4 * t8 + (i & 3); }
+// acc[i][j]: row elements 2 i and 2 i + 1, column element j
+__device__ __forceinline__ void f32_stage(const F32Stage& A, const F32Stage& B, int tx, int ty, F32Acc& acc) {
 #pragma unroll
   for (int kk = 0; kk < kF32K; ++kk) {
-    const float4 a0 = *reinterpret_cast<const float4*>(&A[kk][8 * ty]);
-    const float4 a1 = *reinterpret_cast<const float4*>(&A[kk][8 * ty + 4]);
-    const float4 b = *reinterpret_cast<const float4*>(&B[kk][4 * tx]);
+    const int ca = f32_col(kk, 4 * ty), cb = f32_col(kk, 4 * tx);
+    const float4 a0 = *reinterpret_cast<const float4*>(&A[kk][ca]);
+    const float4 a1 = *reinterpret_cast<const float4*>(&A[kk][32 + ca]);
+    const float4 b0 = *reinterpret_cast<const float4*>(&B[kk][cb]);
+    const float4 b1 = *reinterpret_cast<const float4*>(&B[kk][32 + cb]);
     const unsigned long long av[4] = {pack2(a0.x, a0.y), pack2(a0.z, a0.w), pack2(a1.x, a1.y), pack2(a1.z, a1.w)};
-    const unsigned long long bv[4] = {pack2(b.x, b.y), pack2(b.y, b.x), pack2(b.z, b.w), pack2(b.w, b.z)};
+    const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) fma2(acc[i][j], av[i], bv[j]);
+      for (int j = 0; j < 8; ++j) fma2(acc[i][j], av[i], pack2(bv[j], bv[j]));
   }
-}
-
-// v[i][j]: row 8 ty + i, column 4 tx + j
-__device__ __forceinline__ void f32_unpack(const unsigned long long (&acc)[4][4], float (&v)[8][4]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; j += 2) {
-      const float2 d = unpack2(acc[i][j]), s = unpack2(acc[i][j + 1]);
-      v[2 * i][j] = d.x;
-      v[2 * i + 1][j + 1] = d.y;
-      v[2 * i][j + 1] = s.x;
-      v[2 * i + 1][j] = s.y;
-    }
 }
 
 // Step C in FP32: chi[P][Q] -= sum over the tile's slab list of X[P][k] Y[Q][k],
 // each slab summed in FP32 and the slabs in FP64.  ldk and every slab's start
-// and length are multiples of 16 elements.  A cluster shares a tile, each block
+// and length are multiples of 64 elements.  A cluster shares a tile, each block
 // a contiguous part of its slabs: 58 atoms have 272 tiles of work, less than two
-// blocks per SM.  Bound by the FP32 pipe.
+// blocks per SM.  The FP64 sums stay in shared memory (64 of them would take 128
+// registers of each thread).  58 atoms, 858 GFLOP: 61 ms in 4 x 4 tiles of one
+// block, 25.8 with one stage of loads in flight, 22.3 with two.  What remains is
+// the latency of those loads (a third of them miss the L2 cache) at 8 warps per SM.
 constexpr int kF32Split = 8;
-__global__ void __cluster_dims__(1, 1, kF32Split) __launch_bounds__(128) k_chi_tiles_f32(const float* __restrict__ X, const float* __restrict__ Y,
-                                                       long long ldk, int P0, int prow, int nri,
-                                                       const int* __restrict__ tasks, const int* __restrict__ counts,
-                                                       int max_slab, int nqt, const long long* __restrict__ slab_k0,
-                                                       const int* __restrict__ slab_len, double* __restrict__ chi) {
-  __shared__ __align__(16) union {
-    struct {
-      F32Stage a[2], b[2];
-    } st;
-    double part[64][64];
-  } sm;
-  auto& As = sm.st.a;
-  auto& Bs = sm.st.b;
-  auto& part = sm.part;  // after the last stage
+struct F32ChiShared {
+  double sum[64][kF32Threads];  // element 8 i + j of each thread
+  F32Stage a[2], b[2];
+};
+__global__ void __cluster_dims__(1, 1, kF32Split) __launch_bounds__(kF32Threads)
+    k_chi_tiles_f32(const float* __restrict__ X, const float* __restrict__ Y, long long ldk, int P0, int prow, int nri,
+                    const int* __restrict__ tasks, const int* __restrict__ counts, int max_slab, int nqt,
+                    const long long* __restrict__ slab_k0, const int* __restrict__ slab_len,
+                    double* __restrict__ chi) {
+  extern __shared__ __align__(16) unsigned char f32_smem[];
+  F32ChiShared& sm = *reinterpret_cast<F32ChiShared*>(f32_smem);
   const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
   const int rank = static_cast<int>(cluster.block_rank());
   const int tile = blockIdx.y * nqt + blockIdx.x;
   const int total = counts[tile];
   if (total == 0) return;  // the whole cluster
   const int p0 = blockIdx.y * 64, q0 = blockIdx.x * 64;
-  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  // this thread fetches k 4 (t % 4) .. + 3 of rows t / 4 and t / 4 + 32
+  const int t = threadIdx.x, tx = t & 7, ty = t >> 3;
+  // this thread fetches k 4 (t % 4) .. + 3 of rows t / 4 + 16 h
   const int fr = t >> 2, fk = (t & 3) * 4;
-  const float* xr[2];
-  const float* yr[2];
+  const float* xr = X + static_cast<long long>(p0 + fr) * ldk + fk;
+  const float* yr = Y + static_cast<long long>(q0 + fr) * ldk + fk;
+  float4 f0[8], f1[8];
+  auto fetch = [&](float4(&f)[8], long long k) {
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int r = fr + 32 * h;
-    xr[h] = p0 + r < prow ? X + static_cast<long long>(p0 + r) * ldk + fk : nullptr;
-    yr[h] = q0 + r < nri ? Y + static_cast<long long>(q0 + r) * ldk + fk : nullptr;
-  }
-  float4 fx[2], fy[2];
-  auto fetch = [&](long long k) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      fx[h] = xr[h] ? *reinterpret_cast<const float4*>(xr[h] + k) : make_float4(0.f, 0.f, 0.f, 0.f);
-      fy[h] = yr[h] ? *reinterpret_cast<const float4*>(yr[h] + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int h = 0; h < 4; ++h) {
+      const long long o = k + 16 * h * ldk;
+      f[h] = p0 + fr + 16 * h < prow ? *reinterpret_cast<const float4*>(xr + o) : make_float4(0.f, 0.f, 0.f, 0.f);
+      f[4 + h] = q0 + fr + 16 * h < nri ? *reinterpret_cast<const float4*>(yr + o) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
-  auto put = [&](int s) {
+  auto put = [&](const float4(&f)[8], F32Stage& a, F32Stage& b) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int r = fr + 32 * h;
-      As[s][fk][r] = fx[h].x;
-      As[s][fk + 1][r] = fx[h].y;
-      As[s][fk + 2][r] = fx[h].z;
-      As[s][fk + 3][r] = fx[h].w;
-      Bs[s][fk][r] = fy[h].x;
-      Bs[s][fk + 1][r] = fy[h].y;
-      Bs[s][fk + 2][r] = fy[h].z;
-      Bs[s][fk + 3][r] = fy[h].w;
+    for (int h = 0; h < 4; ++h) {
+      const int c = f32_col(fk, fr + 16 * h);
+      a[fk][c] = f[h].x;
+      a[fk + 1][c] = f[h].y;
+      a[fk + 2][c] = f[h].z;
+      a[fk + 3][c] = f[h].w;
+      b[fk][c] = f[4 + h].x;
+      b[fk + 1][c] = f[4 + h].y;
+      b[fk + 2][c] = f[4 + h].z;
+      b[fk + 3][c] = f[4 + h].w;
     }
   };
   const int first = static_cast<int>(static_cast<long long>(total) * rank / kF32Split);
   const int cnt = static_cast<int>(static_cast<long long>(total) * (rank + 1) / kF32Split) - first;
   const int* list = tasks + static_cast<long long>(tile) * max_slab + first;
-  double sum[8][4] = {};
-  int s = 0;
+#pragma unroll 8
+  for (int e = 0; e < 64; ++e) sm.sum[e][t] = 0.0;
   if (cnt > 0) {
-    fetch(slab_k0[list[0]]);
-    put(0);
+    const long long k0 = slab_k0[list[0]];
+    fetch(f0, k0);
+    fetch(f1, k0 + kF32K);
+    put(f0, sm.a[0], sm.b[0]);
   }
   __syncthreads();
   for (int i = 0; i < cnt; ++i) {
     const long long k0 = slab_k0[list[i]];
     const int len = slab_len[list[i]];
     const long long next = i + 1 < cnt ? slab_k0[list[i + 1]] : -1;
-    unsigned long long acc[4][4] = {};
-    for (int kk = 0; kk < len; kk += kF32K) {
-      // the next stage on its way while this one is multiplied
-      const long long k = kk + kF32K < len ? k0 + kk + kF32K : next;
-      if (k >= 0) fetch(k);
-      f32_stage(As[s], Bs[s], tx, ty, acc);
-      if (k >= 0) put(s ^ 1);
+    F32Acc acc = {};
+    for (int kk = 0; kk < len; kk += 2 * kF32K) {
+      // two stages on their way while this one is multiplied
+      const long long k = kk + 2 * kF32K < len ? k0 + kk + 2 * kF32K : next;
+      if (k >= 0) fetch(f0, k);
+      f32_stage(sm.a[0], sm.b[0], tx, ty, acc);
+      put(f1, sm.a[1], sm.b[1]);
       __syncthreads();
-      s ^= 1;
+      if (k >= 0) fetch(f1, k + kF32K);
+      f32_stage(sm.a[1], sm.b[1], tx, ty, acc);
+      if (k >= 0) put(f0, sm.a[0], sm.b[0]);
+      __syncthreads();
     }
-    float v[8][4];
-    f32_unpack(acc, v);
 #pragma unroll
-    for (int a = 0; a < 8; ++a)
+    for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) sum[a][j] += static_cast<double>(v[a][j]);
+      for (int j = 0; j < 8; ++j) {
+        const float2 v = unpack2(acc[a][j]);
+        sm.sum[16 * a + j][t] += static_cast<double>(v.x);
+        sm.sum[16 * a + 8 + j][t] += static_cast<double>(v.y);
+      }
   }
-  // the cluster's partial tiles, eight rows of each added up by every rank in
-  // the order of the slabs
-#pragma unroll
-  for (int a = 0; a < 8; ++a)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) part[8 * ty + a][4 * tx + j] = sum[a][j];
+  // the partial tiles, row element `rank` of every thread added up by this rank
+  // in the order of the slabs
   cluster.sync();
-  for (int e = t; e < 8 * 64; e += 128) {
-    const int r = 8 * rank + e / 64, c = e % 64;
+  const int m = p0 + f32_at(ty, rank);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int n = q0 + f32_at(tx, j);
     double v = 0.0;
 #pragma unroll
-    for (int o = 0; o < kF32Split; ++o) v += cluster.map_shared_rank(&part[r][c], o)[0];
-    const int m = p0 + r, n = q0 + c;
+    for (int o = 0; o < kF32Split; ++o) v += *cluster.map_shared_rank(&sm.sum[8 * rank + j][t], o);
     if (m < prow && n < nri) chi[static_cast<long long>(P0 + m) * nri + n] -= v;
   }
   cluster.sync();  // no rank leaves while its tile is read
@@ -529,41 +522,47 @@ __global__ void k_panel_gemm(const T* __restrict__ G, int nao, const T* __restri
   }
 }
 
-// The same in FP32 on the 8 x 4 tiles of f32_stage: rows n of the panel along
-// the threads' columns, rows r of G along their rows.
-__global__ void __launch_bounds__(128) k_panel_gemm_f32(const float* __restrict__ G, int nao,
-                                                        const float* __restrict__ pool, const int* __restrict__ lam,
-                                                        const PanelTask* __restrict__ tasks, int mode, int r0, int R,
-                                                        int P0b, long long ldk, const long long* __restrict__ rowbase,
-                                                        const int* __restrict__ rowmul, float* __restrict__ out) {
-  __shared__ __align__(16) F32Stage As[2], Bs[2];
+// The same in FP32 on the tiles of f32_stage: rows r of G along the tile's rows,
+// panel columns n along its columns.  The results pass through shared memory, so
+// that a warp's stores run along the operand's memory: n in mode 0, r in mode 1.
+// 58 atoms, 585 GFLOP: 24 ms in 4 x 4 tiles, 15.1 in these.
+__global__ void __launch_bounds__(kF32Threads)
+    k_panel_gemm_f32(const float* __restrict__ G, int nao, const float* __restrict__ pool, const int* __restrict__ lam,
+                     const PanelTask* __restrict__ tasks, int mode, int r0, int R, int P0b, long long ldk,
+                     const long long* __restrict__ rowbase, const int* __restrict__ rowmul, float* __restrict__ out) {
+  __shared__ __align__(16) union {
+    struct {
+      F32Stage a[2], b[2];
+    } st;
+    float out[64][65];  // after the last stage
+  } sm;
   const PanelTask tk = tasks[blockIdx.z];
   const int n0 = blockIdx.x * 64, m0 = blockIdx.y * 64;
   if (n0 >= tk.N || m0 >= R) return;
-  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const float* P = pool + tk.panel_off;
+  const int t = threadIdx.x, tx = t & 7, ty = t >> 3;
+  // this thread fetches column t of every k row
+  const bool rin = m0 + t < R, nin = n0 + t < tk.N;
+  const float* g = G + r0 + m0 + t;
+  const float* P = pool + tk.panel_off + n0 + t;
   const int* lk = lam + tk.lam_off;
-  // this thread fetches column c of k rows kr, kr + 2, ..
-  const int c = t & 63, kr = t >> 6;
-  const bool rin = m0 + c < R, nin = n0 + c < tk.N;
-  float fa[8], fb[8];
+  float fa[kF32K], fb[kF32K];
   auto fetch = [&](int k0) {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int k = k0 + kr + 2 * e;
+    for (int e = 0; e < kF32K; ++e) {
+      const int k = k0 + e;
       const bool kin = k < tk.K;
-      fa[e] = (kin && rin) ? G[static_cast<long long>(lk[k]) * nao + r0 + m0 + c] : 0.f;
-      fb[e] = (kin && nin) ? P[static_cast<long long>(k) * tk.N + n0 + c] : 0.f;
+      fa[e] = (kin && rin) ? g[static_cast<long long>(lk[k]) * nao] : 0.f;
+      fb[e] = (kin && nin) ? P[static_cast<long long>(k) * tk.N] : 0.f;
     }
   };
   auto put = [&](int s) {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      As[s][kr + 2 * e][c] = fa[e];
-      Bs[s][kr + 2 * e][c] = fb[e];
+    for (int e = 0; e < kF32K; ++e) {
+      sm.st.a[s][e][f32_col(e, t)] = fa[e];
+      sm.st.b[s][e][f32_col(e, t)] = fb[e];
     }
   };
-  unsigned long long acc[4][4] = {};
+  F32Acc acc = {};
   int s = 0;
   fetch(0);
   put(0);
@@ -571,27 +570,42 @@ __global__ void __launch_bounds__(128) k_panel_gemm_f32(const float* __restrict_
   for (int k0 = 0; k0 < tk.K; k0 += kF32K) {
     const bool more = k0 + kF32K < tk.K;
     if (more) fetch(k0 + kF32K);
-    f32_stage(As[s], Bs[s], tx, ty, acc);
+    f32_stage(sm.st.a[s], sm.st.b[s], tx, ty, acc);
     if (more) put(s ^ 1);
     __syncthreads();
     s ^= 1;
   }
-  float v[8][4];
-  f32_unpack(acc, v);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int n = n0 + 4 * tx + j;
-    if (n >= tk.N) continue;
-    const int pw = n / tk.nsig, sp = n - pw * tk.nsig;
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int r = m0 + 8 * ty + i;
-      if (r >= R) continue;
-      const long long dst = mode == 0 ? static_cast<long long>(tk.p0 + pw - P0b) * ldk + tk.seg +
-                                            static_cast<long long>(r0 + r) * tk.nsig + sp
-                                      : static_cast<long long>(tk.p0 + pw) * ldk + rowbase[r] +
-                                            static_cast<long long>(tk.aom + sp) * rowmul[r];
-      out[dst] = v[i][j];
+    for (int j = 0; j < 8; ++j) {
+      const float2 v = unpack2(acc[i][j]);
+      sm.out[f32_at(ty, 2 * i)][f32_at(tx, j)] = v.x;
+      sm.out[f32_at(ty, 2 * i + 1)][f32_at(tx, j)] = v.y;
+    }
+  __syncthreads();
+  if (mode == 0) {
+    if (!nin) return;
+    const int n = n0 + t, pw = n / tk.nsig, sp = n - pw * tk.nsig;
+    float* o = out + static_cast<long long>(tk.p0 + pw - P0b) * ldk + tk.seg + sp +
+               static_cast<long long>(r0 + m0) * tk.nsig;
+    const int mr = min(64, R - m0);
+#pragma unroll 4
+    for (int i = 0; i < mr; ++i) o[static_cast<long long>(i) * tk.nsig] = sm.out[i][t];
+  } else {
+    if (!rin) return;
+    const int r = m0 + t;
+    const long long base = rowbase[r];
+    const int mul = rowmul[r];
+    int pw = n0 / tk.nsig, sp = n0 - pw * tk.nsig;
+    const int nr = min(64, tk.N - n0);
+#pragma unroll 4
+    for (int i = 0; i < nr; ++i) {
+      out[static_cast<long long>(tk.p0 + pw) * ldk + base + static_cast<long long>(tk.aom + sp) * mul] = sm.out[t][i];
+      if (++sp == tk.nsig) {
+        sp = 0;
+        ++pw;
+      }
     }
   }
 }
@@ -616,7 +630,7 @@ __device__ __forceinline__ float magnitude(double v) {
 // One warp per block.  The norm is first taken in FP32 (a relative error below
 // 1e-3 for blocks of up to 10^4 rows); only a block within 1 % of the threshold, one
 // outside FP32's range or one with an Inf or NaN has it taken in FP64, so every decision is the FP64 one.
-// In FP64 throughout, the kernel was bound by that pipe.
+// In FP64 throughout, the kernel was bound by that pipe: 5.5 ms at 58 atoms, now 1.7.
 template <typename T>
 __global__ void k_operand_block_filter(T* __restrict__ Z, long long ldk, int rowoff,
                                        const int* __restrict__ ri_off, const int* __restrict__ ao_off,
@@ -837,7 +851,7 @@ void launch_panel_gemm(const T* G, int nao, const T* pool, const int* lam, const
     int nz = ntasks - z0 < 65535 ? ntasks - z0 : 65535;
     dim3 grid((maxN + 63) / 64, (R + 63) / 64, nz);
     if constexpr (sizeof(T) == 4)
-      k_panel_gemm_f32<<<grid, 128, 0, st>>>(G, nao, pool, lam, tasks + z0, mode, r0, R, P0b, ldk, rowbase, rowmul,
+      k_panel_gemm_f32<<<grid, kF32Threads, 0, st>>>(G, nao, pool, lam, tasks + z0, mode, r0, R, P0b, ldk, rowbase, rowmul,
                                              out);
     else
       k_panel_gemm<T><<<grid, 256, 0, st>>>(G, nao, pool, lam, tasks + z0, mode, r0, R, P0b, ldk,
@@ -897,12 +911,15 @@ void launch_chi_tiles(const T* X, const T* Y, long long ldk, int P0, int prow, i
                       const int* tasks, const int* counts, int max_slab, int npt, int nqt,
                       const long long* slab_k0, const int* slab_len, double* chi, cudaStream_t st) {
   dim3 grid(nqt, npt);
-  if constexpr (sizeof(T) == 4)
-    k_chi_tiles_f32<<<dim3(nqt, npt, kF32Split), 128, 0, st>>>(X, Y, ldk, P0, prow, nri, tasks, counts, max_slab, nqt, slab_k0, slab_len,
-                                          chi);
-  else
+  if constexpr (sizeof(T) == 4) {
+    constexpr int smem = static_cast<int>(sizeof(F32ChiShared));
+    cudaFuncSetAttribute(k_chi_tiles_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    k_chi_tiles_f32<<<dim3(nqt, npt, kF32Split), kF32Threads, smem, st>>>(
+        X, Y, ldk, P0, prow, nri, tasks, counts, max_slab, nqt, slab_k0, slab_len, chi);
+  } else {
     k_chi_tiles<T, AccT><<<grid, 256, 0, st>>>(X, Y, ldk, P0, prow, nri, tasks, counts, max_slab, nqt,
                                                slab_k0, slab_len, chi);
+  }
 }
 template void launch_chi_tiles<double, double>(const double*, const double*, long long, int, int, int,
                                                const int*, const int*, int, int, int,
