@@ -97,6 +97,15 @@ __device__ __forceinline__ uint16_t take_slice(double& v, bool f16) {
   v -= static_cast<double>(__bfloat162float(h));
   return __bfloat16_as_ushort(h);
 }
+// float -> double by integer operations, exact.  The conversion instruction runs
+// on the FP64 pipe: 64 cycles of an SM quarter per warp, 8 thousand for the
+// 128 x 128 sums of a tile.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
+  if (m - 1u < 0x007fffffu || m >= 0x7f800000u) return static_cast<double>(f);  // subnormal, Inf, NaN
+  const unsigned hi = m ? (m >> 3) + 0x38000000u : 0u;
+  return __hiloint2double(static_cast<int>(hi | (u & 0x80000000u)), static_cast<int>(u << 29));
+}
 // acc[j] += TMEM[lane row][taddr column + j], j < 32: one 32-column load and
 // its wait, or (kHalves = 2) two 16-column loads and waits, which keeps 16
 // fewer registers live.  The registers pass through the wait's asm so that
@@ -272,30 +281,15 @@ struct ChiJob {
       // Y row ql; rows past the Y operand read as zeros (TMA fill), so
       // every ql < qlim may be written
       const int q = T.yb + c0 + cc + col;
-      if (unit_first) {
-        // units of one tile may run concurrently when K is split
+      // Added by the L2 cache: units of one tile may run concurrently when K is
+      // split, and an FP64 add here would take the FP64 pipe once more.  45-atom
+      // ribbon: the pipe was busy for 35 % of the kernel, and the MMAs waited.
 #pragma unroll
-        for (int i = 0; i < 32; i += kRowsPer) {
-          const int p = T.ya + quad * 32 + i + sub;
-          if (p < prow && q < qlim)
-            atomicAdd(chi + static_cast<long long>(P0 + p) * nri + q,
-                      -static_cast<double>(f[(i + sub) * kStgPitch + col] * out_scale));
-        }
-      } else {
-        // one owner per tile: all loads in flight, then the stores
-        double old[32 / kRowsPer];
-#pragma unroll
-        for (int i = 0; i < 32 / kRowsPer; ++i) {
-          const int p = T.ya + quad * 32 + kRowsPer * i + sub;
-          old[i] = (p < prow && q < qlim) ? chi[static_cast<long long>(P0 + p) * nri + q] : 0.0;
-        }
-#pragma unroll
-        for (int i = 0; i < 32 / kRowsPer; ++i) {
-          const int p = T.ya + quad * 32 + kRowsPer * i + sub;
-          if (p < prow && q < qlim)
-            chi[static_cast<long long>(P0 + p) * nri + q] =
-                old[i] - static_cast<double>(f[(kRowsPer * i + sub) * kStgPitch + col] * out_scale);
-        }
+      for (int i = 0; i < 32; i += kRowsPer) {
+        const int p = T.ya + quad * 32 + i + sub;
+        if (p < prow && q < qlim)
+          atomicAdd(chi + static_cast<long long>(P0 + p) * nri + q,
+                    widen(-(f[(i + sub) * kStgPitch + col] * out_scale)));
       }
       __syncwarp();
     }
@@ -358,7 +352,7 @@ struct GroupJob {
         const int r = quad * 32 + kRowsPer * i + sub;
         if (r < g.rows && c < g.cols) {
           double* o = out + g.out_off + static_cast<long long>(r) * g.ld + c;
-          *o -= static_cast<double>(f[(kRowsPer * i + sub) * kStgPitch + col] * g.scale);
+          atomicAdd(o, widen(-(f[(kRowsPer * i + sub) * kStgPitch + col] * g.scale)));
         }
       }
       __syncwarp();
