@@ -1365,6 +1365,50 @@ int ensure_ycover(gw_ctx* ctx) {
 
 int tc_results(gw_ctx* ctx, int** err, unsigned long long** stat, double** fc);
 
+// Layout of the step-C operands of a batch in memory: segments of whole
+// sigma-atoms, [segment][row][seg_len], so that a column of TMA boxes (one row
+// of memory pages per few operand rows) touches few pages.  With 118 atoms one
+// row of the plain layout is 3 MB and every row of a box lies in a page of its
+// own: the address translation held step C at 54.8 ms per tau point; rows of
+// 0.8 MB take 31 ms, rows of 0.3 MB no less.
+constexpr long long kSegmentK = 1 << 18;
+struct OperandSegments {
+  int nseg = 1;
+  long long seg_len = 0;         // row pitch, a multiple of 64 elements
+  std::vector<int> seg;          // per sigma-atom of the batch
+  std::vector<long long> off;    // offset in the segment's row
+  std::vector<long long> k0;     // reduction index: seg * seg_len + off
+  long long len() const { return nseg * seg_len; }
+  // memory offsets of the sigma-atoms in an operand of `rows` rows
+  std::vector<long long> offsets(long long rows) const {
+    std::vector<long long> o(seg.size());
+    for (size_t i = 0; i < o.size(); ++i) o[i] = seg[i] * rows * seg_len + off[i];
+    return o;
+  }
+};
+// Segments of about `most` elements (one when the batch has no more, or when
+// the padding to equal lengths would exceed a quarter).
+OperandSegments plan_segments(const Batch& b, long long most) {
+  OperandSegments g;
+  const int ns = b.s1 - b.s0;
+  const long long want = std::max<long long>((b.Kb + most - 1) / most, 1), target = (b.Kb + want - 1) / want;
+  g.nseg = (int)want;
+  g.seg.resize(ns);
+  g.off.resize(ns);
+  g.k0.resize(ns);
+  long long first = 0;
+  for (int i = 0; i < ns; ++i) {
+    const long long len = (i + 1 < ns ? b.seg[i + 1] : b.Kb) - b.seg[i];
+    g.seg[i] = (int)std::min(want - 1, (b.seg[i] + len / 2) / target);
+    if (i > 0 && g.seg[i] != g.seg[i - 1]) first = b.seg[i];
+    g.off[i] = b.seg[i] - first;
+    g.seg_len = std::max(g.seg_len, g.off[i] + len);
+  }
+  if (want > 1 && (g.len() > b.Kb + b.Kb / 4 || g.len() > INT32_MAX)) return plan_segments(b, b.Kb);
+  for (int i = 0; i < ns; ++i) g.k0[i] = g.seg[i] * g.seg_len + g.off[i];
+  return g;
+}
+
 // One batch on the tensor cores: steps A and B straight into bf16 slices,
 // block filter from the accumulated norms, task lists, step C.  gs_occ,
 // gs_virt: slices of G^occ and G^virt, [slices][n_AO][n_AO rounded to 64].
@@ -1390,22 +1434,33 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
   if (prow == 0 || qrow == 0 || Kb == 0) return GW_OK;
   const int kmax = ctx->pt_kmax, gkp = (ctx->nao + 63) / 64 * 64;
   void *xs, *ys;
-  if ((rc = ws(ctx, "Xs", (size_t)slices * prow * Kb * 2, &xs))) return rc;
-  if ((rc = ws(ctx, "Ys", (size_t)slices * qrow * Kb * 2, &ys))) return rc;
-  GW_TRY(cudaMemsetAsync(xs, 0, (size_t)slices * prow * Kb * 2, ctx->stream));
+  OperandSegments g = plan_segments(b, ctx->mlp_mode ? Kb : kSegmentK);
+  if (g.nseg > 1 && (ws(ctx, "Xs", (size_t)slices * prow * g.len() * 2, &xs) ||
+                     ws(ctx, "Ys", (size_t)slices * qrow * g.len() * 2, &ys))) {
+    // no room for the segments' padding
+    gw::work_trim(ctx, "Xs", 0);
+    gw::work_trim(ctx, "Ys", 0);
+    ctx->err.clear();
+    g = plan_segments(b, Kb);
+  }
+  const long long ldk = g.seg_len, Kp = g.len();  // row pitch, elements per row of the padded operands
+  if ((rc = ws(ctx, "Xs", (size_t)slices * prow * Kp * 2, &xs))) return rc;
+  if ((rc = ws(ctx, "Ys", (size_t)slices * qrow * Kp * 2, &ys))) return rc;
+  const std::vector<long long> seg_x = g.offsets(prow), seg_y = g.offsets(qrow);
+  GW_TRY(cudaMemsetAsync(xs, 0, (size_t)slices * prow * Kp * 2, ctx->stream));
   if ((rc = ensure_ycover(ctx))) return rc;
   if (ctx->ycov_ok) {
     // step B writes every (q, s, mu of a covering owner, sigma); zero the rest
     long long* d_seg0;
     int* d_nao0;
-    if ((rc = upload(ctx, "seg_y", b.seg, &d_seg0))) return rc;
+    if ((rc = upload(ctx, "seg_y", seg_y, &d_seg0))) return rc;
     if ((rc = upload(ctx, "n_ao_y", ctx->n_ao, &d_nao0))) return rc;
-    gw::launch_zero_unwritten_y(ys, slices, (long long)qrow * Kb, Kb, b.Q0, qrow, ns, d_seg0, d_nao0,
+    gw::launch_zero_unwritten_y(ys, slices, (long long)qrow * Kp, ldk, b.Q0, qrow, ns, d_seg0, d_nao0,
                                 b.s0, ctx->d_ao_off, b.m0, b.m1, b.Lc, ctx->d_ycov_lo,
                                 ctx->d_ycov_hi, ctx->stream);
     GW_CHECK_LAUNCH();
   } else {
-    GW_TRY(cudaMemsetAsync(ys, 0, (size_t)slices * qrow * Kb * 2, ctx->stream));
+    GW_TRY(cudaMemsetAsync(ys, 0, (size_t)slices * qrow * Kp * 2, ctx->stream));
   }
   const int pa0 = [&] {
     int a = 0;
@@ -1498,7 +1553,7 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
       }
       if (ctx->pt_stream) t.p_row0 = row0A[s];
       t.g_row0 = (int)ta.size() * rows_a;
-      t.seg = b.seg[s - b.s0];
+      t.seg = seg_x[s - b.s0];
       t.s_local = s - b.s0;
       if (staged) {
         // panel rows from pw boundaries: (tile / nsig) whole runs per tile
@@ -1541,13 +1596,13 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
         return fail(ctx, GW_ERR_CUDA, "cuTensorMapEncodeTiled failed for G (step A)");
       const int lrc =
           staged ? gw::launch_panel_tc_staged(f16, (float)(1.0 / (s_go * s_t)), (float)s_x, mg, mpA, d_tiles,
-                                              (int)tiles.size(), d_ta, 0, xs, (long long)prow * Kb, Kb,
+                                              (int)tiles.size(), d_ta, 0, xs, (long long)prow * Kp, ldk,
                                               b.P0, b.Lc, 0, b.s0, nullptr, bx2, ctx->d_atom_of_ri,
                                               ctx->d_atom_of_ao, ctx->d_ao_off, ctx->d_ri_off, d_nao_a,
                                               npa, pa0, b.mu0, b.m0, nmc, ctx->flush_k, d_err, ctx->stream)
                  : gw::launch_panel_tc(slices, f16, (float)(1.0 / (s_go * s_t)), (float)s_x, mg, mpA, d_tiles,
                                        (int)tiles.size(), d_ta, 0, b.nmu, xs,
-                                       (long long)prow * Kb, Kb, b.P0, nullptr, nullptr, nullptr, bx2,
+                                       (long long)prow * Kp, ldk, b.P0, nullptr, nullptr, nullptr, bx2,
                                        ctx->d_atom_of_ri, ctx->d_atom_of_ao, ctx->d_ao_off, n_at, npa,
                                        pa0, b.mu0, b.m0, nmc, ctx->flush_k, d_err, ctx->stream);
       if (lrc) return fail(ctx, GW_ERR_CUDA, "tensor-core step A launch setup failed");
@@ -1632,7 +1687,7 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
     std::vector<int> rowmul(R), rowsl(R);
     for (int s = b.s0; s < b.s1; ++s)
       for (int i = 0; i < ctx->n_ao[s]; ++i) {
-        rowbase[ctx->ao_off[s] - r0 + i] = b.seg[s - b.s0] + i;
+        rowbase[ctx->ao_off[s] - r0 + i] = seg_y[s - b.s0] + i;
         rowmul[ctx->ao_off[s] - r0 + i] = ctx->n_ao[s];
         rowsl[ctx->ao_off[s] - r0 + i] = s - b.s0;
       }
@@ -1657,13 +1712,13 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
         return fail(ctx, GW_ERR_CUDA, "cuTensorMapEncodeTiled failed for G (step B)");
       const int lrc =
           staged_b ? gw::launch_panel_tc_staged(f16, (float)(1.0 / (s_gv * s_t)), (float)s_y, mg, mpB, d_tiles,
-                                              (int)tiles.size(), d_tb, 1, ys, (long long)qrow * Kb, Kb,
+                                              (int)tiles.size(), d_tb, 1, ys, (long long)qrow * Kp, ldk,
                                               b.Q0, b.Lc, r0, b.s0, d_rowbase, by2, ctx->d_atom_of_ri,
                                               ctx->d_atom_of_ao, ctx->d_ao_off, ctx->d_ri_off, d_nao_a,
                                               nqa, qa0, b.mu0, b.m0, nmc, ctx->flush_k, d_err, ctx->stream)
                  : gw::launch_panel_tc(slices, f16, (float)(1.0 / (s_gv * s_t)), (float)s_y, mg, mpB, d_tiles,
                                        (int)tiles.size(), d_tb, 1, R, ys,
-                                       (long long)qrow * Kb, Kb, b.Q0, d_rowbase, d_rowmul, d_rowsl, by2,
+                                       (long long)qrow * Kp, ldk, b.Q0, d_rowbase, d_rowmul, d_rowsl, by2,
                                        ctx->d_atom_of_ri, ctx->d_atom_of_ao, ctx->d_ao_off, n_at, nqa,
                                        qa0, b.mu0, b.m0, nmc, ctx->flush_k, d_err, ctx->stream);
       if (lrc) return fail(ctx, GW_ERR_CUDA, "tensor-core step B launch setup failed");
@@ -1673,8 +1728,8 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
         gw::DeadY* d_dead;
         long long* d_segb;
         if ((rc = upload(ctx, "dead_y", dead, &d_dead))) return rc;
-        if ((rc = upload(ctx, "seg_b", b.seg, &d_segb))) return rc;
-        gw::launch_zero_dead_y(ys, slices, (long long)qrow * Kb, Kb, qrow, d_dead, (int)dead.size(), d_segb,
+        if ((rc = upload(ctx, "seg_y", seg_y, &d_segb))) return rc;
+        gw::launch_zero_dead_y(ys, slices, (long long)qrow * Kp, ldk, qrow, d_dead, (int)dead.size(), d_segb,
                                d_nao_a, b.s0, ctx->stream);
         GW_CHECK_LAUNCH();
         ctx->stats.kernel_launches += 1;
@@ -1694,19 +1749,19 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
   if ((rc = wsT(ctx, "fy", (size_t)ns * nmc * nqt, &fy))) return rc;
   GW_TRY(cudaMemsetAsync(fx, 0, (size_t)ns * nmc * npt, ctx->stream));
   GW_TRY(cudaMemsetAsync(fy, 0, (size_t)ns * nmc * nqt, ctx->stream));
-  long long* d_seg;
+  long long *d_segx, *d_segy;
   int* d_nao;
-  if ((rc = upload(ctx, "seg", b.seg, &d_seg))) return rc;
+  if ((rc = upload(ctx, "seg_x", seg_x, &d_segx)) || (rc = upload(ctx, "seg_y", seg_y, &d_segy))) return rc;
   if ((rc = upload(ctx, "n_ao_b", ctx->n_ao, &d_nao))) return rc;
   // queue of filtered blocks to zero (shared by the two stream-ordered calls)
   int *zlist, *zcount;
   if ((rc = wsT(ctx, "zlist", (size_t)ns * nmc * std::max(npa, nqa), &zlist))) return rc;
   if ((rc = wsT(ctx, "zcount", 1, &zcount))) return rc;
-  gw::launch_slices_block_filter(xs, slices, (long long)prow * Kb, Kb, b.P0, ctx->d_ri_off,
-                                 ctx->d_ao_off, d_nao, b.s0, ns, d_seg, pa0, npa, b.m0, nmc, b.mu0, thr,
+  gw::launch_slices_block_filter(xs, slices, (long long)prow * Kp, ldk, b.P0, ctx->d_ri_off,
+                                 ctx->d_ao_off, d_nao, b.s0, ns, d_segx, pa0, npa, b.m0, nmc, b.mu0, thr,
                                  bx2, bx, fx, npt, tile, zlist, zcount, ctx->stream);
-  gw::launch_slices_block_filter(ys, slices, (long long)qrow * Kb, Kb, b.Q0, ctx->d_ri_off,
-                                 ctx->d_ao_off, d_nao, b.s0, ns, d_seg, qa0, nqa, b.m0, nmc, b.mu0, thr,
+  gw::launch_slices_block_filter(ys, slices, (long long)qrow * Kp, ldk, b.Q0, ctx->d_ri_off,
+                                 ctx->d_ao_off, d_nao, b.s0, ns, d_segy, qa0, nqa, b.m0, nmc, b.mu0, thr,
                                  by2, by, fy, nqt, tile, zlist, zcount, ctx->stream);
   GW_CHECK_LAUNCH();
   std::vector<long long> slab_k0(nslab);
@@ -1715,7 +1770,7 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
   for (int sl = 0; sl < ns; ++sl)
     for (int c = 0; c < per; ++c) {
       const int nsig = ctx->n_ao[b.s0 + sl];
-      slab_k0[sl * per + c] = b.seg[sl] + (long long)c * kSlabAO * nsig;
+      slab_k0[sl * per + c] = g.k0[sl] + (long long)c * kSlabAO * nsig;
       slab_len[sl * per + c] = kSlabAO * nsig;
     }
   long long* d_k0;
@@ -1787,8 +1842,8 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
     ctx->stats.kernel_launches += 4;
   }
   CUtensorMap mx, my;
-  if (gw::make_slice_map(&mx, xs, Kb, prow, slices, tile, f16) ||
-      gw::make_slice_map(&my, ys, Kb, qrow, slices, tile, f16))
+  if (gw::make_slice_map(&mx, xs, ldk, prow, slices * g.nseg, tile, f16) ||
+      gw::make_slice_map(&my, ys, ldk, qrow, slices * g.nseg, tile, f16))
     return fail(ctx, GW_ERR_CUDA, "cuTensorMapEncodeTiled failed for the step-C operands");
   cudaEvent_t ec0, ec1;
   if ((rc = c_event_pair(ctx, 2 * batch_idx, &ec0, &ec1))) return rc;
@@ -1822,7 +1877,7 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
     if (gw::launch_chi_tc_units(slices, f16, (float)(1.0 / (s_x * s_y)), mx, my, w.u_tile, w.u_first,
                                 w.u_count, (int)std::min<size_t>(cap, INT32_MAX), w.n_units, tasks,
                                 counts, nslab, d_k0, d_len, b.P0, prow, nri, b.Q0, qrow, nqt, acc,
-                                ctx->flush_k, ctx->c_dynamic ? d_work : nullptr, d_err, ctx->stream))
+                                (int)ldk, g.nseg, ctx->flush_k, ctx->c_dynamic ? d_work : nullptr, d_err, ctx->stream))
       return fail(ctx, GW_ERR_CUDA, "tensor-core step C launch setup failed");
     GW_CHECK_LAUNCH();
     GW_TRY(cudaEventRecord(ec1, ctx->stream));
@@ -1918,8 +1973,8 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
     GW_TRY(cudaEventRecord(ec0, ctx->stream));
     if (gw::launch_chi_tc_units(slices, f16, (float)(1.0 / (s_x * s_y)), mx, my, d_ut, d_uf, d_uc,
                                 (int)u_tile.size(), nullptr, tasks, counts,
-                                nslab, d_k0, d_len, b.P0, prow, nri, b.Q0, qrow, nqt, acc, ctx->flush_k,
-                                ctx->c_dynamic ? d_work : nullptr, d_err, ctx->stream))
+                                nslab, d_k0, d_len, b.P0, prow, nri, b.Q0, qrow, nqt, acc, (int)ldk, g.nseg,
+                                ctx->flush_k, ctx->c_dynamic ? d_work : nullptr, d_err, ctx->stream))
       return fail(ctx, GW_ERR_CUDA, "tensor-core step C launch setup failed");
   } else {
     int* d_active;
@@ -1927,7 +1982,7 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
     GW_TRY(cudaEventRecord(ec0, ctx->stream));
     if (gw::launch_chi_tc(slices, f16, (float)(1.0 / (s_x * s_y)), mx, my, d_active,
                           (int)active.size(), tasks, counts, nslab, d_k0,
-                          d_len, b.P0, prow, nri, b.Q0, qrow, nqt, acc, ctx->flush_k, d_err,
+                          d_len, b.P0, prow, nri, b.Q0, qrow, nqt, acc, (int)ldk, g.nseg, ctx->flush_k, d_err,
                           ctx->stream))
       return fail(ctx, GW_ERR_CUDA, "tensor-core step C launch setup failed");
   }

@@ -207,8 +207,10 @@ struct ChiJob {
   float out_scale;  // 1 / (scale of the A operand x scale of the B operand)
   const int* n_dev; // optional: number of units in device memory (n_tiles = capacity)
   int* work;        // optional: counter handing the units out in order (zeroed before the launch)
+  int seg_len, nseg; // operands: nseg segments of seg_len reduction elements, each over all rows
   static constexpr bool kPeriodic = true;
   static constexpr bool kTileStaging = false;
+  static constexpr bool kSegmented = true;
   static constexpr bool kDynamic = true;
   static constexpr int kDrainHalves = 2;  // 96 registers: one 32-column load would spill
 
@@ -305,6 +307,7 @@ struct GroupJob {
   int n_tiles;
   double* out;
   static constexpr bool kPeriodic = true;
+  static constexpr bool kSegmented = false;
   static constexpr bool kTileStaging = false;
   static constexpr bool kDynamic = false;
   static constexpr int kDrainHalves = 2;
@@ -406,6 +409,7 @@ struct PanelJob {
   float unscale;              // 1 / (scale of Gg x scale of PT): true Z = acc * unscale
   float out_scale;            // scale of the Z slices
   static constexpr bool kPeriodic = false;
+  static constexpr bool kSegmented = false;
   static constexpr bool kTileStaging = false;
   static constexpr bool kDynamic = false;
   static constexpr int kDrainHalves = 1;
@@ -592,6 +596,7 @@ struct PanelStagedJob {
   int f16;
   float unscale, out_scale;
   static constexpr bool kPeriodic = false;
+  static constexpr bool kSegmented = false;
   static constexpr bool kTileStaging = true;
   static constexpr bool kDynamic = false;
   static constexpr int kDrainHalves = 1;
@@ -1063,10 +1068,15 @@ __global__ void __launch_bounds__(kThreads, 1)
           mbar_expect_tx(&full[stage], L::kStageBytes);
           armed[stage] = true;
           armed_parity[stage] = phase;
-          const int x = it.next();
+          int x = it.next(), z = 0, dz = 1;  // slice s at z + s dz
+          if constexpr (Job::kSegmented) {
+            z = x / job.seg_len;
+            x -= z * job.seg_len;
+            dz = job.nseg;
+          }
           for (int s = 0; s < S; ++s) {
-            tma_load_3d(st + s * L::kTileBytes, &map_a, x, T.ya, s, &full[stage]);
-            tma_load_3d(st + (S + s) * L::kTileBytes, &map_b, x, T.yb, s, &full[stage]);
+            tma_load_3d(st + s * L::kTileBytes, &map_a, x, T.ya, z + s * dz, &full[stage]);
+            tma_load_3d(st + (S + s) * L::kTileBytes, &map_b, x, T.yb, z + s * dz, &full[stage]);
           }
           if (++stage == kStages) {
             stage = 0;
@@ -1870,10 +1880,11 @@ void tc_set_stall_test(int on) { g_stall_test = on; }
 int launch_chi_tc(int slices, int f16, float out_scale, const CUtensorMap& mx, const CUtensorMap& my,
                   const int* tile_list, int n_tiles, const int* tasks, const int* counts, int max_slab,
                   const long long* slab_k0, const int* slab_len, int P0, int prow, int nri, int Q0,
-                  int qrow, int nqt, double* chi, int flush_k, int* err_flag, cudaStream_t st) {
+                  int qrow, int nqt, double* chi, int seg_len, int nseg, int flush_k, int* err_flag,
+                  cudaStream_t st) {
   (void)qrow;
   tc::ChiJob job{tile_list, n_tiles, nullptr, nullptr, tasks, counts, max_slab, slab_k0, slab_len, nqt,
-                 P0, prow, nri, nri - Q0, chi + Q0, out_scale, nullptr, nullptr};
+                 P0, prow, nri, nri - Q0, chi + Q0, out_scale, nullptr, nullptr, seg_len, nseg};
   return launch_persistent(slices, f16, mx, my, job, flush_k, err_flag, st);
 }
 
@@ -1881,11 +1892,11 @@ int launch_chi_tc_units(int slices, int f16, float out_scale, const CUtensorMap&
                         const CUtensorMap& my, const int* unit_tile, const int* unit_first,
                         const int* unit_count, int n_units, const int* n_units_dev, const int* tasks,
                         const int* counts, int max_slab, const long long* slab_k0, const int* slab_len,
-                        int P0, int prow, int nri, int Q0, int qrow, int nqt, double* chi, int flush_k,
-                        int* work, int* err_flag, cudaStream_t st) {
+                        int P0, int prow, int nri, int Q0, int qrow, int nqt, double* chi, int seg_len,
+                        int nseg, int flush_k, int* work, int* err_flag, cudaStream_t st) {
   (void)qrow;
   tc::ChiJob job{unit_tile, n_units, unit_first, unit_count, tasks, counts, max_slab, slab_k0, slab_len,
-                 nqt, P0, prow, nri, nri - Q0, chi + Q0, out_scale, n_units_dev, work};
+                 nqt, P0, prow, nri, nri - Q0, chi + Q0, out_scale, n_units_dev, work, seg_len, nseg};
   if (work && cudaMemsetAsync(work, 0, sizeof(int), st) != cudaSuccess) return -6;
   return launch_persistent(slices, f16, mx, my, job, flush_k, err_flag, st);
 }

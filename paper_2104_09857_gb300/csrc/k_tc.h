@@ -45,7 +45,11 @@ void launch_absmax_rowsum(const double* a, long long ld, int rows, int cols, dou
 int launch_chi_tc(int slices, int f16, float out_scale, const CUtensorMap& mx, const CUtensorMap& my,
                   const int* tile_list, int n_tiles, const int* tasks, const int* counts, int max_slab,
                   const long long* slab_k0, const int* slab_len, int P0, int prow, int nri, int Q0,
-                  int qrow, int nqt, double* chi, int flush_k, int* err_flag, cudaStream_t st);
+                  int qrow, int nqt, double* chi, int seg_len, int nseg, int flush_k, int* err_flag,
+                  cudaStream_t st);
+// mx, my: operands of nseg segments of seg_len reduction elements, dimension 2 of
+// the maps being slice * nseg + segment; slab_k0 counts segment * seg_len +
+// offset (plain operands: nseg = 1, seg_len no less than their length).
 // Step C over work units that split tiles along K: unit u computes tile
 // unit_tile[u] over list entries [unit_first[u], unit_first[u] + unit_count[u])
 // of that tile's task list and adds into chi with FP64 atomics.  The number
@@ -57,8 +61,8 @@ int launch_chi_tc_units(int slices, int f16, float out_scale, const CUtensorMap&
                         const CUtensorMap& my, const int* unit_tile, const int* unit_first,
                         const int* unit_count, int n_units, const int* n_units_dev, const int* tasks,
                         const int* counts, int max_slab, const long long* slab_k0, const int* slab_len,
-                        int P0, int prow, int nri, int Q0, int qrow, int nqt, double* chi, int flush_k,
-                        int* work, int* err_flag, cudaStream_t st);
+                        int P0, int prow, int nri, int Q0, int qrow, int nqt, double* chi, int seg_len,
+                        int nseg, int flush_k, int* work, int* err_flag, cudaStream_t st);
 // Device scratch of launch_plan_units: per tile (ntiles) ucnt, uoff; per unit
 // (capacity ntiles * nslab) t_tile, t_first, t_count, t_key, u_tile, u_first,
 // u_count; per slab (nslab) hist, start; and the counters n_units,

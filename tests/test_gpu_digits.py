@@ -94,6 +94,23 @@ def test_chi_at_the_tile_edges(pkg, last, ri):
                 assert np.linalg.norm(got[j] - ref[j]) <= tol * np.linalg.norm(ref[j]), (form, j)
 
 
+@pytest.mark.parametrize("last", [1, 14])
+def test_chi_operands_in_segments(pkg, last):
+    """519 and 532 primary functions: a batch's reduction length (299 and 306
+    thousand) passes one operand segment of the tensor-core forms."""
+    sysm = System("long", np.array([[1.4 * i, 0.0, 0.0] for i in range(38)]), ["C"] * 38)
+    sysm.n_ao = np.array([14] * 37 + [last], dtype=np.int32)
+    sysm.n_ri = np.array([1] * 37 + [3], dtype=np.int32)
+    case = case_from_system(sysm, 1, 1e-9, 7)
+    case.tau = np.array([0.5])
+    ref = oc.chi_dense(case)
+    with pkg.Context(0) as ctx:
+        ctx.load_case(case)
+        for form in ("fp16x3", "bf16x6"):
+            got = ctx.chi_tau(case.thr, form).cpu().numpy()
+            assert np.linalg.norm(got - ref) <= 1e-6 * np.linalg.norm(ref), form
+
+
 @pytest.mark.parametrize("form", ["fp64", "fp32"])
 @pytest.mark.parametrize("thr", [0.0, 1e-18, 1e4])
 def test_filter_outside_the_quick_norms(pkg, form, thr):
