@@ -39,7 +39,7 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 WORKLOAD = "ribbon300"
-N_PRODUCTS = {"fp32": 1, "bf16x3": 3, "bf16x6": 6, "fp16x3": 3, "fp64": 1}
+N_PRODUCTS = {"fp32": 1, "bf16x3": 3, "bf16x6": 6, "fp16x3": 3, "fp64": 36}
 SPLIT_FORMS = ("bf16x3", "bf16x6", "fp16x3")
 
 
@@ -250,16 +250,16 @@ def _roof(flops, seconds, prec, peaks, peak_src, kernel, traffic, alu=None):
     """Roofline object of one kernel: achieved = useful flops / its device
     time over the timed region (the same per average launch)."""
     achieved = flops / seconds / 1e12 if seconds > 0 else None
-    if prec in SPLIT_FORMS:
-        # binary16 and bf16 share the dense tensor rate (kind::f16)
+    if prec in SPLIT_FORMS or prec == "fp64":
+        # binary16 and bf16 share the dense tensor rate (kind::f16); FP64 is 36
+        # products of 8-bit digits held in binary16
         peak = peaks["bf16_tflops_sustained"] / N_PRODUCTS[prec]
         note = (f"{peak_src} bf16 sustained (= f16 rate) / {N_PRODUCTS[prec]} products per useful "
                 f"product")
         bound = "tensor"
     else:
         peak = alu[prec]["tflops"] if alu else None
-        note = (f"measured {'FFMA' if prec == 'fp32' else 'DFMA'} throughput of this GPU "
-                f"(libgwpeaks)") if peak else "not measured"
+        note = "measured FFMA throughput of this GPU (libgwpeaks)" if peak else "not measured"
         bound = "alu"
     return {"kernel": kernel, "bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak if (achieved and peak) else None,

@@ -48,7 +48,8 @@ enum gw_status {
 /* Arithmetic of the contraction steps (Eq. 3).  Green's functions are always
  * built in FP64; chi is always accumulated across blocks in FP64. */
 enum gw_precision {
-  GW_FP64 = 0,   /* FP64 operands, FP64 accumulation (CUDA cores)                  */
+  GW_FP64 = 0,   /* FP64 operands and results: products of 8-bit digits on the
+                    tensor cores, summed exactly as integers, one rounding each    */
   GW_FP32 = 1,   /* FP32 operands, FP32 accumulation per block slab (CUDA cores)   */
   GW_BF16X3 = 2, /* two-term BF16 split, 3 products per product, FP32 accumulation
                     on the tensor cores (tcgen05)                                  */
@@ -130,7 +131,8 @@ int gw_set_greens(gw_ctx* ctx, const double* C, const double* eps, int n_occ,
  * norm is < thr is dropped (thr = 0: nothing is dropped, exact zeros are still
  * skipped).  chi is formed on atom blocks atom(P) <= atom(Q) and mirrored.
  *
- * precision (enum gw_precision): GW_FP64 and GW_FP32 on the CUDA cores;
+ * precision (enum gw_precision): GW_FP64 as digit products on the tensor cores,
+ * GW_FP32 on the CUDA cores;
  * GW_BF16X3, GW_BF16X6 and GW_FP16X3 as split 16-bit products on the tensor
  * cores with FP64 accumulation of chi across work units.  screening:
  * GW_SCREEN_BOUND (the exact filter above) or GW_SCREEN_MLP (tensor-core forms
@@ -160,7 +162,7 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
  * (real, phases removed as for chi; W even in tau; RI metric = identity).
  * W_tau[n_tau][n_ri][n_ri]: device if w_on_device else host (e.g. the output
  * of gw_chi_to_w).  Filter: 3c, G and (mu-atom, P-atom) blocks of B^n with
- * norm < thr are dropped.  precision: GW_FP64 (CUDA cores) or GW_BF16X3 /
+ * norm < thr are dropped.  precision: GW_FP64 or GW_BF16X3 /
  * GW_BF16X6 / GW_FP16X3 (the two products B W and (B W) B^T on the tensor
  * cores as split 16-bit tile jobs with FP64 outputs; G, B^n and the traces
  * stay FP64).
@@ -268,8 +270,8 @@ int gw_ri_metric(gw_ctx* ctx, const double* S, int n_mat, const double* M, int m
  * gw_sigma_tau):
  *   Sigma_{mu nu}(+i tau) = -sum (mu lam|P) G^occ_{lam sig}(tau) W_PQ(tau) (sig nu|Q)
  *   Sigma_{mu nu}(-i tau) = +sum (mu lam|P) G^virt_{lam sig}(tau) W_PQ(tau) (sig nu|Q)
- * for every tau point of gw_set_greens.  FP64 dense route on the CUDA cores
- * for molecules (n_AO^2 n_RI <= 3*2^30 and n_AO <= 2047, GW_ERR_INVALID_ARG
+ * for every tau point of gw_set_greens.  FP64 dense route for
+ * molecules (n_AO^2 n_RI <= 3*2^30 and n_AO <= 2047, GW_ERR_INVALID_ARG
  * otherwise; three arrays of n_AO^2 n_RI doubles on the device).  Filter: 3c
  * blocks and G blocks with Frobenius norm < thr are dropped.  W_tau:
  * [n_tau][n_ri][n_ri], device if w_on_device else host.  sigma_out:
@@ -298,9 +300,8 @@ int gw_sigma_x(gw_ctx* ctx, const double* V, int v_on_device, const int* orbital
  * per tau point, each of the two products of Eq. 10 -- Y = B^n W and
  * Z = Y B^nT, every (molecule, orbital) pair -- is one persistent
  * tensor-core launch over all pairs' tiles, and the traces with G^occ and
- * G^virt one more launch; B^n is formed once per molecule from its FP64
- * panels, which are then released (one molecule's panels are resident at a
- * time).  GW_FP64 runs gw_sigma_tau's FP64 route molecule by molecule.
+ * G^virt one more launch; B^n is formed once per molecule from its stored 3c
+ * blocks.  GW_FP64 runs gw_sigma_tau's FP64 route molecule by molecule.
  * Runs on the stream of ctxs[0]; messages go to ctxs[0]'s gw_last_error.
  * Errors: GW_ERR_INVALID_ARG (null or mismatched arguments, devices or tau
  * counts, orbital index), GW_ERR_ORDER (a context without inputs),
