@@ -2579,7 +2579,16 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
     gw::TraceRange trace_tau("chi: one tau point");
     GW_TRY(cudaEventRecord(ev[0], ctx->stream));
     ctx->cur_tau = ctx->tau[j];
-    if ((rc = gw::greens_fp64(ctx, *ctx, ctx->tau[j], cso, csv, go, gv, ctx->stream))) return rc;
+    // The forms that round G take the sums of the FP64 pipe, not the digits: the
+    // 16-bit slices resolve the smallest elements to 2^-38 of the largest only, so
+    // the last bit of G moves the norm of a small block of X or Y by up to 1e-3,
+    // and with it blocks at the threshold (2 of 36 ribbons of 58 atoms changed by
+    // more than their sums' rounding).  Costs 0.2 ms per tau point at 602 functions.
+    if (precision == GW_FP64) {
+      if ((rc = gw::greens_fp64(ctx, *ctx, ctx->tau[j], cso, csv, go, gv, ctx->stream))) return rc;
+    } else {
+      gw::launch_greens(ctx->d_C, ctx->d_eps, nao, ctx->n_occ, ctx->mu, ctx->tau[j], cso, csv, go, gv, ctx->stream);
+    }
     GW_CHECK_LAUNCH();
     ctx->stats.kernel_launches += 3;
     double h[4] = {0, 0, 0, 0};
