@@ -19,12 +19,11 @@
 // closer to the exact value, and it does not depend on how K is split:
 // partial sums are integers, so split units may add in any order.
 //
-// Layout: a cluster of two CTAs takes 128 x 128 outputs, 64 columns each;
+// Layout: two neighbouring CTAs take 128 x 128 outputs, 64 columns each;
 // stages of 32 reduction elements with all eight digits of both operands
 // (96 KB, two stages).  64 columns per CTA and not 128: the two integers of
-// 128 x 128 outputs would take the whole register file.  The A operand is the
-// same for both: each CTA loads four of its digits and multicasts them to the
-// pair, which cuts the L2 traffic of a stage from 96 to 64 KB per CTA.
+// 128 x 128 outputs would take the whole register file.  Both load the A
+// operand; that they run side by side keeps its second read in the L2 cache.
 // MMAs: a digit of A meets two neighbouring digits of B at once, whose rows
 // follow one another in shared memory, and adds into two neighbouring
 // diagonals, 64 accumulator columns each: N = 128 takes 64 cycles where two
@@ -58,7 +57,7 @@ namespace emu {
 using namespace gw::tc;
 
 constexpr int kS = kEmuSlices;
-constexpr int kM = kEmuTileM, kN = kEmuTileN / 2;  // a CTA takes half of a cluster's columns
+constexpr int kM = kEmuTileM, kN = kEmuTileN / 2;  // a CTA takes half of a tile's columns
 constexpr int kN2 = kEmuTileN;
 constexpr int kChunk = 32;  // reduction elements of a stage (64-byte rows)
 constexpr int kSub = kChunk / kMmaK;
@@ -466,9 +465,9 @@ struct GemmJob {
     return T;
   }
   __device__ bool skip(int ya, int yb) const { return tri && yb >= ya + kM + tri_off; }
-  __device__ void half(Tile& T, int rank) const {
-    T.yb += rank * kN;
-    T.rb += rank * kN;
+  __device__ void half(Tile& T, int side) const {
+    T.yb += side * kN;
+    T.rb += side * kN;
   }
   __device__ int nchunks(const Tile& T) const { return T.n; }
   struct Iter {
@@ -598,9 +597,9 @@ struct Panel64Job {
     T.n = (tk.K + kChunk - 1) / kChunk;
     return T;
   }
-  __device__ void half(Tile& T, int rank) const {
-    T.yb += rank * kN;
-    T.b0 += rank * kN;
+  __device__ void half(Tile& T, int side) const {
+    T.yb += side * kN;
+    T.b0 += side * kN;
   }
   __device__ int nchunks(const Tile& T) const { return T.n; }
   struct Iter {
@@ -694,7 +693,7 @@ struct Chi64Job {
     for (int i = 0; i < T.cnt; ++i) T.n += slab_len[T.list[i]] / kChunk;
     return T;
   }
-  __device__ void half(Tile& T, int rank) const { T.yb += rank * kN; }
+  __device__ void half(Tile& T, int side) const { T.yb += side * kN; }
   __device__ int nchunks(const Tile& T) const { return T.n; }
   struct Iter {
     const Chi64Job* j;
@@ -854,7 +853,7 @@ __device__ __forceinline__ bool add_pair(int p, int q, uint64_t* acc_full, uint6
 }
 
 template <class Job>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, 1)
     k_emu(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const Job job,
           int* __restrict__ err_flag) {
   extern __shared__ uint8_t smem_raw[];
@@ -872,7 +871,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 2);  // both CTAs have read their copy of the stage
+      mbar_init(&empty[s], 1);
     }
     for (int b = 0; b < kPairs; ++b) {
       mbar_init(&acc_full[b], 1);
@@ -889,11 +888,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync();  // the peer's barriers are initialised
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const int n_items = job.items();
-  const int rank = blockIdx.x & 1, first = blockIdx.x >> 1, step = gridDim.x >> 1;
+  const int side = blockIdx.x & 1, first = blockIdx.x >> 1, step = gridDim.x >> 1;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -904,7 +902,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       bool ok = true;
       for (int t = first; t < n_items && ok; t += step) {
         typename Job::Tile T = job.tile(t);
-        job.half(T, rank);
+        job.half(T, side);
         const int n = job.nchunks(T);
         typename Job::Iter it;
         it.init(&job, T);
@@ -918,9 +916,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           armed[stage] = true;
           armed_parity[stage] = phase;
           const int x = it.next();
-          // this CTA's half of A's digits to both CTAs, its own columns of B
-          const int s0 = rank * (kS / 2);
-          tma_load_3d_pair(st + s0 * kABytes, &map_a, x, T.ya, s0, &full[stage]);
+          tma_load_3d(st, &map_a, x, T.ya, 0, &full[stage]);
           tma_load_3d(st + kS * kABytes, &map_b, x, T.yb, 0, &full[stage]);
           if (++stage == kStages) {
             stage = 0;
@@ -928,10 +924,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           }
         }
       }
-      // both CTAs' releases of the last stages have arrived here: none is on
-      // its way to a CTA that has left
-      for (int s = 0; s < kStages && ok; ++s)
-        if (armed[s]) ok = mbar_wait(&empty[s], armed_parity[s], abort_flag);
       if (!ok) {
         *abort_flag = 1;
         atomicOr(err_flag, 1);
@@ -988,7 +980,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           issued = true;
         }
         if (!ok) break;
-        if (lead) mma_commit_pair(&empty[stage]);
+        if (lead) mma_commit(&empty[stage]);
         __syncwarp();
         if (last) aphase ^= 1u;
         if (++stage == kStages) {
@@ -1017,7 +1009,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       typename Job::Tile T = job.tile(t);
       const int n = job.nchunks(T);
       if (n == 0) continue;
-      job.half(T, rank);
+      job.half(T, side);
       // exponents of this lane's row and of column c0 + lane % 16, loaded here:
       // beside the stores they would be fetched one by one
       const int er = job.row_exp(T, quad * 32 + lane), ec = job.col_exp(T, c0 + lane % kCols);
@@ -1049,7 +1041,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync();  // neither CTA leaves while the other may write to it
   tc_fence_after();
   if (warp == 1) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
@@ -1075,7 +1066,7 @@ int launch(const CUtensorMap& ma, const CUtensorMap& mb, const Job& job, int n_i
 }
 
 // K splits of an m x n product: the number of units that makes the last wave
-// over the 76 clusters short.  Costs in stages (about 1.7 us each): a unit's
+// over the 76 pairs of CTAs short.  Costs in stages (about 1.7 us each): a unit's
 // start and end about 3, clearing the partial sums about 3 in all.
 int k_splits(long long m, long long n, int K, int nz) {
   const long long tiles = ((m + kM - 1) / kM) * ((n + kN2 - 1) / kN2) * nz;
@@ -1133,7 +1124,7 @@ int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, 
   const int m = static_cast<int>(A.s.rows), n = static_cast<int>(B.s.rows);
   if (m <= 0 || n <= 0) return 0;
   CUtensorMap ma, mb;
-  if (make_digit_map(&ma, A.dig, A.kp, A.s.nz > 1 ? A.stride_rows : A.s.rows, A.stride_rows, kEmuSlices, emu::kChunk, emu::kM, kEmuSlices / 2) ||
+  if (make_digit_map(&ma, A.dig, A.kp, A.s.nz > 1 ? A.stride_rows : A.s.rows, A.stride_rows, kEmuSlices, emu::kChunk, emu::kM, kEmuSlices) ||
       make_digit_map(&mb, B.dig, B.kp, B.s.nz > 1 ? B.stride_rows : B.s.rows, B.stride_rows, kEmuSlices, emu::kChunk,
                      emu::kN, kEmuSlices))
     return -2;
@@ -1215,11 +1206,10 @@ int launch_panel64(const Panel64Args& p, int* err_flag, cudaStream_t st) {
   if (p.n_tiles == 0) return 0;
   CUtensorMap mp, mg;
   const bool x = p.mode == 0;
-  const int whole = kEmuSlices, part = kEmuSlices / 2;  // digits per load of the B and A operand
   if (make_digit_map(&mp, p.panel_dig, p.kp, p.panel_rows, p.panel_rows, kEmuSlices, emu::kChunk,
-                     x ? emu::kM : emu::kN, x ? part : whole) ||
+                     x ? emu::kM : emu::kN, kEmuSlices) ||
       make_digit_map(&mg, p.g_dig, p.g_kp, p.g_rows, p.g_rows, kEmuSlices, emu::kChunk, x ? emu::kN : emu::kM,
-                     x ? whole : part))
+                     kEmuSlices))
     return -2;
   emu::Panel64Job j{p.tiles, p.n_tiles, p.mode, p.R,  p.r0,   p.P0b, p.tasks, p.ldk, p.rowbase,
                     p.rowmul, p.panel_exps, p.g_exps, p.out, p.pool, p.G, p.lam, p.nao};
@@ -1229,7 +1219,7 @@ int launch_panel64(const Panel64Args& p, int* err_flag, cudaStream_t st) {
 int launch_chi64(const EmuOp& x, const EmuOp& y, const Chi64Args& c, int* err_flag, cudaStream_t st) {
   CUtensorMap mx, my;
   if (make_digit_map(&mx, x.dig, x.kp, x.s.rows, x.stride_rows, kEmuSlices, emu::kChunk, emu::kM,
-                     kEmuSlices / 2) ||
+                     kEmuSlices) ||
       make_digit_map(&my, y.dig, y.kp, y.s.rows, y.stride_rows, kEmuSlices, emu::kChunk, emu::kN, kEmuSlices))
     return -2;
   emu::Chi64Job j{c.units.u_tile, c.units.u_first, c.units.u_count, c.units.n_units, c.tasks, c.counts, c.nslab,
