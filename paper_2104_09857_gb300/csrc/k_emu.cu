@@ -814,7 +814,7 @@ template <bool kHi>
 __device__ __forceinline__ bool add_pair(int p, int q, uint64_t* acc_full, uint64_t* acc_empty, uint32_t parity,
                                          volatile int* abort_flag, uint32_t row_addr, int lane,
                                          long long (&hi)[kCols], uint32_t (&lo)[kCols]) {
-  if (!mbar_wait(&acc_full[p], parity, abort_flag)) return false;
+  if (!mbar_wait_warp(&acc_full[p], parity, abort_flag)) return false;
   tc_fence_after();
   const int w0 = q ? 1 << 8 : 1 << 24, w1 = q ? 1 : 1 << 16;
 #pragma unroll
@@ -944,7 +944,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const typename Job::Tile T = job.tile(t);
       const int n = __reduce_max_sync(0xffffffffu, job.nchunks(T));
       for (int i = 0; i < n && ok; ++i) {
-        ok = __all_sync(0xffffffffu, mbar_wait(&full[stage], phase, abort_flag));
+        ok = mbar_wait_warp(&full[stage], phase, abort_flag);
         if (!ok) break;
         tc_fence_after();
         const bool first = (i % kGroup) == 0, last = (i % kGroup) == kGroup - 1 || i == n - 1;
@@ -954,7 +954,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int p = 0; p < kPairs; ++p) {
           if (first) {
-            ok = __all_sync(0xffffffffu, mbar_wait(&acc_empty[p], aphase, abort_flag));
+            ok = mbar_wait_warp(&acc_empty[p], aphase, abort_flag);
             if (!ok) break;
             tc_fence_after();
           }

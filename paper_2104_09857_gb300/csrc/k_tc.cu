@@ -778,7 +778,7 @@ struct PanelStagedJob {
         __syncwarp();
         if (lane == 0) mbar_arrive(ep.freed);
       }
-      if (!mbar_wait(ep.freed, static_cast<uint32_t>(ep.tile_no - 1) & 1u, ep.abort)) return false;
+      if (!mbar_wait_warp(ep.freed, static_cast<uint32_t>(ep.tile_no - 1) & 1u, ep.abort)) return false;
     }
     // row keys uniform across the warp's valid rows?
     const int rk0 = __shfl_sync(0xffffffffu, rk, 0);
@@ -819,7 +819,7 @@ struct PanelStagedJob {
       __syncwarp();
       if (lane == 0) mbar_arrive(ep.staged);
       if (ep.warp != 0) return true;
-      if (!mbar_wait(ep.staged, static_cast<uint32_t>(ep.tile_no) & 1u, ep.abort)) return false;
+      if (!mbar_wait_warp(ep.staged, static_cast<uint32_t>(ep.tile_no) & 1u, ep.abort)) return false;
       const int nsig = t_nsig;
       const int pitch = kTileN * nsig + kRunSkew;
       const long long d0 = static_cast<long long>(t_p0 + pw0 - P0b) * ldk + t_seg +
@@ -845,7 +845,7 @@ struct PanelStagedJob {
     // striding over them
     __syncwarp();
     if (lane == 0) mbar_arrive(ep.staged);
-    if (!mbar_wait(ep.staged, static_cast<uint32_t>(ep.tile_no) & 1u, ep.abort)) return false;
+    if (!mbar_wait_warp(ep.staged, static_cast<uint32_t>(ep.tile_no) & 1u, ep.abort)) return false;
     int U0 = 0;  // first region of the current group of 32 atoms
     for (int base = sf; base <= sl; base += 32) {
       if (base > sf) {
@@ -958,7 +958,7 @@ struct Sched {
   // the MMA issuer warp and the epilogue warps (all 32 lanes)
   __device__ int consume_warp(int lane, bool& ok) {
     if (!counter) return next_static();
-    if (!mbar_wait(&full[s], ph, abort)) {
+    if (!mbar_wait_warp(&full[s], ph, abort)) {
       ok = false;
       return -1;
     }
@@ -1120,7 +1120,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int js = 0;
       int sub = 0;  // MMA steps into the drain interval
       for (int i = 0; i < n; ++i) {
-        ok = __all_sync(kAll, mbar_wait(&full[stage], phase, abort_flag));
+        ok = mbar_wait_warp(&full[stage], phase, abort_flag);
         if (!ok) break;
         tc_fence_after();
         const uint64_t da = desc_sw128(smem_u32(operands + stage * L::kStageBytes));
@@ -1130,8 +1130,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         while (k < kSub) {
           const int mb = chunk % kAccBufs;
           if (sub == 0) {
-            ok = __all_sync(kAll, mbar_wait(&acc_empty[mb], ((static_cast<uint32_t>(chunk / kAccBufs)) & 1u) ^ 1u,
-                                            abort_flag));
+            ok = mbar_wait_warp(&acc_empty[mb], ((static_cast<uint32_t>(chunk / kAccBufs)) & 1u) ^ 1u, abort_flag);
             if (!ok) break;
             tc_fence_after();
           }
@@ -1206,7 +1205,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     (void)ep;
     // test hook: a dependency that is never satisfied; the bounded wait
     // gives up and the kernel reports a time-out instead of hanging
-    bool ok = cad.stall ? mbar_wait(never, 0, abort_flag) : true;
+    bool ok = cad.stall ? mbar_wait_warp(never, 0, abort_flag) : true;
     for (int t = ok ? sch.consume_warp(lane, ok) : -1; t >= 0 && ok; t = sch.consume_warp(lane, ok)) {
       const typename Job::Tile T = job.tile(t);
       const long long n = job.nsteps(T);
@@ -1215,7 +1214,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int j = 0; j < kEpiCols; ++j) acc[j] = 0.f;
       for (long long c = 0; c < nch; ++c, ++chunk) {
         const int mb = chunk % kAccBufs;
-        if (!mbar_wait(&acc_full[mb], static_cast<uint32_t>(chunk / kAccBufs) & 1u, abort_flag)) {
+        if (!mbar_wait_warp(&acc_full[mb], static_cast<uint32_t>(chunk / kAccBufs) & 1u, abort_flag)) {
           ok = false;
           break;
         }

@@ -56,6 +56,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     if (global_ns() - t0 > kWaitLimitNs) return false;
   }
 }
+// The same by all 32 lanes of a warp: false in every lane if it is false in one.
+// Near the limit, or while an abort comes in, some lanes may see the phase and
+// others give up; what follows a warp's wait are warp-wide instructions
+// (tcgen05.ld, shuffles, __syncwarp), which all of its lanes must reach.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0;
+}
 // Bounded wait without abort check (clean-up after an abort).
 __device__ __forceinline__ void mbar_wait_cleanup(uint64_t* bar, uint32_t parity) {
   const uint64_t t0 = global_ns();
