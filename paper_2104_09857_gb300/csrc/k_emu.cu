@@ -855,7 +855,7 @@ __device__ __forceinline__ bool add_pair(int p, int q, uint64_t* acc_full, uint6
 template <class Job>
 __global__ void __launch_bounds__(kThreads, 1)
     k_emu(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, const Job job,
-          int* __restrict__ err_flag) {
+          int stall, int* __restrict__ err_flag) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -865,7 +865,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* acc_full = empty + kStages;
   uint64_t* acc_empty = acc_full + kPairs;
   uint64_t* drain = acc_empty + kPairs;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+  uint64_t* never = drain + 1;  // arrived at by nothing (stall test hook)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(never + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = __reduce_max_sync(0xffffffffu, threadIdx.x / 32), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -878,6 +879,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&acc_empty[b], kEpiWarps);
     }
     mbar_init(drain, 1);
+    mbar_init(never, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -1004,7 +1006,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     unsigned long long* stg = reinterpret_cast<unsigned long long*>(staging + (warp - 2) * kStgBytes);
     const uint32_t row_addr = tmem + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(c0);
     uint32_t aphase = 0;
-    bool ok = true;
+    // test hook: the bounded wait gives up and the kernel reports a time-out
+    bool ok = stall ? mbar_wait_warp(never, 0, abort_flag) : true;
     for (int t = first; t < n_items && ok; t += step) {
       typename Job::Tile T = job.tile(t);
       const int n = job.nchunks(T);
@@ -1061,7 +1064,7 @@ int launch(const CUtensorMap& ma, const CUtensorMap& mb, const Job& job, int n_i
       return -1;
     attr_set.fetch_or(bit, std::memory_order_release);
   }
-  k_emu<Job><<<2 * std::min(n_items, std::max(sms / 2, 1)), kThreads, kSmem, st>>>(ma, mb, job, err_flag);
+  k_emu<Job><<<2 * std::min(n_items, std::max(sms / 2, 1)), kThreads, kSmem, st>>>(ma, mb, job, tc_stall_test(), err_flag);
   return 0;
 }
 

@@ -1875,6 +1875,7 @@ int make_digit_map(CUtensorMap* map, const void* base, long long k_len, long lon
 int tc_tile_rows() { return tc::kTileM; }
 
 void tc_set_stall_test(int on) { g_stall_test = on; }
+int tc_stall_test() { return g_stall_test; }
 
 int launch_chi_tc(int slices, int f16, float out_scale, const CUtensorMap& mx, const CUtensorMap& my,
                   const int* tile_list, int n_tiles, const int* tasks, const int* counts, int max_slab,

@@ -25,10 +25,11 @@ int make_digit_map(CUtensorMap* map, const void* base, long long k_len, long lon
                    int slices, int box_k, int box_rows, int box_slices);
 // Rows (and columns) of one step-C tile of the tensor-core kernel.
 int tc_tile_rows();
-// Test hook (process-wide): while on, every tensor-core kernel launched has
+// Test hook (of the calling host thread): while on, every tensor-core kernel launched has
 // its epilogue wait first on a barrier that nothing arrives at, so that the
 // bounded waits expire (about 2 s) and the kernel returns its error flag.
 void tc_set_stall_test(int on);
+int tc_stall_test();
 // 2^(14 - ceil(log2 bound)): scales a value of magnitude <= bound to <= 2^14
 // (1 for a zero or non-finite bound).
 double pow2_scale(double bound);
