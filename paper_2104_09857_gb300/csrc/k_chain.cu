@@ -92,27 +92,19 @@ __global__ void k_set_identity(double* __restrict__ a, int n) {
 constexpr int kNb = 32;
 constexpr int kOuter = 2 * kNb;
 
-// 1 / sqrt(p) for a normal p > 0: the FP32 reciprocal square root of the
-// mantissa (exponent made even and taken apart), then one third-order step
-// y (1 + e/2 + 3 e^2/8), e = 1 - p y^2, which leaves e^3 ~ 2^-66.
-__device__ __forceinline__ double inv_sqrt(double p) {
-  const int hi = __double2hiint(p);
-  const int ex = ((hi >> 20) - 1023) & ~1;  // even exponent
-  const double m = __hiloint2double(hi - (ex << 20), __double2loint(p));  // in [1, 4)
-  const double y0 = static_cast<double>(rsqrtf(static_cast<float>(m)));
-  const double e = fma(-m * y0, y0, 1.0);
-  const double y = fma(y0 * e, fma(e, 0.375, 0.5), y0);
-  return __hiloint2double(__double2hiint(y) - ((ex / 2) << 20), __double2loint(y));
-}
-
 // Cholesky factor of the b x b diagonal block at (k0, k0) of every matrix, to
 // fac[k0 * 32..] (row-major, pitch 32) and the reciprocals of its diagonal to
 // fac[(n + 32) * 32 + k0..].  One CTA per matrix; formed by every CTA of the
-// solve below instead, the CTAs of an SM would queue for its FP64 pipe.
+// solve below instead, the CTAs of an SM would queue for its FP64 pipe.  The
+// columns of the block are scaled by rsqrt (one unit in the last place), a
+// square root and a division per pivot would lie on the serial chain; the
+// diagonal and its reciprocals are rounded roots and quotients, taken for all
+// pivots at once at the end.
 __global__ void __launch_bounds__(128) k_chol_factor(const double* __restrict__ a0, int n, long long z_stride, int k0,
                                                      int b, double* __restrict__ fac0, long long fac_z,
                                                      int* __restrict__ err) {
   __shared__ double d[kNb][kNb + 1];
+  __shared__ double piv[kNb];
   const double* a = a0 + blockIdx.x * z_stride;
   double* fac = fac0 + blockIdx.x * fac_z;
   double* rd = fac + (static_cast<long long>(n) + kNb) * kNb + k0;
@@ -129,15 +121,10 @@ __global__ void __launch_bounds__(128) k_chol_factor(const double* __restrict__ 
       bad = true;
       p = 1.0;
     }
-    // a subnormal pivot (outside inv_sqrt's range) by the library's root
-    const double y = p < 2.2250738585072014e-308 ? 1.0 / sqrt(p) : inv_sqrt(p);
-    __syncthreads();  // every thread has read the pivot
+    const double y = rsqrt(p);
     if (warp == 0) {
       if (lane > j) d[lane][j] *= y;
-      if (lane == j) {
-        d[j][j] = p * y;
-        rd[j] = y;
-      }
+      if (lane == j) piv[j] = p;
     }
     __syncthreads();
     const double l = d[lane][j];
@@ -146,6 +133,12 @@ __global__ void __launch_bounds__(128) k_chol_factor(const double* __restrict__ 
     __syncthreads();
   }
   if (bad && threadIdx.x == 0) atomicOr(err, 1);
+  if (warp == 0 && lane < b) {
+    const double r = sqrt(piv[lane]);
+    d[lane][lane] = r;
+    rd[lane] = 1.0 / r;
+  }
+  __syncthreads();
   for (int i = threadIdx.x; i < kNb * kNb; i += blockDim.x)
     fac[static_cast<long long>(k0) * kNb + i] = d[i >> 5][i & 31];
 }

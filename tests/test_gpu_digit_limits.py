@@ -44,3 +44,17 @@ def test_stall_times_out_and_context_recovers(pkg):
         ctx.set_option("test_stall_tc", 0)
         got = ctx.chi_tau(case.thr, "fp64").cpu().numpy()
     assert _rel(got, ref) <= 1e-10
+
+
+def test_cholesky_pivots_are_rounded_roots(pkg):
+    """With chi = 0, W^c = L L^T - V is the factorisation's own error.  For a
+    diagonal V a correctly rounded root errs by 2^-53 of itself, its square by
+    twice that and one more rounding: 3 2^-53 of V, to first order."""
+    n, tau = 300, np.array([1.0])
+    v = np.exp(np.random.default_rng(3).uniform(np.log(1e-6), np.log(1e6), n))
+    with pkg.Context(0) as ctx:
+        ctx.set_basis(np.arange(30.0).reshape(10, 3), np.ones(10, dtype=np.int32), np.full(10, n // 10, dtype=np.int32))
+        ctx.set_greens(np.eye(10), np.linspace(-1.0, 1.0, 10), 5, 0.0, tau)
+        w = ctx.chi_to_w(np.zeros((1, n, n)), np.diag(v), np.ones((1, 1)), np.ones((1, 1))).cpu().numpy()[0]
+    assert not np.any(w - np.diag(np.diag(w)))
+    assert np.abs(np.diag(w) / v).max() <= 3 * 2.0 ** -53 * (1 + 1e-9)
