@@ -1041,7 +1041,8 @@ int chi_one_batch_digits(gw_ctx* ctx, const Batch& b, const double* g_occ, const
   gw::EmuSrc sy = sx;
   sy.src = Y;
   sy.rows = nri;
-  if ((rc = gw::emu_prep(ctx, "X", sx, &ox, ctx->stream)) || (rc = gw::emu_prep(ctx, "Y", sy, &oy, ctx->stream)))
+  if ((rc = gw::emu_prep_segments(ctx, "X", sx, d_seg, ns, &ox, ctx->stream)) ||
+      (rc = gw::emu_prep_segments(ctx, "Y", sy, d_seg, ns, &oy, ctx->stream)))
     return rc;
   // task lists, work units, step C
   std::vector<long long> slab_k0(nslab);
@@ -1075,27 +1076,30 @@ int chi_one_batch_digits(gw_ctx* ctx, const Batch& b, const double* g_occ, const
                          tm, tn, per, 0, n_at, 0, nao, ctx->d_atom_of_ao, ctx->stream);
   gw::launch_count_c(bx, by, ns, 0, n_at, pa0, npa, 0, n_at, d_nri, d_nao, b.s0, d_fc, ctx->stream);
   // Units of about 1/8 of an SM's share, at least 1024 elements (a unit's
-  // atomics cost about as much as 64); with many tiles a unit is a tile, and
-  // adds into chi itself.  Partial sums are integers, so either way chi is
-  // the same to the last bit, run after run.
+  // atomics cost about as much as 64); with many tiles a unit is a tile.
+  // Partial sums are integers, so either way chi is the same to the last bit,
+  // run after run.
   int split = INT32_MAX;
   if (ntiles < 152 * 16)
     split = (int)std::min<double>(std::max(1024.0, 0.6 * ntiles * (double)Kb / (152 * 8)), 1 << 30);
-  void* part = nullptr;
-  if (split != INT32_MAX && (rc = ws(ctx, "d64_part", (size_t)prow * nri * 16, &part))) return rc;
+  void* part;
+  int* pair;
+  if ((rc = ws(ctx, "d64_part", (size_t)prow * nri * 16, &part)) ||
+      (rc = wsT(ctx, "d64_pair", (size_t)prow * nri, &pair)))
+    return rc;
   GW_TRY(cudaMemsetAsync(tstat, 0, 3 * sizeof(unsigned long long), ctx->stream));
   gw::launch_plan_units(tlist, counts, kacc, d_len, ntiles, nslab, split, w, tstat, ctx->stream);
   GW_CHECK_LAUNCH();
   cudaEvent_t ec0, ec1;
   if ((rc = c_event_pair(ctx, 2 * batch_idx, &ec0, &ec1))) return rc;
   GW_TRY(cudaEventRecord(ec0, ctx->stream));
-  gw::Chi64Args c{w, tlist, counts, nslab, nqt, b.P0, prow, nri, d_k0, d_len, acc, part};
+  gw::Chi64Args c{w, tlist, counts, nslab, nqt, b.P0, prow, nri, per, d_k0, d_len, acc, part, pair};
   if (gw::launch_chi64(ox, oy, c, d_err, ctx->stream))
     return fail(ctx, GW_ERR_CUDA, "FP64 step C: launch setup failed");
   GW_CHECK_LAUNCH();
   GW_TRY(cudaEventRecord(ec1, ctx->stream));
   ctx->stats.c_launches += 1;
-  ctx->stats.kernel_launches += 13;
+  ctx->stats.kernel_launches += 14;
   std::vector<double> h_fc((size_t)ns * n_at);
   unsigned long long h_stat[3];
   GW_TRY(cudaMemcpyAsync(h_fc.data(), d_fc, h_fc.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));

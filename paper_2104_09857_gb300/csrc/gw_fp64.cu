@@ -34,21 +34,39 @@ int emu_begin(gw_ctx* ctx, cudaStream_t st) {
   return GW_OK;
 }
 
-int emu_prep(gw_ctx* ctx, const char* name, const EmuSrc& s, EmuOp* op, cudaStream_t st) {
+namespace {
+// digits of `rows` rows of length K and n_exps exponents in buffers of this name
+int digit_buffers(gw_ctx* ctx, const char* name, long long rows, int K, long long n_exps, EmuOp* op) {
   void* p;
   int rc;
   const std::string n = std::string("w.dig.") + name;
-  if ((rc = work_buffer(ctx, n.c_str(), std::max<size_t>(emu_dig_bytes(s.rows * s.nz, s.K), 16), &p))) return rc;
+  if ((rc = work_buffer(ctx, n.c_str(), std::max<size_t>(emu_dig_bytes(rows, K), 16), &p))) return rc;
   op->dig = p;
-  if ((rc = work_buffer(ctx, (n + ".e").c_str(), std::max<size_t>(s.rows * s.nz, 1) * 2 * sizeof(int), &p))) return rc;
+  if ((rc = work_buffer(ctx, (n + ".e").c_str(), std::max<size_t>(n_exps, 1) * sizeof(int), &p))) return rc;
   op->exps = static_cast<int*>(p);
-  launch_emu_prep(*op, s, st);
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) {
-    ctx->err = std::string("FP64 operand preparation: ") + cudaGetErrorString(e);
-    return GW_ERR_CUDA;
-  }
   return GW_OK;
+}
+int prep_launched(gw_ctx* ctx) {
+  const cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) return GW_OK;
+  ctx->err = std::string("FP64 operand preparation: ") + cudaGetErrorString(e);
+  return GW_ERR_CUDA;
+}
+}  // namespace
+
+int emu_prep(gw_ctx* ctx, const char* name, const EmuSrc& s, EmuOp* op, cudaStream_t st) {
+  const int rc = digit_buffers(ctx, name, s.rows * s.nz, s.K, s.rows * s.nz * 2, op);
+  if (rc) return rc;
+  launch_emu_prep(*op, s, st);
+  return prep_launched(ctx);
+}
+
+int emu_prep_segments(gw_ctx* ctx, const char* name, const EmuSrc& s, const long long* seg, int n_seg, EmuOp* op,
+                      cudaStream_t st) {
+  const int rc = digit_buffers(ctx, name, s.rows, s.K, s.rows * n_seg, op);
+  if (rc) return rc;
+  launch_emu_prep_segments(*op, s, seg, n_seg, st);
+  return prep_launched(ctx);
 }
 
 int emu_mm(gw_ctx* ctx, const EmuOp& A, const EmuOp& B, const EmuGemm& g, cudaStream_t st) {

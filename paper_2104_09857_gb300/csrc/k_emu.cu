@@ -17,7 +17,11 @@
 // rounds once at the end.  Against a sequential FP64 sum (error about
 // 0.2 * 2^-53 |a| |b| of the rows' 2-norms for random signs) the result is
 // closer to the exact value, and it does not depend on how K is split:
-// partial sums are integers, so split units may add in any order.
+// partial sums are integers, so split units may add in any order.  That holds
+// in the norm: the error of an element is 2^-61 of the product of its rows'
+// largest magnitudes, also where the element itself is far below that product
+// and an FP64 sum's error with it.  Step C of chi, whose rows fall off with
+// distance, therefore has exponents per part of a row (Chi64Job).
 //
 // Layout: two neighbouring CTAs take 128 x 128 outputs, 64 columns each;
 // stages of 32 reduction elements with all eight digits of both operands
@@ -180,6 +184,41 @@ __global__ void __launch_bounds__(256) k_prep_rows(const double* __restrict__ sr
 #pragma unroll
       for (int i = 0; i < kS; ++i)
         *reinterpret_cast<uint4*>(dig + (i * rows + r) * kp + k) = q[i];
+    }
+  }
+}
+
+// Rows of a row-major matrix with an exponent per segment of a row: segment i
+// starts at element seg[i] (a multiple of 64) and ends where the next begins.
+// exps[i * rows + r].  One CTA per segment of a row.
+__global__ void __launch_bounds__(256) k_prep_segments(const double* __restrict__ src, long long ld, long long rows,
+                                                       int K, const long long* __restrict__ seg, int n_seg,
+                                                       __half* __restrict__ dig, int* __restrict__ exps) {
+  __shared__ int red[8];
+  for (long long i = blockIdx.x; i < rows * n_seg; i += gridDim.x) {
+    const long long r = i / n_seg;
+    const int s = static_cast<int>(i - r * n_seg);
+    const long long k0 = seg[s];
+    const int len = static_cast<int>((s + 1 < n_seg ? seg[s + 1] : K) - k0);
+    const double* x = src + r * ld + k0;
+    int be = 0;
+    for (int k = threadIdx.x; k < len; k += 256) be = max(be, biased_exp(x[k]));
+    be = __reduce_max_sync(0xffffffffu, be);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = be;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < 8; ++w) be = max(be, red[w]);
+    const int e = row_exp(be);
+    if (threadIdx.x == 0) exps[s * rows + r] = e;
+    for (int k = 8 * threadIdx.x; k < len; k += 8 * 256) {
+      double v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = x[k + j];
+      uint4 q[kS];
+      digits8(v, e, q);
+#pragma unroll
+      for (int j = 0; j < kS; ++j) *reinterpret_cast<uint4*>(dig + (j * rows + r) * K + k0 + k) = q[j];
     }
   }
 }
@@ -392,12 +431,13 @@ __device__ __forceinline__ void by_rows(unsigned long long* stg, int lane, const
   }
   __syncwarp();
 }
-// The (hi, lo) of 32 rows into 64-bit partial sums: element (r, c) at part +
-// 2 (r * n + c) for r < rows, c < n; r, c: the warp's first row and column.
-// only: the one unit of its tile, which stores and does not add.
+// The (hi, lo) of 32 rows, value(j, hi, lo) for column j, into 64-bit partial
+// sums: element (r, c) at part + 2 (r * n + c) for r < rows, c < n; r, c: the
+// warp's first row and column.  only: the one unit of its tile, which stores
+// and does not add.
+template <class V>
 __device__ __forceinline__ void add_partial(unsigned long long* part, bool only, long long n, int rows, int r, int c,
-                                            int lane, long long (&hi)[kCols], uint32_t (&lo)[kCols],
-                                            unsigned long long* stg) {
+                                            int lane, const V& value, unsigned long long* stg) {
   const int k = lane & 7;
   unsigned long long* p = part + ((r + (lane >> 3)) * n + c + (k >> 1)) * 2 + (k & 1);
   const int left = rows - r - (lane >> 3);
@@ -406,8 +446,11 @@ __device__ __forceinline__ void add_partial(unsigned long long* part, bool only,
     unsigned long long v[8];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      v[2 * j] = static_cast<unsigned long long>(hi[h + j]);
-      v[2 * j + 1] = lo[h + j];
+      long long hi;
+      uint32_t lo;
+      value(h + j, hi, lo);
+      v[2 * j] = static_cast<unsigned long long>(hi);
+      v[2 * j + 1] = lo;
     }
     const bool in = c + h + (k >> 1) < n;
     by_rows(stg, lane, v, [](int) { return 0.0; }, [&](int i, unsigned long long x, double) {
@@ -464,6 +507,7 @@ struct GemmJob {
     if (skip(T.ra, T.rb)) T.n = 0;
     return T;
   }
+  __device__ bool next(Tile&) const { return false; }
   __device__ bool skip(int ya, int yb) const { return tri && yb >= ya + kM + tri_off; }
   __device__ void half(Tile& T, int side) const {
     T.yb += side * kN;
@@ -512,7 +556,12 @@ struct GemmJob {
                         int er, int ec, unsigned long long* stg) const {
     const int r = T.ra + row0, c = T.rb + c0;
     if (part) {
-      add_partial(part + static_cast<long long>(T.z) * m * n * 2, ks == 1, n, m, r, c, lane, hi, lo, stg);
+      add_partial(part + static_cast<long long>(T.z) * m * n * 2, ks == 1, n, m, r, c, lane,
+                  [&](int j, long long& h, uint32_t& l) {
+                    h = hi[j];
+                    l = lo[j];
+                  },
+                  stg);
       return;
     }
     const int left = m - r - (lane >> 3);
@@ -597,6 +646,7 @@ struct Panel64Job {
     T.n = (tk.K + kChunk - 1) / kChunk;
     return T;
   }
+  __device__ bool next(Tile&) const { return false; }
   __device__ void half(Tile& T, int side) const {
     T.yb += side * kN;
     T.b0 += side * kN;
@@ -664,34 +714,82 @@ struct Panel64Job {
 
 // ---------------------------------------------------------------------------
 // step C in FP64: chi[P][Q] -= sum over the unit's slabs of X[P][k] Y[Q][k]
+//
+// X and Y of two distant auxiliary functions overlap only where both are far
+// below their largest magnitudes: digits below one exponent per row would leave
+// such an element of chi an error of 2^-61 of the product of the rows' maxima
+// (58-atom ribbon: 1.9e-10 of chi between its ends, FP64 sums 4e-14).  So the
+// rows have an exponent per sigma-atom, over which they vary little where they
+// matter, and the sums over one sigma-atom (a piece of a unit) are shifted to
+// the larger of all pieces' scales, 2^(pair - 68) with pair the largest sum of
+// the two exponents, before they are added as integers.
 // ---------------------------------------------------------------------------
+// (hi 2^32 + lo) / 2^s rounded to nearest, s >= 0.
+__device__ __forceinline__ void shift_round(long long& hi, uint32_t& lo, int s) {
+  if (s <= 0) return;
+  if (s > 95) {
+    hi = 0;
+    lo = 0;
+    return;
+  }
+  const uint32_t sg = static_cast<uint32_t>(static_cast<int32_t>(static_cast<unsigned long long>(hi) >> 32) >> 31);
+  uint32_t w2 = static_cast<uint32_t>(static_cast<unsigned long long>(hi) >> 32), w1 = static_cast<uint32_t>(hi),
+           w0 = lo;
+  // by s - 1, then one is added and the last bit goes
+  const int t = s - 1, words = t >> 5, bits = t & 31;
+  const uint32_t a = words == 0 ? w0 : (words == 1 ? w1 : w2);
+  const uint32_t b = words == 0 ? w1 : (words == 1 ? w2 : sg), c = words == 0 ? w2 : sg;
+  w0 = __funnelshift_r(a, b, bits);
+  w1 = __funnelshift_r(b, c, bits);
+  w2 = __funnelshift_r(c, sg, bits);
+  asm("add.cc.u32 %0, %0, 1;\n\taddc.cc.u32 %1, %1, 0;\n\taddc.u32 %2, %2, 0;" : "+r"(w0), "+r"(w1), "+r"(w2));
+  lo = __funnelshift_r(w0, w1, 1);
+  w1 = __funnelshift_r(w1, w2, 1);
+  w2 = static_cast<uint32_t>(static_cast<int32_t>(w2) >> 1);
+  hi = static_cast<long long>((static_cast<unsigned long long>(w2) << 32) | w1);
+}
+
 struct Chi64Job {
   const int *unit_tile, *unit_first, *unit_count, *n_units;
   const int* tasks;
   const int* counts;
   int nslab, nqt, P0, prow, nri;
+  int per;  // slabs of a sigma-atom
   const long long* slab_k0;
   const int* slab_len;
-  const int *ex, *ey;
+  const int *ex, *ey;  // exponents [sigma-atom][row]
+  const int* pair;     // [nri][prow]: exponent of element (P, Q)'s integers
   double* chi;
-  unsigned long long* part;  // units of one tile add here; null: a unit is a whole tile
+  unsigned long long* part;
   const double *X, *Y;
   long long ldk;
   struct Tile {
-    int ya, yb, n, cnt, id;
-    const int* list;
+    int ya, yb, n, id;
+    const int* list;  // the piece's entries, and how many the unit has from here on
+    int cnt, left, atom;
   };
   __device__ int items() const { return *n_units; }
+  __device__ void piece(Tile& T) const {
+    T.atom = T.list[0] / per;
+    T.n = 0;
+    for (T.cnt = 0; T.cnt < T.left && T.list[T.cnt] / per == T.atom; ++T.cnt) T.n += slab_len[T.list[T.cnt]] / kChunk;
+  }
   __device__ Tile tile(int u) const {
     Tile T;
     T.id = unit_tile[u];
     T.ya = T.id / nqt * kM;
     T.yb = T.id % nqt * kN2;
-    T.cnt = unit_count[u];
+    T.left = unit_count[u];
     T.list = tasks + static_cast<long long>(T.id) * nslab + unit_first[u];
-    T.n = 0;
-    for (int i = 0; i < T.cnt; ++i) T.n += slab_len[T.list[i]] / kChunk;
+    piece(T);
     return T;
+  }
+  __device__ bool next(Tile& T) const {
+    T.left -= T.cnt;
+    T.list += T.cnt;
+    if (T.left <= 0) return false;
+    piece(T);
+    return true;
   }
   __device__ void half(Tile& T, int side) const { T.yb += side * kN; }
   __device__ int nchunks(const Tile& T) const { return T.n; }
@@ -731,51 +829,67 @@ struct Chi64Job {
         s = fma(X[p * ldk + slab_k0[l[i]] + k], Y[q * ldk + slab_k0[l[i]] + k], s);
     return s;
   }
-  __device__ double value(int id, int p, int q, long long hi, long long lo, int a, int b) const {
-    return (a == kBad || b == kBad) ? direct(id, p, q) : sums_to_double(hi, lo, a + b + kUnit);
+  __device__ int row_exp(const Tile& T, int row) const {
+    return T.ya + row < prow ? ex[static_cast<long long>(T.atom) * prow + T.ya + row] : kOut;
   }
-  __device__ int row_exp(const Tile& T, int row) const { return T.ya + row < prow ? ex[T.ya + row] : kOut; }
-  __device__ int col_exp(const Tile& T, int c) const { return T.yb + c < nri ? ey[T.yb + c] : kOut; }
+  __device__ int col_exp(const Tile& T, int c) const {
+    return T.yb + c < nri ? ey[static_cast<long long>(T.atom) * nri + T.yb + c] : kOut;
+  }
   __device__ void write(long long (&hi)[kCols], uint32_t (&lo)[kCols], const Tile& T, int row0, int lane, int c0,
                         int er, int ec, unsigned long long* stg) const {
     const int p0 = T.ya + row0, q0 = T.yb + c0;
-    if (part) {
-      add_partial(part, false, nri, prow, p0, q0, lane, hi, lo, stg);
-      return;
-    }
-    const int left = prow - p0 - (lane >> 3);
     const Exps es(er, ec);
-#pragma unroll
-    for (int h = 0; h < kCols; h += 8) {
-      unsigned long long v[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        double x = fixed_to_double(hi[h + j], lo[h + j], es.sum(h + j));
-        if (es.in(h + j) && es.bad(h + j)) x = direct(T.id, p0 + lane, q0 + h + j);
-        v[j] = static_cast<unsigned long long>(__double_as_longlong(x));
-      }
-      const int q = q0 + h + (lane & 7);
-      const bool in = q < nri;
-      const long long ld = nri;
-      double* c = chi + (P0 + p0 + (lane >> 3)) * ld + q;
-      by_rows(
-          stg, lane, v, [&](int i) { return in && 4 * i < left ? c[4 * i * ld] : 0.0; },
-          [&](int i, unsigned long long x, double old) {
-            if (in && 4 * i < left) c[4 * i * ld] = old - __longlong_as_double(static_cast<long long>(x));
-          });
-    }
+    const int* e = pair + static_cast<long long>(q0) * prow + p0 + lane;
+    add_partial(part, false, nri, prow, p0, q0, lane,
+                [&](int j, long long& h, uint32_t& l) {
+                  h = hi[j];
+                  l = lo[j];
+                  const int scale = es.sum(j) - kUnit;
+                  if (es.in(j)) {
+                    const int to = e[static_cast<long long>(j) * prow];
+                    if (to != kBad) shift_round(h, l, to - scale);
+                  }
+                },
+                stg);
   }
 };
-__global__ void k_chi64_finish(const Chi64Job j) {
-  const long long n = static_cast<long long>(j.prow) * j.nri;
-  for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-       i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int p = static_cast<int>(i / j.nri), q = static_cast<int>(i % j.nri);
+// pair[q][p] = the largest sum over the sigma-atoms of ex[s][p] + ey[s][q], kBad
+// where one of them is.
+__global__ void __launch_bounds__(256) k_pair_exps(const int* __restrict__ ex, const int* __restrict__ ey, int ns,
+                                                   int prow, int nri, int* __restrict__ pair) {
+  const int p = blockIdx.x * 32 + (threadIdx.x & 31);
+  const int q0 = blockIdx.y * 32 + (threadIdx.x >> 5) * 4;
+  if (p >= prow) return;
+  int m[4] = {kOut, kOut, kOut, kOut};
+  for (int s = 0; s < ns; ++s) {
+    const int a = ex[static_cast<long long>(s) * prow + p];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (q0 + i < nri) {
+        const int b = ey[static_cast<long long>(s) * nri + q0 + i];
+        m[i] = max(m[i], a == kBad || b == kBad ? kBad : a + b);
+      }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (q0 + i < nri) pair[static_cast<long long>(q0 + i) * prow + p] = m[i];
+}
+__global__ void __launch_bounds__(256) k_chi64_finish(const Chi64Job j) {
+  __shared__ int t[32][33];
+  const int q0 = blockIdx.x * 32, p0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int i = ty; i < 32; i += 8)
+    if (q0 + i < j.nri && p0 + tx < j.prow) t[i][tx] = j.pair[static_cast<long long>(q0 + i) * j.prow + p0 + tx];
+  __syncthreads();
+  for (int i = ty; i < 32; i += 8) {
+    const int p = p0 + i, q = q0 + tx;
+    if (p >= j.prow || q >= j.nri) continue;
     const int id = p / kM * j.nqt + q / kN2;
     if (j.counts[id] == 0) continue;
-    const ulonglong2 v = reinterpret_cast<const ulonglong2*>(j.part)[i];
+    const ulonglong2 v = reinterpret_cast<const ulonglong2*>(j.part)[static_cast<long long>(p) * j.nri + q];
+    const int e = t[tx][i];
     j.chi[static_cast<long long>(j.P0 + p) * j.nri + q] -=
-        j.value(id, p, q, static_cast<long long>(v.x), static_cast<long long>(v.y), j.ex[p], j.ey[q]);
+        e == kBad ? j.direct(id, p, q)
+                  : sums_to_double(static_cast<long long>(v.x), static_cast<long long>(v.y), e + kUnit);
   }
 }
 
@@ -905,26 +1019,28 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int t = first; t < n_items && ok; t += step) {
         typename Job::Tile T = job.tile(t);
         job.half(T, side);
-        const int n = job.nchunks(T);
-        typename Job::Iter it;
-        it.init(&job, T);
-        for (int i = 0; i < n; ++i) {
-          if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag)) {
-            ok = false;
-            break;
+        do {
+          const int n = job.nchunks(T);
+          typename Job::Iter it;
+          it.init(&job, T);
+          for (int i = 0; i < n; ++i) {
+            if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag)) {
+              ok = false;
+              break;
+            }
+            uint8_t* st = smem + stage * kStageBytes;
+            mbar_expect_tx(&full[stage], kStageBytes);
+            armed[stage] = true;
+            armed_parity[stage] = phase;
+            const int x = it.next();
+            tma_load_3d(st, &map_a, x, T.ya, 0, &full[stage]);
+            tma_load_3d(st + kS * kABytes, &map_b, x, T.yb, 0, &full[stage]);
+            if (++stage == kStages) {
+              stage = 0;
+              phase ^= 1u;
+            }
           }
-          uint8_t* st = smem + stage * kStageBytes;
-          mbar_expect_tx(&full[stage], kStageBytes);
-          armed[stage] = true;
-          armed_parity[stage] = phase;
-          const int x = it.next();
-          tma_load_3d(st, &map_a, x, T.ya, 0, &full[stage]);
-          tma_load_3d(st + kS * kABytes, &map_b, x, T.yb, 0, &full[stage]);
-          if (++stage == kStages) {
-            stage = 0;
-            phase ^= 1u;
-          }
-        }
+        } while (ok && job.next(T));
       }
       if (!ok) {
         *abort_flag = 1;
@@ -943,53 +1059,55 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t phase = 0, aphase = 1;
     bool ok = true, issued = false;
     for (int t = first; t < n_items && ok; t += step) {
-      const typename Job::Tile T = job.tile(t);
-      const int n = __reduce_max_sync(0xffffffffu, job.nchunks(T));
-      for (int i = 0; i < n && ok; ++i) {
-        ok = mbar_wait_warp(&full[stage], phase, abort_flag);
-        if (!ok) break;
-        tc_fence_after();
-        const bool first = (i % kGroup) == 0, last = (i % kGroup) == kGroup - 1 || i == n - 1;
-        const uint64_t da = desc_sw64(smem_u32(smem + stage * kStageBytes));
-        const uint32_t a_lo = static_cast<uint32_t>(da), hi = static_cast<uint32_t>(da >> 32);
-        const uint32_t b_lo = a_lo + static_cast<uint32_t>((kS * kABytes) >> 4);
+      typename Job::Tile T = job.tile(t);
+      do {
+        const int n = __reduce_max_sync(0xffffffffu, job.nchunks(T));
+        for (int i = 0; i < n && ok; ++i) {
+          ok = mbar_wait_warp(&full[stage], phase, abort_flag);
+          if (!ok) break;
+          tc_fence_after();
+          const bool first = (i % kGroup) == 0, last = (i % kGroup) == kGroup - 1 || i == n - 1;
+          const uint64_t da = desc_sw64(smem_u32(smem + stage * kStageBytes));
+          const uint32_t a_lo = static_cast<uint32_t>(da), hi = static_cast<uint32_t>(da >> 32);
+          const uint32_t b_lo = a_lo + static_cast<uint32_t>((kS * kABytes) >> 4);
 #pragma unroll
-        for (int p = 0; p < kPairs; ++p) {
-          if (first) {
-            ok = mbar_wait_warp(&acc_empty[p], aphase, abort_flag);
-            if (!ok) break;
-            tc_fence_after();
+          for (int p = 0; p < kPairs; ++p) {
+            if (first) {
+              ok = mbar_wait_warp(&acc_empty[p], aphase, abort_flag);
+              if (!ok) break;
+              tc_fence_after();
+            }
+            if (lead) {
+              // digit a of A with digits 2p - a and 2p - a + 1 of B, whose rows
+              // follow one another, into the two accumulators side by side; the
+              // last digit of A only meets digit 0
+              const uint32_t acc = tmu + static_cast<uint32_t>(2 * p * kN);
+#pragma unroll
+              for (int a = 0; a <= 2 * p + 1; ++a)
+#pragma unroll
+                for (int k = 0; k < kSub; ++k) {
+                  const uint32_t da_lo = a_lo + static_cast<uint32_t>((a * kABytes + k * kMmaK * 2) >> 4);
+                  if (a <= 2 * p)
+                    mma_f16_lo(acc, da_lo, b_lo + static_cast<uint32_t>(((2 * p - a) * kBBytes + k * kMmaK * 2) >> 4),
+                               hi, two, (a | k) ? 1u : (first ? 0u : 1u));
+                  else
+                    mma_f16_lo(acc + kN, da_lo, b_lo + static_cast<uint32_t>((k * kMmaK * 2) >> 4), hi, one, 1u);
+                }
+              if (last) mma_commit(&acc_full[p]);
+            }
+            __syncwarp();
+            issued = true;
           }
-          if (lead) {
-            // digit a of A with digits 2p - a and 2p - a + 1 of B, whose rows
-            // follow one another, into the two accumulators side by side; the
-            // last digit of A only meets digit 0
-            const uint32_t acc = tmu + static_cast<uint32_t>(2 * p * kN);
-#pragma unroll
-            for (int a = 0; a <= 2 * p + 1; ++a)
-#pragma unroll
-              for (int k = 0; k < kSub; ++k) {
-                const uint32_t da_lo = a_lo + static_cast<uint32_t>((a * kABytes + k * kMmaK * 2) >> 4);
-                if (a <= 2 * p)
-                  mma_f16_lo(acc, da_lo, b_lo + static_cast<uint32_t>(((2 * p - a) * kBBytes + k * kMmaK * 2) >> 4),
-                             hi, two, (a | k) ? 1u : (first ? 0u : 1u));
-                else
-                  mma_f16_lo(acc + kN, da_lo, b_lo + static_cast<uint32_t>((k * kMmaK * 2) >> 4), hi, one, 1u);
-              }
-            if (last) mma_commit(&acc_full[p]);
-          }
+          if (!ok) break;
+          if (lead) mma_commit(&empty[stage]);
           __syncwarp();
-          issued = true;
+          if (last) aphase ^= 1u;
+          if (++stage == kStages) {
+            stage = 0;
+            phase ^= 1u;
+          }
         }
-        if (!ok) break;
-        if (lead) mma_commit(&empty[stage]);
-        __syncwarp();
-        if (last) aphase ^= 1u;
-        if (++stage == kStages) {
-          stage = 0;
-          phase ^= 1u;
-        }
-      }
+      } while (ok && job.next(T));
     }
     if (!ok && lead) {
       *abort_flag = 1;
@@ -1010,32 +1128,35 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool ok = stall ? mbar_wait_warp(never, 0, abort_flag) : true;
     for (int t = first; t < n_items && ok; t += step) {
       typename Job::Tile T = job.tile(t);
-      const int n = job.nchunks(T);
-      if (n == 0) continue;
+      if (job.nchunks(T) == 0) continue;
       job.half(T, side);
-      // exponents of this lane's row and of column c0 + lane % 16, loaded here:
-      // beside the stores they would be fetched one by one
-      const int er = job.row_exp(T, quad * 32 + lane), ec = job.col_exp(T, c0 + lane % kCols);
-      // value = hi 2^32 + lo: 48 registers for 16 columns
-      long long hi[kCols];
-      uint32_t lo[kCols];
+      do {
+        const int n = job.nchunks(T);
+        // exponents of this lane's row and of column c0 + lane % 16, loaded here:
+        // beside the stores they would be fetched one by one
+        const int er = job.row_exp(T, quad * 32 + lane), ec = job.col_exp(T, c0 + lane % kCols);
+        // value = hi 2^32 + lo: 48 registers for 16 columns
+        long long hi[kCols];
+        uint32_t lo[kCols];
 #pragma unroll
-      for (int j = 0; j < kCols; ++j) {
-        hi[j] = 0;
-        lo[j] = 0;
-      }
-      for (int i = 0; i < n && ok; i += kGroup, aphase ^= 1u) {
-        // pairs 0 and 1 (diagonals 0-3) into hi, 2 and 3 into lo; rolled, for
-        // the instruction cache
+        for (int j = 0; j < kCols; ++j) {
+          hi[j] = 0;
+          lo[j] = 0;
+        }
+        for (int i = 0; i < n && ok; i += kGroup, aphase ^= 1u) {
+          // pairs 0 and 1 (diagonals 0-3) into hi, 2 and 3 into lo; rolled, for
+          // the instruction cache
 #pragma unroll 1
-        for (int p = 0; p < kPairs / 2 && ok; ++p)
-          ok = add_pair<true>(p, p, acc_full, acc_empty, aphase, abort_flag, row_addr, lane, hi, lo);
+          for (int p = 0; p < kPairs / 2 && ok; ++p)
+            ok = add_pair<true>(p, p, acc_full, acc_empty, aphase, abort_flag, row_addr, lane, hi, lo);
 #pragma unroll 1
-        for (int p = 0; p < kPairs / 2 && ok; ++p)
-          ok = add_pair<false>(kPairs / 2 + p, p, acc_full, acc_empty, aphase, abort_flag, row_addr, lane, hi, lo);
-      }
+          for (int p = 0; p < kPairs / 2 && ok; ++p)
+            ok = add_pair<false>(kPairs / 2 + p, p, acc_full, acc_empty, aphase, abort_flag, row_addr, lane, hi, lo);
+        }
+        if (!ok) break;
+        job.write(hi, lo, T, quad * 32, lane, c0, er, ec, stg);
+      } while (job.next(T));
       if (!ok) break;
-      job.write(hi, lo, T, quad * 32, lane, c0, er, ec, stg);
     }
     if (!ok) {
       *abort_flag = 1;
@@ -1111,6 +1232,16 @@ void launch_emu_prep(EmuOp& op, const EmuSrc& s, cudaStream_t st) {
     emu::k_col_exps<<<dim3(gx, gy), 256, 0, st>>>(s.src, s.ld, s.rows, s.K, be);
     emu::k_prep_cols<<<dim3(gx, op.kp / 64), 256, 0, st>>>(s.src, s.ld, s.rows, s.K, op.kp, be, dig, op.exps);
   }
+}
+
+void launch_emu_prep_segments(EmuOp& op, const EmuSrc& s, const long long* seg, int n_seg, cudaStream_t st) {
+  op.s = s;
+  op.stride_rows = s.rows;
+  op.kp = s.K;
+  if (s.rows <= 0 || n_seg <= 0) return;
+  const unsigned grid = static_cast<unsigned>(std::min<long long>(s.rows * n_seg, 152 * 64));
+  emu::k_prep_segments<<<grid, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, seg, n_seg, static_cast<__half*>(op.dig),
+                                             op.exps);
 }
 
 // Sums go out as integers and a second kernel rounds them, also where K is not
@@ -1226,15 +1357,14 @@ int launch_chi64(const EmuOp& x, const EmuOp& y, const Chi64Args& c, int* err_fl
       make_digit_map(&my, y.dig, y.kp, y.s.rows, y.stride_rows, kEmuSlices, emu::kChunk, emu::kN, kEmuSlices))
     return -2;
   emu::Chi64Job j{c.units.u_tile, c.units.u_first, c.units.u_count, c.units.n_units, c.tasks, c.counts, c.nslab,
-                  c.nqt, c.P0, c.prow, c.nri, c.slab_k0, c.slab_len, x.exps, y.exps, c.chi,
+                  c.nqt, c.P0, c.prow, c.nri, c.per, c.slab_k0, c.slab_len, x.exps, y.exps, c.pair, c.chi,
                   static_cast<unsigned long long*>(c.part), x.s.src, y.s.src, x.s.ld};
-  if (c.part) cudaMemsetAsync(c.part, 0, static_cast<size_t>(c.prow) * c.nri * 16, st);
+  cudaMemsetAsync(c.part, 0, static_cast<size_t>(c.prow) * c.nri * 16, st);
+  const unsigned gp = static_cast<unsigned>((c.prow + 31) / 32), gq = static_cast<unsigned>((c.nri + 31) / 32);
+  emu::k_pair_exps<<<dim3(gp, gq), 256, 0, st>>>(x.exps, y.exps, c.nslab / c.per, c.prow, c.nri, c.pair);
   const int rc = emu::launch(mx, my, j, INT32_MAX, err_flag, st);
   if (rc) return rc;
-  if (c.part) {
-    const long long blocks = (static_cast<long long>(c.prow) * c.nri + 255) / 256;
-    emu::k_chi64_finish<<<static_cast<unsigned>(std::min<long long>(blocks, 152 * 16)), 256, 0, st>>>(j);
-  }
+  emu::k_chi64_finish<<<dim3(gq, gp), 256, 0, st>>>(j);
   return 0;
 }
 

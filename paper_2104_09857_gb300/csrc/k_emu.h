@@ -78,6 +78,11 @@ size_t emu_gemm_ws_bytes(long long m, long long n, int K, int nz = 1);
 int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, int* err_flag,
                     cudaStream_t st);
 
+// The same with an exponent per segment of a row, for step C: segment i starts at
+// element seg[i] of the row (a multiple of 64; in device memory).  s.K is a
+// multiple of 64, op.exps holds n_seg * s.rows ints, [segment][row].
+void launch_emu_prep_segments(EmuOp& op, const EmuSrc& s, const long long* seg, int n_seg, cudaStream_t st);
+
 // One panel problem of the FP64 steps A / B: digits of the panel's rows from
 // p_row0, of G's rows (gathered on its lambda functions) from g_row0.
 struct PanelTask64 {
@@ -114,17 +119,18 @@ struct Panel64Args {
   int nao;
 };
 int launch_panel64(const Panel64Args& p, int* err_flag, cudaStream_t st);
-// Step C over work units (k_tc.h, launch_plan_units) of 128 x 128 tiles.  part:
-// 16 bytes per (X row, RI function) of partial sums, or null when a unit is a
-// whole tile.
+// Step C over work units (k_tc.h, launch_plan_units) of 128 x 128 tiles, operands
+// with an exponent per sigma-atom (`per` slabs).  Scratch per (X row, RI
+// function): part 16 bytes of partial sums, pair 4 of their exponent.
 struct Chi64Args {
   UnitScratch units;
   const int *tasks, *counts;
-  int nslab, nqt, P0, prow, nri;
+  int nslab, nqt, P0, prow, nri, per;
   const long long* slab_k0;
   const int* slab_len;
   double* chi;
   void* part;
+  int* pair;
 };
 int launch_chi64(const EmuOp& x, const EmuOp& y, const Chi64Args& c, int* err_flag, cudaStream_t st);
 
@@ -133,6 +139,8 @@ int launch_chi64(const EmuOp& x, const EmuOp& y, const Chi64Args& c, int* err_fl
 int emu_begin(gw_ctx* ctx, cudaStream_t st);
 int emu_flag(gw_ctx* ctx, int** err);  // the error flag of the launchers
 int emu_prep(gw_ctx* ctx, const char* name, const EmuSrc& s, EmuOp* op, cudaStream_t st);
+int emu_prep_segments(gw_ctx* ctx, const char* name, const EmuSrc& s, const long long* seg, int n_seg, EmuOp* op,
+                      cudaStream_t st);
 int emu_mm(gw_ctx* ctx, const EmuOp& A, const EmuOp& B, const EmuGemm& g, cudaStream_t st);
 // Product of two matrices.  Operands beyond 4 GB of digits go in row chunks;
 // keep (may be null): on a later call with the same A, its digits are reused

@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 from oracle import chi as oc  # noqa: E402
-from synth import make_case  # noqa: E402
+from synth import System, case_from_system, make_case  # noqa: E402
 
 
 @pytest.fixture(scope="module")
@@ -58,3 +58,40 @@ def test_cholesky_pivots_are_rounded_roots(pkg):
         w = ctx.chi_to_w(np.zeros((1, n, n)), np.diag(v), np.ones((1, 1)), np.ones((1, 1))).cpu().numpy()[0]
     assert not np.any(w - np.diag(np.diag(w)))
     assert np.abs(np.diag(w) / v).max() <= 3 * 2.0 ** -53 * (1 + 1e-9)
+
+
+def test_chi_of_distant_functions(pkg):
+    """Every element of chi along a chain of 33 Angstrom, over which chi falls by
+    1e-10, to an FP64 sum's accuracy: with S = sum |X| |Y| (Green's functions of
+    positive orbitals, so that their sums do not cancel), n operations of
+    rounding 2^-53 each err by n 2^-53 S; chi is K = n_AO^2 of them, X and Y each
+    n_AO + n_AO (G), the oracle's own sums the same again."""
+    n, rng = 24, np.random.default_rng(9)
+    sysm = System("chain", np.array([[1.4 * i, 0.0, 0.0] for i in range(n)]), ["C"] * n)
+    sysm.n_ao = np.full(n, 2, dtype=np.int32)
+    sysm.n_ri = np.full(n, 2, dtype=np.int32)
+    case = case_from_system(sysm, 1, 0.0, 7)
+    nao, tau = 2 * n, 0.5
+    x = np.repeat(sysm.xyz[:, 0], 2)
+    at = np.concatenate([sysm.xyz[:, 0], sysm.xyz[:, 0]])  # one occupied, one virtual orbital per atom
+    c = rng.uniform(0.5, 1.0, (nao, nao)) * np.exp(-0.8 * np.abs(x[:, None] - at[None]))
+    eps = np.concatenate([np.linspace(-1.0, -0.2, n), np.linspace(0.2, 1.0, n)])
+    t = case.t3c
+    d = oc.dense_three_center(sysm.n_ao, sysm.n_ri, t.blocks, t.offsets, t.data)
+    h = c * np.exp(-0.5 * tau * np.abs(eps))
+    go, gv = h[:, :n] @ h[:, :n].T, h[:, n:] @ h[:, n:].T
+
+    def sums(t3):
+        m = np.einsum("ml,lsp->msp", go, t3).reshape(nao * nao, -1)
+        q = np.einsum("sl,mlq->msq", gv, t3).reshape(nao * nao, -1)
+        return m.T @ q
+
+    ref, bound = -sums(d), sums(np.abs(d))
+    with pkg.Context(0) as ctx:
+        ctx.set_basis(sysm.xyz, sysm.n_ao, sysm.n_ri)
+        ctx.set_3c_tensor(t.blocks, t.data)
+        ctx.set_greens(c, eps, n, 0.0, np.array([tau]))
+        got = ctx.chi_tau(0.0, "fp64").cpu().numpy()[0]
+    up = np.arange(nao)[:, None] // 2 <= np.arange(nao)[None] // 2
+    assert bound[0, -1] <= 1e-9 * bound.max()
+    assert (np.abs(got - ref)[up] / bound[up]).max() <= 2 * (nao * nao + 4 * nao) * 2.0 ** -53
