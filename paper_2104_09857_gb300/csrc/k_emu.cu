@@ -190,28 +190,37 @@ __global__ void __launch_bounds__(256) k_prep_rows(const double* __restrict__ sr
 
 // Rows of a row-major matrix with an exponent per segment of a row: segment i
 // starts at element seg[i] (a multiple of 64) and ends where the next begins.
-// exps[i * rows + r].  One CTA per segment of a row.
+// exps[i * rows + r].  kWarps (1 or 8) warps per segment of a row, which they
+// read twice (the second time from cache).
+template <int kWarps>
 __global__ void __launch_bounds__(256) k_prep_segments(const double* __restrict__ src, long long ld, long long rows,
                                                        int K, const long long* __restrict__ seg, int n_seg,
                                                        __half* __restrict__ dig, int* __restrict__ exps) {
+  constexpr int kPer = 8 / kWarps, kN = 32 * kWarps;  // segments of a CTA, threads of a segment
   __shared__ int red[8];
-  for (long long i = blockIdx.x; i < rows * n_seg; i += gridDim.x) {
+  const int warp = threadIdx.x >> 5, t = threadIdx.x % kN;
+  for (long long i0 = static_cast<long long>(blockIdx.x) * kPer; i0 < rows * n_seg;
+       i0 += static_cast<long long>(gridDim.x) * kPer) {
+    const long long i = i0 + warp / kWarps;
+    if (i >= rows * n_seg) continue;  // kPer > 1: no barrier below
     const long long r = i / n_seg;
     const int s = static_cast<int>(i - r * n_seg);
     const long long k0 = seg[s];
     const int len = static_cast<int>((s + 1 < n_seg ? seg[s + 1] : K) - k0);
     const double* x = src + r * ld + k0;
     int be = 0;
-    for (int k = threadIdx.x; k < len; k += 256) be = max(be, biased_exp(x[k]));
+    for (int k = t; k < len; k += kN) be = max(be, biased_exp(x[k]));
     be = __reduce_max_sync(0xffffffffu, be);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = be;
-    __syncthreads();
+    if (kWarps > 1) {
+      __syncthreads();
+      if (t % 32 == 0) red[warp] = be;
+      __syncthreads();
 #pragma unroll
-    for (int w = 0; w < 8; ++w) be = max(be, red[w]);
+      for (int w = 0; w < kWarps; ++w) be = max(be, red[w]);
+    }
     const int e = row_exp(be);
-    if (threadIdx.x == 0) exps[s * rows + r] = e;
-    for (int k = 8 * threadIdx.x; k < len; k += 8 * 256) {
+    if (t == 0) exps[s * rows + r] = e;
+    for (int k = 8 * t; k < len; k += 8 * kN) {
       double v[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] = x[k + j];
@@ -861,6 +870,7 @@ __global__ void __launch_bounds__(256) k_pair_exps(const int* __restrict__ ex, c
   const int q0 = blockIdx.y * 32 + (threadIdx.x >> 5) * 4;
   if (p >= prow) return;
   int m[4] = {kOut, kOut, kOut, kOut};
+#pragma unroll 4
   for (int s = 0; s < ns; ++s) {
     const int a = ex[static_cast<long long>(s) * prow + p];
 #pragma unroll
@@ -880,16 +890,25 @@ __global__ void __launch_bounds__(256) k_chi64_finish(const Chi64Job j) {
   for (int i = ty; i < 32; i += 8)
     if (q0 + i < j.nri && p0 + tx < j.prow) t[i][tx] = j.pair[static_cast<long long>(q0 + i) * j.prow + p0 + tx];
   __syncthreads();
-  for (int i = ty; i < 32; i += 8) {
-    const int p = p0 + i, q = q0 + tx;
-    if (p >= j.prow || q >= j.nri) continue;
-    const int id = p / kM * j.nqt + q / kN2;
-    if (j.counts[id] == 0) continue;
-    const ulonglong2 v = reinterpret_cast<const ulonglong2*>(j.part)[static_cast<long long>(p) * j.nri + q];
-    const int e = t[tx][i];
-    j.chi[static_cast<long long>(j.P0 + p) * j.nri + q] -=
-        e == kBad ? j.direct(id, p, q)
-                  : sums_to_double(static_cast<long long>(v.x), static_cast<long long>(v.y), e + kUnit);
+  const int q = q0 + tx;
+  ulonglong2 v[4];
+  double old[4];
+  bool on[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int p = p0 + ty + 8 * i;
+    on[i] = p < j.prow && q < j.nri && j.counts[p / kM * j.nqt + q / kN2] != 0;
+    if (!on[i]) continue;
+    v[i] = reinterpret_cast<const ulonglong2*>(j.part)[static_cast<long long>(p) * j.nri + q];
+    old[i] = j.chi[static_cast<long long>(j.P0 + p) * j.nri + q];
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (!on[i]) continue;
+    const int p = p0 + ty + 8 * i, e = t[tx][ty + 8 * i];
+    j.chi[static_cast<long long>(j.P0 + p) * j.nri + q] =
+        old[i] - (e == kBad ? j.direct(p / kM * j.nqt + q / kN2, p, q)
+                            : sums_to_double(static_cast<long long>(v[i].x), static_cast<long long>(v[i].y), e + kUnit));
   }
 }
 
@@ -1239,9 +1258,14 @@ void launch_emu_prep_segments(EmuOp& op, const EmuSrc& s, const long long* seg, 
   op.stride_rows = s.rows;
   op.kp = s.K;
   if (s.rows <= 0 || n_seg <= 0) return;
-  const unsigned grid = static_cast<unsigned>(std::min<long long>(s.rows * n_seg, 152 * 64));
-  emu::k_prep_segments<<<grid, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, seg, n_seg, static_cast<__half*>(op.dig),
-                                             op.exps);
+  __half* dig = static_cast<__half*>(op.dig);
+  const bool wide = s.K / n_seg >= 2048;  // a CTA per segment, else a warp
+  const long long blocks = wide ? s.rows * n_seg : (s.rows * n_seg + 7) / 8;
+  const unsigned grid = static_cast<unsigned>(std::min<long long>(blocks, 152 * 64));
+  if (wide)
+    emu::k_prep_segments<8><<<grid, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, seg, n_seg, dig, op.exps);
+  else
+    emu::k_prep_segments<1><<<grid, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, seg, n_seg, dig, op.exps);
 }
 
 // Sums go out as integers and a second kernel rounds them, also where K is not
