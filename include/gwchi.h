@@ -482,6 +482,9 @@ int gw_get_stats(const gw_ctx* ctx, gw_stats* out);
  * Fault-injection hooks for tests (no effect on results when 0):
  *   "test_fail_alloc"  1: the next new device work buffer fails to allocate
  *                      (the call returns GW_ERR_OOM; the hook then clears)
+ *   "test_device_bytes"  what the work buffers and the panels' digits of the
+ *                      context may hold together (0: no limit); allocations
+ *                      beyond fail as on a device of that size
  *   "test_stall_tc"    1: in gw_chi_tau, every tensor-core kernel waits first
  *                      on a dependency that is never met; its bounded waits
  *                      expire after about 2 s and the call returns

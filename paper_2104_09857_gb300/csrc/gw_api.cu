@@ -56,6 +56,13 @@ int fail(gw_ctx* ctx, int code, const std::string& msg) {
   return code;
 }
 
+// device bytes in the named buffers and the panels' digits
+double held_bytes(const gw_ctx* ctx) {
+  double b = ctx->d_pd ? (double)ctx->pd_bytes : 0.0;
+  for (const auto& kv : ctx->work) b += (double)kv.second.second;
+  return b;
+}
+
 // named device scratch buffer, grown on demand
 int ws(gw_ctx* ctx, const char* name, size_t bytes, void** out) {
   auto& wb = ctx->work;
@@ -72,14 +79,18 @@ int ws(gw_ctx* ctx, const char* name, size_t bytes, void** out) {
   void* p = nullptr;
   if (bytes > 0 && ctx->test_fail_alloc) {
     ctx->test_fail_alloc = 0;
+    ctx->alloc_injected = true;
     ctx->err = std::string("cudaMalloc of work buffer '") + name + "' (" + std::to_string(bytes) +
                " bytes): injected failure (option test_fail_alloc)";
     return GW_ERR_OOM;
   }
   if (bytes > 0) {
-    cudaError_t e = cudaMalloc(&p, bytes);
+    cudaError_t e = cudaErrorMemoryAllocation;
+    if (ctx->test_device_bytes == 0.0 || held_bytes(ctx) + (double)bytes <= ctx->test_device_bytes)
+      e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
+      ctx->alloc_injected = false;
       ctx->err = std::string("cudaMalloc of work buffer '") + name + "' (" +
                  std::to_string(bytes) + " bytes): " + cudaGetErrorString(e);
       return GW_ERR_OOM;
@@ -866,6 +877,8 @@ int ensure_panel_digits(gw_ctx* ctx) {
   const size_t bytes = gw::emu_dig_bytes(rows, kmax);
   size_t free_b = 0, total_b = 0;
   cudaMemGetInfo(&free_b, &total_b);
+  if (ctx->test_device_bytes > 0.0)
+    free_b = (size_t)std::max(0.0, std::min((double)free_b, ctx->test_device_bytes - held_bytes(ctx)));
   const double operands = std::min(ctx->batch_bytes, (double)kDigitElem * 2.0 * ctx->nri * ctx->naop * (double)ctx->nao);
   const double need = (double)bytes + 8.0 * rows + operands + 32.0 * ctx->nri * (double)ctx->nri +
                       64.0 * ctx->nao * (double)ctx->nao + 1e9;
@@ -877,6 +890,7 @@ int ensure_panel_digits(gw_ctx* ctx) {
     return GW_OK;
   }
   ctx->d_pd = dig;
+  ctx->pd_bytes = bytes + (size_t)rows * sizeof(int);
   ctx->d_pd_exps = static_cast<int*>(exps);
   ctx->pd_rows = rows;
   ctx->pd_kp = kp;
@@ -892,8 +906,10 @@ int ensure_panel_digits(gw_ctx* ctx) {
   long long* d_row0;
   int *d_be, rc;
   if ((rc = upload(ctx, "pd_desc", pd, &d_desc)) || (rc = upload(ctx, "pd_row0", row0, &d_row0)) ||
-      (rc = wsT(ctx, "pd_be", (size_t)rows, &d_be)))
-    return rc;
+      (rc = wsT(ctx, "pd_be", (size_t)rows, &d_be))) {
+    free_panel_digits(ctx);
+    return gw::memory_short(ctx, rc) ? GW_OK : rc;
+  }
   gw::launch_panel_digits(ctx->d_panel64, d_desc, d_row0, (int)pd.size(), max_n, kmax, rows, kp, d_be, ctx->d_pd,
                           ctx->d_pd_exps, ctx->stream);
   GW_CHECK_LAUNCH();
@@ -902,7 +918,21 @@ int ensure_panel_digits(gw_ctx* ctx) {
   return GW_OK;
 }
 
+// Everything that only the digit products need goes back, and the call goes on
+// with the CUDA-core kernels: what an allocation that fails on the digit route
+// turns into.  False where it was the test hook's failure, which is reported.
+bool leave_digits(gw_ctx* ctx, int rc) {
+  if (!gw::memory_short(ctx, rc)) return false;
+  cudaStreamSynchronize(ctx->stream);
+  gw::work_trim(ctx, "w.dig.", 0);
+  gw::work_trim(ctx, "d64_", 0);
+  free_panel_digits(ctx);
+  ctx->err.clear();
+  return true;
+}
+
 // One batch in FP64 by digit products.  op_o, op_v: digits of G^occ, G^virt.
+// GW_ERR_OOM leaves acc as it was.
 int chi_one_batch_digits(gw_ctx* ctx, const Batch& b, const double* g_occ, const double* g_virt,
                          const gw::EmuOp& op_o, const gw::EmuOp& op_v, double thr, double* acc,
                          std::vector<double>& fc_host, size_t batch_idx) {
@@ -2089,6 +2119,7 @@ int tc_finish_tau(gw_ctx* ctx, const std::vector<unsigned long long>& h, std::ve
 }  // namespace
 
 namespace gw {
+bool memory_short(const gw_ctx* ctx, int rc) { return rc == GW_ERR_OOM && !ctx->alloc_injected; }
 int plan_bn_lists(gw_ctx* ctx, double thr) {
   if (ctx->d_t3f)
     return fail(ctx, GW_ERR_UNSUPPORTED,
@@ -2404,6 +2435,11 @@ int gw_set_option(gw_ctx* ctx, const char* key, double value) {
     ctx->test_fail_alloc = value != 0.0;
     return GW_OK;
   }
+  if (!strcmp(key, "test_device_bytes")) {
+    if (!(value >= 0)) return fail(ctx, GW_ERR_INVALID_ARG, "test_device_bytes must be >= 0");
+    ctx->test_device_bytes = value;
+    return GW_OK;
+  }
   if (!strcmp(key, "test_stall_tc")) {
     ctx->test_stall = value != 0.0;
     return GW_OK;
@@ -2547,7 +2583,7 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
     ctx->last_precision = precision;
   }
   if (f64 && (rc = ensure_panel_digits(ctx))) return rc;
-  const bool digits = f64 && ctx->pd_ok;
+  bool digits = f64 && ctx->pd_ok;
   if (!f64 && !tcpath && (rc = ensure_panel32(ctx))) return rc;
   if (tcpath && (rc = ensure_pt(ctx, precision == GW_BF16X6 ? 3 : 2, f16))) return rc;
   const int nao = ctx->nao, nri = ctx->nri, n_at = ctx->n_at;
@@ -2650,9 +2686,11 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
       s.src = go;
       s.ld = s.rows = nao;
       s.K = nao;
-      if ((rc = gw::emu_prep(ctx, "go", s, &op_o, ctx->stream))) return rc;
+      rc = gw::emu_prep(ctx, "go", s, &op_o, ctx->stream);
       s.src = gv;
-      if ((rc = gw::emu_prep(ctx, "gv", s, &op_v, ctx->stream))) return rc;
+      if (!rc) rc = gw::emu_prep(ctx, "gv", s, &op_v, ctx->stream);
+      if (rc && !leave_digits(ctx, rc)) return rc;
+      digits = rc == GW_OK;
       ctx->stats.kernel_launches += 2;
     }
     double fa = 0.0, fb = 0.0;
@@ -2676,8 +2714,10 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
       }
       fa += ba;
       fb += bb;
+      if (digits && (rc = chi_one_batch_digits(ctx, b, go, gv, op_o, op_v, thr, acc, fc, bi)))
+        digits = !leave_digits(ctx, rc);
       if (digits)
-        rc = chi_one_batch_digits(ctx, b, go, gv, op_o, op_v, thr, acc, fc, bi);
+        ;  // done, or rc says why not
       else if (f64)
         rc = chi_one_batch<double>(ctx, b, go, gv, ctx->d_panel64, thr, acc, fc, precision, bi);
       else if (tcpath)

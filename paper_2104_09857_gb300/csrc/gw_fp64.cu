@@ -138,6 +138,7 @@ int greens_fp64(gw_ctx* ctx, const gw_ctx& mol, double tau, double* cso, double*
     return GW_OK;
   }
   launch_scale_orbitals(mol.d_C, mol.d_eps, n, occ, mol.mu, tau, cso, csv, st);
+  // (where their digits do not fit, on the FP64 pipes after all)
   for (int v = 0; v < 2; ++v) {
     EmuSrc s;
     s.src = v ? csv : cso;
@@ -146,11 +147,16 @@ int greens_fp64(gw_ctx* ctx, const gw_ctx& mol, double tau, double* cso, double*
     s.rows = n;
     EmuOp op;
     int rc = emu_prep(ctx, "orbitals", s, &op, st);
-    if (rc) return rc;
     EmuGemm g;
     g.C = v ? g_virt : g_occ;
     g.ldc = n;
-    if ((rc = emu_mm(ctx, op, op, g, st))) return rc;
+    if (!rc) rc = emu_mm(ctx, op, op, g, st);
+    if (memory_short(ctx, rc)) {
+      ctx->err.clear();
+      launch_greens(mol.d_C, mol.d_eps, n, occ, mol.mu, tau, cso, csv, g_occ, g_virt, st);
+      return GW_OK;
+    }
+    if (rc) return rc;
   }
   return GW_OK;
 }

@@ -107,6 +107,9 @@ int plan_bn_lists(gw_ctx* ctx, double thr);
 // FP64 calls ("w." names) stay only while they are small beside the operand
 // batches of chi.
 int work_buffer(gw_ctx* ctx, const char* name, size_t bytes, void** out);
+// rc is an allocation that failed, and not for the test hook: what needs less
+// memory may be tried instead.
+bool memory_short(const gw_ctx* ctx, int rc);
 void work_trim(gw_ctx* ctx, const char* prefix, size_t keep);
 constexpr size_t kWorkKeep = size_t(1) << 30;
 
@@ -215,6 +218,7 @@ struct gw_ctx {
   // the panels as digits for the FP64 products (row pd_row0[owner] + n)
   bool pd_ok = false;
   void* d_pd = nullptr;
+  size_t pd_bytes = 0;
   int* d_pd_exps = nullptr;
   long long pd_rows = 0;
   int pd_kp = 0;
@@ -305,8 +309,10 @@ struct gw_ctx {
   std::map<std::string, std::pair<void*, std::vector<char>>> uploaded;
   std::vector<cudaEvent_t> events;
 
-  // test hooks (options "test_fail_alloc", "test_stall_tc")
+  // test hooks (options "test_fail_alloc", "test_device_bytes", "test_stall_tc")
   int test_fail_alloc = 0;  // the next new work-buffer allocation fails
+  bool alloc_injected = false;     // the last allocation that failed was that one
+  double test_device_bytes = 0.0;  // what the named buffers may hold (0: no limit)
   int test_stall = 0;       // tensor-core kernels wait on a dependency never met
 
   gw_stats stats{};

@@ -95,3 +95,39 @@ def test_chi_of_distant_functions(pkg):
     up = np.arange(nao)[:, None] // 2 <= np.arange(nao)[None] // 2
     assert bound[0, -1] <= 1e-9 * bound.max()
     assert (np.abs(got - ref)[up] / bound[up]).max() <= 2 * (nao * nao + 4 * nao) * 2.0 ** -53
+
+
+def _digits(ctx):
+    """The last call's products were digits (36 of them per multiply-add)."""
+    s = ctx.stats()
+    return s["flops_issued"] > 16 * s["flops_useful"]
+
+
+def test_chi_without_room_for_a_batch_of_digits(pkg):
+    """A batch whose digits do not fit goes through the CUDA-core kernels; the
+    call fails only where their operands do not fit either."""
+    from paper_2104_09857_gb300 import _lib
+
+    case = make_case("benzene", n_tau=2)
+    ref = oc.chi_dense(case)
+    seen = []
+    for limit in 2e6 * 1.25 ** np.arange(24):
+        with pkg.Context(0) as ctx:
+            ctx.load_case(case)
+            ctx.set_option("batch_atoms", 1)
+            ctx.chi_tau(case.thr, "fp64", 0, 1)  # the panels' digits are there
+            ctx.set_option("batch_atoms", 0)
+            ctx.set_option("test_device_bytes", limit)
+            try:
+                got = ctx.chi_tau(case.thr, "fp64").cpu().numpy()
+            except _lib.GwError as e:
+                assert e.code == -5  # GW_ERR_OOM
+                seen.append("none")
+            else:
+                assert _rel(got, ref) <= 1e-10
+                seen.append("digits" if _digits(ctx) else "cores")
+            ctx.set_option("test_device_bytes", 0)
+            got = ctx.chi_tau(case.thr, "fp64").cpu().numpy()
+            assert _rel(got, ref) <= 1e-10 and _digits(ctx)
+    order = [k for i, k in enumerate(seen) if i == 0 or seen[i - 1] != k]
+    assert order == ["none", "cores", "digits"], seen
