@@ -74,7 +74,9 @@ typedef struct gw_stats {
                             counted)                                              */
   double flops_a, flops_b, flops_c;  /* the same, per step                       */
   double flops_issued;   /* arithmetic the kernels actually issued (padded tiles,
-                            all split products)                                   */
+                            all split products; GW_FP64: 36 digit products per
+                            product, or one where the digits did not fit and the
+                            CUDA-core kernels ran)                                */
   double ms_greens, ms_step_ab, ms_filter, ms_step_c, ms_total; /* last chi call */
   double ms_step_c_kernel; /* device time of the step-C kernels alone           */
   long long c_launches;  /* step-C kernel launches in the last call            */

@@ -854,9 +854,59 @@ int chi_one_batch(gw_ctx* ctx, const Batch& b, const T* g_occ, const T* g_virt, 
 // Bytes of an operand element there: FP64 and eight 16-bit digits.
 constexpr size_t kDigitElem = 8 + 2 * gw::kEmuSlices;
 
+// Where every panel's lambda functions are all of them, G's own digits serve
+// steps A and B; else they are gathered per panel.
+bool whole_panels(const gw_ctx* ctx) {
+  for (const PanelDesc& d : ctx->panels)
+    if (d.K != 0 && d.K != ctx->nao) return false;
+  return true;
+}
+
+// Bytes that the digit route of gw_chi_tau takes beside the panels' digits (of
+// pitch kp) and the buffers that the context already holds, which it uses again.
+double digit_route_bytes(gw_ctx* ctx, int kp) {
+  const double nao = ctx->nao, nri = ctx->nri, n_at = ctx->n_at;
+  std::map<std::string, double> need;
+  const auto want = [&](const char* name, double bytes) { need[name] = std::max(need[name], bytes); };
+  const bool whole = whole_panels(ctx);
+  for (const Batch& b : plan_batches(ctx, kDigitElem, ctx->batch_bytes, 0)) {
+    const double prow = b.P1 - b.P0, k = (double)b.Kb, ns = b.s1 - b.s0, R = ctx->ao_off[b.s1] - ctx->ao_off[b.s0];
+    want("X", 8 * prow * k);
+    want("Y", 8 * nri * k);
+    want("w.dig.X", 2.0 * gw::kEmuSlices * prow * k);
+    want("w.dig.Y", 2.0 * gw::kEmuSlices * nri * k);
+    want("w.dig.X.e", 4 * prow * ns);
+    want("w.dig.Y.e", 4 * nri * ns);
+    if (!whole) want("d64_gg", 2.0 * gw::kEmuSlices * std::max(ns * nao, n_at * R) * kp);
+    want("d64_part", 16 * prow * nri);
+    want("d64_pair", 4 * prow * nri);
+    const double tiles = std::ceil(prow / gw::kEmuTileM) * std::ceil(nri / gw::kEmuTileN), cap = tiles * b.nslab;
+    want("tasks", 4 * cap);
+    for (const char* u : {"u_ttile", "u_tfirst", "u_tcount", "u_tkey", "u_tile", "u_first", "u_count"}) want(u, 4 * cap);
+    want("bx", ns * n_at * n_at);
+    want("by", ns * n_at * n_at);
+    want("fx", ns * n_at * prow / gw::kEmuTileM);
+    want("fy", ns * n_at * nri / gw::kEmuTileN);
+  }
+  const double g_digits = 2.0 * gw::kEmuSlices * nao * gw::emu_kp(ctx->nao);
+  for (const char* g : {"w.dig.go", "w.dig.gv", "w.dig.orbitals"}) want(g, g_digits);
+  for (const char* g : {"g_occ", "g_virt", "cso", "csv"}) want(g, 8 * nao * nao);
+  for (const char* c : {"chi_acc", "chi_stage"}) want(c, 8 * nri * nri);
+  want("w.part", 96e6);  // partial sums of G's products (k_emu.cu)
+  double more = 0.0;
+  for (const auto& n : need) {
+    const auto it = ctx->work.find(n.first);
+    // a buffer that is too small is freed before it grows
+    const double have = it == ctx->work.end() ? 0.0 : (double)it->second.second;
+    if (have < n.second) more += n.second - have;
+  }
+  return more;
+}
+
 // ctx->pd_ok afterwards: the digits are there.  They take 16 bytes per panel
-// element beside the FP64 pool's 8; where that and one batch of operands do
-// not fit in free memory the call stays on the CUDA-core kernels.
+// element beside the FP64 pool's 8; where that and the batches do not fit in
+// free memory the call stays on the CUDA-core kernels (gw_stats: flops_issued
+// counts 36 products per multiply-add with the digits, one without).
 int ensure_panel_digits(gw_ctx* ctx) {
   if (ctx->pd_ok) return GW_OK;
   free_panel_digits(ctx);
@@ -879,9 +929,8 @@ int ensure_panel_digits(gw_ctx* ctx) {
   cudaMemGetInfo(&free_b, &total_b);
   if (ctx->test_device_bytes > 0.0)
     free_b = (size_t)std::max(0.0, std::min((double)free_b, ctx->test_device_bytes - held_bytes(ctx)));
-  const double operands = std::min(ctx->batch_bytes, (double)kDigitElem * 2.0 * ctx->nri * ctx->naop * (double)ctx->nao);
-  const double need = (double)bytes + 8.0 * rows + operands + 32.0 * ctx->nri * (double)ctx->nri +
-                      64.0 * ctx->nao * (double)ctx->nao + 1e9;
+  // (1 GB to spare for the tables of the plan and the caller)
+  const double need = (double)bytes + 8.0 * rows + digit_route_bytes(ctx, kp) + (ctx->test_device_bytes > 0.0 ? 0 : 1e9);
   if (need > (double)free_b) return GW_OK;
   void *dig = nullptr, *exps = nullptr;
   if (cudaMalloc(&dig, bytes) != cudaSuccess || cudaMalloc(&exps, (size_t)rows * sizeof(int)) != cudaSuccess) {
@@ -947,9 +996,7 @@ int chi_one_batch_digits(gw_ctx* ctx, const Batch& b, const double* g_occ, const
   if ((rc = wsT(ctx, "X", (size_t)prow * Kb, &X)) || (rc = wsT(ctx, "Y", (size_t)nri * Kb, &Y))) return rc;
   GW_TRY(cudaMemsetAsync(X, 0, (size_t)prow * Kb * sizeof(double), ctx->stream));
   GW_TRY(cudaMemsetAsync(Y, 0, (size_t)nri * Kb * sizeof(double), ctx->stream));
-  // where every panel's lambda functions are all of them, G's own digits serve
-  bool whole = true;
-  for (const PanelDesc& d : ctx->panels) whole = whole && (d.K == 0 || d.K == nao);
+  const bool whole = whole_panels(ctx);
   const int r0 = ctx->ao_off[b.s0], R = ctx->ao_off[b.s1] - r0;
   std::vector<gw::PanelTask64> tasks[2];
   std::vector<int4> tiles[2];

@@ -131,3 +131,31 @@ def test_chi_without_room_for_a_batch_of_digits(pkg):
             assert _rel(got, ref) <= 1e-10 and _digits(ctx)
     order = [k for i, k in enumerate(seen) if i == 0 or seen[i - 1] != k]
     assert order == ["none", "cores", "digits"], seen
+
+
+def test_route_does_not_depend_on_earlier_calls(pkg):
+    """The memory that a plan with digits needs is not counted twice where the
+    context holds its buffers already: the smallest device on which the digits
+    are taken serves a second threshold as well."""
+    case = make_case("ribbon28", n_tau=2)
+
+    def routes(limit):
+        with pkg.Context(0) as ctx:
+            ctx.load_case(case)
+            ctx.set_option("test_device_bytes", limit)
+            out = []
+            for thr in (1e-6, 1e-9, 1e-6):
+                got = ctx.chi_tau(thr, "fp64", 0, 1).cpu().numpy()
+                out.append(_digits(ctx))
+            return out, got
+
+    ref = oc.chi_dense(case, thr=1e-6)[:1]
+    lo, hi = 1.5e9, 2e10  # the CUDA cores' X and Y fit; everything does
+    assert routes(hi)[0] == [True] * 3
+    for _ in range(7):
+        mid = (lo * hi) ** 0.5
+        taken, got = routes(mid)
+        assert _rel(got, ref) <= 1e-10
+        assert taken[2] == taken[0]
+        # 1e-9 keeps more blocks than 1e-6: it may need more
+        lo, hi = (lo, mid) if taken[0] else (mid, hi)
