@@ -88,6 +88,8 @@ int ws(gw_ctx* ctx, const char* name, size_t bytes, void** out) {
     cudaError_t e = cudaErrorMemoryAllocation;
     if (ctx->test_device_bytes == 0.0 || held_bytes(ctx) + (double)bytes <= ctx->test_device_bytes)
       e = cudaMalloc(&p, bytes);
+    // the panels' digits are a copy that the next FP64 chi can make again
+    if (e != cudaSuccess && gw::give_back_digits(ctx)) return ws(ctx, name, bytes, out);
     if (e != cudaSuccess) {
       cudaGetLastError();
       ctx->alloc_injected = false;
@@ -156,6 +158,24 @@ void free_panel_digits(gw_ctx* ctx) {
   ctx->pd_ok = false;
 }
 
+// Panel digits beyond this are given back when a call of gw_chi_tau ends.  Making
+// them again takes 0.33 ms per GB (2.9 GB of a 40-atom ribbon: 0.94 ms) of calls
+// that at this size take 0.3 s per tau point and more.
+constexpr size_t kPanelDigitsKeep = size_t(16) << 30;
+
+// While a call multiplies with the panels' digits.
+struct DigitsInUse {
+  gw_ctx* ctx;
+  DigitsInUse(gw_ctx* c, bool use) : ctx(c) { ctx->pd_in_use = use; }
+  ~DigitsInUse() {
+    ctx->pd_in_use = false;
+    if (ctx->d_pd && ctx->pd_bytes > kPanelDigitsKeep) {
+      cudaStreamSynchronize(ctx->stream);
+      free_panel_digits(ctx);
+    }
+  }
+};
+
 void reset_tensor(gw_ctx* ctx) {
   free_dev(ctx->d_t3);
   free_dev(ctx->d_t3f);
@@ -219,7 +239,7 @@ int plan_panels(gw_ctx* ctx, double thr) {
   ctx->panels_ok = false;
   ctx->panels_thr = -1.0;
   ctx->pt_ok = false;
-  ctx->pd_ok = false;
+  free_panel_digits(ctx);
   ctx->bn_ok = false;
   ctx->panel32_ok = false;
   ctx->ycov_valid = false;
@@ -360,7 +380,7 @@ int build_panels(gw_ctx* ctx, double thr) {
   free_dev(ctx->d_panel32);
   ctx->d_panel64 = nullptr;
   ctx->d_panel32 = nullptr;
-  GW_TRY(cudaMalloc(&ctx->d_panel64, std::max<long long>(off, 1) * sizeof(double)));
+  GW_TRY(gw::device_alloc(ctx, (void**)&ctx->d_panel64, std::max<long long>(off, 1) * sizeof(double)));
   GW_TRY(cudaMemsetAsync(ctx->d_panel64, 0, std::max<long long>(off, 1) * sizeof(double), ctx->stream));
   int *d_kept, *d_ldB, *d_ldA;
   long long *d_dstB, *d_dstA;
@@ -2166,6 +2186,18 @@ int tc_finish_tau(gw_ctx* ctx, const std::vector<unsigned long long>& h, std::ve
 }  // namespace
 
 namespace gw {
+cudaError_t device_alloc(gw_ctx* ctx, void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess && give_back_digits(ctx)) e = cudaMalloc(p, bytes);
+  return e;
+}
+bool give_back_digits(gw_ctx* ctx) {
+  if (!ctx->d_pd || ctx->pd_in_use) return false;
+  cudaGetLastError();
+  cudaStreamSynchronize(ctx->stream);
+  free_panel_digits(ctx);
+  return true;
+}
 bool memory_short(const gw_ctx* ctx, int rc) { return rc == GW_ERR_OOM && !ctx->alloc_injected; }
 int plan_bn_lists(gw_ctx* ctx, double thr) {
   if (ctx->d_t3f)
@@ -2555,7 +2587,7 @@ int gw_mlp_log(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
     return fail(ctx, GW_ERR_INVALID_ARG, "gw_mlp_log: tau range out of bounds");
   GW_TRY(cudaSetDevice(ctx->device));
   double* chi = nullptr;
-  GW_TRY(cudaMalloc(&chi, std::max<size_t>((size_t)tau_count * ctx->nri * ctx->nri, 1) * sizeof(double)));
+  GW_TRY(gw::device_alloc(ctx, (void**)&chi, std::max<size_t>((size_t)tau_count * ctx->nri * ctx->nri, 1) * sizeof(double)));
   ctx->mlp_log_feat.clear();
   ctx->mlp_log_tgt.clear();
   ctx->mlp_mode = 1;
@@ -2631,6 +2663,7 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
   }
   if (f64 && (rc = ensure_panel_digits(ctx))) return rc;
   bool digits = f64 && ctx->pd_ok;
+  const DigitsInUse in_use(ctx, digits);
   if (!f64 && !tcpath && (rc = ensure_panel32(ctx))) return rc;
   if (tcpath && (rc = ensure_pt(ctx, precision == GW_BF16X6 ? 3 : 2, f16))) return rc;
   const int nao = ctx->nao, nri = ctx->nri, n_at = ctx->n_at;

@@ -98,7 +98,7 @@ extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const doub
   if (chi_on_device) {
     chi = chi_tau;
   } else {
-    CH_TRY(cudaMalloc(&b_chi.p, (size_t)n_tau * nn * 8));
+    CH_TRY(gw::device_alloc(ctx, &b_chi.p, (size_t)n_tau * nn * 8));
     CH_TRY(cudaMemcpyAsync(b_chi.p, chi_tau, (size_t)n_tau * nn * 8, cudaMemcpyHostToDevice, st));
     chi = (const double*)b_chi.p;
   }
@@ -106,7 +106,7 @@ extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const doub
   if (out_on_device) {
     wout = w_tau_out;
   } else {
-    CH_TRY(cudaMalloc(&b_w.p, (size_t)n_tau * nn * 8));
+    CH_TRY(gw::device_alloc(ctx, &b_w.p, (size_t)n_tau * nn * 8));
     wout = (double*)b_w.p;
   }
   CH_TRY(cudaMemsetAsync(wout, 0, (size_t)n_tau * nn * 8, st));
@@ -216,13 +216,13 @@ extern "C" int gw_ri_metric(gw_ctx* ctx, const double* S, int n_mat, const doubl
     return rc;
   const double* m = M;
   if (!m_on_device) {
-    CH_TRY(cudaMalloc(&b_m.p, (size_t)n_mat * nn * 8));
+    CH_TRY(gw::device_alloc(ctx, &b_m.p, (size_t)n_mat * nn * 8));
     CH_TRY(cudaMemcpyAsync(b_m.p, M, (size_t)n_mat * nn * 8, cudaMemcpyHostToDevice, st));
     m = (const double*)b_m.p;
   }
   double* o = out;
   if (!out_on_device) {
-    CH_TRY(cudaMalloc(&b_o.p, (size_t)n_mat * nn * 8));
+    CH_TRY(gw::device_alloc(ctx, &b_o.p, (size_t)n_mat * nn * 8));
     o = (double*)b_o.p;
   }
   CH_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));

@@ -84,8 +84,8 @@ extern "C" int gw_evgw(gw_ctx* ctx, const double* V, int n_omega, const double* 
   const size_t per_tau = static_cast<size_t>(ctx->nri) * ctx->nri;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return ev_fail(ctx, GW_ERR_CUDA, "cudaSetDevice");
   DevBuf chi, w;
-  if (cudaMalloc(&chi.p, std::max<size_t>(per_tau * n_tau, 1) * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&w.p, std::max<size_t>(per_tau * n_tau, 1) * sizeof(double)) != cudaSuccess)
+  if (gw::device_alloc(ctx, &chi.p, std::max<size_t>(per_tau * n_tau, 1) * sizeof(double)) != cudaSuccess ||
+      gw::device_alloc(ctx, &w.p, std::max<size_t>(per_tau * n_tau, 1) * sizeof(double)) != cudaSuccess)
     return ev_fail(ctx, GW_ERR_OOM, "device buffers for chi and W");
 
   std::vector<double> sx(n_orb), sig(static_cast<size_t>(n_orb) * n_tau * 2), e(n_orb), prev(n_orb),

@@ -107,6 +107,11 @@ int plan_bn_lists(gw_ctx* ctx, double thr);
 // FP64 calls ("w." names) stay only while they are small beside the operand
 // batches of chi.
 int work_buffer(gw_ctx* ctx, const char* name, size_t bytes, void** out);
+// cudaMalloc for a call's own arrays: where it fails, once more without the
+// digits of the panels (give_back_digits: true if there were any and no call is
+// using them).
+cudaError_t device_alloc(gw_ctx* ctx, void** p, size_t bytes);
+bool give_back_digits(gw_ctx* ctx);
 // rc is an allocation that failed, and not for the test hook: what needs less
 // memory may be tried instead.
 bool memory_short(const gw_ctx* ctx, int rc);
@@ -219,6 +224,7 @@ struct gw_ctx {
   bool pd_ok = false;
   void* d_pd = nullptr;
   size_t pd_bytes = 0;
+  bool pd_in_use = false;
   int* d_pd_exps = nullptr;
   long long pd_rows = 0;
   int pd_kp = 0;

@@ -121,16 +121,16 @@ extern "C" int gw_sigma_ao_tau(gw_ctx* ctx, const double* W_tau, int w_on_device
   int rc = gw::emu_begin(ctx, st);
   if (rc) return rc;
   DevBuf b_t, b_z, b_u, b_go, b_gv, b_cso, b_csv, b_fl, b_w, b_out;
-  SA_TRY(cudaMalloc(&b_t.p, std::max<long long>(dense, 1) * 8));
-  SA_TRY(cudaMalloc(&b_z.p, std::max<long long>(dense, 1) * 8));
-  SA_TRY(cudaMalloc(&b_u.p, std::max<long long>(dense, 1) * 8));
-  SA_TRY(cudaMalloc(&b_go.p, nn_ao * 8));
-  SA_TRY(cudaMalloc(&b_gv.p, nn_ao * 8));
-  SA_TRY(cudaMalloc(&b_cso.p, static_cast<size_t>(nao) * std::max(ctx->n_occ, 1) * 8));
-  SA_TRY(cudaMalloc(&b_csv.p, static_cast<size_t>(nao) * std::max(nao - ctx->n_occ, 1) * 8));
-  SA_TRY(cudaMalloc(&b_fl.p, 2 * static_cast<size_t>(n_at) * n_at));
-  if (!w_on_device) SA_TRY(cudaMalloc(&b_w.p, nn_ri * 8));
-  if (!out_on_device) SA_TRY(cudaMalloc(&b_out.p, 2 * nn_ao * 8));
+  SA_TRY(gw::device_alloc(ctx, &b_t.p, std::max<long long>(dense, 1) * 8));
+  SA_TRY(gw::device_alloc(ctx, &b_z.p, std::max<long long>(dense, 1) * 8));
+  SA_TRY(gw::device_alloc(ctx, &b_u.p, std::max<long long>(dense, 1) * 8));
+  SA_TRY(gw::device_alloc(ctx, &b_go.p, nn_ao * 8));
+  SA_TRY(gw::device_alloc(ctx, &b_gv.p, nn_ao * 8));
+  SA_TRY(gw::device_alloc(ctx, &b_cso.p, static_cast<size_t>(nao) * std::max(ctx->n_occ, 1) * 8));
+  SA_TRY(gw::device_alloc(ctx, &b_csv.p, static_cast<size_t>(nao) * std::max(nao - ctx->n_occ, 1) * 8));
+  SA_TRY(gw::device_alloc(ctx, &b_fl.p, 2 * static_cast<size_t>(n_at) * n_at));
+  if (!w_on_device) SA_TRY(gw::device_alloc(ctx, &b_w.p, nn_ri * 8));
+  if (!out_on_device) SA_TRY(gw::device_alloc(ctx, &b_out.p, 2 * nn_ao * 8));
   double* T = static_cast<double*>(b_t.p);
   double* Z = static_cast<double*>(b_z.p);
   double* U = static_cast<double*>(b_u.p);

@@ -159,3 +159,34 @@ def test_route_does_not_depend_on_earlier_calls(pkg):
         assert taken[2] == taken[0]
         # 1e-9 keeps more blocks than 1e-6: it may need more
         lo, hi = (lo, mid) if taken[0] else (mid, hi)
+
+
+def test_other_calls_get_the_panel_digits_memory(pkg):
+    """A call that finds no memory takes back the panels' digits of an earlier
+    FP64 chi before it gives up: afterwards there are device sizes at which chi
+    has to do without them (were they still there, it would need nothing new)."""
+    from paper_2104_09857_gb300 import _lib
+    from synth.chain_inputs import synthetic_w
+
+    case = make_case("benzene", n_tau=1)
+    ref = oc.chi_dense(case)
+    w = synthetic_w(case.system.nri_total, case.tau, 5)
+    taken = []
+    for limit in 2e7 * 1.2 ** np.arange(24):
+        with pkg.Context(0) as ctx:
+            ctx.load_case(case)
+            ctx.chi_tau(case.thr, "fp64")
+            assert _digits(ctx)
+            ctx.set_option("test_device_bytes", 1)
+            with pytest.raises(_lib.GwError) as e:
+                ctx.sigma_tau(w, [case.n_occ], case.thr)
+            assert e.value.code == -5  # GW_ERR_OOM
+            ctx.set_option("test_device_bytes", limit)
+            try:
+                got = ctx.chi_tau(case.thr, "fp64").cpu().numpy()
+            except _lib.GwError as e:
+                assert e.code == -5
+            else:
+                assert _rel(got, ref) <= 1e-10
+                taken.append(_digits(ctx))
+    assert not taken[0] and taken[-1], taken
