@@ -487,6 +487,9 @@ int gw_get_stats(const gw_ctx* ctx, gw_stats* out);
  *   "test_device_bytes"  what the work buffers and the panels' digits of the
  *                      context may hold together (0: no limit); allocations
  *                      beyond fail as on a device of that size
+ *   "test_digit_bytes"  bound on the digits that an FP64 product holds of one
+ *                      operand at a time, and on the matrices that one sweep of
+ *                      gw_chi_to_w factors together (0: 4 GB and 1 GB)
  *   "test_stall_tc"    1: in gw_chi_tau, every tensor-core kernel waits first
  *                      on a dependency that is never met; its bounded waits
  *                      expire after about 2 s and the call returns

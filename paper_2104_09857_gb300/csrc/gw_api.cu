@@ -2519,6 +2519,11 @@ int gw_set_option(gw_ctx* ctx, const char* key, double value) {
     ctx->test_device_bytes = value;
     return GW_OK;
   }
+  if (!strcmp(key, "test_digit_bytes")) {
+    if (!(value >= 0)) return fail(ctx, GW_ERR_INVALID_ARG, "test_digit_bytes must be >= 0");
+    ctx->test_digit_bytes = value;
+    return GW_OK;
+  }
   if (!strcmp(key, "test_stall_tc")) {
     ctx->test_stall = value != 0.0;
     return GW_OK;

@@ -38,21 +38,10 @@ int chain_buffer(gw_ctx* ctx, const char* name, size_t count, T** out) {
   return rc;
 }
 
-// g.C = Q Q^T from one set of digits where they are whole
-int square(gw_ctx* ctx, const gw::EmuSrc& q, const gw::EmuGemm& g, cudaStream_t st) {
-  if (gw::emu_dig_bytes(q.rows, q.K) > (size_t(4) << 30)) return gw::emu_product(ctx, q, q, g, nullptr, st);
-  gw::EmuOp op;
-  const int rc = gw::emu_prep(ctx, "a", q, &op, st);
-  return rc ? rc : gw::emu_mm(ctx, op, op, g, st);
-}
-
-}  // namespace
-
-extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const double* gamma,
-                           const double* delta, const double* chi_tau, int chi_on_device,
-                           double* w_tau_out, int out_on_device) {
-  if (!ctx) return GW_ERR_INVALID_ARG;
-  gw::TraceRange trace("gw_chi_to_w");
+// gw_chi_to_w with the frequencies factored together in groups of up to `group`
+// bytes of [eps; L] (at least one).
+int chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const double* gamma, const double* delta,
+             const double* chi_tau, int chi_on_device, double* w_tau_out, int out_on_device, size_t group) {
   ctx->err.clear();
   if (ctx->n_at == 0 || !ctx->have_greens) {
     ctx->err = "gw_chi_to_w: call gw_set_basis and gw_set_greens first (the tau grid)";
@@ -83,7 +72,7 @@ extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const doub
   // context's work buffers.  nb frequencies are factored together: all of
   // them within 1 GB (the sweep's chain of small kernels is then paid once),
   // one at a time for large matrices, whose sweeps fill the chip by themselves.
-  const int nb = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_omega, (size_t(1) << 30) / (2 * nn * 8)));
+  const int nb = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_omega, group / (2 * nn * 8)));
   double *v, *low, *m, *t, *ww, *g, *d;
   int* err;
   int rc;
@@ -162,7 +151,7 @@ extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const doub
       q.ldc = n;
       q.tri = 1;
       s_row.src = m + (size_t)(k - k0) * 2 * nn + nn;
-      if ((rc = square(ctx, s_row, q, st))) return rc;
+      if ((rc = gw::emu_product(ctx, s_row, s_row, q, nullptr, st))) return rc;
       // W^c(i tau_j) += delta_jk W^c(i omega_k)
       gw::chain_add_symmetric(ww, v, d + k, n_omega, n_tau, n, wout, st);
       CH_TRY(cudaGetLastError());
@@ -183,6 +172,25 @@ extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const doub
 // S^-1 M S^-1 for n_mat symmetric matrices M (chi~ of Eq. 5, W~ of Eq. 10,
 // V~ of Eq. 11), FP64: S = R R^T (blocked Cholesky), R^-1 by a triangular
 // solve on the identity, S^-1 = R^-T R^-1, then two products per matrix.
+}  // namespace
+
+extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const double* gamma,
+                           const double* delta, const double* chi_tau, int chi_on_device,
+                           double* w_tau_out, int out_on_device) {
+  if (!ctx) return GW_ERR_INVALID_ARG;
+  gw::TraceRange trace("gw_chi_to_w");
+  const auto call = [&](size_t group) {
+    return chi_to_w(ctx, V, n_omega, gamma, delta, chi_tau, chi_on_device, w_tau_out, out_on_device, group);
+  };
+  int rc = call(ctx->test_digit_bytes > 0.0 ? (size_t)ctx->test_digit_bytes : size_t(1) << 30);
+  if (gw::memory_short(ctx, rc)) {
+    // once more, one frequency at a time
+    gw::work_trim(ctx, "w.", 0);
+    rc = call(0);
+  }
+  return rc;
+}
+
 extern "C" int gw_ri_metric(gw_ctx* ctx, const double* S, int n_mat, const double* M, int m_on_device,
                             double* out, int out_on_device) {
   if (!ctx) return GW_ERR_INVALID_ARG;
@@ -248,7 +256,7 @@ extern "C" int gw_ri_metric(gw_ctx* ctx, const double* S, int n_mat, const doubl
   p.C = si;
   p.ldc = n;
   p.ktri = 1;
-  if ((rc = square(ctx, s_q, p, st))) return rc;
+  if ((rc = gw::emu_product(ctx, s_q, s_q, p, nullptr, st))) return rc;
   gw::EmuOp keep;
   for (int k = 0; k < n_mat; ++k) {
     // t = S^-1 M, then t S^-1 (S^-1 symmetric: its rows are its columns)

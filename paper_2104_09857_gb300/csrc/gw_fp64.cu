@@ -88,31 +88,34 @@ int emu_mm(gw_ctx* ctx, const EmuOp& A, const EmuOp& B, const EmuGemm& g, cudaSt
   return GW_OK;
 }
 
-int emu_product(gw_ctx* ctx, const EmuSrc& A, const EmuSrc& B, const EmuGemm& g, EmuOp* keep, cudaStream_t st) {
-  auto chunk = [](const EmuSrc& s) {
-    const size_t row = emu_dig_bytes(1, s.K);
-    // whole tiles of rows
-    return static_cast<long long>(std::max<size_t>(kMaxDigits / row / kEmuTileM, 1)) * kEmuTileM;
-  };
-  const long long ca = chunk(A), cb = chunk(B);
-  auto part = [](const EmuSrc& s, long long r0, long long n) {
-    EmuSrc p = s;
-    p.src = s.src + (s.trans ? r0 : r0 * s.ld);
-    p.rows = std::min(n, s.rows - r0);
-    return p;
-  };
+namespace {
+// Rows of s whose digits take up to `most` bytes, in whole tiles and at least one.
+long long chunk_rows(const EmuSrc& s, size_t most) {
+  return static_cast<long long>(std::max<size_t>(most / emu_dig_bytes(1, s.K) / kEmuTileM, 1)) * kEmuTileM;
+}
+EmuSrc row_chunk(const EmuSrc& s, long long r0, long long n) {
+  EmuSrc p = s;
+  p.src = s.src + (s.trans ? r0 : r0 * s.ld);
+  p.rows = std::min(n, s.rows - r0);
+  return p;
+}
+// the product with at most `most` bytes of digits of each operand at a time
+int product_in_chunks(gw_ctx* ctx, const EmuSrc& A, const EmuSrc& B, const EmuGemm& g, EmuOp* keep, size_t most,
+                      cudaStream_t st) {
+  const long long ca = chunk_rows(A, most), cb = chunk_rows(B, most);
+  const bool square = A.src == B.src && A.ld == B.ld && A.rows == B.rows && A.K == B.K && A.trans == B.trans;
   int rc;
   for (long long r0 = 0; r0 < A.rows; r0 += ca) {
     EmuOp a;
     if (keep && keep->dig && A.rows <= ca) {
       a = *keep;
     } else {
-      if ((rc = emu_prep(ctx, keep ? "kept" : "a", part(A, r0, ca), &a, st))) return rc;
+      if ((rc = emu_prep(ctx, keep ? "kept" : "a", row_chunk(A, r0, ca), &a, st))) return rc;
       if (keep && A.rows <= ca) *keep = a;
     }
     for (long long c0 = 0; c0 < B.rows; c0 += cb) {
-      EmuOp b;
-      if ((rc = emu_prep(ctx, "b", part(B, c0, cb), &b, st))) return rc;
+      EmuOp b = a;
+      if (!(square && c0 == r0) && (rc = emu_prep(ctx, "b", row_chunk(B, c0, cb), &b, st))) return rc;
       EmuGemm h = g;
       h.C = g.C + r0 * g.ldc + (g.cblk ? 0 : c0);
       h.col0 = g.col0 + c0;
@@ -123,6 +126,24 @@ int emu_product(gw_ctx* ctx, const EmuSrc& A, const EmuSrc& B, const EmuGemm& g,
     }
   }
   return GW_OK;
+}
+}  // namespace
+
+int emu_product(gw_ctx* ctx, const EmuSrc& A, const EmuSrc& B, const EmuGemm& g, EmuOp* keep, cudaStream_t st) {
+  size_t most = ctx->test_digit_bytes > 0.0 ? static_cast<size_t>(ctx->test_digit_bytes) : kMaxDigits;
+  for (;;) {
+    const int rc = product_in_chunks(ctx, A, B, g, keep, most, st);
+    // where the digits do not fit, in half as large chunks (the product does not
+    // depend on them); C must not have been added to
+    const bool smaller = chunk_rows(A, most) > kEmuTileM || chunk_rows(B, most) > kEmuTileM;
+    if (!memory_short(ctx, rc) || g.beta != 0.0 || !smaller) return rc;
+    // (only this product's: a caller may hold others, or kept ones of another)
+    work_trim(ctx, "w.dig.b", 0);
+    work_trim(ctx, keep ? "w.dig.kept" : "w.dig.a", 0);
+    if (keep) keep->dig = nullptr;
+    ctx->err.clear();
+    most = std::min(most, std::max(emu_dig_bytes(A.rows, A.K), emu_dig_bytes(B.rows, B.K))) / 2;
+  }
 }
 
 // From kGreensDigits primary functions on, the digit products: about 10 us of

@@ -315,9 +315,10 @@ struct gw_ctx {
   std::map<std::string, std::pair<void*, std::vector<char>>> uploaded;
   std::vector<cudaEvent_t> events;
 
-  // test hooks (options "test_fail_alloc", "test_device_bytes", "test_stall_tc")
+  // test hooks (options "test_fail_alloc", "test_device_bytes", "test_digit_bytes", "test_stall_tc")
   int test_fail_alloc = 0;  // the next new work-buffer allocation fails
   bool alloc_injected = false;     // the last allocation that failed was that one
+  double test_digit_bytes = 0.0;   // digits of one operand, and of a group of frequencies (0: the built-in limits)
   double test_device_bytes = 0.0;  // what the named buffers may hold (0: no limit)
   int test_stall = 0;       // tensor-core kernels wait on a dependency never met
 

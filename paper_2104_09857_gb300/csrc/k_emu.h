@@ -142,9 +142,10 @@ int emu_prep(gw_ctx* ctx, const char* name, const EmuSrc& s, EmuOp* op, cudaStre
 int emu_prep_segments(gw_ctx* ctx, const char* name, const EmuSrc& s, const long long* seg, int n_seg, EmuOp* op,
                       cudaStream_t st);
 int emu_mm(gw_ctx* ctx, const EmuOp& A, const EmuOp& B, const EmuGemm& g, cudaStream_t st);
-// Product of two matrices.  Operands beyond 4 GB of digits go in row chunks;
-// keep (may be null): on a later call with the same A, its digits are reused
-// where they are whole (keep->dig set by the first call).
+// Product of two matrices.  Operands beyond 4 GB of digits, or whose digits do
+// not fit the device, go in row chunks; one matrix on both sides has one set of
+// digits.  keep (may be null): on a later call with the same A, its digits are
+// reused where they are whole (keep->dig set by the first call).
 int emu_product(gw_ctx* ctx, const EmuSrc& A, const EmuSrc& B, const EmuGemm& g, EmuOp* keep,
                 cudaStream_t st);
 // G^occ(tau), G^virt(tau) of Eq. 2 from the orbitals of mol (ctx: the context

@@ -190,3 +190,130 @@ def test_other_calls_get_the_panel_digits_memory(pkg):
                 assert _rel(got, ref) <= 1e-10
                 taken.append(_digits(ctx))
     assert not taken[0] and taken[-1], taken
+
+
+def _spd(rng, n):
+    b = rng.standard_normal((n, n))
+    return b @ b.T / n + np.eye(n)
+
+
+@pytest.fixture(scope="module")
+def dense_inputs():
+    """chi(i tau), V, transforms, S and M of n = 300 auxiliary functions."""
+    rng = np.random.default_rng(21)
+    n = 300
+    m = rng.standard_normal((2, n, n))
+    return {"n": n, "tau": np.array([0.1, 1.0, 8.0]), "chi": -np.stack([_spd(rng, n) * f for f in (1.0, 0.5, 0.1)]),
+            "v": _spd(rng, n), "gamma": rng.standard_normal((3, 3)) ** 2, "delta": rng.standard_normal((3, 3)),
+            "m": m + m.transpose(0, 2, 1)}
+
+
+def _dense_calls(ctx, d):
+    from paper_2104_09857_gb300 import _lib
+
+    w = ctx.chi_to_w(d["chi"], d["v"], d["gamma"], d["delta"]).cpu().numpy()
+    return w, np.asarray(_lib.gw_ri_metric(ctx.ctx, d["v"], d["m"]))
+
+
+def _dense_context(pkg, d):
+    ctx = pkg.Context(0)
+    ctx.set_basis(np.arange(30.0).reshape(10, 3), np.ones(10, dtype=np.int32),
+                  np.full(10, d["n"] // 10, dtype=np.int32))
+    ctx.set_greens(np.eye(10), np.linspace(-1.0, 1.0, 10), 5, 0.0, d["tau"])
+    return ctx
+
+
+def test_row_chunks_and_frequency_groups_change_nothing(pkg, dense_inputs):
+    """Products in chunks of 128 rows and sweeps of one frequency at a time: sums
+    of digits are exact, so every bit is that of the whole product."""
+    from paper_2104_09857_gb300 import _lib
+    from synth.chain_inputs import synthetic_w
+
+    case = make_case("benzene", n_tau=1)
+    w = synthetic_w(case.system.nri_total, case.tau, 5)
+    nao = case.system.nao_total
+    got = []
+    for limit in (0, 7e5):
+        with _dense_context(pkg, dense_inputs) as ctx:
+            ctx.set_option("test_digit_bytes", limit)
+            got.append(list(_dense_calls(ctx, dense_inputs)))
+        with pkg.Context(0) as ctx:
+            ctx.load_case(case)
+            ctx.set_option("test_digit_bytes", limit)
+            got[-1].append(np.asarray(_lib.gw_sigma_ao_tau(ctx.ctx, w, 1, nao, case.thr)))
+    for whole, chunks in zip(*got):
+        assert np.array_equal(whole, chunks)
+
+
+def test_products_without_room_for_whole_digits(pkg, dense_inputs):
+    """On a device that does not hold an operand's digits whole the products go
+    in smaller chunks: chi_to_w and the metric run, to the same bits, with less
+    than their matrices, the partial sums and both operands' digits."""
+    from paper_2104_09857_gb300 import _lib
+
+    d, n = dense_inputs, dense_inputs["n"]
+    nn, digits = 8.0 * n * n, 16.0 * n * 320
+    with _dense_context(pkg, d) as ctx:
+        ref = _dense_calls(ctx, d)
+    ran = []
+    for limit in 6 * nn * 1.05 ** np.arange(40):
+        with _dense_context(pkg, d) as ctx:
+            ctx.set_option("test_device_bytes", limit)
+            try:
+                got = _dense_calls(ctx, d)
+            except _lib.GwError as e:
+                assert e.code == -5, limit
+            else:
+                assert all(np.array_equal(a, b) for a, b in zip(got, ref))
+                ran.append(limit)
+    # V, L, [eps; L] of one frequency and two products; a sweep's panel as digits
+    # and the partial sums of its update; two operands
+    rows = 2 * n - 64
+    assert ran and ran[0] < 6 * nn + rows * (64 + n - 64) * 16 + 2 * digits, ran
+
+
+@pytest.mark.parametrize("n", [2, 29, 30])
+def test_chain_of_one_frequency_and_few_functions(pkg, n):
+    """Two atoms, one frequency: the smallest chains."""
+    from oracle import chain as och
+
+    rng = np.random.default_rng(n)
+    v, chi = _spd(rng, n), -_spd(rng, n)[None]
+    one = np.ones((1, 1))
+    ref, _ = och.chi_to_w(chi, v, one, one)
+    with pkg.Context(0) as ctx:
+        ctx.set_basis(np.array([[0.0, 0.0, 0.0], [1.4, 0.0, 0.0]]), np.ones(2, dtype=np.int32),
+                      np.array([n - n // 2, n // 2], dtype=np.int32))
+        ctx.set_greens(np.eye(2), np.array([-1.0, 1.0]), 1, 0.0, np.array([1.0]))
+        got = ctx.chi_to_w(chi, v, one, one).cpu().numpy()
+    assert np.linalg.norm(got - ref) <= 1e-10 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("where", ["tensor", "orbitals"])
+def test_non_finite_chi(pkg, where):
+    """Operands that no fixed-point form holds take the plain sums, in the panels
+    and in step C: elements of magnitude 1e200 overflow G (to Inf) or T's
+    products, and what they do not reach is as without them."""
+    case = make_case("chain_CHCH", n_tau=1)
+    with pkg.Context(0) as ctx:
+        ctx.load_case(case)
+        want = ctx.chi_tau(0.0, "fp64").cpu().numpy()[0]
+        big = 1e200 if where == "tensor" else 1e160
+        if where == "tensor":  # T^2 overflows: the elements of chi with the last auxiliary function
+            data = case.t3c.data.copy()
+            last = case.t3c.blocks[:, 2] == case.system.n_atoms - 1
+            for i in np.nonzero(last)[0]:
+                blk = data[case.t3c.offsets[i]:case.t3c.offsets[i + 1]].reshape(-1, case.system.n_ri[-1])
+                blk[:, -1] *= big
+            ctx.set_3c_tensor(case.t3c.blocks, data)
+        else:  # G overflows
+            c = case.C.copy()
+            c[0] *= big
+            ctx.set_greens(c, case.eps, case.n_occ, case.mu_fermi, case.tau)
+        got = ctx.chi_tau(0.0, "fp64").cpu().numpy()[0]
+    if where == "tensor":
+        assert not np.isfinite(got[-1, -1])
+        assert np.abs(got[:-1, :-1] - want[:-1, :-1]).max() <= 1e-14 * np.abs(want).max()
+        assert np.abs(got[:-1, -1] / big - want[:-1, -1]).max() <= 1e-13 * np.abs(want).max()
+    else:
+        assert not np.isfinite(got).any()
