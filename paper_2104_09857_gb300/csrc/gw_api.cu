@@ -1510,6 +1510,29 @@ OperandSegments plan_segments(const Batch& b, long long most) {
   return g;
 }
 
+// bytes of X and Y of a batch in rows of `len` elements
+double operand_bytes(const Batch& b, long long len, size_t elem_bytes) {
+  return (double)((b.P1 - b.P0) + (b.Q1 - b.Q0)) * (double)len * elem_bytes;
+}
+// Batches whose X and Y stay within the byte budget in segments too (a batch of
+// one owner may need more either way): planned again for the share of it that
+// the padding leaves.
+std::vector<Batch> plan_batches_segments(gw_ctx* ctx, size_t elem_bytes) {
+  const double budget = ctx->batch_bytes;
+  double most = budget;
+  std::vector<Batch> batches;
+  for (int attempt = 0; attempt < 4; ++attempt) {
+    batches = plan_batches_tc(ctx, elem_bytes, most, gw::tc_tile_rows());
+    double worst = 1.0;
+    for (const Batch& b : batches)
+      if (operand_bytes(b, b.Kb, elem_bytes) <= budget)
+        worst = std::max(worst, operand_bytes(b, plan_segments(b, kSegmentK).len(), elem_bytes) / budget);
+    if (worst == 1.0) break;
+    most /= worst;
+  }
+  return batches;
+}
+
 // One batch on the tensor cores: steps A and B straight into bf16 slices,
 // block filter from the accumulated norms, task lists, step C.  gs_occ,
 // gs_virt: slices of G^occ and G^virt, [slices][n_AO][n_AO rounded to 64].
@@ -1536,6 +1559,8 @@ int chi_one_batch_tc(gw_ctx* ctx, const Batch& b, const void* gs_occ, const void
   const int kmax = ctx->pt_kmax, gkp = (ctx->nao + 63) / 64 * 64;
   void *xs, *ys;
   OperandSegments g = plan_segments(b, ctx->mlp_mode ? Kb : kSegmentK);
+  if (operand_bytes(b, g.len(), 2 * slices) > std::max(ctx->batch_bytes, operand_bytes(b, Kb, 2 * slices)))
+    g = plan_segments(b, Kb);
   if (g.nseg > 1 && (ws(ctx, "Xs", (size_t)slices * prow * g.len() * 2, &xs) ||
                      ws(ctx, "Ys", (size_t)slices * qrow * g.len() * 2, &ys))) {
     // no room for the segments' padding
@@ -2676,7 +2701,8 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
   const size_t esz = f64 ? (digits ? kDigitElem : sizeof(double))
                          : precision == GW_BF16X6 ? 6 : tcpath ? 4 : sizeof(float);
   std::vector<Batch> batches =
-      tcpath ? plan_batches_tc(ctx, esz, ctx->batch_bytes, gw::tc_tile_rows())
+      tcpath ? (ctx->mlp_mode ? plan_batches_tc(ctx, esz, ctx->batch_bytes, gw::tc_tile_rows())
+                              : plan_batches_segments(ctx, esz))
              : plan_batches(ctx, esz, ctx->batch_bytes, 0);
   ctx->stats.n_batches = (int)batches.size();
 

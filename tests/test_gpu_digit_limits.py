@@ -317,3 +317,22 @@ def test_non_finite_chi(pkg, where):
         assert np.abs(got[:-1, -1] / big - want[:-1, -1]).max() <= 1e-13 * np.abs(want).max()
     else:
         assert not np.isfinite(got).any()
+
+
+def test_segments_stay_within_the_operand_budget(pkg):
+    """X and Y of 519 functions take one batch of exactly batch_bytes without the
+    padding of their segments: with it they take two."""
+    sysm = System("long", np.array([[1.4 * i, 0.0, 0.0] for i in range(38)]), ["C"] * 38)
+    sysm.n_ao = np.array([14] * 37 + [1], dtype=np.int32)
+    sysm.n_ri = np.array([1] * 37 + [3], dtype=np.int32)
+    case = case_from_system(sysm, 1, 1e-9, 7)
+    case.tau = np.array([0.5])
+    ref = oc.chi_dense(case)
+    plain = 4 * (40 + 40) * (576 * 519)  # two 16-bit slices, rows of X and Y, padded functions x functions
+    with pkg.Context(0) as ctx:
+        ctx.load_case(case)
+        for room, batches in ((1.2, 1), (1.0, 2)):
+            ctx.set_option("batch_bytes", plain * room)
+            got = ctx.chi_tau(case.thr, "fp16x3").cpu().numpy()
+            assert ctx.stats()["n_batches"] == batches
+            assert np.linalg.norm(got - ref) <= 1e-6 * np.linalg.norm(ref)
