@@ -88,7 +88,7 @@ int ws(gw_ctx* ctx, const char* name, size_t bytes, void** out) {
     cudaError_t e = cudaErrorMemoryAllocation;
     if (ctx->test_device_bytes == 0.0 || held_bytes(ctx) + (double)bytes <= ctx->test_device_bytes)
       e = cudaMalloc(&p, bytes);
-    // the panels' digits are a copy that the next FP64 chi can make again
+    // the digits of chi are copies that the next FP64 chi makes again
     if (e != cudaSuccess && gw::give_back_digits(ctx)) return ws(ctx, name, bytes, out);
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -893,10 +893,10 @@ double digit_route_bytes(gw_ctx* ctx, int kp) {
     const double prow = b.P1 - b.P0, k = (double)b.Kb, ns = b.s1 - b.s0, R = ctx->ao_off[b.s1] - ctx->ao_off[b.s0];
     want("X", 8 * prow * k);
     want("Y", 8 * nri * k);
-    want("w.dig.X", 2.0 * gw::kEmuSlices * prow * k);
-    want("w.dig.Y", 2.0 * gw::kEmuSlices * nri * k);
-    want("w.dig.X.e", 4 * prow * ns);
-    want("w.dig.Y.e", 4 * nri * ns);
+    want("d64_X", 2.0 * gw::kEmuSlices * prow * k);
+    want("d64_Y", 2.0 * gw::kEmuSlices * nri * k);
+    want("d64_X.e", 4 * prow * ns);
+    want("d64_Y.e", 4 * nri * ns);
     if (!whole) want("d64_gg", 2.0 * gw::kEmuSlices * std::max(ns * nao, n_at * R) * kp);
     want("d64_part", 16 * prow * nri);
     want("d64_pair", 4 * prow * nri);
@@ -909,7 +909,7 @@ double digit_route_bytes(gw_ctx* ctx, int kp) {
     want("fy", ns * n_at * nri / gw::kEmuTileN);
   }
   const double g_digits = 2.0 * gw::kEmuSlices * nao * gw::emu_kp(ctx->nao);
-  for (const char* g : {"w.dig.go", "w.dig.gv", "w.dig.orbitals"}) want(g, g_digits);
+  for (const char* g : {"d64_go", "d64_gv", "w.dig.orbitals"}) want(g, g_digits);
   for (const char* g : {"g_occ", "g_virt", "cso", "csv"}) want(g, 8 * nao * nao);
   for (const char* c : {"chi_acc", "chi_stage"}) want(c, 8 * nri * nri);
   want("w.part", 96e6);  // partial sums of G's products (k_emu.cu)
@@ -994,8 +994,8 @@ bool leave_digits(gw_ctx* ctx, int rc) {
   if (!gw::memory_short(ctx, rc)) return false;
   cudaStreamSynchronize(ctx->stream);
   gw::work_trim(ctx, "w.dig.", 0);
-  gw::work_trim(ctx, "d64_", 0);
-  free_panel_digits(ctx);
+  ctx->pd_in_use = false;
+  gw::give_back_digits(ctx);
   ctx->err.clear();
   return true;
 }
@@ -1138,8 +1138,8 @@ int chi_one_batch_digits(gw_ctx* ctx, const Batch& b, const double* g_occ, const
   gw::EmuSrc sy = sx;
   sy.src = Y;
   sy.rows = nri;
-  if ((rc = gw::emu_prep_segments(ctx, "X", sx, d_seg, ns, &ox, ctx->stream)) ||
-      (rc = gw::emu_prep_segments(ctx, "Y", sy, d_seg, ns, &oy, ctx->stream)))
+  if ((rc = gw::emu_prep_segments(ctx, "d64_X", sx, d_seg, ns, &ox, ctx->stream)) ||
+      (rc = gw::emu_prep_segments(ctx, "d64_Y", sy, d_seg, ns, &oy, ctx->stream)))
     return rc;
   // task lists, work units, step C
   std::vector<long long> slab_k0(nslab);
@@ -2217,10 +2217,13 @@ cudaError_t device_alloc(gw_ctx* ctx, void** p, size_t bytes) {
   return e;
 }
 bool give_back_digits(gw_ctx* ctx) {
-  if (!ctx->d_pd || ctx->pd_in_use) return false;
+  const auto first = ctx->work.lower_bound("d64_");
+  const bool batch = first != ctx->work.end() && first->first.compare(0, 4, "d64_") == 0;
+  if ((!ctx->d_pd && !batch) || ctx->pd_in_use) return false;
   cudaGetLastError();
   cudaStreamSynchronize(ctx->stream);
   free_panel_digits(ctx);
+  work_trim(ctx, "d64_", 0);
   return true;
 }
 bool memory_short(const gw_ctx* ctx, int rc) { return rc == GW_ERR_OOM && !ctx->alloc_injected; }
@@ -2797,9 +2800,9 @@ int gw_chi_tau(gw_ctx* ctx, int tau_first, int tau_count, double thr, int precis
       s.src = go;
       s.ld = s.rows = nao;
       s.K = nao;
-      rc = gw::emu_prep(ctx, "go", s, &op_o, ctx->stream);
+      rc = gw::emu_prep(ctx, "d64_go", s, &op_o, ctx->stream);
       s.src = gv;
-      if (!rc) rc = gw::emu_prep(ctx, "gv", s, &op_v, ctx->stream);
+      if (!rc) rc = gw::emu_prep(ctx, "d64_gv", s, &op_v, ctx->stream);
       if (rc && !leave_digits(ctx, rc)) return rc;
       digits = rc == GW_OK;
       ctx->stats.kernel_launches += 2;

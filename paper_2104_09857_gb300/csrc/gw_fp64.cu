@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 #include <string>
 
 #include "gw_internal.h"
@@ -35,11 +36,12 @@ int emu_begin(gw_ctx* ctx, cudaStream_t st) {
 }
 
 namespace {
-// digits of `rows` rows of length K and n_exps exponents in buffers of this name
+// Digits of `rows` rows of length K and n_exps exponents in buffers of this name,
+// which go when the call ends (gw::WorkTrim) unless they are chi's ("d64_").
 int digit_buffers(gw_ctx* ctx, const char* name, long long rows, int K, long long n_exps, EmuOp* op) {
   void* p;
   int rc;
-  const std::string n = std::string("w.dig.") + name;
+  const std::string n = std::string(std::strncmp(name, "d64_", 4) ? "w.dig." : "") + name;
   if ((rc = work_buffer(ctx, n.c_str(), std::max<size_t>(emu_dig_bytes(rows, K), 16), &p))) return rc;
   op->dig = p;
   if ((rc = work_buffer(ctx, (n + ".e").c_str(), std::max<size_t>(n_exps, 1) * sizeof(int), &p))) return rc;

@@ -108,8 +108,8 @@ int plan_bn_lists(gw_ctx* ctx, double thr);
 // batches of chi.
 int work_buffer(gw_ctx* ctx, const char* name, size_t bytes, void** out);
 // cudaMalloc for a call's own arrays: where it fails, once more without the
-// digits of the panels (give_back_digits: true if there were any and no call is
-// using them).
+// digits that FP64 chi keeps, of the panels and of its last batch (give_back_digits:
+// true if there were any and no call is using them).
 cudaError_t device_alloc(gw_ctx* ctx, void** p, size_t bytes);
 bool give_back_digits(gw_ctx* ctx);
 // rc is an allocation that failed, and not for the test hook: what needs less
