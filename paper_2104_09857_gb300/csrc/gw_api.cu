@@ -1138,8 +1138,9 @@ int chi_one_batch_digits(gw_ctx* ctx, const Batch& b, const double* g_occ, const
   gw::EmuSrc sy = sx;
   sy.src = Y;
   sy.rows = nri;
-  if ((rc = gw::emu_prep_segments(ctx, "d64_X", sx, d_seg, ns, &ox, ctx->stream)) ||
-      (rc = gw::emu_prep_segments(ctx, "d64_Y", sy, d_seg, ns, &oy, ctx->stream)))
+  const int longest = ctx->naop * *std::max_element(ctx->n_ao.begin() + b.s0, ctx->n_ao.begin() + b.s1);
+  if ((rc = gw::emu_prep_segments(ctx, "d64_X", sx, d_seg, ns, longest, &ox, ctx->stream)) ||
+      (rc = gw::emu_prep_segments(ctx, "d64_Y", sy, d_seg, ns, longest, &oy, ctx->stream)))
     return rc;
   // task lists, work units, step C
   std::vector<long long> slab_k0(nslab);
@@ -1196,7 +1197,7 @@ int chi_one_batch_digits(gw_ctx* ctx, const Batch& b, const double* g_occ, const
   GW_CHECK_LAUNCH();
   GW_TRY(cudaEventRecord(ec1, ctx->stream));
   ctx->stats.c_launches += 1;
-  ctx->stats.kernel_launches += 14;
+  ctx->stats.kernel_launches += 16;
   std::vector<double> h_fc((size_t)ns * n_at);
   unsigned long long h_stat[3];
   GW_TRY(cudaMemcpyAsync(h_fc.data(), d_fc, h_fc.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));

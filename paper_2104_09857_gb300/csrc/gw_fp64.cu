@@ -63,11 +63,11 @@ int emu_prep(gw_ctx* ctx, const char* name, const EmuSrc& s, EmuOp* op, cudaStre
   return prep_launched(ctx);
 }
 
-int emu_prep_segments(gw_ctx* ctx, const char* name, const EmuSrc& s, const long long* seg, int n_seg, EmuOp* op,
-                      cudaStream_t st) {
+int emu_prep_segments(gw_ctx* ctx, const char* name, const EmuSrc& s, const long long* seg, int n_seg, int max_len,
+                      EmuOp* op, cudaStream_t st) {
   const int rc = digit_buffers(ctx, name, s.rows, s.K, s.rows * n_seg, op);
   if (rc) return rc;
-  launch_emu_prep_segments(*op, s, seg, n_seg, st);
+  launch_emu_prep_segments(*op, s, seg, n_seg, max_len, st);
   return prep_launched(ctx);
 }
 

@@ -190,45 +190,62 @@ __global__ void __launch_bounds__(256) k_prep_rows(const double* __restrict__ sr
 
 // Rows of a row-major matrix with an exponent per segment of a row: segment i
 // starts at element seg[i] (a multiple of 64) and ends where the next begins.
-// exps[i * rows + r].  kWarps (1 or 8) warps per segment of a row, which they
-// read twice (the second time from cache).
-template <int kWarps>
-__global__ void __launch_bounds__(256) k_prep_segments(const double* __restrict__ src, long long ld, long long rows,
-                                                       int K, const long long* __restrict__ seg, int n_seg,
-                                                       __half* __restrict__ dig, int* __restrict__ exps) {
-  constexpr int kPer = 8 / kWarps, kN = 32 * kWarps;  // segments of a CTA, threads of a segment
-  __shared__ int red[8];
-  const int warp = threadIdx.x >> 5, t = threadIdx.x % kN;
-  for (long long i0 = static_cast<long long>(blockIdx.x) * kPer; i0 < rows * n_seg;
-       i0 += static_cast<long long>(gridDim.x) * kPer) {
-    const long long i = i0 + warp / kWarps;
-    if (i >= rows * n_seg) continue;  // kPer > 1: no barrier below
-    const long long r = i / n_seg;
-    const int s = static_cast<int>(i - r * n_seg);
+// First exps[i * rows + r], a warp per segment of a row.
+__global__ void __launch_bounds__(256) k_segment_exps(const double* __restrict__ src, long long ld, long long rows,
+                                                      int K, const long long* __restrict__ seg, int n_seg,
+                                                      int* __restrict__ exps) {
+  const int lane = threadIdx.x & 31;
+  for (long long i = blockIdx.x * 8LL + threadIdx.x / 32; i < rows * n_seg; i += gridDim.x * 8LL) {
+    const int s = static_cast<int>(i / rows);
     const long long k0 = seg[s];
     const int len = static_cast<int>((s + 1 < n_seg ? seg[s + 1] : K) - k0);
-    const double* x = src + r * ld + k0;
+    const double2* x = reinterpret_cast<const double2*>(src + (i - s * rows) * ld + k0);
     int be = 0;
-    for (int k = t; k < len; k += kN) be = max(be, biased_exp(x[k]));
+#pragma unroll 4
+    for (int k = lane; k < len / 2; k += 32) {
+      const double2 v = x[k];
+      be = max(be, max(biased_exp(v.x), biased_exp(v.y)));
+    }
     be = __reduce_max_sync(0xffffffffu, be);
-    if (kWarps > 1) {
-      __syncthreads();
-      if (t % 32 == 0) red[warp] = be;
-      __syncthreads();
+    if (lane == 0) exps[i] = row_exp(be);
+  }
+}
+// Then the digits, in blocks of one stage's 32 elements, [block][digit][row][32]: a
+// tile of them is eight contiguous pieces of 8 KB.  In rows of K elements a tile's
+// 1024 rows lay in pages of their own from some 50 atoms on, and every CTA reads
+// its own tiles: step C took 28 ms where it now takes 21 (58 atoms).  A CTA takes
+// 16 rows x 512 elements of segment blockIdx.z, so that it reads and writes within
+// some thirty pages: 5.4 ms for both operands with the exponents' pass.  A row's
+// whole segment per CTA, in one pass, wrote to 200 pages and took 7.5 ms.
+constexpr int kSegRows = 16, kSegK = 512;
+__global__ void __launch_bounds__(256) k_segment_digits(const double* __restrict__ src, long long ld, long long rows,
+                                                        int K, const long long* __restrict__ seg, int n_seg,
+                                                        const int* __restrict__ exps, __half* __restrict__ dig) {
+  const int s = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long k0 = seg[s];
+  const int len = static_cast<int>((s + 1 < n_seg ? seg[s + 1] : K) - k0);
+  // a warp: 8 rows x one block, four lanes with 8 elements each per row
+  const long long r = static_cast<long long>(blockIdx.x) * kSegRows + (warp & 1) * 8 + lane / 4;
+  if (r >= rows) return;
+  const int e = exps[s * rows + r];
+  const double* x = src + r * ld + k0;
+  __half* out = dig + (k0 / kChunk * kS * rows + r) * kChunk + lane % 4 * 8;
+#pragma unroll 1
+  for (int b = warp / 2; b < kSegK / kChunk; b += 4) {
+    const int k = static_cast<int>(blockIdx.y) * kSegK + b * kChunk;
+    if (k >= len) break;
+    double v[8];
 #pragma unroll
-      for (int w = 0; w < kWarps; ++w) be = max(be, red[w]);
+    for (int j = 0; j < 4; ++j) {
+      const double2 w = *reinterpret_cast<const double2*>(x + k + lane % 4 * 8 + 2 * j);
+      v[2 * j] = w.x;
+      v[2 * j + 1] = w.y;
     }
-    const int e = row_exp(be);
-    if (t == 0) exps[s * rows + r] = e;
-    for (int k = 8 * t; k < len; k += 8 * kN) {
-      double v[8];
+    uint4 q[kS];
+    digits8(v, e, q);
+    __half* o = out + static_cast<long long>(k / kChunk) * kS * rows * kChunk;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = x[k + j];
-      uint4 q[kS];
-      digits8(v, e, q);
-#pragma unroll
-      for (int j = 0; j < kS; ++j) *reinterpret_cast<uint4*>(dig + (j * rows + r) * K + k0 + k) = q[j];
-    }
+    for (int j = 0; j < kS; ++j) *reinterpret_cast<uint4*>(o + j * rows * kChunk) = q[j];
   }
 }
 
@@ -490,6 +507,7 @@ struct GemmJob {
   const double *A, *B;
   long long lda, ldb;
   int ta, tb;
+  static constexpr bool kBlocked = false;  // digits in rows of K elements
 
   struct Tile {
     int ya, yb, c0, n;  // rows of the stacked digits
@@ -639,6 +657,7 @@ struct Panel64Job {
   const double *pool, *G;
   const int* lam;
   int nao;
+  static constexpr bool kBlocked = false;
   struct Tile {
     int ya, yb, n, task, a0, b0;
   };
@@ -772,6 +791,7 @@ struct Chi64Job {
   unsigned long long* part;
   const double *X, *Y;
   long long ldk;
+  static constexpr bool kBlocked = true;  // digits as k_segment_digits lays them
   struct Tile {
     int ya, yb, n, id;
     const int* list;  // the piece's entries, and how many the unit has from here on
@@ -863,9 +883,14 @@ struct Chi64Job {
   }
 };
 // pair[q][p] = the largest sum over the sigma-atoms of ex[s][p] + ey[s][q], kBad
-// where one of them is.
+// where one of them is; part = 0.
 __global__ void __launch_bounds__(256) k_pair_exps(const int* __restrict__ ex, const int* __restrict__ ey, int ns,
-                                                   int prow, int nri, int* __restrict__ pair) {
+                                                   int prow, int nri, int* __restrict__ pair,
+                                                   ulonglong2* __restrict__ part) {
+  for (int i = threadIdx.x >> 5; i < 32; i += 8) {
+    const int pp = blockIdx.x * 32 + i, qq = blockIdx.y * 32 + (threadIdx.x & 31);
+    if (pp < prow && qq < nri) part[static_cast<long long>(pp) * nri + qq] = make_ulonglong2(0, 0);
+  }
   const int p = blockIdx.x * 32 + (threadIdx.x & 31);
   const int q0 = blockIdx.y * 32 + (threadIdx.x >> 5) * 4;
   if (p >= prow) return;
@@ -1051,9 +1076,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_expect_tx(&full[stage], kStageBytes);
             armed[stage] = true;
             armed_parity[stage] = phase;
-            const int x = it.next();
-            tma_load_3d(st, &map_a, x, T.ya, 0, &full[stage]);
-            tma_load_3d(st + kS * kABytes, &map_b, x, T.yb, 0, &full[stage]);
+            int x = it.next(), z = 0;
+            if constexpr (Job::kBlocked) {
+              z = x / kChunk * kS;
+              x = 0;
+            }
+            tma_load_3d(st, &map_a, x, T.ya, z, &full[stage]);
+            tma_load_3d(st + kS * kABytes, &map_b, x, T.yb, z, &full[stage]);
             if (++stage == kStages) {
               stage = 0;
               phase ^= 1u;
@@ -1253,19 +1282,19 @@ void launch_emu_prep(EmuOp& op, const EmuSrc& s, cudaStream_t st) {
   }
 }
 
-void launch_emu_prep_segments(EmuOp& op, const EmuSrc& s, const long long* seg, int n_seg, cudaStream_t st) {
+void launch_emu_prep_segments(EmuOp& op, const EmuSrc& s, const long long* seg, int n_seg, int max_len,
+                              cudaStream_t st) {
   op.s = s;
   op.stride_rows = s.rows;
   op.kp = s.K;
   if (s.rows <= 0 || n_seg <= 0) return;
-  __half* dig = static_cast<__half*>(op.dig);
-  const bool wide = s.K / n_seg >= 2048;  // a CTA per segment, else a warp
-  const long long blocks = wide ? s.rows * n_seg : (s.rows * n_seg + 7) / 8;
-  const unsigned grid = static_cast<unsigned>(std::min<long long>(blocks, 152 * 64));
-  if (wide)
-    emu::k_prep_segments<8><<<grid, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, seg, n_seg, dig, op.exps);
-  else
-    emu::k_prep_segments<1><<<grid, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, seg, n_seg, dig, op.exps);
+  const long long warps = s.rows * n_seg;
+  emu::k_segment_exps<<<static_cast<unsigned>(std::min<long long>((warps + 7) / 8, 152 * 64)), 256, 0, st>>>(
+      s.src, s.ld, s.rows, s.K, seg, n_seg, op.exps);
+  const dim3 grid(static_cast<unsigned>((s.rows + emu::kSegRows - 1) / emu::kSegRows),
+                  static_cast<unsigned>((max_len + emu::kSegK - 1) / emu::kSegK), n_seg);
+  emu::k_segment_digits<<<grid, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, seg, n_seg, op.exps,
+                                              static_cast<__half*>(op.dig));
 }
 
 // Sums go out as integers and a second kernel rounds them, also where K is not
@@ -1376,16 +1405,16 @@ int launch_panel64(const Panel64Args& p, int* err_flag, cudaStream_t st) {
 
 int launch_chi64(const EmuOp& x, const EmuOp& y, const Chi64Args& c, int* err_flag, cudaStream_t st) {
   CUtensorMap mx, my;
-  if (make_digit_map(&mx, x.dig, x.kp, x.s.rows, x.stride_rows, kEmuSlices, emu::kChunk, emu::kM,
-                     kEmuSlices) ||
-      make_digit_map(&my, y.dig, y.kp, y.s.rows, y.stride_rows, kEmuSlices, emu::kChunk, emu::kN, kEmuSlices))
+  const int planes = x.kp / emu::kChunk * kEmuSlices;
+  if (make_digit_map(&mx, x.dig, emu::kChunk, x.s.rows, x.s.rows, planes, emu::kChunk, emu::kM, kEmuSlices) ||
+      make_digit_map(&my, y.dig, emu::kChunk, y.s.rows, y.s.rows, planes, emu::kChunk, emu::kN, kEmuSlices))
     return -2;
   emu::Chi64Job j{c.units.u_tile, c.units.u_first, c.units.u_count, c.units.n_units, c.tasks, c.counts, c.nslab,
                   c.nqt, c.P0, c.prow, c.nri, c.per, c.slab_k0, c.slab_len, x.exps, y.exps, c.pair, c.chi,
                   static_cast<unsigned long long*>(c.part), x.s.src, y.s.src, x.s.ld};
-  cudaMemsetAsync(c.part, 0, static_cast<size_t>(c.prow) * c.nri * 16, st);
   const unsigned gp = static_cast<unsigned>((c.prow + 31) / 32), gq = static_cast<unsigned>((c.nri + 31) / 32);
-  emu::k_pair_exps<<<dim3(gp, gq), 256, 0, st>>>(x.exps, y.exps, c.nslab / c.per, c.prow, c.nri, c.pair);
+  emu::k_pair_exps<<<dim3(gp, gq), 256, 0, st>>>(x.exps, y.exps, c.nslab / c.per, c.prow, c.nri, c.pair,
+                                                  static_cast<ulonglong2*>(c.part));
   const int rc = emu::launch(mx, my, j, INT32_MAX, err_flag, st);
   if (rc) return rc;
   emu::k_chi64_finish<<<dim3(gq, gp), 256, 0, st>>>(j);

@@ -79,9 +79,12 @@ int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, 
                     cudaStream_t st);
 
 // The same with an exponent per segment of a row, for step C: segment i starts at
-// element seg[i] of the row (a multiple of 64; in device memory).  s.K is a
-// multiple of 64, op.exps holds n_seg * s.rows ints, [segment][row].
-void launch_emu_prep_segments(EmuOp& op, const EmuSrc& s, const long long* seg, int n_seg, cudaStream_t st);
+// element seg[i] of the row (a multiple of 64; in device memory) and is max_len
+// long at most.  s.K and s.ld are multiples of 64, s.src is aligned to 16 bytes;
+// op.exps holds n_seg * s.rows ints, [segment][row]; the digits lie as
+// k_segment_digits says.
+void launch_emu_prep_segments(EmuOp& op, const EmuSrc& s, const long long* seg, int n_seg, int max_len,
+                              cudaStream_t st);
 
 // One panel problem of the FP64 steps A / B: digits of the panel's rows from
 // p_row0, of G's rows (gathered on its lambda functions) from g_row0.
@@ -139,8 +142,8 @@ int launch_chi64(const EmuOp& x, const EmuOp& y, const Chi64Args& c, int* err_fl
 int emu_begin(gw_ctx* ctx, cudaStream_t st);
 int emu_flag(gw_ctx* ctx, int** err);  // the error flag of the launchers
 int emu_prep(gw_ctx* ctx, const char* name, const EmuSrc& s, EmuOp* op, cudaStream_t st);
-int emu_prep_segments(gw_ctx* ctx, const char* name, const EmuSrc& s, const long long* seg, int n_seg, EmuOp* op,
-                      cudaStream_t st);
+int emu_prep_segments(gw_ctx* ctx, const char* name, const EmuSrc& s, const long long* seg, int n_seg, int max_len,
+                      EmuOp* op, cudaStream_t st);
 int emu_mm(gw_ctx* ctx, const EmuOp& A, const EmuOp& B, const EmuGemm& g, cudaStream_t st);
 // Product of two matrices.  Operands beyond 4 GB of digits, or whose digits do
 // not fit the device, go in row chunks; one matrix on both sides has one set of
