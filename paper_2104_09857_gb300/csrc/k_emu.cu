@@ -63,7 +63,7 @@ using namespace gw::tc;
 constexpr int kS = kEmuSlices;
 constexpr int kM = kEmuTileM, kN = kEmuTileN / 2;  // a CTA takes half of a tile's columns
 constexpr int kN2 = kEmuTileN;
-constexpr int kChunk = 32;  // reduction elements of a stage (64-byte rows)
+constexpr int kChunk = kEmuBlock;  // reduction elements of a stage (64-byte rows)
 constexpr int kSub = kChunk / kMmaK;
 constexpr int kStages = 2;
 constexpr int kGroup = 4;  // stages of one exact accumulation
@@ -189,25 +189,42 @@ __global__ void __launch_bounds__(256) k_prep_rows(const double* __restrict__ sr
 }
 
 // Rows of a row-major matrix with an exponent per segment of a row: segment i
-// starts at element seg[i] (a multiple of 64) and ends where the next begins.
-// First exps[i * rows + r], a warp per segment of a row.
+// starts at element seg[i] (a multiple of 64) and ends where the next begins; seg
+// null: one segment, of K elements and zeros up to a multiple of 64.  kPairs: 16
+// bytes may be loaded at once (src, ld and the ends are even).  First
+// exps[i * rows + r], a warp per piece of a segment of a row; with several pieces
+// exps holds values below every exponent before.
+constexpr int kSegPiece = 8192;
+template <bool kPairs>
 __global__ void __launch_bounds__(256) k_segment_exps(const double* __restrict__ src, long long ld, long long rows,
-                                                      int K, const long long* __restrict__ seg, int n_seg,
+                                                      int K, const long long* __restrict__ seg, int n_seg, int pieces,
                                                       int* __restrict__ exps) {
   const int lane = threadIdx.x & 31;
-  for (long long i = blockIdx.x * 8LL + threadIdx.x / 32; i < rows * n_seg; i += gridDim.x * 8LL) {
-    const int s = static_cast<int>(i / rows);
-    const long long k0 = seg[s];
-    const int len = static_cast<int>((s + 1 < n_seg ? seg[s + 1] : K) - k0);
-    const double2* x = reinterpret_cast<const double2*>(src + (i - s * rows) * ld + k0);
+  const long long r = blockIdx.x * 8LL + threadIdx.x / 32;
+  if (r >= rows) return;
+  for (int j = blockIdx.y; j < n_seg * pieces; j += gridDim.y) {
+    const int s = pieces == 1 ? j : j / pieces;
+    const long long k0 = seg ? seg[s] : 0;
+    const int end = static_cast<int>((s + 1 < n_seg ? seg[s + 1] : K) - k0);
+    const int from = (j - s * pieces) * kSegPiece, len = min(end - from, kSegPiece);
+    const double* x = src + r * ld + k0 + from;
     int be = 0;
+    if (kPairs) {
 #pragma unroll 4
-    for (int k = lane; k < len / 2; k += 32) {
-      const double2 v = x[k];
-      be = max(be, max(biased_exp(v.x), biased_exp(v.y)));
+      for (int k = lane; k < len / 2; k += 32) {
+        const double2 v = reinterpret_cast<const double2*>(x)[k];
+        be = max(be, max(biased_exp(v.x), biased_exp(v.y)));
+      }
+    } else {
+#pragma unroll 8
+      for (int k = lane; k < len; k += 32) be = max(be, biased_exp(x[k]));
     }
     be = __reduce_max_sync(0xffffffffu, be);
-    if (lane == 0) exps[i] = row_exp(be);
+    if (lane != 0) continue;
+    if (pieces == 1)
+      exps[s * rows + r] = row_exp(be);
+    else
+      atomicMax(exps + s * rows + r, row_exp(be));
   }
 }
 // Then the digits, in blocks of one stage's 32 elements, [block][digit][row][32]: a
@@ -218,11 +235,12 @@ __global__ void __launch_bounds__(256) k_segment_exps(const double* __restrict__
 // some thirty pages: 5.4 ms for both operands with the exponents' pass.  A row's
 // whole segment per CTA, in one pass, wrote to 200 pages and took 7.5 ms.
 constexpr int kSegRows = 16, kSegK = 512;
+template <bool kPairs>
 __global__ void __launch_bounds__(256) k_segment_digits(const double* __restrict__ src, long long ld, long long rows,
                                                         int K, const long long* __restrict__ seg, int n_seg,
                                                         const int* __restrict__ exps, __half* __restrict__ dig) {
   const int s = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long k0 = seg[s];
+  const long long k0 = seg ? seg[s] : 0;
   const int len = static_cast<int>((s + 1 < n_seg ? seg[s + 1] : K) - k0);
   // a warp: 8 rows x one block, four lanes with 8 elements each per row
   const long long r = static_cast<long long>(blockIdx.x) * kSegRows + (warp & 1) * 8 + lane / 4;
@@ -232,18 +250,24 @@ __global__ void __launch_bounds__(256) k_segment_digits(const double* __restrict
   __half* out = dig + (k0 / kChunk * kS * rows + r) * kChunk + lane % 4 * 8;
 #pragma unroll 1
   for (int b = warp / 2; b < kSegK / kChunk; b += 4) {
-    const int k = static_cast<int>(blockIdx.y) * kSegK + b * kChunk;
-    if (k >= len) break;
+    const int block = static_cast<int>(blockIdx.y) * (kSegK / kChunk) + b, k = block * kChunk + lane % 4 * 8;
+    if (block * kChunk >= (len + 63) / 64 * 64) break;
     double v[8];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const double2 w = *reinterpret_cast<const double2*>(x + k + lane % 4 * 8 + 2 * j);
-      v[2 * j] = w.x;
-      v[2 * j + 1] = w.y;
+    for (int j = 0; j < 8; j += 2) {
+      if (kPairs) {
+        double2 w = make_double2(0.0, 0.0);
+        if (k + j < len) w = *reinterpret_cast<const double2*>(x + k + j);
+        v[j] = w.x;
+        v[j + 1] = w.y;
+      } else {
+        v[j] = k + j < len ? x[k + j] : 0.0;
+        v[j + 1] = k + j + 1 < len ? x[k + j + 1] : 0.0;
+      }
     }
     uint4 q[kS];
     digits8(v, e, q);
-    __half* o = out + static_cast<long long>(k / kChunk) * kS * rows * kChunk;
+    __half* o = out + static_cast<long long>(block) * kS * rows * kChunk;
 #pragma unroll
     for (int j = 0; j < kS; ++j) *reinterpret_cast<uint4*>(o + j * rows * kChunk) = q[j];
   }
@@ -507,7 +531,9 @@ struct GemmJob {
   const double *A, *B;
   long long lda, ldb;
   int ta, tb;
-  static constexpr bool kBlocked = false;  // digits in rows of K elements
+  int blocked_a, blocked_b;  // digits in blocks (k_segment_digits), not in rows
+  __device__ bool a_blocked() const { return blocked_a; }
+  __device__ bool b_blocked() const { return blocked_b; }
 
   struct Tile {
     int ya, yb, c0, n;  // rows of the stacked digits
@@ -657,7 +683,8 @@ struct Panel64Job {
   const double *pool, *G;
   const int* lam;
   int nao;
-  static constexpr bool kBlocked = false;
+  __device__ static bool a_blocked() { return false; }
+  __device__ static bool b_blocked() { return false; }
   struct Tile {
     int ya, yb, n, task, a0, b0;
   };
@@ -791,7 +818,8 @@ struct Chi64Job {
   unsigned long long* part;
   const double *X, *Y;
   long long ldk;
-  static constexpr bool kBlocked = true;  // digits as k_segment_digits lays them
+  __device__ static bool a_blocked() { return true; }
+  __device__ static bool b_blocked() { return true; }
   struct Tile {
     int ya, yb, n, id;
     const int* list;  // the piece's entries, and how many the unit has from here on
@@ -1076,13 +1104,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_expect_tx(&full[stage], kStageBytes);
             armed[stage] = true;
             armed_parity[stage] = phase;
-            int x = it.next(), z = 0;
-            if constexpr (Job::kBlocked) {
-              z = x / kChunk * kS;
-              x = 0;
-            }
-            tma_load_3d(st, &map_a, x, T.ya, z, &full[stage]);
-            tma_load_3d(st + kS * kABytes, &map_b, x, T.yb, z, &full[stage]);
+            const int x = it.next(), z = x / kChunk * kS;
+            const bool ba = job.a_blocked(), bb = job.b_blocked();
+            tma_load_3d(st, &map_a, ba ? 0 : x, T.ya, ba ? z : 0, &full[stage]);
+            tma_load_3d(st + kS * kABytes, &map_b, bb ? 0 : x, T.yb, bb ? z : 0, &full[stage]);
             if (++stage == kStages) {
               stage = 0;
               phase ^= 1u;
@@ -1237,6 +1262,14 @@ int launch(const CUtensorMap& ma, const CUtensorMap& mb, const Job& job, int n_i
   return 0;
 }
 
+// tensor map of an operand's tiles of box_rows rows x one stage x all digits
+int operand_map(CUtensorMap* map, const EmuOp& op, int box_rows) {
+  const long long rows = op.s.nz > 1 ? op.stride_rows : op.s.rows;
+  if (op.blocked)
+    return make_digit_map(map, op.dig, kChunk, rows, op.stride_rows, op.kp / kChunk * kS, kChunk, box_rows, kS);
+  return make_digit_map(map, op.dig, op.kp, rows, op.stride_rows, kS, kChunk, box_rows, kS);
+}
+
 // K splits of an m x n product: the number of units that makes the last wave
 // over the 76 pairs of CTAs short.  Costs in stages (about 1.7 us each): a unit's
 // start and end about 3, clearing the partial sums about 3 in all.
@@ -1257,11 +1290,36 @@ int k_splits(long long m, long long n, int K, int nz) {
 
 }  // namespace emu
 
+void launch_emu_prep_segments(EmuOp& op, const EmuSrc& s, const long long* seg, int n_seg, int max_len,
+                              cudaStream_t st) {
+  op.s = s;
+  op.stride_rows = s.rows;
+  op.kp = emu_kp(s.K);
+  op.blocked = true;
+  if (s.rows <= 0 || n_seg <= 0) return;
+  const int pieces = std::max(1, (max_len + emu::kSegPiece - 1) / emu::kSegPiece);
+  const dim3 ge(static_cast<unsigned>((s.rows + 7) / 8), static_cast<unsigned>(std::min(n_seg * pieces, 65535)));
+  if (pieces > 1) cudaMemsetAsync(op.exps, 0x80, static_cast<size_t>(s.rows) * n_seg * sizeof(int), st);
+  const dim3 gd(static_cast<unsigned>((s.rows + emu::kSegRows - 1) / emu::kSegRows),
+                static_cast<unsigned>((emu_kp(max_len) + emu::kSegK - 1) / emu::kSegK), n_seg);
+  __half* dig = static_cast<__half*>(op.dig);
+  if (s.ld % 2 == 0 && s.K % 2 == 0 && reinterpret_cast<uintptr_t>(s.src) % 16 == 0) {
+    emu::k_segment_exps<true><<<ge, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, seg, n_seg, pieces, op.exps);
+    emu::k_segment_digits<true><<<gd, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, seg, n_seg, op.exps, dig);
+  } else {
+    emu::k_segment_exps<false><<<ge, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, seg, n_seg, pieces, op.exps);
+    emu::k_segment_digits<false><<<gd, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, seg, n_seg, op.exps, dig);
+  }
+}
+
 void launch_emu_prep(EmuOp& op, const EmuSrc& s, cudaStream_t st) {
+  // long rows in blocks (a whole row is the one segment)
+  if (!s.trans && s.nz == 1 && s.K >= kEmuBlockedK) return launch_emu_prep_segments(op, s, nullptr, 1, s.K, st);
   op.s = s;
   const long long rows = s.rows * s.nz;
   op.stride_rows = rows;
   op.kp = emu_kp(s.K);
+  op.blocked = false;
   if (rows <= 0) return;
   __half* dig = static_cast<__half*>(op.dig);
   if (!s.trans) {
@@ -1282,21 +1340,6 @@ void launch_emu_prep(EmuOp& op, const EmuSrc& s, cudaStream_t st) {
   }
 }
 
-void launch_emu_prep_segments(EmuOp& op, const EmuSrc& s, const long long* seg, int n_seg, int max_len,
-                              cudaStream_t st) {
-  op.s = s;
-  op.stride_rows = s.rows;
-  op.kp = s.K;
-  if (s.rows <= 0 || n_seg <= 0) return;
-  const long long warps = s.rows * n_seg;
-  emu::k_segment_exps<<<static_cast<unsigned>(std::min<long long>((warps + 7) / 8, 152 * 64)), 256, 0, st>>>(
-      s.src, s.ld, s.rows, s.K, seg, n_seg, op.exps);
-  const dim3 grid(static_cast<unsigned>((s.rows + emu::kSegRows - 1) / emu::kSegRows),
-                  static_cast<unsigned>((max_len + emu::kSegK - 1) / emu::kSegK), n_seg);
-  emu::k_segment_digits<<<grid, 256, 0, st>>>(s.src, s.ld, s.rows, s.K, seg, n_seg, op.exps,
-                                              static_cast<__half*>(op.dig));
-}
-
 // Sums go out as integers and a second kernel rounds them, also where K is not
 // split, as long as they stay in the L2 cache: beside the accumulators there
 // are few registers left for the conversion, which takes 20000 cycles per tile
@@ -1311,10 +1354,7 @@ int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, 
   const int m = static_cast<int>(A.s.rows), n = static_cast<int>(B.s.rows);
   if (m <= 0 || n <= 0) return 0;
   CUtensorMap ma, mb;
-  if (make_digit_map(&ma, A.dig, A.kp, A.s.nz > 1 ? A.stride_rows : A.s.rows, A.stride_rows, kEmuSlices, emu::kChunk, emu::kM, kEmuSlices) ||
-      make_digit_map(&mb, B.dig, B.kp, B.s.nz > 1 ? B.stride_rows : B.s.rows, B.stride_rows, kEmuSlices, emu::kChunk,
-                     emu::kN, kEmuSlices))
-    return -2;
+  if (emu::operand_map(&ma, A, emu::kM) || emu::operand_map(&mb, B, emu::kN)) return -2;
   emu::GemmJob j{};
   j.m = m;
   j.n = n;
@@ -1350,6 +1390,8 @@ int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, 
   j.A = A.s.src;
   j.lda = A.s.ld;
   j.ta = A.s.trans;
+  j.blocked_a = A.blocked;
+  j.blocked_b = B.blocked;
   j.B = B.s.src;
   j.ldb = B.s.ld;
   j.tb = B.s.trans;
@@ -1405,10 +1447,7 @@ int launch_panel64(const Panel64Args& p, int* err_flag, cudaStream_t st) {
 
 int launch_chi64(const EmuOp& x, const EmuOp& y, const Chi64Args& c, int* err_flag, cudaStream_t st) {
   CUtensorMap mx, my;
-  const int planes = x.kp / emu::kChunk * kEmuSlices;
-  if (make_digit_map(&mx, x.dig, emu::kChunk, x.s.rows, x.s.rows, planes, emu::kChunk, emu::kM, kEmuSlices) ||
-      make_digit_map(&my, y.dig, emu::kChunk, y.s.rows, y.s.rows, planes, emu::kChunk, emu::kN, kEmuSlices))
-    return -2;
+  if (emu::operand_map(&mx, x, emu::kM) || emu::operand_map(&my, y, emu::kN)) return -2;
   emu::Chi64Job j{c.units.u_tile, c.units.u_first, c.units.u_count, c.units.n_units, c.tasks, c.counts, c.nslab,
                   c.nqt, c.P0, c.prow, c.nri, c.per, c.slab_k0, c.slab_len, x.exps, y.exps, c.pair, c.chi,
                   static_cast<unsigned long long*>(c.part), x.s.src, y.s.src, x.s.ld};

@@ -14,6 +14,10 @@ constexpr int kEmuSlices = 8;   // digits per operand element
 constexpr int kEmuProducts = 36;  // digit pairs of a product
 constexpr int kEmuTileM = 128;  // rows (A operand) and columns (B operand) of a tile
 constexpr int kEmuTileN = 128;
+constexpr int kEmuBlock = 32;     // reduction elements of a stage
+// Rows of this length and more are kept in blocks: a tile's 1024 rows of digits
+// would lie 128 KB apart.
+constexpr int kEmuBlockedK = 65536;
 
 // A matrix to be used as an operand: rows x K, element (r, k) at
 // src[r * ld + k], or src[k * ld + r] when trans.
@@ -28,7 +32,8 @@ struct EmuSrc {
   long long z_stride = 0;
 };
 // The same as digits: [kEmuSlices][stride_rows][kp] binary16, kp a multiple of
-// 64, zero for k >= K, and per row the power of two above its largest
+// 64, zero for k >= K (blocked: in blocks of kEmuBlock elements of all rows, as
+// k_segment_digits says), and per row the power of two above its largest
 // magnitude.  The FP64 values are read again only for rows that hold an Inf
 // or NaN.
 struct EmuOp {
@@ -36,12 +41,13 @@ struct EmuOp {
   int* exps = nullptr;
   long long stride_rows = 0;
   int kp = 0;
+  bool blocked = false;
   EmuSrc s;
   EmuOp slice_rows(long long r0, long long n) const;  // rows [r0, r0 + n)
 };
 inline EmuOp EmuOp::slice_rows(long long r0, long long n) const {
   EmuOp o = *this;
-  o.dig = static_cast<char*>(dig) + r0 * kp * 2;
+  o.dig = static_cast<char*>(dig) + r0 * (blocked ? kEmuBlock : kp) * 2;
   o.exps = exps + r0;
   o.s.src = s.src + (s.trans ? r0 : r0 * s.ld);
   o.s.rows = n;
@@ -80,9 +86,8 @@ int launch_emu_gemm(const EmuOp& A, const EmuOp& B, const EmuGemm& g, void* ws, 
 
 // The same with an exponent per segment of a row, for step C: segment i starts at
 // element seg[i] of the row (a multiple of 64; in device memory) and is max_len
-// long at most.  s.K and s.ld are multiples of 64, s.src is aligned to 16 bytes;
-// op.exps holds n_seg * s.rows ints, [segment][row]; the digits lie as
-// k_segment_digits says.
+// long at most (seg null: the row is one segment).  s.nz = 1, not s.trans;
+// op.exps holds n_seg * s.rows ints, [segment][row]; the digits lie in blocks.
 void launch_emu_prep_segments(EmuOp& op, const EmuSrc& s, const long long* seg, int n_seg, int max_len,
                               cudaStream_t st);
 

@@ -336,3 +336,24 @@ def test_segments_stay_within_the_operand_budget(pkg):
             got = ctx.chi_tau(case.thr, "fp16x3").cpu().numpy()
             assert ctx.stats()["n_batches"] == batches
             assert np.linalg.norm(got - ref) <= 1e-6 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("nao,nri", [(255, 257), (256, 256), (257, 257)])
+def test_long_rows_of_digits(pkg, nao, nri):
+    """The last product of the AO self-energy at n_AO n_RI = 65535, 65536 and
+    66049: rows of digits, the first length in blocks, an odd one."""
+    from oracle import sigma as osg
+    from paper_2104_09857_gb300 import _lib
+    from synth.chain_inputs import synthetic_w
+
+    n = 17
+    sysm = System("chain", np.array([[1.4 * i, 0.0, 0.0] for i in range(n)]), ["C"] * n)
+    sysm.n_ao = np.array([15] * 16 + [nao - 240], dtype=np.int32)
+    sysm.n_ri = np.array([15] * 16 + [nri - 240], dtype=np.int32)
+    case = case_from_system(sysm, 1, 1e-9, 7)
+    w = synthetic_w(nri, case.tau, 5)
+    ref = osg.sigma_ao_dense(case, w, thr=case.thr)
+    with pkg.Context(0) as ctx:
+        ctx.load_case(case)
+        got = np.asarray(_lib.gw_sigma_ao_tau(ctx.ctx, w, 1, nao, case.thr)).reshape(np.shape(ref))
+    assert np.linalg.norm(got - ref) <= 1e-10 * np.linalg.norm(ref)
