@@ -1173,13 +1173,20 @@ int chi_one_batch_digits(gw_ctx* ctx, const Batch& b, const double* g_occ, const
   gw::launch_build_tasks(fx, fy, nslab, npt, nqt, b.P0, prow, 0, nri, ctx->d_atom_of_ri, d_len, tlist, counts, kacc,
                          tm, tn, per, 0, n_at, 0, nao, ctx->d_atom_of_ao, ctx->stream);
   gw::launch_count_c(bx, by, ns, 0, n_at, pa0, npa, 0, n_at, d_nri, d_nao, b.s0, d_fc, ctx->stream);
-  // Units of about 1/8 of an SM's share, at least 1024 elements (a unit's
-  // atomics cost about as much as 64); with many tiles a unit is a tile.
-  // Partial sums are integers, so either way chi is the same to the last bit,
-  // run after run.
+  // Units of 1/16 of a CTA pair's share of 0.6 of all tiles' reduction elements
+  // (about what the lists keep: the tiles above the diagonal); with many tiles a
+  // unit is a tile.  Step C in ms at 0.3, 0.6 and 2: 6.31, 6.32, 6.80 (40-atom
+  // ribbon), 6.43, 6.25, 6.18 (45-atom cluster), 21.5, 21.1, 21.1 (58-atom ribbon).
+  // At least 1024 elements, for the atomics of a unit; 512 with fewer than 16 tiles,
+  // where the units are a wave or two.  At 512, 1024 and 2048 with nine tiles or
+  // less: 0.078, 0.121, 0.170 (8-atom ring), 0.173, 0.207, 0.177 (12), 0.393, 0.434,
+  // 0.455 (16); with 16 and more: 0.656, 0.603, 0.625 (20-atom ring), 0.642, 0.599,
+  // 0.642 (20-atom ribbon), 1.110, 0.982, 1.065 (24-atom ring); from 28 atoms on the
+  // first line decides.  Partial sums are integers, so chi is the same to the last
+  // bit either way, run after run.
   int split = INT32_MAX;
   if (ntiles < 152 * 16)
-    split = (int)std::min<double>(std::max(1024.0, 0.6 * ntiles * (double)Kb / (152 * 8)), 1 << 30);
+    split = (int)std::min<double>(std::max(ntiles < 16 ? 512.0 : 1024.0, 0.6 * ntiles * (double)Kb / (152 * 8)), 1 << 30);
   void* part;
   int* pair;
   if ((rc = ws(ctx, "d64_part", (size_t)prow * nri * 16, &part)) ||

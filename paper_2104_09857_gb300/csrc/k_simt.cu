@@ -316,6 +316,11 @@ __device__ __forceinline__ void f32_stage(const F32Stage& A, const F32Stage& B, 
 // registers of each thread).  58 atoms, 858 GFLOP: 61 ms in 4 x 4 tiles of one
 // block, 25.8 with one stage of loads in flight, 22.3 with two.  What remains is
 // the latency of those loads (a third of them miss the L2 cache) at 8 warps per SM.
+// Clusters of 1, 2, 4 and 8, ms: 12-atom ring 0.92, 0.57, 0.29, 0.16; ribbons of 20
+// atoms 2.96, 1.56, 0.93, 0.80, of 40 11.9, 9.0, 8.4, 6.5, of 58 37, 34, 21.1, 22.3,
+// of 100 181, 151, 146, 150; 45-atom cluster 13.3, 9.7, 8.9, 7.2.  Eight loses 6 %
+// at most where there are many tiles (shorter parts that end together keep the CTAs
+// on the same slabs), so it is taken at every size.
 constexpr int kF32Split = 8;
 struct F32ChiShared {
   double sum[64][kF32Threads];  // element 8 i + j of each thread
