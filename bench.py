@@ -246,11 +246,17 @@ def alu_peaks():
     return out
 
 
-def _roof(flops, seconds, prec, peaks, peak_src, kernel, traffic, alu=None):
+def _digits(st):
+    """Whether FP64 ran as digit products (36 issued per useful product) and not,
+    for want of memory, on the CUDA cores (one)."""
+    return st["flops_issued"] > 16 * st["flops_useful"]
+
+
+def _roof(flops, seconds, prec, peaks, peak_src, kernel, traffic, alu=None, digits=True):
     """Roofline object of one kernel: achieved = useful flops / its device
     time over the timed region (the same per average launch)."""
     achieved = flops / seconds / 1e12 if seconds > 0 else None
-    if prec in SPLIT_FORMS or prec == "fp64":
+    if prec in SPLIT_FORMS or (prec == "fp64" and digits):
         # binary16 and bf16 share the dense tensor rate (kind::f16); FP64 is 36
         # products of 8-bit digits held in binary16
         peak = peaks["bf16_tflops_sustained"] / N_PRODUCTS[prec]
@@ -259,7 +265,8 @@ def _roof(flops, seconds, prec, peaks, peak_src, kernel, traffic, alu=None):
         bound = "tensor"
     else:
         peak = alu[prec]["tflops"] if alu else None
-        note = "measured FFMA throughput of this GPU (libgwpeaks)" if peak else "not measured"
+        note = (f"measured {'FFMA' if prec == 'fp32' else 'DFMA'} throughput of this GPU "
+                f"(libgwpeaks)") if peak else "not measured"
         bound = "alu"
     return {"kernel": kernel, "bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak if (achieved and peak) else None,
@@ -458,9 +465,9 @@ def run_ours(args):
     traffic = _traffic(prec, {"a": agg["flops_a"], "b": agg["flops_b"], "c": agg["flops_c"],
                               "batches": float(nb)})
     roof_ab = _roof(agg["flops_a"] + agg["flops_b"], agg["ms_step_ab"] / 1e3, prec, peaks, peak_src,
-                    "steps A/B (panel job; time includes the two G gathers)", traffic.get("ab"), alu)
+                    "steps A/B (panel job; time includes the two G gathers)", traffic.get("ab"), alu, _digits(agg))
     roof_c = _roof(agg["flops_c"], agg["ms_step_c_kernel"] / 1e3, prec, peaks, peak_src,
-                   "step C (chi job)", traffic.get("c"), alu)
+                   "step C (chi job)", traffic.get("c"), alu, _digits(agg))
     for r, n_l in ((roof_ab, 2 * nb), (roof_c, nb)):
         r["launches"] = n_l
     if agg["ms_step_ab"] >= agg["ms_step_c_kernel"]:
@@ -528,8 +535,9 @@ def run_ours(args):
             forms[form] = {"ms_per_tau": f_ms, "useful_tflops": st["flops_useful"] / f_ms / 1e9,
                            "rel_frobenius": rel, "rel_element": el,
                            "roofline_step_c": _roof(st["flops_c"], st["ms_step_c_kernel"] / 1e3, form,
-                                                    peaks, peak_src, "step C", None, alu)}
+                                                    peaks, peak_src, "step C", None, alu, _digits(st))}
             if form == "fp64":
+                forms[form]["route"] = "digit products" if _digits(st) else "CUDA cores"
                 forms[form]["speedup_timed_form_over_fp64"] = f_ms / ms_per_tau
         forms["tau_index"] = jm
         forms["sample"] = f"diagonal chi blocks of RI atoms {atoms_m} at tau index {jm}"

@@ -49,7 +49,11 @@ enum gw_status {
  * built in FP64; chi is always accumulated across blocks in FP64. */
 enum gw_precision {
   GW_FP64 = 0,   /* FP64 operands and results: products of 8-bit digits on the
-                    tensor cores, summed exactly as integers, one rounding each    */
+                    tensor cores, summed exactly as integers, one rounding each.
+                    The digits hold 62 bits below the largest magnitude of an
+                    operand's row (step C of Eq. 3: of its part on one
+                    sigma-atom): an element's error is 2^-61 of the product of
+                    the two rows' largest magnitudes, not of the element         */
   GW_FP32 = 1,   /* FP32 operands, FP32 accumulation per block slab (CUDA cores)   */
   GW_BF16X3 = 2, /* two-term BF16 split, 3 products per product, FP32 accumulation
                     on the tensor cores (tcgen05)                                  */
