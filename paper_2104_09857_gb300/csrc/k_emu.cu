@@ -39,7 +39,7 @@
 // Eight-bit digits and not nine: seven nine-bit digits need 28 products but a
 // drain every 32 elements, and the drains' float-to-integer conversions (16
 // per cycle and SM) were then the limit.
-// Measured at 4096^3: 3.2 ms, 43 TFLOP/s (one digit pair per MMA: 4.2 ms;
+// Measured at 4096^3: 3.06 ms, 45 TFLOP/s (one digit pair per MMA: 4.2 ms;
 // without the elected lane and with nine-bit digits: 6.2 ms; the FP64 pipe:
 // 137 ms).
 #include <cuda.h>
