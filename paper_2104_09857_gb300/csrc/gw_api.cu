@@ -963,6 +963,12 @@ int ensure_panel_digits(gw_ctx* ctx) {
   ctx->d_pd_exps = static_cast<int*>(exps);
   ctx->pd_rows = rows;
   ctx->pd_kp = kp;
+  // being made: not to be given back to the allocations below
+  struct Making {
+    gw_ctx* ctx;
+    ~Making() { ctx->pd_in_use = false; }
+  } making{ctx};
+  ctx->pd_in_use = true;
   // panels without rows are left out of the launch
   std::vector<PanelDesc> pd;
   std::vector<long long> row0;

@@ -168,10 +168,6 @@ int chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const double* gamma, con
   }
   return GW_OK;
 }
-
-// S^-1 M S^-1 for n_mat symmetric matrices M (chi~ of Eq. 5, W~ of Eq. 10,
-// V~ of Eq. 11), FP64: S = R R^T (blocked Cholesky), R^-1 by a triangular
-// solve on the identity, S^-1 = R^-T R^-1, then two products per matrix.
 }  // namespace
 
 extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const double* gamma,
@@ -191,6 +187,9 @@ extern "C" int gw_chi_to_w(gw_ctx* ctx, const double* V, int n_omega, const doub
   return rc;
 }
 
+// S^-1 M S^-1 for n_mat symmetric matrices M (chi~ of Eq. 5, W~ of Eq. 10,
+// V~ of Eq. 11), FP64: S = R R^T (blocked Cholesky), R^-1 by a triangular
+// solve on the identity, S^-1 = R^-T R^-1, then two products per matrix.
 extern "C" int gw_ri_metric(gw_ctx* ctx, const double* S, int n_mat, const double* M, int m_on_device,
                             double* out, int out_on_device) {
   if (!ctx) return GW_ERR_INVALID_ARG;
